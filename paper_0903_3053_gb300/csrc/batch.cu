@@ -125,29 +125,29 @@ __device__ void run_ising(const GroupMember &m, int chain, int G, int rank, cons
         if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(lat);
             for (uint32_t u = start; u < units; u += stride)
-                int8_group<0, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                int8_unit<0, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
             group_barrier(G, cluster);
             if (measure)
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_group<1, true, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, true, kLdBatch>(s, ch, ks, u, sweep, anti, up);
             else
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_group<1, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
         } else {
             uint32_t *p0 = reinterpret_cast<uint32_t *>(lat), *p1 = p0 + nw;
             for (uint32_t u = start; u < units; u += stride) {
-                const uint32_t yy = u / ch.W, w = u - yy * ch.W;
+                const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * ch.W;
                 msc_row_pair<0, false, kLdBatch>(p0, p1, yy, w, ch, ks, sweep, anti, up);
             }
             group_barrier(G, cluster);
             if (measure)
                 for (uint32_t u = start; u < units; u += stride) {
-                    const uint32_t yy = u / ch.W, w = u - yy * ch.W;
+                    const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * ch.W;
                     msc_row_pair<1, true, kLdBatch>(p1, p0, yy, w, ch, ks, sweep, anti, up);
                 }
             else
                 for (uint32_t u = start; u < units; u += stride) {
-                    const uint32_t yy = u / ch.W, w = u - yy * ch.W;
+                    const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * ch.W;
                     msc_row_pair<1, false, kLdBatch>(p1, p0, yy, w, ch, ks, sweep, anti, up);
                 }
         }

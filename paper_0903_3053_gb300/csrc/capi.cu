@@ -427,6 +427,7 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
             ch.key = PhiloxKey{(uint32_t)chains[k].seed, (uint32_t)(chains[k].seed >> 32)};
             ch.chain_id = chains[k].chain_id;
             ch.spin_off = p.lat_off[k];
+            ch.div_half = make_fastdiv(ch.Lx / 2);
         }
         e = cudaMemcpyAsync(c->d_chains, c->ising.data(), sizeof(IsingChain) * n_chains, cudaMemcpyHostToDevice,
                             c->stream);

@@ -49,9 +49,9 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
         if (t < groups) {
             const PhiloxSchedule ks = philox_schedule(ch.key);
             if (measure)
-                int8_group<C, true>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, true>(s, ch, ks, t, sweep, anti, up);
             else
-                int8_group<C, false>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, false>(s, ch, ks, t, sweep, anti, up);
         }
     } else {
         const uint32_t W = ch.W, nw = W * ch.Ly;
@@ -88,11 +88,12 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 }
 
 // Two launch-bound flavours of the same half-sweep: blocks of at most 256
-// threads with 8 resident per SM (32 registers: full occupancy also for the
-// measuring colour-1 kernel, +1.7% on the MSC benchmark batch), and blocks of
-// up to 1024 threads for callers that ask for them.
+// threads with 8 resident per SM for the 32-spin words (32 registers: full
+// occupancy also for the measuring colour-1 kernel, +1.7% on the MSC benchmark
+// batch) and 6 for int8 (40 registers, no spills), and blocks of up to 1024
+// threads for callers that ask for them.
 template <int C, int LAYOUT>
-__global__ void __launch_bounds__(256, 8) k_half_sweep(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
+__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 ? 8 : 6) k_half_sweep(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
 template <int C, int LAYOUT>
 __global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
 
@@ -115,11 +116,15 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
     const uint32_t bytes = LAYOUT == MC_LAYOUT_INT8 ? ch.Lx * ch.Ly : 8u * ch.Ly * ch.W;
     uint32_t *gl = reinterpret_cast<uint32_t *>(a.lattice + ch.spin_off);
     uint32_t *sl = reinterpret_cast<uint32_t *>(smem);
+    __shared__ uint32_t sums[2][2];
+    if (threadIdx.x < 4)
+        sums[threadIdx.x >> 1][threadIdx.x & 1] = 0;
     for (uint32_t u = threadIdx.x; u < bytes / 4; u += blockDim.x)
         sl[u] = gl[u];
     __syncthreads();
     const PhiloxSchedule ks = philox_schedule(ch.key);
     const unsigned long long base = a.state->sweep_base;
+    int buf = 0;
     for (uint32_t t = 0; t < n_sweeps; ++t) {
         const uint32_t sweep = (uint32_t)(base + t);
         const bool measure = every != 0 && ((t + 1) % every) == 0;
@@ -128,47 +133,56 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
             int8_t *s = reinterpret_cast<int8_t *>(smem);
             const uint32_t groups = (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
             for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                int8_group<0, false>(s, ch, ks, g, sweep, anti, up);
+                int8_unit<0, false>(s, ch, ks, g, sweep, anti, up);
             __syncthreads();
             if (measure) {
                 for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                    int8_group<1, true>(s, ch, ks, g, sweep, anti, up);
+                    int8_unit<1, true>(s, ch, ks, g, sweep, anti, up);
             } else {
                 for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                    int8_group<1, false>(s, ch, ks, g, sweep, anti, up);
+                    int8_unit<1, false>(s, ch, ks, g, sweep, anti, up);
             }
         } else {
             const uint32_t W = ch.W, nw = W * ch.Ly, pairs = W * (ch.Ly >> 1);
             uint32_t *p0 = sl, *p1 = sl + nw;
             for (uint32_t u = threadIdx.x; u < pairs; u += blockDim.x) {
-                const uint32_t yy = u / W, w = u - yy * W;
+                const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * W;
                 msc_row_pair<0, false>(p0, p1, yy, w, ch, ks, sweep, anti, up);
             }
             __syncthreads();
             if (measure) {
                 for (uint32_t u = threadIdx.x; u < pairs; u += blockDim.x) {
-                    const uint32_t yy = u / W, w = u - yy * W;
+                    const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * W;
                     msc_row_pair<1, true>(p1, p0, yy, w, ch, ks, sweep, anti, up);
                 }
             } else {
                 for (uint32_t u = threadIdx.x; u < pairs; u += blockDim.x) {
-                    const uint32_t yy = u / W, w = u - yy * W;
+                    const uint32_t yy = fast_div(32 * u, ch.div_half), w = u - yy * W;
                     msc_row_pair<1, false>(p1, p0, yy, w, ch, ks, sweep, anti, up);
                 }
             }
         }
+        if (measure) { // the warps add up in the sums' current buffer; no barrier besides the sweep's own
+            anti = __reduce_add_sync(0xffffffffu, anti);
+            up = __reduce_add_sync(0xffffffffu, up);
+            if ((threadIdx.x & 31) == 0) {
+                atomicAdd(&sums[buf][0], anti);
+                atomicAdd(&sums[buf][1], up);
+            }
+        }
+        __syncthreads();
         if (measure) {
-            block_sum2(anti, up);
             if (threadIdx.x == 0) {
                 const unsigned long long r = a.state->rec_head + (t + 1) / every - 1;
                 DevRecord *rec = &a.series[(long long)k * a.cap + (long long)(r % (unsigned long long)a.cap)];
                 rec->sweep = (long long)(base + t);
-                rec->a = anti;
-                rec->b = up;
+                rec->a = sums[buf][0];
+                rec->b = sums[buf][1];
                 rec->d0 = rec->d1 = rec->d2 = 0.0;
+                sums[buf][0] = sums[buf][1] = 0; // next added to two measurements later, past further barriers
             }
+            buf ^= 1;
         }
-        __syncthreads();
     }
     for (uint32_t u = threadIdx.x; u < bytes / 4; u += blockDim.x)
         gl[u] = sl[u];

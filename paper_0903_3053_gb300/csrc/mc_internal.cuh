@@ -32,6 +32,7 @@ struct IsingChain {
     uint32_t pad0;
     uint64_t spin_off;  // byte offset of the chain's spins in the lattice region
     double beta;        // coupling (the Metropolis-Hastings step of the learned proposal needs it)
+    FastDiv div_half;   // by Lx / 2: colour-linear site index -> row
 };
 
 // Per-chain descriptor of a 4D SU(2) chain.

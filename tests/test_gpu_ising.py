@@ -105,6 +105,32 @@ def test_ragged_and_degenerate_shapes(layout, shape, mode):
     np.testing.assert_array_equal(series["M"][0], M[4::5])
 
 
+@pytest.mark.parametrize("shape", [(8, 2), (8, 8), (24, 2), (40, 6), (16, 130), (520, 14)])
+@pytest.mark.parametrize("beta", [0.0, 0.35, 3.0, 6.0])
+@pytest.mark.parametrize("launch", ["grid", "resident", "group"])
+def test_int8_rows_of_whole_groups(shape, beta, launch):
+    """Rows of whole Philox groups (Lx % 8 == 0) are updated four sites at a time:
+    one group per row (both in-row neighbours wrap), two rows (both vertical
+    neighbours are one row), group counts that leave the last warp ragged, and
+    thresholds at 2^32 - 1 (beta = 0) and 0 (beta = 3: dE = 8 only; 6: both)."""
+    s = oracle.ising_init(shape, seed=21, chain=3, hot=True)
+    E, M = oracle.ising_run(s, beta, 21, 3, 0, 9)
+    b = mc.Batch([mc.ising(shape, beta, seed=21, chain_id=3)], layout=mc.MC_LAYOUT_INT8, series_capacity=9)
+    if launch == "group":
+        g = mc.Group([b])
+        g.configure(2, 64, 0.0)  # one chain shared by two CTAs
+        g.sweep(9, 1)
+        g.close()
+    else:
+        b.set_mode(mc.MC_MODE_GRID if launch == "grid" else mc.MC_MODE_RESIDENT)
+        b.sweep(9, 1)
+    rec = b.read_series()
+    np.testing.assert_array_equal(b.get_config(0), s)
+    np.testing.assert_array_equal(rec["E"][0], E)
+    np.testing.assert_array_equal(rec["M"][0], M)
+    b.close()
+
+
 @pytest.mark.parametrize("threads", [32, 64, 128, 512, 1024])
 def test_block_size_invariance(threads):
     chains = [mc.ising((256, 128), 0.44, seed=3, chain_id=0)]
