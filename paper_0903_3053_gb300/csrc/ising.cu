@@ -58,13 +58,15 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
         uint32_t *base = reinterpret_cast<uint32_t *>(a.lattice + ch.spin_off);
         uint32_t *pc = base + (size_t)C * nw;
         const uint32_t *po = base + (size_t)(1 - C) * nw;
-        if (t < W * (ch.Ly >> 1)) { // one thread per row pair and word column
+        const uint32_t np = ch.Ly >> 1, nt = (np + a.row_pairs - 1) / a.row_pairs;
+        if (t < W * nt) { // one thread per word column and a.row_pairs row pairs
             const PhiloxSchedule ks = philox_schedule(ch.key);
-            const uint32_t yy = t / W, w = t - yy * W;
+            const uint32_t q = fast_div(32 * t, ch.div_half), w = t - q * W; // t / W: half a row is 32 W sites
+            const uint32_t yy0 = q * a.row_pairs, yy1 = min(np, yy0 + a.row_pairs);
             if (measure)
-                msc_row_pair<C, true>(pc, po, yy, w, ch, ks, sweep, anti, up);
+                msc_row_pairs<C, true>(pc, po, yy0, yy1, w, ch, ks, sweep, anti, up);
             else
-                msc_row_pair<C, false>(pc, po, yy, w, ch, ks, sweep, anti, up);
+                msc_row_pairs<C, false>(pc, po, yy0, yy1, w, ch, ks, sweep, anti, up);
         }
     }
     if (!a.measure)
@@ -88,12 +90,13 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 }
 
 // Two launch-bound flavours of the same half-sweep: blocks of at most 256
-// threads with 8 resident per SM for the 32-spin words (32 registers: full
-// occupancy also for the measuring colour-1 kernel, +1.7% on the MSC benchmark
-// batch) and 6 for int8 (40 registers, no spills), and blocks of up to 1024
-// threads for callers that ask for them.
+// threads with 4 resident per SM for the 32-spin words (64 registers, so that the
+// Philox key schedule stays in registers; the kernel is bound by the schedulers'
+// dispatch, which 32 warps per SM keep busy: a 32768^2 chain 730 us per sweep
+// against 757 with 8 blocks and 32 registers) and 6 for int8 (40 registers, no
+// spills), and blocks of up to 1024 threads for callers that ask for them.
 template <int C, int LAYOUT>
-__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 ? 8 : 6) k_half_sweep(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
+__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 ? 4 : 6) k_half_sweep(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
 template <int C, int LAYOUT>
 __global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
 
@@ -391,11 +394,29 @@ static uint32_t grid_units(const mc_ctx *c, const IsingChain &ch)
 {
     if (c->layout == MC_LAYOUT_INT8)
         return (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
-    return (ch.Ly >> 1) * ch.W; // row pairs x words
+    return ((ch.Ly >> 1) + c->row_pairs - 1) / c->row_pairs * ch.W; // runs of row pairs x words
 }
+
+// 32-spin words, row pairs per thread: more of them spread a thread's prologue
+// (chain lookup, descriptor, indices, key schedule) over more words and load each
+// neighbour row once, fewer keep the last wave of blocks even.  As many, up to 8,
+// as leave 2^18 threads (1.7 full waves of 1024 threads on 152 SMs).  Measured us
+// per measured sweep with 1 / 2 / 4 / 8 row pairs: one 4096^2 chain (131072 row
+// pairs) 18.2 / 20.0 / - / -, one 8192^2 or four 4096^2 chains (524288) 54.6 / 52.3 / 57.7 /
+// 58.8, one 16384^2 chain (2097152) 199.5 / - / - / 189.2.
+constexpr uint64_t kRowPairThreads = 1u << 18;
+constexpr int kMaxRowPairs = 8;
 
 void ising_plan_grid(mc_ctx *c)
 {
+    c->row_pairs = 1;
+    if (c->layout == MC_LAYOUT_MSC32) {
+        uint64_t pairs = 0;
+        for (const auto &ch : c->ising)
+            pairs += (uint64_t)ch.W * (ch.Ly >> 1);
+        while (c->row_pairs < kMaxRowPairs && pairs / (2 * c->row_pairs) >= kRowPairThreads)
+            c->row_pairs *= 2;
+    }
     c->block_start.assign(c->n_chains + 1, 0);
     uint32_t acc = 0;
     for (int k = 0; k < c->n_chains; ++k) {
@@ -500,6 +521,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     a.state = c->d_state;
     a.cap = c->cap;
     a.tries = nullptr;
+    a.row_pairs = (uint32_t)c->row_pairs;
     if (mode == MC_MODE_RESIDENT) {
         int smem = 0;
         if (!ising_resident_fits(c, &smem))

@@ -175,20 +175,23 @@ __device__ __forceinline__ void int8_unit(int8_t *s, const IsingChain &ch, const
 // Philox block is drawn (a per-block skip branch costs more than it saves).
 // Every site is compared with both thresholds, as two carry chains that build
 // the masks g2 = (r >= T2) and g4 = (r >= T4) with site b at bit b (sites are
-// visited from 31 down to 0); a site with one anti-aligned neighbour (dE = 4)
-// flips iff r < T2, one with none (dE = 8) iff r < T4, and since T4 <= T2
-// the flip mask is ge2 | ~g4 | (eq1 & ~g2).  (A per-site select of the
-// threshold followed by one compare measured 12% slower.)
+// visited from 31 down to 0).  A site with two or more anti-aligned neighbours
+// flips, one with one (dE = 4) iff r < T2, one with none (dE = 8) iff r < T4;
+// since T4 <= T2, r < T4 flips in every case.  (A per-site select of the
+// threshold followed by one compare measured 12% slower; predicates in place
+// of the carry chains 20% slower: an integer add takes one dispatch cycle of a
+// scheduler, a compare, logic or multiply instruction two.)  Bound by that dispatch:
+// a 4-site Philox block is 17 wide multiplies and 19 three-input xors, 72 cycles
+// per warp, its compares 16 more; 103 cycles measured (110 with a thread per row
+// pair and the neighbour count as half adders): 1.365e12 -> 1.47e12 flips/s on a
+// 32768^2 chain.
 template <int C>
 __device__ __forceinline__ uint32_t msc_word(uint32_t s, uint32_t nu, uint32_t nd, uint32_t ns, uint32_t side,
                                              uint32_t blk0, uint32_t sweep, const IsingChain &ch,
                                              const PhiloxSchedule &ks)
 {
     const uint32_t a1 = s ^ nu, a2 = s ^ nd, a3 = s ^ ns, a4 = s ^ side; // 1 = anti-aligned
-    const uint32_t s12 = a1 ^ a2, c12 = a1 & a2, s34 = a3 ^ a4, c34 = a3 & a4;
-    const uint32_t ge2 = c12 | c34 | (s12 & s34); // >= 2 anti-aligned: dE <= 0, always flip
-    const uint32_t eq0 = ~(a1 | a2 | a3 | a4);    // dE = 8
-    const uint32_t eq1 = ~(ge2 | eq0);            // dE = 4
+    const uint32_t x = a1 ^ a2 ^ a3, m = (a1 & a2) | (a3 & (a1 | a2)); // 2 m + x = a1 + a2 + a3
     const uint32_t nT2 = 0u - ch.T2, nT4 = 0u - ch.T4;
     uint32_t g2 = 0, g4 = 0;
 #pragma unroll
@@ -203,44 +206,63 @@ __device__ __forceinline__ uint32_t msc_word(uint32_t s, uint32_t nu, uint32_t n
         g2 = ~0u;
     if (ch.T4 == 0)
         g4 = ~0u;
-    return s ^ (ge2 | ~g4 | (eq1 & ~g2));
+    return s ^ ((x & a4) | m | ~g4 | ((x ^ a4) & ~g2));
 }
 
-// Update words (2 yy, w) and (2 yy + 1, w) of plane C.  The two rows share the
-// other plane's rows 2 yy and 2 yy + 1 as neighbours, so six loads serve both
-// words.  Row y holds sites x = 2 j + ((y + C) & 1): offset C on the even row,
-// 1 - C on the odd one, which decides the side (j - 1 or j + 1) neighbour.
+// Update words (y, w) of plane C for the row pairs y = 2 yy, 2 yy + 1 with yy0 <=
+// yy < yy1.  The two rows of a pair share the other plane's rows 2 yy and 2 yy +
+// 1 as neighbours and the next pair shares rows 2 yy + 1 and 2 yy + 2, so each row
+// of the other plane is loaded once.  Row y holds sites x = 2 j + ((y + C) & 1):
+// offset C on the even row, 1 - C on the odd one, which decides the side (j - 1
+// or j + 1) neighbour.
+template <int C, bool MEASURE, int LD = kLdPlain>
+__device__ __forceinline__ void msc_row_pairs(uint32_t *pc, const uint32_t *po, uint32_t yy0, uint32_t yy1, uint32_t w,
+                                              const IsingChain &ch, const PhiloxSchedule &ks, uint32_t sweep,
+                                              uint32_t &anti, uint32_t &up)
+{
+    const uint32_t W = ch.W, Ly = ch.Ly, bpr = ch.Lx >> 3; // bpr: Philox blocks per row of one colour
+    const uint32_t wl = dec_wrap(w, W), wr = inc_wrap(w, W);
+    uint32_t y0 = 2 * yy0, r0 = y0 * W, blk = y0 * bpr + 8 * w;
+    uint32_t om = lat_load<LD>(&po[dec_wrap(y0, Ly) * W + w]), o0 = lat_load<LD>(&po[r0 + w]);
+#pragma unroll 1
+    for (uint32_t yy = yy0; yy < yy1; ++yy) {
+        const uint32_t r1 = r0 + W, r2 = y0 + 2 == Ly ? 0u : r1 + W;
+        const uint32_t o1 = lat_load<LD>(&po[r1 + w]), op = lat_load<LD>(&po[r2 + w]);
+        uint32_t side0, side1;
+        if (C == 0) {
+            side0 = (o0 << 1) | (lat_load<LD>(&po[r0 + wl]) >> 31);
+            side1 = (o1 >> 1) | (lat_load<LD>(&po[r1 + wr]) << 31);
+        } else {
+            side0 = (o0 >> 1) | (lat_load<LD>(&po[r0 + wr]) << 31);
+            side1 = (o1 << 1) | (lat_load<LD>(&po[r1 + wl]) >> 31);
+        }
+        const uint32_t s0 = lat_load<LD>(&pc[r0 + w]), s1 = lat_load<LD>(&pc[r1 + w]);
+        const uint32_t n0 = msc_word<C>(s0, om, o1, o0, side0, blk, sweep, ch, ks);
+        const uint32_t n1 = msc_word<C>(s1, o0, op, o1, side1, blk + bpr, sweep, ch, ks);
+        if (n0 != s0)
+            pc[r0 + w] = n0;
+        if (n1 != s1)
+            pc[r1 + w] = n1;
+        if (MEASURE) {
+            anti += __popc(n0 ^ om) + __popc(n0 ^ o1) + __popc(n0 ^ o0) + __popc(n0 ^ side0) + __popc(n1 ^ o0) +
+                    __popc(n1 ^ op) + __popc(n1 ^ o1) + __popc(n1 ^ side1);
+            up += __popc(n0) + __popc(o0) + __popc(n1) + __popc(o1);
+        }
+        om = o1;
+        o0 = op;
+        y0 += 2;
+        r0 += 2 * W;
+        blk += 2 * bpr;
+    }
+}
+
+// One row pair.
 template <int C, bool MEASURE, int LD = kLdPlain>
 __device__ __forceinline__ void msc_row_pair(uint32_t *pc, const uint32_t *po, uint32_t yy, uint32_t w,
                                              const IsingChain &ch, const PhiloxSchedule &ks, uint32_t sweep,
                                              uint32_t &anti, uint32_t &up)
 {
-    const uint32_t W = ch.W, Ly = ch.Ly, y0 = 2 * yy, y1 = y0 + 1;
-    const uint32_t om = lat_load<LD>(&po[dec_wrap(y0, Ly) * W + w]);
-    const uint32_t o0 = lat_load<LD>(&po[y0 * W + w]);
-    const uint32_t o1 = lat_load<LD>(&po[y1 * W + w]);
-    const uint32_t op = lat_load<LD>(&po[inc_wrap(y1, Ly) * W + w]);
-    uint32_t side0, side1;
-    if (C == 0) {
-        side0 = (o0 << 1) | (lat_load<LD>(&po[y0 * W + dec_wrap(w, W)]) >> 31);
-        side1 = (o1 >> 1) | (lat_load<LD>(&po[y1 * W + inc_wrap(w, W)]) << 31);
-    } else {
-        side0 = (o0 >> 1) | (lat_load<LD>(&po[y0 * W + inc_wrap(w, W)]) << 31);
-        side1 = (o1 << 1) | (lat_load<LD>(&po[y1 * W + dec_wrap(w, W)]) >> 31);
-    }
-    const uint32_t s0 = lat_load<LD>(&pc[y0 * W + w]), s1 = lat_load<LD>(&pc[y1 * W + w]);
-    const uint32_t bpr = ch.Lx >> 3; // Philox blocks per row of one colour
-    const uint32_t n0 = msc_word<C>(s0, om, o1, o0, side0, y0 * bpr + 8 * w, sweep, ch, ks);
-    const uint32_t n1 = msc_word<C>(s1, o0, op, o1, side1, y1 * bpr + 8 * w, sweep, ch, ks);
-    if (n0 != s0)
-        pc[y0 * W + w] = n0;
-    if (n1 != s1)
-        pc[y1 * W + w] = n1;
-    if (MEASURE) {
-        anti += __popc(n0 ^ om) + __popc(n0 ^ o1) + __popc(n0 ^ o0) + __popc(n0 ^ side0) + __popc(n1 ^ o0) +
-                __popc(n1 ^ op) + __popc(n1 ^ o1) + __popc(n1 ^ side1);
-        up += __popc(n0) + __popc(o0) + __popc(n1) + __popc(o1);
-    }
+    msc_row_pairs<C, MEASURE, LD>(pc, po, yy, yy + 1, w, ch, ks, sweep, anti, up);
 }
 
 // Gather the neighbours of word (y, w) of plane C from the other plane `po`.

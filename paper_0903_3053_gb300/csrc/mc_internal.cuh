@@ -133,6 +133,7 @@ struct SweepArgs {
     uint32_t rec_k;              // index of this record within the running call
     uint8_t *tries;              // SU(2) try record base, or nullptr
     uint32_t block_base;         // first block of this launch in the block table
+    uint32_t row_pairs;          // MSC32 grid mode: row pairs per thread
 };
 
 }  // namespace mc
@@ -171,6 +172,7 @@ struct mc_ctx {
     std::vector<uint32_t> block_start, meas_start;
     std::vector<std::pair<int, int>> groups; // SU(2) launch groups of chains [first, last)
     uint32_t grid_blocks = 0, meas_blocks = 0;
+    int row_pairs = 1;                   // MSC32 grid mode: row pairs per thread
     // run bookkeeping
     long long sweeps_done = 0;
     long long rec_written = 0, rec_read = 0;
