@@ -165,10 +165,6 @@ __device__ void run_ising(const GroupMember &m, int chain, int G, int rank, cons
 // SU(2) measurement in the batch kernel: one x1 pair of sites per thread step
 // (su2_pair_plaquettes, 29 link loads per pair) measured 0.451 against 0.459 ms
 // per measured sweep of the batched workload for one site per step.
-#ifndef MC_GROUP_PAIR_PLAQ
-#define MC_GROUP_PAIR_PLAQ 1
-#endif
-
 __device__ void run_su2(const GroupMember &m, int chain, int item, int G, int rank, const GroupArgs &g,
                         cg::cluster_group &cluster)
 {
@@ -193,13 +189,8 @@ __device__ void run_su2(const GroupMember &m, int chain, int item, int G, int ra
             }
         if (g.every != 0 && ((t + 1) % g.every) == 0) {
             long long ps = 0, pt = 0;
-#if MC_GROUP_PAIR_PLAQ
             for (uint32_t j = start; j < ch.nh; j += stride) // one x1 pair of sites per step
                 su2_pair_plaquettes<kLdBatch>(U, ch, j, ps, pt);
-#else
-            for (uint32_t s = start; s < 2 * ch.nh; s += stride)
-                su2_site_plaquettes<kLdBatch>(U, ch, s, ps, pt);
-#endif
             block_sum2ll(ps, pt);
             if (threadIdx.x == 0) {
                 part[2 * rank] = ps;

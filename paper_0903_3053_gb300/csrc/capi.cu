@@ -118,7 +118,7 @@ bool validate(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t ca
 
 struct Plan {
     size_t state, chains, block_start, meas_start, series, scratch_rec, partials, staging, tries, lattice, total;
-    size_t partial_count, staging_bytes;
+    size_t staging_bytes;
     std::vector<size_t> lat_off, tries_off;
 };
 
@@ -152,12 +152,10 @@ Plan make_plan(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t c
         } else {
             const size_t sites = (size_t)d.L[0] * d.L[1] * d.L[2] * d.L[3];
             staging = std::max(staging, sites * 4 * 16);
-            // >= kSu2ResidentMaxCluster blocks: the resident mode keeps one partial pair per CTA of a chain
-            meas_blocks += std::max<size_t>((sites / 2 + kPlaqThreads - 1) / kPlaqThreads, kSu2ResidentMaxCluster);
+            meas_blocks += (sites / 2 + kPlaqThreads - 1) / kPlaqThreads;
         }
     }
-    p.partial_count = 2 * meas_blocks;
-    p.partials = take(p.partial_count * sizeof(long long));
+    p.partials = take(2 * meas_blocks * sizeof(long long)); // Polyakov loop: at most one per 256 spatial sites
     p.staging_bytes = staging;
     p.staging = take(staging);
     p.tries_off.assign(n, 0);
@@ -225,9 +223,10 @@ int resolve_mode(mc_ctx *c)
     if (c->kind == MC_KIND_SU2) {
         if (c->record_tries) // the per-link try record is kept by the grid kernels only
             return MC_MODE_GRID;
-        if (c->mode != MC_MODE_AUTO)
-            return c->mode;
-        return su2_resident_auto(c) ? MC_MODE_RESIDENT : MC_MODE_GRID;
+        // Automatic: always the chained phase launches.  The single-launch mode, whose phases are separated by
+        // cluster barriers, is slower from 2^4 (22 against 15 us per measured sweep) over 8^4 (28 against 16; 64
+        // chains 274 against 52) up; it remains for callers that want one launch per call.
+        return c->mode == MC_MODE_RESIDENT ? MC_MODE_RESIDENT : MC_MODE_GRID;
     }
     if (c->mode != MC_MODE_AUTO)
         return c->mode;
@@ -408,7 +407,6 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
     c->d_series = reinterpret_cast<DevRecord *>(c->ws + p.series);
     c->d_scratch_rec = reinterpret_cast<DevRecord *>(c->ws + p.scratch_rec);
     c->d_partials = reinterpret_cast<long long *>(c->ws + p.partials);
-    c->partial_count = p.partial_count;
     c->d_staging = c->ws + p.staging;
     c->staging_bytes = p.staging_bytes;
     c->d_tries = reinterpret_cast<uint8_t *>(c->ws + p.tries);
@@ -448,6 +446,10 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
             ch.div1 = make_fastdiv((uint32_t)ch.L[1]);
             ch.div2 = make_fastdiv((uint32_t)ch.L[2]);
             ch.div3 = make_fastdiv((uint32_t)ch.L[3]);
+            ch.step2 = 8u * (uint32_t)ch.L[1];
+            ch.step3 = ch.step2 * (uint32_t)ch.L[2];
+            ch.step0 = ch.step3 * (uint32_t)ch.L[3];
+            ch.bytes = ch.step0 * (uint32_t)ch.L[0];
         }
         e = cudaMemcpyAsync(c->d_chains, c->su2.data(), sizeof(Su2Chain) * n_chains, cudaMemcpyHostToDevice,
                             c->stream);

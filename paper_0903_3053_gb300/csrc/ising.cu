@@ -43,6 +43,7 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
     const uint32_t sweep = (uint32_t)(a.state->sweep_base + a.k);
     const bool measure = (C == 1) && a.measure;
     uint32_t anti = 0, up = 0;
+    chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between calls)
     if (LAYOUT == MC_LAYOUT_INT8) {
         int8_t *s = reinterpret_cast<int8_t *>(a.lattice + ch.spin_off);
         const uint32_t groups = (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
@@ -103,10 +104,8 @@ __global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a) { half_swe
 template <int C, int LAYOUT>
 void launch_half_sweep(mc_ctx *c, const SweepArgs &a)
 {
-    if (c->threads <= 256)
-        k_half_sweep<C, LAYOUT><<<c->grid_blocks, c->threads, 0, c->ls>>>(a);
-    else
-        k_half_sweep_big<C, LAYOUT><<<c->grid_blocks, c->threads, 0, c->ls>>>(a);
+    launch_chained(c, c->threads <= 256 ? k_half_sweep<C, LAYOUT> : k_half_sweep_big<C, LAYOUT>, c->grid_blocks,
+                   (unsigned)c->threads, a);
 }
 
 // ------------------------------------------------------------------ resident mode
@@ -522,6 +521,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     a.cap = c->cap;
     a.tries = nullptr;
     a.row_pairs = (uint32_t)c->row_pairs;
+    a.release = 1;
     if (mode == MC_MODE_RESIDENT) {
         int smem = 0;
         if (!ising_resident_fits(c, &smem))

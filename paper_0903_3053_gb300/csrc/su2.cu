@@ -35,58 +35,111 @@
 namespace mc {
 namespace {
 
-// 256 threads, at least 6 blocks per SM (40 registers; ptxas spills 12-48
-// bytes per thread, about 1% of the kernel's load requests): the phase is bound
-// by the latency of the 18 neighbour-link loads, and 48 resident warps hide it
-// better than the 40 an unconstrained build allows (+14% measured on 4 x 32^4).
-template <int P, int MU, bool REC>
-__global__ void __launch_bounds__(256, 6) k_phase(SweepArgs a)
+// Chain descriptors of small batches as kernel parameters: the block's chain is
+// found by comparisons with parameters, and the extents, steps, divisors and keys
+// come from the constant bank instead of a binary search and some twenty dependent
+// loads per thread: 16 against 20 us per measured sweep of 16 chains of 4^4, 55 against
+// 61 for one 4 x 24^3 chain with overrelaxation; no difference where the launch is long
+// (4 x 32^4).  Larger batches look the chain up in memory.
+constexpr int kTableChains = 16;
+struct ChainTable {
+    uint32_t start[kTableChains]; // first block of each chain (2^32 - 1 past the last)
+    Su2Chain ch[kTableChains];
+};
+struct NoTable {
+};
+
+__device__ __forceinline__ const Su2Chain &block_chain(const SweepArgs &, const ChainTable &tab, uint32_t b, int &k, uint32_t &b0)
 {
-    const uint32_t b = blockIdx.x + a.block_base;
-    const int k = find_chain(a.block_start, a.n_chains, b);
-    const Su2Chain ch = static_cast<const Su2Chain *>(a.chains)[k];
-    const uint32_t e = (b - a.block_start[k]) * blockDim.x + threadIdx.x;
+    k = 0;
+#pragma unroll
+    for (int i = 1; i < kTableChains; ++i)
+        k += b >= tab.start[i] ? 1 : 0;
+    b0 = tab.start[k];
+    return tab.ch[k];
+}
+__device__ __forceinline__ Su2Chain block_chain(const SweepArgs &a, const NoTable &, uint32_t b, int &k, uint32_t &b0)
+{
+    k = find_chain(a.block_start, a.n_chains, b);
+    b0 = a.block_start[k];
+    return static_cast<const Su2Chain *>(a.chains)[k];
+}
+
+// The record of this launch's sweep of chain k.
+__device__ __forceinline__ DevRecord *sweep_record(const SweepArgs &a, int k)
+{
+    const unsigned long long slot = (a.state->rec_head + a.rec_k) % (unsigned long long)a.cap;
+    return &a.series[(long long)k * a.cap + (long long)slot];
+}
+
+// Blocks of up to 256 threads, MINB per SM.  The 18 neighbour links of an update
+// are in flight together only when the registers hold them: 64 registers (MINB =
+// 4, 32 warps per SM) take 503 us per heat-bath sweep of 4 x 32^4 against 528 with
+// 40 registers and 48 warps, and a launch whose blocks are all resident with 85
+// (MINB = 3) is shorter still: 8^4 13.5 against 15.1 us per sweep (20.3 with 40
+// registers), 20 x 24 x 20 x 24 31.8 against 35.4, but 522 us for 4 x 32^4.  Bound by
+// the schedulers' dispatch (~1150 cycles per warp and link: FP32 420, Philox 220,
+// the divergent retries 20%) with the DRAM traffic of a 256 MiB lattice at 60% of
+// its floor; launch and link-load latency on small lattices.
+template <int P, int MU, bool REC, int MINB, typename TAB>
+__global__ void __launch_bounds__(256, MINB) k_phase(const __grid_constant__ SweepArgs a, const __grid_constant__ TAB tab)
+{
+    int k;
+    uint32_t b0;
+    const auto &ch = block_chain(a, tab, blockIdx.x, k, b0);
+    const uint32_t e = (blockIdx.x - b0) * blockDim.x + threadIdx.x;
     if (e >= ch.nh)
         return;
     float4 *U = reinterpret_cast<float4 *>(a.lattice + ch.link_off);
     const PhiloxSchedule ks = philox_schedule(ch.key);
-    su2_update_link<P, MU, kLdReadOnly, REC>(U, ch, ks, e, (uint32_t)(a.state->sweep_base + a.k), a.tries, a.state);
+    su2_update_link<P, MU, kLdPlain, REC, false, 3, true>(U, ch, ks, e, (uint32_t)(a.state->sweep_base + a.k), a.tries,
+                                                          a.state, a.release != 0);
+    if (P == 1 && MU == 0 && a.measure && e == 0) { // the plaquette kernel of this sweep adds into the record
+        DevRecord *rec = sweep_record(a, k);
+        rec->sweep = (long long)(a.state->sweep_base + a.k);
+        rec->a = rec->b = 0;
+        rec->d0 = rec->d1 = rec->d2 = 0.0;
+    }
 }
 
-// Overrelaxation phase: same thread layout as k_phase, no random numbers.
-template <int P, int MU>
-__global__ void __launch_bounds__(256, 6) k_or_phase(SweepArgs a)
+// Overrelaxation phase: same thread layout as k_phase, no random numbers; 4 blocks
+// per SM for the same reason (52 against 55 us per phase of 4 x 32^4, 1.6 against 2.2
+// of 8^4 with 40 registers).
+template <int P, int MU, typename TAB>
+__global__ void __launch_bounds__(256, 4) k_or_phase(const __grid_constant__ SweepArgs a, const __grid_constant__ TAB tab)
 {
-    const uint32_t b = blockIdx.x + a.block_base;
-    const int k = find_chain(a.block_start, a.n_chains, b);
-    const Su2Chain ch = static_cast<const Su2Chain *>(a.chains)[k];
-    const uint32_t e = (b - a.block_start[k]) * blockDim.x + threadIdx.x;
+    int k;
+    uint32_t b0;
+    const auto &ch = block_chain(a, tab, blockIdx.x, k, b0);
+    const uint32_t e = (blockIdx.x - b0) * blockDim.x + threadIdx.x;
     if (e >= ch.nh)
         return;
     float4 *U = reinterpret_cast<float4 *>(a.lattice + ch.link_off);
-    su2_overrelax_link<P, MU, kLdReadOnly>(U, ch, e);
+    su2_overrelax_link<P, MU, kLdPlain, true>(U, ch, e, a.release != 0);
 }
 
 // ------------------------------------------------------------------ plaquette
-// Per-block partial sums of (1/2) Tr U_munu(x) of Eq. (3), spatial and temporal
-// separately (the two values per measuring thread of Sec. 2.4).  One thread per
-// x1 pair of sites (su2_pair_plaquettes), kPlaqThreads pairs per block, at
-// least 8 blocks per SM: 74 us instead of 96 us for one site per thread on
-// 4 x 32^4, where the kernel is bound by the latency of its link loads.
-// Products in FP32, sums in exact int64 fixed point (plaq_fixed);
-// partial[2 b], partial[2 b + 1].
-__global__ void __launch_bounds__(kPlaqThreads, 8) k_plaquette(const Su2Chain *chains, const uint32_t *meas_start,
-                                                               int n_chains, const char *lattice, long long *partial,
-                                                               uint32_t block_base)
+// Sums of (1/2) Tr U_munu(x) of Eq. (3), spatial and temporal separately (the two
+// values per measuring thread of Sec. 2.4).  One thread per x1 pair of sites
+// (su2_pair_plaquettes), kPlaqThreads pairs per block, at least 6 blocks per SM (80
+// registers for the 29 links in flight: 74 us per measurement of 4 x 32^4, 78 with 8
+// or 5 blocks, 85 with 4; 96 us for one site per thread): bound by the latency of
+// its link loads.  Products in FP32, sums in exact int64
+// fixed point (plaq_fixed), so that the blocks add them straight into the
+// chain's record in any order.  The record (zeroed by the sweep's first phase) is the
+// sweep's, or `out` for chain `only` (zeroed by the caller).
+__global__ void __launch_bounds__(kPlaqThreads, 6) k_plaquette(const __grid_constant__ SweepArgs a,
+                                                               const uint32_t *meas_start, int only, DevRecord *out)
 {
     __shared__ long long ss[kPlaqThreads / 32], st[kPlaqThreads / 32];
-    const uint32_t blk = blockIdx.x + block_base;
-    const int k = find_chain(meas_start, n_chains, blk);
-    const Su2Chain ch = chains[k];
+    const uint32_t blk = only >= 0 ? meas_start[only] + blockIdx.x : blockIdx.x;
+    const int k = only >= 0 ? only : find_chain(meas_start, a.n_chains, blk);
+    const Su2Chain ch = static_cast<const Su2Chain *>(a.chains)[k];
     const uint32_t j = (blk - meas_start[k]) * kPlaqThreads + threadIdx.x;
     long long ps = 0, pt = 0;
+    chain_wait(a.release != 0);
     if (j < ch.nh)
-        su2_pair_plaquettes<kLdReadOnly>(reinterpret_cast<const float4 *>(lattice + ch.link_off), ch, j, ps, pt);
+        su2_pair_plaquettes<kLdPlain>(reinterpret_cast<const float4 *>(a.lattice + ch.link_off), ch, j, ps, pt);
     ps = warp_sum_ll(ps);
     pt = warp_sum_ll(pt);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -96,58 +149,15 @@ __global__ void __launch_bounds__(kPlaqThreads, 8) k_plaquette(const Su2Chain *c
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long a = 0, b = 0;
+        long long sa = 0, sb = 0;
         for (int i = 0; i < kPlaqThreads / 32; ++i) {
-            a += ss[i];
-            b += st[i];
+            sa += ss[i];
+            sb += st[i];
         }
-        partial[2 * blk] = a;
-        partial[2 * blk + 1] = b;
+        DevRecord *rec = out ? out : sweep_record(a, k);
+        atomicAdd(&rec->a, (unsigned long long)sa); // the exact sums; P, P_s, P_t are formed on the host
+        atomicAdd(&rec->b, (unsigned long long)sb);
     }
-}
-
-// One block per chain (blockIdx.x = chain index, or `only` when >= 0): exact sum
-// of the chain's partials, written as P, P_s, P_t.
-__global__ void __launch_bounds__(256) k_plaquette_final(const Su2Chain *chains, const uint32_t *meas_start,
-                                                         const long long *partial, DevRecord *series, long long cap,
-                                                         const DevState *state, uint32_t ksweep, uint32_t rec_k,
-                                                         int only, DevRecord *out)
-{
-    __shared__ long long ss[8], st[8];
-    const int k = only >= 0 ? only : (int)blockIdx.x;
-    const uint32_t b0 = meas_start[k], b1 = meas_start[k + 1];
-    long long a = 0, b = 0;
-    for (uint32_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-        a += partial[2 * i];
-        b += partial[2 * i + 1];
-    }
-    a = warp_sum_ll(a);
-    b = warp_sum_ll(b);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        ss[w] = a;
-        st[w] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0)
-        return;
-    long long A = 0, B = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-        A += ss[i];
-        B += st[i];
-    }
-    DevRecord *rec = out;
-    long long sweep = (long long)(state->sweep_base + ksweep);
-    if (!rec) {
-        const unsigned long long slot = (state->rec_head + rec_k) % (unsigned long long)cap;
-        rec = &series[(long long)k * cap + (long long)slot];
-    } else {
-        sweep = (long long)state->sweep_base - 1;
-    }
-    rec->sweep = sweep;
-    rec->a = (unsigned long long)A; // the exact sums; P, P_s, P_t are formed on the host
-    rec->b = (unsigned long long)B;
-    rec->d0 = rec->d1 = rec->d2 = 0.0;
 }
 
 // ------------------------------------------------------------------ Polyakov loop
@@ -266,37 +276,57 @@ __global__ void k_su2_io(Su2Chain ch, float4 *U, float4 *canon, int to_lattice)
 
 inline unsigned blocks_for(size_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
-template <int P>
-void launch_phase(mc_ctx *c, const SweepArgs &a, int mu, unsigned nblocks)
+template <int P, bool REC, int MINB, typename TAB>
+void launch_phase(mc_ctx *c, const SweepArgs &a, const TAB &tab, int mu)
 {
     if (prof_begin(c) != cudaSuccess)
         return;
-    const bool rec = a.tries != nullptr;
-    switch (mu * 2 + (rec ? 1 : 0)) {
-    case 0: k_phase<P, 0, false><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 1: k_phase<P, 0, true><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 2: k_phase<P, 1, false><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 3: k_phase<P, 1, true><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 4: k_phase<P, 2, false><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 5: k_phase<P, 2, true><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 6: k_phase<P, 3, false><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    default: k_phase<P, 3, true><<<nblocks, c->threads, 0, c->ls>>>(a); break;
+    const unsigned nt = (unsigned)c->threads;
+    switch (mu) {
+    case 0: launch_chained(c, k_phase<P, 0, REC, MINB, TAB>, c->grid_blocks, nt, a, tab); break;
+    case 1: launch_chained(c, k_phase<P, 1, REC, MINB, TAB>, c->grid_blocks, nt, a, tab); break;
+    case 2: launch_chained(c, k_phase<P, 2, REC, MINB, TAB>, c->grid_blocks, nt, a, tab); break;
+    default: launch_chained(c, k_phase<P, 3, REC, MINB, TAB>, c->grid_blocks, nt, a, tab); break;
     }
     prof_end(c);
 }
 
-template <int P>
-void launch_or_phase(mc_ctx *c, const SweepArgs &a, int mu, unsigned nblocks)
+template <int P, typename TAB>
+void launch_or_phase(mc_ctx *c, const SweepArgs &a, const TAB &tab, int mu)
 {
     if (prof_begin(c) != cudaSuccess)
         return;
+    const unsigned nt = (unsigned)c->threads;
     switch (mu) {
-    case 0: k_or_phase<P, 0><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 1: k_or_phase<P, 1><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    case 2: k_or_phase<P, 2><<<nblocks, c->threads, 0, c->ls>>>(a); break;
-    default: k_or_phase<P, 3><<<nblocks, c->threads, 0, c->ls>>>(a); break;
+    case 0: launch_chained(c, k_or_phase<P, 0, TAB>, c->grid_blocks, nt, a, tab); break;
+    case 1: launch_chained(c, k_or_phase<P, 1, TAB>, c->grid_blocks, nt, a, tab); break;
+    case 2: launch_chained(c, k_or_phase<P, 2, TAB>, c->grid_blocks, nt, a, tab); break;
+    default: launch_chained(c, k_or_phase<P, 3, TAB>, c->grid_blocks, nt, a, tab); break;
     }
     prof_end(c);
+}
+
+// The phases of one compound sweep: heat-bath, then n_or overrelaxation sweeps,
+// each over the odd sites first (Sec. 2.4).  The last phase before a measurement
+// keeps the plaquette kernel's blocks out until it is done: set up early they
+// crowd the SMs that its own blocks leave first (20 x 24 x 20 x 24: 50 against 60 us
+// per measured sweep).
+template <bool REC, int MINB, typename TAB>
+void launch_sweep(mc_ctx *c, const SweepArgs &a, const TAB &tab)
+{
+    for (int r = 0; r <= c->n_or; ++r)
+        for (int ph = 0; ph < 8; ++ph) {
+            SweepArgs b = a;
+            b.release = !(a.measure && r == c->n_or && ph == 7);
+            if (r == 0 && ph < 4)
+                launch_phase<1, REC, MINB>(c, b, tab, ph);
+            else if (r == 0)
+                launch_phase<0, REC, MINB>(c, b, tab, ph - 4);
+            else if (ph < 4)
+                launch_or_phase<1>(c, b, tab, ph);
+            else
+                launch_or_phase<0>(c, b, tab, ph - 4);
+        }
 }
 
 }  // namespace
@@ -304,11 +334,9 @@ void launch_or_phase(mc_ctx *c, const SweepArgs &a, int mu, unsigned nblocks)
 // =========================================================================== host
 size_t su2_config_bytes(const Su2Chain &ch) { return (size_t)2 * ch.nh * 4 * sizeof(float4); }
 
-// Block tables.  All chains of the batch form one launch group: sweeping
-// L2-sized groups of chains one after another (to keep each group's links
-// L2-resident across its eight phases) was measured slower on 4 x 32^4 -- the
-// phase kernel is issue-bound, and four one-chain launches per phase add tail
-// waves -- so the group list holds a single entry.
+// Block tables.  All chains of the batch share each launch: sweeping L2-sized
+// groups of chains one after another (to keep each group's links L2-resident
+// across its eight phases) was measured slower on 4 x 32^4.
 void su2_plan_grid(mc_ctx *c)
 {
     c->block_start.assign(c->n_chains + 1, 0);
@@ -324,7 +352,6 @@ void su2_plan_grid(mc_ctx *c)
     c->meas_start[c->n_chains] = macc;
     c->grid_blocks = acc;
     c->meas_blocks = macc;
-    c->groups.assign(1, std::make_pair(0, c->n_chains));
 }
 
 cudaError_t su2_init_launch(mc_ctx *c, const mc_chain_desc *desc)
@@ -337,22 +364,7 @@ cudaError_t su2_init_launch(mc_ctx *c, const mc_chain_desc *desc)
     return cudaGetLastError();
 }
 
-// Per-block plaquette partial sums for chains [k0, k1).
-static void plaquette_partials(mc_ctx *c, int k0, int k1)
-{
-    const uint32_t b0 = c->meas_start[k0], b1 = c->meas_start[k1];
-    k_plaquette<<<b1 - b0, kPlaqThreads, 0, c->ls>>>(static_cast<const Su2Chain *>(c->d_chains), c->d_meas_start, c->n_chains,
-                                            c->d_lattice, c->d_partials, b0);
-}
-
-static void plaquette_final(mc_ctx *c, uint32_t ksweep, uint32_t rec_k, int only, DevRecord *out)
-{
-    const unsigned nb = only >= 0 ? 1u : (unsigned)c->n_chains;
-    k_plaquette_final<<<nb, 256, 0, c->ls>>>(static_cast<const Su2Chain *>(c->d_chains), c->d_meas_start,
-                                             c->d_partials, c->d_series, c->cap, c->d_state, ksweep, rec_k, only, out);
-}
-
-cudaError_t su2_sweep_enqueue(mc_ctx *c, long long n, int every)
+static SweepArgs sweep_args(const mc_ctx *c)
 {
     SweepArgs a{};
     a.chains = c->d_chains;
@@ -363,27 +375,39 @@ cudaError_t su2_sweep_enqueue(mc_ctx *c, long long n, int every)
     a.state = c->d_state;
     a.cap = c->cap;
     a.tries = c->record_tries ? c->d_tries : nullptr;
+    a.release = 1;
+    return a;
+}
+
+cudaError_t su2_sweep_enqueue(mc_ctx *c, long long n, int every)
+{
+    SweepArgs a = sweep_args(c);
+    ChainTable tab;
+    const bool table = c->n_chains <= kTableChains;
+    for (int k = 0; table && k < kTableChains; ++k) {
+        tab.start[k] = k < c->n_chains ? c->block_start[k] : 0xFFFFFFFFu;
+        tab.ch[k] = c->su2[k < c->n_chains ? k : 0];
+    }
+    // every block resident at 3 x 256 threads per SM: the 85-register phase kernel
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool resident = (long long)c->grid_blocks * c->threads <= 768ll * sms;
     for (long long t = 0; t < n; ++t) {
         a.k = (uint32_t)t;
-        const bool measure = every > 0 && ((t + 1) % every) == 0;
-        for (const auto &g : c->groups) {
-            a.block_base = c->block_start[g.first];
-            const unsigned nb = c->block_start[g.second] - c->block_start[g.first];
-            for (int mu = 0; mu < 4; ++mu)
-                launch_phase<1>(c, a, mu, nb); // odd sites first (Sec. 2.4)
-            for (int mu = 0; mu < 4; ++mu)
-                launch_phase<0>(c, a, mu, nb);
-            for (int r = 0; r < c->n_or; ++r) { // overrelaxation sweeps, same phase order
-                for (int mu = 0; mu < 4; ++mu)
-                    launch_or_phase<1>(c, a, mu, nb);
-                for (int mu = 0; mu < 4; ++mu)
-                    launch_or_phase<0>(c, a, mu, nb);
-            }
-            if (measure)
-                plaquette_partials(c, g.first, g.second);
-        }
-        if (measure)
-            plaquette_final(c, (uint32_t)t, (uint32_t)((t + 1) / every - 1), -1, nullptr);
+        a.measure = every > 0 && ((t + 1) % every) == 0;
+        a.rec_k = a.measure ? (uint32_t)((t + 1) / every - 1) : 0u;
+        if (c->record_tries)
+            launch_sweep<true, 4>(c, a, NoTable{});
+        else if (!table)
+            launch_sweep<false, 4>(c, a, NoTable{});
+        else if (resident)
+            launch_sweep<false, 3>(c, a, tab);
+        else
+            launch_sweep<false, 4>(c, a, tab);
+        if (a.measure)
+            launch_chained(c, k_plaquette, c->meas_blocks, (unsigned)kPlaqThreads, a,
+                           static_cast<const uint32_t *>(c->d_meas_start), -1, static_cast<DevRecord *>(nullptr));
     }
     return cudaGetLastError();
 }
@@ -401,8 +425,11 @@ cudaError_t su2_polyakov_launch(mc_ctx *c, int chain, DevRecord *out)
 
 cudaError_t su2_measure_launch(mc_ctx *c, int chain, DevRecord *out)
 {
-    plaquette_partials(c, chain, chain + 1);
-    plaquette_final(c, 0, 0, chain, out);
+    const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(DevRecord), c->ls);
+    if (e != cudaSuccess)
+        return e;
+    k_plaquette<<<c->meas_start[chain + 1] - c->meas_start[chain], kPlaqThreads, 0, c->ls>>>(
+        sweep_args(c), c->d_meas_start, chain, out);
     return cudaGetLastError();
 }
 

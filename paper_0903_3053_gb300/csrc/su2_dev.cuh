@@ -38,106 +38,87 @@ __device__ __forceinline__ float4 qscale(float4 a, float s)
     return make_float4(__fmul_rn(a.x, s), __fmul_rn(a.y, s), __fmul_rn(a.z, s), __fmul_rn(a.w, s));
 }
 
-struct Site {
-    int x[4];
+// A site and its neighbours, as byte offsets into the (parity, mu) link arrays.
+// A step along directions 2, 3 or 0 moves the index within the parity by a constant
+// (wrapped at the ends); the index s >> 1 is the same for both sites of an x1
+// pair, so a step along direction 1 moves it only when it leaves the pair.  Each
+// coordinate's steps are independent of the others', and one offset serves the
+// arrays of every direction.  (Canonical indices, neighbour by neighbour, with an
+// array index each took 2.4x the integer instructions.)
+struct LinkSite {
+    uint32_t o;            // offset of the site
+    uint32_t fw[4], bw[4]; // what a step forward / backward along each direction adds to it (mod 2^32)
+    uint32_t b;            // parity of x1: the canonical index is 2 e + b
+    uint32_t par;          // parity of the site
 };
 
-__device__ __forceinline__ Site site_from_parity_index(const Su2Chain &ch, int p, uint32_t e)
+// Coordinates of the x1 pair e = x1/2 + (L1/2) (x2 + L2 (x3 + L3 x0)), the
+// steps that its two sites share, and the site with x1 parity b or of parity p.
+__device__ __forceinline__ LinkSite link_pair(const Su2Chain &ch, uint32_t e, uint32_t &x1h)
 {
-    // e = x1/2 + (L1/2) (x2 + L2 (x3 + L3 x0)); magic-number divisions (fastdiv.cuh)
-    uint32_t q1, x1h, q2, x2, x0, x3;
+    uint32_t q1, q2, x2, x0, x3; // magic-number divisions (fastdiv.cuh)
     fast_divmod(e, ch.div1h, q1, x1h);
     fast_divmod(q1, ch.div2, q2, x2);
     fast_divmod(q2, ch.div3, x0, x3);
-    Site s;
-    s.x[0] = (int)x0;
-    s.x[2] = (int)x2;
-    s.x[3] = (int)x3;
-    s.x[1] = 2 * (int)x1h + ((p + s.x[0] + s.x[2] + s.x[3]) & 1);
+    LinkSite s;
+    s.o = 16u * e;
+    s.par = (x0 + x2 + x3) & 1u; // of the pair's even-x1 site
+    s.fw[2] = x2 + 1 == ch.div2.d ? ch.step2 - ch.step3 : ch.step2;
+    s.bw[2] = x2 == 0 ? ch.step3 - ch.step2 : 0u - ch.step2;
+    s.fw[3] = x3 + 1 == ch.div3.d ? ch.step3 - ch.step0 : ch.step3;
+    s.bw[3] = x3 == 0 ? ch.step0 - ch.step3 : 0u - ch.step3;
+    s.fw[0] = x0 + 1 == (uint32_t)ch.L[0] ? ch.step0 - ch.bytes : ch.step0;
+    s.bw[0] = x0 == 0 ? ch.bytes - ch.step0 : 0u - ch.step0;
     return s;
 }
-
-__device__ __forceinline__ uint32_t canonical(const Su2Chain &ch, const Site &s)
+__device__ __forceinline__ LinkSite link_of_pair(const Su2Chain &ch, LinkSite s, uint32_t x1h, uint32_t b)
 {
-    return (uint32_t)(s.x[1] + ch.L[1] * (s.x[2] + ch.L[2] * (s.x[3] + ch.L[3] * s.x[0])));
-}
-
-template <int D>
-__device__ __forceinline__ Site step(const Su2Chain &ch, Site s, int dir)
-{
-    s.x[D] += dir;
-    if (s.x[D] == ch.L[D])
-        s.x[D] = 0;
-    else if (s.x[D] < 0)
-        s.x[D] = ch.L[D] - 1;
+    s.b = b;
+    s.par ^= b;
+    s.fw[1] = b ? (x1h + 1 == ch.div1h.d ? 16u - ch.step2 : 16u) : 0u;
+    s.bw[1] = b ? 0u : (x1h == 0 ? ch.step2 - 16u : 0u - 16u);
     return s;
 }
+__device__ __forceinline__ LinkSite link_site(const Su2Chain &ch, int p, uint32_t e)
+{
+    uint32_t x1h;
+    const LinkSite s = link_pair(ch, e, x1h);
+    return link_of_pair(ch, s, x1h, s.par ^ (uint32_t)p);
+}
 
+// The link in direction `dir` of the parity-`par` site at byte offset o.
 template <int LD>
-__device__ __forceinline__ float4 load_link(const float4 *U, uint32_t nh, int par, int dir, uint32_t e)
+__device__ __forceinline__ float4 link_at(const float4 *U, const Su2Chain &ch, int par, int dir, uint32_t o)
 {
-    return lat_load<LD>(&U[(size_t)(par * 4 + dir) * nh + e]);
-}
-
-// Canonical index strides: direction mu moves the canonical index by st[mu].
-struct Strides {
-    uint32_t st[4];
-};
-
-__device__ __forceinline__ Strides strides_of(const Su2Chain &ch)
-{
-    Strides g;
-    g.st[1] = 1u;
-    g.st[2] = (uint32_t)ch.L[1];
-    g.st[3] = (uint32_t)(ch.L[1] * ch.L[2]);
-    g.st[0] = (uint32_t)(ch.L[1] * ch.L[2] * ch.L[3]);
-    return g;
-}
-
-// Canonical index of x + e_D / x - e_D, given x's coordinate along D.
-template <int D>
-__device__ __forceinline__ uint32_t fwd(const Su2Chain &ch, const Strides &g, int xd, uint32_t s)
-{
-    return xd + 1 == ch.L[D] ? s - (uint32_t)(ch.L[D] - 1) * g.st[D] : s + g.st[D];
-}
-template <int D>
-__device__ __forceinline__ uint32_t bwd(const Su2Chain &ch, const Strides &g, int xd, uint32_t s)
-{
-    return xd == 0 ? s + (uint32_t)(ch.L[D] - 1) * g.st[D] : s - g.st[D];
+    const char *base = reinterpret_cast<const char *>(U) + (size_t)(par * 4 + dir) * ch.bytes;
+    return lat_load<LD>(reinterpret_cast<const float4 *>(base + o));
 }
 
 // The two staples of Eq. (6) in the (MU, NU) plane:
 //   U_nu(x) U_mu(x+nu) U_nu(x+mu)^+  +  U_nu(x-nu)^+ U_mu(x-nu) U_nu(x-nu+mu).
 // x + nu, x + mu and x - nu have parity 1 - P; x - nu + mu has parity P.
 template <int MU, int NU, int P, int LD>
-__device__ __forceinline__ float4 staple_pair(const float4 *__restrict__ U, const Su2Chain &ch, const Strides &g,
-                                              const Site &x, uint32_t s, uint32_t spm, uint32_t e)
+__device__ __forceinline__ float4 staple_pair(const float4 *__restrict__ U, const Su2Chain &ch, const LinkSite &x)
 {
     constexpr int Q = 1 - P;
-    const uint32_t nh = ch.nh;
-    const uint32_t spn = fwd<NU>(ch, g, x.x[NU], s);
-    const uint32_t smn = bwd<NU>(ch, g, x.x[NU], s);
-    const uint32_t smnpm = fwd<MU>(ch, g, x.x[MU], smn); // x - nu has the same MU coordinate as x
-    const float4 a = load_link<LD>(U, nh, P, NU, e);
-    const float4 b = load_link<LD>(U, nh, Q, MU, spn >> 1);
-    const float4 c = load_link<LD>(U, nh, Q, NU, spm >> 1);
-    const float4 d = load_link<LD>(U, nh, Q, NU, smn >> 1);
-    const float4 f = load_link<LD>(U, nh, Q, MU, smn >> 1);
-    const float4 h = load_link<LD>(U, nh, P, NU, smnpm >> 1);
+    const uint32_t pm = x.o + x.fw[MU], pn = x.o + x.fw[NU], mn = x.o + x.bw[NU], mnpm = mn + x.fw[MU];
+    const float4 a = link_at<LD>(U, ch, P, NU, x.o);
+    const float4 b = link_at<LD>(U, ch, Q, MU, pn);
+    const float4 c = link_at<LD>(U, ch, Q, NU, pm);
+    const float4 d = link_at<LD>(U, ch, Q, NU, mn);
+    const float4 f = link_at<LD>(U, ch, Q, MU, mn);
+    const float4 h = link_at<LD>(U, ch, P, NU, mnpm);
     return qadd(qmul(qmul(a, b), qdag(c)), qmul(qmul(qdag(d), f), h));
 }
 
 template <int MU, int P, int LD>
-__device__ __forceinline__ float4 staple(const float4 *__restrict__ U, const Su2Chain &ch, const Site &x, uint32_t s,
-                                         uint32_t e)
+__device__ __forceinline__ float4 staple(const float4 *__restrict__ U, const Su2Chain &ch, const LinkSite &x)
 {
-    const Strides g = strides_of(ch);
-    const uint32_t spm = fwd<MU>(ch, g, x.x[MU], s);
     float4 W = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (MU != 0) W = qadd(W, staple_pair<MU, 0, P, LD>(U, ch, g, x, s, spm, e));
-    if (MU != 1) W = qadd(W, staple_pair<MU, 1, P, LD>(U, ch, g, x, s, spm, e));
-    if (MU != 2) W = qadd(W, staple_pair<MU, 2, P, LD>(U, ch, g, x, s, spm, e));
-    if (MU != 3) W = qadd(W, staple_pair<MU, 3, P, LD>(U, ch, g, x, s, spm, e));
+    if (MU != 0) W = qadd(W, staple_pair<MU, 0, P, LD>(U, ch, x));
+    if (MU != 1) W = qadd(W, staple_pair<MU, 1, P, LD>(U, ch, x));
+    if (MU != 2) W = qadd(W, staple_pair<MU, 2, P, LD>(U, ch, x));
+    if (MU != 3) W = qadd(W, staple_pair<MU, 3, P, LD>(U, ch, x));
     return W;
 }
 
@@ -202,21 +183,25 @@ __device__ __forceinline__ KpFirstTry kp_first_try(uint32_t e, uint32_t sweep, u
 }
 
 // Heat-bath draw of a0: tries 0 .. kKpTries - 1 by Kennedy-Pendleton (skipped
-// when alpha = 0; try 0 from its precomputed part f), then Creutz up to
+// when alpha = 0; the first AHEAD tries from their precomputed parts f), then Creutz up to
 // kKpTries + kCreutzTries - 1; returns the try taken, or kFailed.  One loop
 // over both samplers (measured ~2% faster on 4 x 32^4 than a loop per
 // sampler); the same draws as heatbath_try for every t.
+template <int AHEAD>
 __device__ __forceinline__ int draw_a0(float alpha, uint32_t e, uint32_t sweep, uint32_t sel, const Su2Chain &ch,
-                                       const PhiloxSchedule &ks, const KpFirstTry &f, float &a0)
+                                       const PhiloxSchedule &ks, const KpFirstTry (&f)[AHEAD], float &a0)
 {
     if (alpha > 0.f) {
-        float a;
-        if (kp_accept(f, alpha, a)) {
-            a0 = a;
-            return 0;
+#pragma unroll
+        for (int t = 0; t < AHEAD; ++t) {
+            float a;
+            if (kp_accept(f[t], alpha, a)) {
+                a0 = a;
+                return t;
+            }
         }
     }
-    for (int t = alpha > 0.f ? 1 : kKpTries; t < kKpTries + kCreutzTries; ++t) {
+    for (int t = alpha > 0.f ? AHEAD : kKpTries; t < kKpTries + kCreutzTries; ++t) {
         float a;
         if (heatbath_try(t, alpha, e, sweep, sel, ch, ks, a)) {
             a0 = a;
@@ -226,8 +211,6 @@ __device__ __forceinline__ int draw_a0(float alpha, uint32_t e, uint32_t sweep, 
     return kFailed;
 }
 
-// Staple of the link U_MU(x) at site e of parity P (Eq. (6)) as V = W / |W| and
-// alpha = beta |W| (V = 1 for a vanishing staple); sc = canonical site index.
 // V = W / |W| and alpha = beta |W| of a staple W (V = 1 for a vanishing staple);
 // one reciprocal square root serves both.
 __device__ __forceinline__ void staple_to_heatbath(const float4 &W, float beta, float4 &V, float &alpha)
@@ -241,16 +224,6 @@ __device__ __forceinline__ void staple_to_heatbath(const float4 &W, float beta, 
         kn = __fmul_rn(k2, inv);
     }
     alpha = __fmul_rn(beta, kn);
-}
-
-template <int P, int MU, int LD>
-__device__ __forceinline__ void su2_link_staple(const float4 *U, const Su2Chain &ch, uint32_t e, float4 &V,
-                                                float &alpha, uint32_t &sc)
-{
-    const Site x = site_from_parity_index(ch, P, e);
-    sc = canonical(ch, x);
-    const float4 W = staple<MU, P, LD>(U, ch, x, sc, e);
-    staple_to_heatbath(W, ch.beta, V, alpha);
 }
 
 // Uniform direction on S^2 for the vector part of X in Eq. (5): cos theta =
@@ -290,10 +263,10 @@ __device__ __forceinline__ float4 heatbath_link(float a0, const float4 &V, const
 // Heat-bath draw and store for a link whose staple is (V, alpha) and whose
 // direction is d: a0 by Kennedy-Pendleton / Creutz, U = X V, reprojection
 // (Eqs. (5), (7)).  Returns the try taken (kFailed: link unchanged, counted).
-template <int P, int MU, bool INLINE_FAIL>
+template <int P, int MU, bool INLINE_FAIL, int AHEAD>
 __device__ __forceinline__ int su2_link_draw(float4 *U, const Su2Chain &ch, const PhiloxSchedule &ks, uint32_t e,
                                              uint32_t sweep, float4 V, float alpha, const S2Direction &d,
-                                             const KpFirstTry &f, DevState *state)
+                                             const KpFirstTry (&f)[AHEAD], DevState *state)
 {
     const uint32_t sel = ((uint32_t)P << 12) | ((uint32_t)MU << 8);
     float a0 = 0.f;
@@ -317,9 +290,10 @@ __device__ __forceinline__ int su2_link_draw(float4 *U, const Su2Chain &ch, cons
 // INLINE_FAIL: count a failed update with an inlined atomic (the persistent
 // batch kernel, where the out-of-line call costs a stack frame) instead of
 // count_heatbath_failure.
-template <int P, int MU, int LD, bool REC, bool INLINE_FAIL = false, int EARLY = 2>
+// CHAINED: the links are read only after chain_wait (the phase kernels).
+template <int P, int MU, int LD, bool REC, bool INLINE_FAIL = false, int EARLY = 2, bool CHAINED = false>
 __device__ __forceinline__ void su2_update_link(float4 *U, const Su2Chain &ch, const PhiloxSchedule &ks, uint32_t e,
-                                                uint32_t sweep, uint8_t *tries, DevState *state)
+                                                uint32_t sweep, uint8_t *tries, DevState *state, bool release = false)
 {
     // The direction and the alpha-free part of the first heat-bath try do not
     // depend on the staple: computed first (EARLY = 2), their Philox blocks,
@@ -327,23 +301,28 @@ __device__ __forceinline__ void su2_update_link(float4 *U, const Su2Chain &ch, c
     // (0.609 against 0.650 ms per sweep of 4 x 32^4, identical links).  EARLY
     // = 1 moves only the direction, 0 neither; the draws are the same.
     const uint32_t sel = ((uint32_t)P << 12) | ((uint32_t)MU << 8);
+    constexpr int AHEAD = EARLY >= 3 ? EARLY - 1 : 1;
     S2Direction d;
-    KpFirstTry f;
+    KpFirstTry f[AHEAD];
     if (EARLY >= 1)
         d = su2_direction<P, MU>(ch, ks, e, sweep);
     if (EARLY >= 2)
-        f = kp_first_try(e, sweep, sel, ch, ks);
+#pragma unroll
+        for (int t = 0; t < AHEAD; ++t)
+            f[t] = kp_first_try(e, sweep, sel | (uint32_t)t, ch, ks);
     float4 V;
     float alpha;
-    uint32_t sc;
-    su2_link_staple<P, MU, LD>(U, ch, e, V, alpha, sc);
+    const LinkSite x = link_site(ch, P, e);
+    if (CHAINED)
+        chain_wait(release);
+    staple_to_heatbath(staple<MU, P, LD>(U, ch, x), ch.beta, V, alpha);
     if (EARLY < 2)
-        f = kp_first_try(e, sweep, sel, ch, ks);
+        f[0] = kp_first_try(e, sweep, sel, ch, ks);
     if (EARLY < 1)
         d = su2_direction<P, MU>(ch, ks, e, sweep);
-    const int t = su2_link_draw<P, MU, INLINE_FAIL>(U, ch, ks, e, sweep, V, alpha, d, f, state);
+    const int t = su2_link_draw<P, MU, INLINE_FAIL, AHEAD>(U, ch, ks, e, sweep, V, alpha, d, f, state);
     if (REC)
-        tries[ch.tries_off + (size_t)sc * 4 + MU] = (uint8_t)t;
+        tries[ch.tries_off + (size_t)(2 * e + x.b) * 4 + MU] = (uint8_t)t; // canonical site 2 e + b
 }
 
 // Overrelaxation of the link U_MU(x) at site e of parity P (the
@@ -351,14 +330,15 @@ __device__ __forceinline__ void su2_update_link(float4 *U, const Su2Chain &ch, c
 // reflection U' = V U^dag V, V = W / |W|, keeps Re Tr(U W^dag) and so the
 // action; deterministic, no random numbers.  A vanishing staple leaves the link
 // as it is.  The result is reprojected onto SU(2).
-template <int P, int MU, int LD>
-__device__ __forceinline__ void su2_overrelax_link(float4 *U, const Su2Chain &ch, uint32_t e)
+template <int P, int MU, int LD, bool CHAINED = false>
+__device__ __forceinline__ void su2_overrelax_link(float4 *U, const Su2Chain &ch, uint32_t e, bool release = false)
 {
     float4 V;
     {
-        const Site x = site_from_parity_index(ch, P, e);
-        const uint32_t sc = canonical(ch, x);
-        const float4 W = staple<MU, P, LD>(U, ch, x, sc, e);
+        const LinkSite x = link_site(ch, P, e);
+        if (CHAINED)
+            chain_wait(release);
+        const float4 W = staple<MU, P, LD>(U, ch, x);
         const float k2 = qdot(W, W);
         if (!(k2 > 0.f))
             return;
@@ -453,131 +433,40 @@ __device__ __forceinline__ void plaquettes_of(const float4 (&Ux)[4], const float
         }
 }
 
-__device__ __forceinline__ Site site_of_canonical(const Su2Chain &ch, uint32_t s)
-{
-    uint32_t q1, q2, c[4];
-    fast_divmod(s, ch.div1, q1, c[1]);
-    fast_divmod(q1, ch.div2, q2, c[2]);
-    fast_divmod(q2, ch.div3, c[0], c[3]);
-    Site x;
-    for (int m = 0; m < 4; ++m)
-        x.x[m] = (int)c[m];
-    return x;
-}
-
-// Spatial and temporal fixed-point sums of (1/2) Tr U_munu(x) over the six
-// plaquettes with corner at canonical site s, added to ps and pt; FP32 products.
-template <int LD>
-__device__ __forceinline__ void su2_site_plaquettes(const float4 *U, const Su2Chain &ch, uint32_t s, long long &ps,
-                                                    long long &pt)
-{
-    const Site x = site_of_canonical(ch, s);
-    const int p = (x.x[0] + x.x[1] + x.x[2] + x.x[3]) & 1, q = 1 - p;
-    const uint32_t e = s >> 1;
-    float4 Ux[4], Uf[4][4]; // Uf[mu][nu] = U_nu(x + mu)
-    Site xf[4];
-    xf[0] = step<0>(ch, x, +1);
-    xf[1] = step<1>(ch, x, +1);
-    xf[2] = step<2>(ch, x, +1);
-    xf[3] = step<3>(ch, x, +1);
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu)
-        Ux[mu] = load_link<LD>(U, ch.nh, p, mu, e);
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        const uint32_t ef = canonical(ch, xf[mu]) >> 1;
-#pragma unroll
-        for (int nu = 0; nu < 4; ++nu)
-            if (nu != mu)
-                Uf[mu][nu] = load_link<LD>(U, ch.nh, q, nu, ef);
-    }
-    plaquettes_of(Ux, Uf, ps, pt);
-}
-
-// The same sums for the two sites of an x1 pair, canonical 2j and 2j + 1 (L1 is
-// even, so both lie in one row and have opposite parities; both have index j
-// within their parity).  The second site's own links are the first site's
-// forward links along x1, so the pair takes 29 link loads instead of 32, and
-// one thread carries two independent products chains.
+// Spatial and temporal fixed-point sums of the plaquettes with corner at the two
+// sites of x1 pair j (L1 is even: both lie in one row, have opposite parities and
+// index j within them), added to ps and pt; FP32 products.  The second site's own
+// links are the first site's forward links along x1, so the pair takes 29 link
+// loads instead of 32; the steps along the other directions are shared, and one
+// thread carries two independent chains of products.
 template <int LD>
 __device__ __forceinline__ void su2_pair_plaquettes(const float4 *U, const Su2Chain &ch, uint32_t j, long long &ps,
                                                     long long &pt)
 {
-    const Site x = site_of_canonical(ch, 2 * j);
-    Site y = x;
-    y.x[1] += 1;
-    const int p0 = (x.x[0] + x.x[1] + x.x[2] + x.x[3]) & 1, p1 = 1 - p0;
-    const uint32_t nh = ch.nh;
+    uint32_t x1h;
+    const LinkSite x = link_pair(ch, j, x1h);
+    const LinkSite y = link_of_pair(ch, x, x1h, 1u);
+    const int p0 = (int)x.par, p1 = 1 - p0;
+    const uint32_t f0 = x.o + x.fw[0], f1 = x.o + y.fw[1], f2 = x.o + x.fw[2], f3 = x.o + x.fw[3];
     float4 U0[4], U1[4], F0[4][4], F1[4][4]; // F0[mu][nu] = U_nu(x + mu), F1[mu][nu] = U_nu(y + mu)
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        U0[mu] = load_link<LD>(U, nh, p0, mu, j);
-        U1[mu] = load_link<LD>(U, nh, p1, mu, j);
+        U0[mu] = link_at<LD>(U, ch, p0, mu, x.o);
+        U1[mu] = link_at<LD>(U, ch, p1, mu, x.o);
     }
 #pragma unroll
-    for (int nu = 0; nu < 4; ++nu)
-        F0[1][nu] = U1[nu];
-    const uint32_t e00 = canonical(ch, step<0>(ch, x, +1)) >> 1, e02 = canonical(ch, step<2>(ch, x, +1)) >> 1,
-                   e03 = canonical(ch, step<3>(ch, x, +1)) >> 1;
-    const uint32_t e10 = canonical(ch, step<0>(ch, y, +1)) >> 1, e11 = canonical(ch, step<1>(ch, y, +1)) >> 1,
-                   e12 = canonical(ch, step<2>(ch, y, +1)) >> 1, e13 = canonical(ch, step<3>(ch, y, +1)) >> 1;
-#pragma unroll
     for (int nu = 0; nu < 4; ++nu) {
-        if (nu != 0) F0[0][nu] = load_link<LD>(U, nh, p1, nu, e00);
-        if (nu != 2) F0[2][nu] = load_link<LD>(U, nh, p1, nu, e02);
-        if (nu != 3) F0[3][nu] = load_link<LD>(U, nh, p1, nu, e03);
-        if (nu != 0) F1[0][nu] = load_link<LD>(U, nh, p0, nu, e10);
-        if (nu != 1) F1[1][nu] = load_link<LD>(U, nh, p0, nu, e11);
-        if (nu != 2) F1[2][nu] = load_link<LD>(U, nh, p0, nu, e12);
-        if (nu != 3) F1[3][nu] = load_link<LD>(U, nh, p0, nu, e13);
+        F0[1][nu] = U1[nu];
+        if (nu != 0) F0[0][nu] = link_at<LD>(U, ch, p1, nu, f0);
+        if (nu != 2) F0[2][nu] = link_at<LD>(U, ch, p1, nu, f2);
+        if (nu != 3) F0[3][nu] = link_at<LD>(U, ch, p1, nu, f3);
+        if (nu != 0) F1[0][nu] = link_at<LD>(U, ch, p0, nu, f0);
+        if (nu != 1) F1[1][nu] = link_at<LD>(U, ch, p0, nu, f1);
+        if (nu != 2) F1[2][nu] = link_at<LD>(U, ch, p0, nu, f2);
+        if (nu != 3) F1[3][nu] = link_at<LD>(U, ch, p0, nu, f3);
     }
     plaquettes_of(U0, F0, ps, pt);
     plaquettes_of(U1, F1, ps, pt);
-}
-
-// Canonical index of the neighbour x + e_D of site x (canonical index s).
-template <int D>
-__device__ __forceinline__ uint32_t canonical_fwd(const Su2Chain &ch, const Site &x, uint32_t s)
-{
-    return fwd<D>(ch, strides_of(ch), x.x[D], s);
-}
-
-// One plaquette, plane (MU, NU) at canonical site s, added in fixed point to pt
-// (MU = 0) or ps: the value plaquettes_of computes for that plane.
-template <int MU, int NU, int LD>
-__device__ __forceinline__ void su2_plane_plaquette(const float4 *U, const Su2Chain &ch, const Site &x, uint32_t s,
-                                                    long long &ps, long long &pt)
-{
-    const int p = (x.x[0] + x.x[1] + x.x[2] + x.x[3]) & 1;
-    const uint32_t nh = ch.nh, e = s >> 1;
-    const float4 umu = load_link<LD>(U, nh, p, MU, e);
-    const float4 unu = load_link<LD>(U, nh, p, NU, e);
-    const float4 unu_f = load_link<LD>(U, nh, 1 - p, NU, canonical_fwd<MU>(ch, x, s) >> 1);
-    const float4 umu_f = load_link<LD>(U, nh, 1 - p, MU, canonical_fwd<NU>(ch, x, s) >> 1);
-    const long long h = plaq_fixed(plaquette_value(umu, unu_f, unu, umu_f));
-    if (MU == 0)
-        pt += h;
-    else
-        ps += h;
-}
-
-// Plaquette number u of a chain, u = plane N + s (N = 2 nh sites; planes in
-// the order (0,1), (0,2), (0,3), (1,2), (1,3), (2,3)), so that consecutive
-// threads take consecutive sites of one plane; added in fixed point to ps / pt.
-template <int LD>
-__device__ __forceinline__ void su2_plaquette_unit(const float4 *U, const Su2Chain &ch, uint32_t u, long long &ps,
-                                                   long long &pt)
-{
-    const uint32_t n = 2u * ch.nh, plane = u / n, s = u - plane * n;
-    const Site x = site_of_canonical(ch, s);
-    switch (plane) {
-    case 0: su2_plane_plaquette<0, 1, LD>(U, ch, x, s, ps, pt); break;
-    case 1: su2_plane_plaquette<0, 2, LD>(U, ch, x, s, ps, pt); break;
-    case 2: su2_plane_plaquette<0, 3, LD>(U, ch, x, s, ps, pt); break;
-    case 3: su2_plane_plaquette<1, 2, LD>(U, ch, x, s, ps, pt); break;
-    case 4: su2_plane_plaquette<1, 3, LD>(U, ch, x, s, ps, pt); break;
-    default: su2_plane_plaquette<2, 3, LD>(U, ch, x, s, ps, pt); break;
-    }
 }
 
 }  // namespace

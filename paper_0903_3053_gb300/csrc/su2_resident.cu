@@ -82,16 +82,13 @@ __device__ __forceinline__ void staple_warps_barrier()
 template <int P, int MU>
 __device__ __forceinline__ float4 staple_pair_nth(const float4 *U, const Su2Chain &ch, uint32_t e, int r)
 {
-    const Site x = site_from_parity_index(ch, P, e);
-    const uint32_t s = canonical(ch, x);
-    const Strides g = strides_of(ch);
-    const uint32_t spm = fwd<MU>(ch, g, x.x[MU], s);
+    const LinkSite x = link_site(ch, P, e);
     constexpr int N0 = MU == 0 ? 1 : 0, N1 = MU <= 1 ? 2 : 1, N2 = MU <= 2 ? 3 : 2;
     if (r == 0)
-        return staple_pair<MU, N0, P, kLdCoherent>(U, ch, g, x, s, spm, e);
+        return staple_pair<MU, N0, P, kLdCoherent>(U, ch, x);
     if (r == 1)
-        return staple_pair<MU, N1, P, kLdCoherent>(U, ch, g, x, s, spm, e);
-    return staple_pair<MU, N2, P, kLdCoherent>(U, ch, g, x, s, spm, e);
+        return staple_pair<MU, N1, P, kLdCoherent>(U, ch, x);
+    return staple_pair<MU, N2, P, kLdCoherent>(U, ch, x);
 }
 
 // Random numbers of one pass (phase (P, MU), links e0 .. e0 + 127, sweep) into
@@ -208,30 +205,32 @@ __device__ __forceinline__ void resident_pass_rt(int phase, float4 *U, const Su2
     }
 }
 
-// The four links of plaquette unit u (u = plane N + s, as su2_plaquette_unit),
-// in the order plaquette_value takes them; temporal: the plane contains mu = 0.
+// The four links of plaquette unit u = plane N + s (N = 2 nh sites; planes in the
+// order (0,1), (0,2), (0,3), (1,2), (1,3), (2,3), so that consecutive threads take
+// consecutive sites of one plane), in the order plaquette_value takes them;
+// returns whether the plane is temporal (contains mu = 0).
 template <int MU, int NU>
-__device__ __forceinline__ void plane_links(const float4 *U, const Su2Chain &ch, const Site &x, uint32_t s,
-                                            float4 (&q)[4])
+__device__ __forceinline__ void plane_links(const float4 *U, const Su2Chain &ch, const LinkSite &x, float4 (&q)[4])
 {
-    const int p = (x.x[0] + x.x[1] + x.x[2] + x.x[3]) & 1;
-    const uint32_t nh = ch.nh, e = s >> 1;
-    q[0] = load_link<kLdCoherent>(U, nh, p, MU, e);
-    q[1] = load_link<kLdCoherent>(U, nh, 1 - p, NU, canonical_fwd<MU>(ch, x, s) >> 1);
-    q[2] = load_link<kLdCoherent>(U, nh, p, NU, e);
-    q[3] = load_link<kLdCoherent>(U, nh, 1 - p, MU, canonical_fwd<NU>(ch, x, s) >> 1);
+    const int p = (int)x.par;
+    q[0] = link_at<kLdCoherent>(U, ch, p, MU, x.o);
+    q[1] = link_at<kLdCoherent>(U, ch, 1 - p, NU, x.o + x.fw[MU]);
+    q[2] = link_at<kLdCoherent>(U, ch, p, NU, x.o);
+    q[3] = link_at<kLdCoherent>(U, ch, 1 - p, MU, x.o + x.fw[NU]);
 }
 __device__ __forceinline__ bool unit_links(const float4 *U, const Su2Chain &ch, uint32_t u, float4 (&q)[4])
 {
     const uint32_t n = 2u * ch.nh, plane = u / n, s = u - plane * n;
-    const Site x = site_of_canonical(ch, s);
+    uint32_t x1h;
+    const LinkSite pr = link_pair(ch, s >> 1, x1h);
+    const LinkSite x = link_of_pair(ch, pr, x1h, s & 1u);
     switch (plane) {
-    case 0: plane_links<0, 1>(U, ch, x, s, q); break;
-    case 1: plane_links<0, 2>(U, ch, x, s, q); break;
-    case 2: plane_links<0, 3>(U, ch, x, s, q); break;
-    case 3: plane_links<1, 2>(U, ch, x, s, q); break;
-    case 4: plane_links<1, 3>(U, ch, x, s, q); break;
-    default: plane_links<2, 3>(U, ch, x, s, q); break;
+    case 0: plane_links<0, 1>(U, ch, x, q); break;
+    case 1: plane_links<0, 2>(U, ch, x, q); break;
+    case 2: plane_links<0, 3>(U, ch, x, q); break;
+    case 3: plane_links<1, 2>(U, ch, x, q); break;
+    case 4: plane_links<1, 3>(U, ch, x, q); break;
+    default: plane_links<2, 3>(U, ch, x, q); break;
     }
     return plane < 3;
 }
@@ -368,20 +367,6 @@ int resident_cluster(const mc_ctx *c)
 }
 
 }  // namespace
-
-// Automatic choice: one pass per phase (<= 2048 links per phase and chain:
-// 8^4 and the 4 x 8^3, 8 x 8^3 lattices of Table 1; measured 1.2-1.35x faster
-// than the grid launches there, and slower from two passes on) and no
-// per-link try record.
-bool su2_resident_auto(const mc_ctx *c)
-{
-    if (c->kind != MC_KIND_SU2 || c->record_tries)
-        return false;
-    for (const auto &ch : c->su2)
-        if (ch.nh > (uint32_t)kSu2ResidentMaxCluster * kResLinks)
-            return false;
-    return true;
-}
 
 // Cluster size for this context: the smallest power of two giving one pass
 // per phase (at most 16), lowered until the device can place such a cluster of

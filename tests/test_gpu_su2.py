@@ -396,3 +396,42 @@ def test_resident_mode_bit_identical_to_grid(case):
     auto = _run_mode(chains, mc.MC_MODE_AUTO, n, every, n_or)
     for a, b_ in zip(ref[0], auto[0]):
         np.testing.assert_array_equal(a, b_)
+
+
+@pytest.mark.parametrize("case", ["one", "extent_2", "sixteen", "seventeen", "all_resident", "several_waves"])
+def test_chained_phase_kernels_agree(case):
+    """The phase kernels with the chain descriptors as parameters (up to 16
+    chains), with a lookup in memory (more), in the launch bound for launches that
+    are resident at once and in the other one, against the try-recording
+    instantiation (whose links the oracle checks): the same links, records and
+    failure counts, with measurements between heat-bath and overrelaxation sweeps."""
+    beta = [0.0, 1.5, 2.3, 2.6]
+    shapes = {"one": [(4, 6, 2, 8)], "extent_2": [(2, 2, 2, 2), (2, 4, 6, 2), (10, 2, 2, 4)],
+              "sixteen": [(4, 4, 2, 6), (2, 6, 4, 4)] * 8, "seventeen": [(4, 4, 2, 6)] * 16 + [(6, 2, 4, 2)],
+              "all_resident": [(20, 24, 20, 24)], "several_waves": [(24, 24, 24, 24), (8, 32, 16, 10)]}[case]
+    chains = [mc.su2(L, beta[(i + 2) % 4], seed=30 + i, chain_id=i) for i, L in enumerate(shapes)]
+    out = []
+    for record in (True, False):
+        b = mc.Batch(chains, series_capacity=8)
+        b.record_tries(record)
+        b.sweep(3, 1)
+        b.set_overrelax(2)
+        b.sweep(4, 2)
+        b.sweep(4, 2)  # replayed
+        out.append((b.read_series(), [b.get_config(k) for k in range(len(chains))], b.failed_updates(),
+                    [b.measure(k) for k in range(len(chains))]))
+        b.close()
+    for f in ("sweep", "P", "Ps", "Pt"):
+        np.testing.assert_array_equal(out[0][0][f], out[1][0][f])
+    for x, y in zip(out[0][1], out[1][1]):
+        np.testing.assert_array_equal(x, y)
+    assert out[0][2:] == out[1][2:]
+    for k in range(len(chains)):  # the last record is the final configuration's
+        assert out[1][0]["P"][k, -1] == out[1][3][k]["P"] == oracle_plaquette_close(out[1][1][k], chains[k].L, out[1][3][k]["P"])
+
+
+def oracle_plaquette_close(q, L, P):
+    """P if the oracle's plaquette of the links agrees with it to FP32 rounding."""
+    want = oracle.su2_plaquette(q.astype(np.float64), L)[0]
+    assert abs(want - P) < 1e-6
+    return P
