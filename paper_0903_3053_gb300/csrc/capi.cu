@@ -180,15 +180,18 @@ Plan make_plan(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t c
     return p;
 }
 
+// Wait for the context's stream and report a latched device fault.  The run state
+// comes back in stream order into the context's page-locked block, so that one wait
+// serves both (12 us for a kernel and its check; 19 with a second, pageable copy
+// after the wait).
 mc_status check_device(mc_ctx *c)
 {
-    cudaError_t e = cudaStreamSynchronize(c->stream);
+    cudaError_t e = cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess)
         return cuda_fail(e, "stream synchronize");
-    DevState st;
-    e = cudaMemcpy(&st, c->d_state, sizeof(st), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "read device state");
+    const DevState &st = *c->h_state;
     if (st.err_code != 0) {
         char buf[160];
         snprintf(buf, sizeof buf, "device fault latched: code %d info %d", st.err_code, st.err_info);
@@ -202,6 +205,7 @@ void destroy_graphs(mc_ctx *c)
     for (auto &kv : c->graphs)
         cudaGraphExecDestroy(kv.second);
     c->graphs.clear();
+    c->swept.clear();
 }
 
 void free_ctx(mc_ctx *c)
@@ -215,6 +219,8 @@ void free_ctx(mc_ctx *c)
         cudaEventDestroy(c->fence_out);
     if (c->cap_stream)
         cudaStreamDestroy(c->cap_stream);
+    if (c->h_state)
+        cudaFreeHost(c->h_state);
     delete c;
 }
 
@@ -266,32 +272,49 @@ cudaError_t sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     return mode == MC_MODE_RESIDENT ? su2_resident_enqueue(c, n, every) : su2_sweep_enqueue(c, n, every);
 }
 
-// Capture `n` sweeps (+ state advance) into a graph, or replay a cached one.
+cudaError_t enqueue_chunk(mc_ctx *c, long long n, int every, int mode)
+{
+    const cudaError_t e = sweep_enqueue(c, n, every, mode);
+    return e != cudaSuccess ? e : advance_state_launch(c, n, every > 0 ? n / every : 0);
+}
+
+// Whether work issued on `s` is being captured into a graph of the caller's.
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// `n` sweeps and the advance of the run state: launched one by one the first
+// time a (n, every, mode, ...) is asked for, captured into a graph the second time
+// and replayed from then on.  A graph pays for itself only when replayed: recording
+// and instantiating one costs ~3 us per launch in it, a launch ~2 us (50 measured
+// sweeps of a 1024 x 512 chain on a new context, configuration and series read
+// back: 551 -> 283 us; 20 of 8^4 at four beta 1159 -> 597).
 mc_status run_chunk(mc_ctx *c, long long n, int every, int mode)
 {
     if (c->profiling) { // direct launches, each sweep kernel bracketed by events
-        cudaError_t ek = sweep_enqueue(c, n, every, mode);
-        if (ek == cudaSuccess)
-            ek = advance_state_launch(c, n, every > 0 ? n / every : 0);
+        cudaError_t ek = enqueue_chunk(c, n, every, mode);
         if (ek != cudaSuccess)
             return cuda_fail(ek, "enqueue sweep kernels");
         return MC_OK;
     }
-    // Graphs are recorded and replayed on a private stream (capture is not
+    // Launched, recorded and replayed on a private stream (capture is not
     // permitted on the legacy default stream a caller may pass), fenced with
     // events against the caller's stream so stream order is preserved.
     const auto key = std::make_tuple(n, every, mode, c->threads, c->record_tries, c->n_or);
     auto it = c->graphs.find(key);
-    if (it == c->graphs.end()) {
+    if (it == c->graphs.end() && c->swept.count(key) && !capturing(c->stream)) {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess)
             return cuda_fail(e, "begin graph capture");
         c->ls = c->cap_stream;
-        cudaError_t ek = sweep_enqueue(c, n, every, mode);
-        const long long recs = every > 0 ? n / every : 0;
-        if (ek == cudaSuccess)
-            ek = advance_state_launch(c, n, recs);
+        const cudaError_t ek = enqueue_chunk(c, n, every, mode);
         c->ls = c->stream;
         e = cudaStreamEndCapture(c->cap_stream, &g);
         if (ek != cudaSuccess) {
@@ -311,14 +334,24 @@ mc_status run_chunk(mc_ctx *c, long long n, int every, int mode)
     cudaError_t e = cudaEventRecord(c->fence_in, c->stream);
     if (e == cudaSuccess)
         e = cudaStreamWaitEvent(c->cap_stream, c->fence_in, 0);
+    if (e == cudaSuccess) {
+        if (it != c->graphs.end()) {
+            e = cudaGraphLaunch(it->second, c->cap_stream);
+        } else {
+            c->ls = c->cap_stream;
+            e = enqueue_chunk(c, n, every, mode);
+            c->ls = c->stream;
+            c->swept.insert(key);
+        }
+    }
+    // also after a failed launch: what was enqueued stays ordered before the caller's next work
+    cudaError_t ef = cudaEventRecord(c->fence_out, c->cap_stream);
+    if (ef == cudaSuccess)
+        ef = cudaStreamWaitEvent(c->stream, c->fence_out, 0);
     if (e == cudaSuccess)
-        e = cudaGraphLaunch(it->second, c->cap_stream);
-    if (e == cudaSuccess)
-        e = cudaEventRecord(c->fence_out, c->cap_stream);
-    if (e == cudaSuccess)
-        e = cudaStreamWaitEvent(c->stream, c->fence_out, 0);
+        e = ef;
     if (e != cudaSuccess)
-        return cuda_fail(e, "graph launch");
+        return cuda_fail(e, "launch sweeps");
     return MC_OK;
 }
 
@@ -394,6 +427,8 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
         e = cudaEventCreateWithFlags(&c->fence_in, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&c->fence_out, cudaEventDisableTiming);
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void **>(&c->h_state), sizeof(DevState), cudaHostAllocDefault);
     if (e != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(e, "create capture stream");
@@ -850,11 +885,7 @@ mc_status mc_su2_failed_updates(mc_ctx *c, int64_t *count)
     mc_status s = check_device(c);
     if (s != MC_OK)
         return s;
-    DevState st;
-    cudaError_t e = cudaMemcpy(&st, c->d_state, sizeof st, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "read device state");
-    *count = (int64_t)st.hb_failures;
+    *count = (int64_t)c->h_state->hb_failures;
     return MC_OK;
 }
 

@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <map>
+#include <set>
 #include <string>
 #include <tuple>
 #include <utility>
@@ -200,6 +201,8 @@ struct mc_ctx {
     int n_or = 0;                        // SU(2): overrelaxation sweeps after each heat-bath sweep
     int su2_res_cluster = 0;             // SU(2) resident mode: CTAs per chain (0 = not prepared)
     std::map<std::tuple<long long, int, int, int, bool, int>, cudaGraphExec_t> graphs;
+    std::set<std::tuple<long long, int, int, int, bool, int>> swept; // launched once, not recorded yet
+    mc::DevState *h_state = nullptr;     // page-locked copy of the run state (check_device)
     // kernel timing (mc_profile_enable)
     bool profiling = false;
     std::vector<cudaEvent_t> events; // pairs: [2i] before, [2i+1] after launch i
