@@ -131,7 +131,7 @@ MC_API mc_status mc_sweep(mc_ctx *ctx, int64_t n_sweeps, int32_t measure_every);
  * lattices that fit there; SU(2): one thread-block cluster of up to 16 CTAs
  * per chain, the phases of Sec. 2.4 separated by the hardware cluster barrier,
  * any lattice size, one launch per call) or MC_MODE_AUTO (Ising: resident for
- * small lattices; SU(2): always grid, whose chained launches are faster).  An SU(2) context that records heat-bath
+ * small lattices, and for larger ones in batches of many; SU(2): always grid, whose chained launches are faster).  An SU(2) context that records heat-bath
  * tries (mc_su2_record_tries) always sweeps in grid mode.  threads_per_block
  * = 0 keeps the default (256 for Ising, 128 for SU(2), at most 256 for SU(2)):
  * the block size of grid mode, and for Ising resident mode the largest block.

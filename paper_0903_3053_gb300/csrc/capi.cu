@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -208,6 +209,50 @@ void destroy_graphs(mc_ctx *c)
     c->swept.clear();
 }
 
+// Page-locked run-state copies of the contexts, 64 to an allocation (registering a
+// page takes ~40 us); an allocation goes back when its last context is destroyed.
+struct StateSlab {
+    DevState *base;
+    uint64_t used;
+};
+std::mutex g_slab_mutex;
+std::vector<StateSlab> g_slabs;
+
+cudaError_t take_host_state(DevState **out)
+{
+    std::lock_guard<std::mutex> lock(g_slab_mutex);
+    for (StateSlab &s : g_slabs)
+        if (s.used != ~0ull) {
+            const int i = __builtin_ctzll(~s.used);
+            s.used |= 1ull << i;
+            *out = s.base + i;
+            return cudaSuccess;
+        }
+    void *p = nullptr;
+    const cudaError_t e = cudaHostAlloc(&p, 64 * sizeof(DevState), cudaHostAllocPortable);
+    if (e == cudaSuccess) {
+        g_slabs.push_back(StateSlab{static_cast<DevState *>(p), 1ull});
+        *out = static_cast<DevState *>(p);
+    }
+    return e;
+}
+
+void give_host_state(DevState *p)
+{
+    std::lock_guard<std::mutex> lock(g_slab_mutex);
+    for (size_t k = 0; k < g_slabs.size(); ++k) {
+        StateSlab &s = g_slabs[k];
+        if (p < s.base || p >= s.base + 64)
+            continue;
+        s.used &= ~(1ull << (p - s.base));
+        if (s.used == 0) {
+            cudaFreeHost(s.base);
+            g_slabs.erase(g_slabs.begin() + (long)k);
+        }
+        return;
+    }
+}
+
 void free_ctx(mc_ctx *c)
 {
     destroy_graphs(c);
@@ -220,7 +265,7 @@ void free_ctx(mc_ctx *c)
     if (c->cap_stream)
         cudaStreamDestroy(c->cap_stream);
     if (c->h_state)
-        cudaFreeHost(c->h_state);
+        give_host_state(c->h_state);
     delete c;
 }
 
@@ -236,14 +281,7 @@ int resolve_mode(mc_ctx *c)
     }
     if (c->mode != MC_MODE_AUTO)
         return c->mode;
-    int smem = 0;
-    if (!ising_resident_fits(c, &smem))
-        return MC_MODE_GRID;
-    uint64_t max_sites = 0;
-    for (const auto &ch : c->ising)
-        max_sites = std::max<uint64_t>(max_sites, (uint64_t)ch.Lx * ch.Ly);
-    // small lattices: launch latency dominates a grid-mode sweep
-    return max_sites <= 65536 ? MC_MODE_RESIDENT : MC_MODE_GRID;
+    return ising_resident_auto(c) ? MC_MODE_RESIDENT : MC_MODE_GRID;
 }
 
 mc_status upload_tables(mc_ctx *c)
@@ -428,7 +466,7 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&c->fence_out, cudaEventDisableTiming);
     if (e == cudaSuccess)
-        e = cudaHostAlloc(reinterpret_cast<void **>(&c->h_state), sizeof(DevState), cudaHostAllocDefault);
+        e = take_host_state(&c->h_state);
     if (e != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(e, "create capture stream");

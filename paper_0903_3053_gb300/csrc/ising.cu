@@ -28,13 +28,16 @@
 // anti-aligned bonds (every bond joins exactly one colour-1 site) and pairs
 // itself with one colour-0 site for the magnetisation; exact integer sums via
 // warp reductions and one 64-bit atomic per CTA.
+#include <algorithm>
+
 #include "ising_dev.cuh"
 
 namespace mc {
 namespace {
 
 // ------------------------------------------------------------------ grid mode
-template <int C, int LAYOUT>
+// PAIRS (int8): threads take a.row_pairs row pairs of a group column, else a group.
+template <int C, int LAYOUT, bool PAIRS>
 __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 {
     const int k = find_chain(a.block_start, a.n_chains, blockIdx.x);
@@ -46,13 +49,12 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
     chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between calls)
     if (LAYOUT == MC_LAYOUT_INT8) {
         int8_t *s = reinterpret_cast<int8_t *>(a.lattice + ch.spin_off);
-        const uint32_t groups = (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
-        if (t < groups) {
+        if (t < int8_units<PAIRS>(ch, a.row_pairs)) {
             const PhiloxSchedule ks = philox_schedule(ch.key);
             if (measure)
-                int8_unit<C, true>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, true, PAIRS>(s, ch, ks, t, a.row_pairs, sweep, anti, up);
             else
-                int8_unit<C, false>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, false, PAIRS>(s, ch, ks, t, a.row_pairs, sweep, anti, up);
         }
     } else {
         const uint32_t W = ch.W, nw = W * ch.Ly;
@@ -91,21 +93,27 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 }
 
 // Two launch-bound flavours of the same half-sweep: blocks of at most 256
-// threads with 4 resident per SM for the 32-spin words (64 registers, so that the
-// Philox key schedule stays in registers; the kernel is bound by the schedulers'
-// dispatch, which 32 warps per SM keep busy: a 32768^2 chain 730 us per sweep
-// against 757 with 8 blocks and 32 registers) and 6 for int8 (40 registers, no
+// threads with 4 resident per SM (64 registers, so that the Philox key schedule
+// stays in registers; the kernel is bound by the schedulers' dispatch, which 32
+// warps per SM keep busy: a 32768^2 chain in 32-spin words 730 us per sweep against
+// 757 with 8 blocks and 32 registers) or 6 for int8 groups (40 registers, no
 // spills), and blocks of up to 1024 threads for callers that ask for them.
-template <int C, int LAYOUT>
-__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 ? 4 : 6) k_half_sweep(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
-template <int C, int LAYOUT>
-__global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a) { half_sweep<C, LAYOUT>(a); }
+template <int C, int LAYOUT, bool PAIRS>
+__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 || PAIRS ? 4 : 6) k_half_sweep(SweepArgs a)
+{
+    half_sweep<C, LAYOUT, PAIRS>(a);
+}
+template <int C, int LAYOUT, bool PAIRS>
+__global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a)
+{
+    half_sweep<C, LAYOUT, PAIRS>(a);
+}
 
-template <int C, int LAYOUT>
+template <int C, int LAYOUT, bool PAIRS>
 void launch_half_sweep(mc_ctx *c, const SweepArgs &a)
 {
-    launch_chained(c, c->threads <= 256 ? k_half_sweep<C, LAYOUT> : k_half_sweep_big<C, LAYOUT>, c->grid_blocks,
-                   (unsigned)c->threads, a);
+    launch_chained(c, c->threads <= 256 ? k_half_sweep<C, LAYOUT, PAIRS> : k_half_sweep_big<C, LAYOUT, PAIRS>,
+                   c->grid_blocks, (unsigned)c->threads, a);
 }
 
 // ------------------------------------------------------------------ resident mode
@@ -133,16 +141,16 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
         uint32_t anti = 0, up = 0;
         if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(smem);
-            const uint32_t groups = (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
-            for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                int8_unit<0, false>(s, ch, ks, g, sweep, anti, up);
+            const uint32_t units = int8_units<false>(ch, 1);
+            for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
+                int8_unit<0, false>(s, ch, ks, u, 1, sweep, anti, up);
             __syncthreads();
             if (measure) {
-                for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                    int8_unit<1, true>(s, ch, ks, g, sweep, anti, up);
+                for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
+                    int8_unit<1, true>(s, ch, ks, u, 1, sweep, anti, up);
             } else {
-                for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
-                    int8_unit<1, false>(s, ch, ks, g, sweep, anti, up);
+                for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
+                    int8_unit<1, false>(s, ch, ks, u, 1, sweep, anti, up);
             }
         } else {
             const uint32_t W = ch.W, nw = W * ch.Ly, pairs = W * (ch.Ly >> 1);
@@ -392,30 +400,32 @@ size_t ising_config_bytes(const IsingChain &ch, int fmt)
 static uint32_t grid_units(const mc_ctx *c, const IsingChain &ch)
 {
     if (c->layout == MC_LAYOUT_INT8)
-        return (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
+        return c->row_pairs ? int8_units<true>(ch, (uint32_t)c->row_pairs) : int8_units<false>(ch, 1);
     return ((ch.Ly >> 1) + c->row_pairs - 1) / c->row_pairs * ch.W; // runs of row pairs x words
 }
 
-// 32-spin words, row pairs per thread: more of them spread a thread's prologue
+// Row pairs per thread: more of them spread a thread's prologue
 // (chain lookup, descriptor, indices, key schedule) over more words and load each
 // neighbour row once, fewer keep the last wave of blocks even.  As many, up to 8,
 // as leave 2^18 threads (1.7 full waves of 1024 threads on 152 SMs).  Measured us
 // per measured sweep with 1 / 2 / 4 / 8 row pairs: one 4096^2 chain (131072 row
 // pairs) 18.2 / 20.0 / - / -, one 8192^2 or four 4096^2 chains (524288) 54.6 / 52.3 / 57.7 /
-// 58.8, one 16384^2 chain (2097152) 199.5 / - / - / 189.2.
+// 58.8, one 16384^2 chain (2097152) 199.5 / - / - / 189.2; int8, one 4096^2 chain (1048576)
+// 32.3 / - / 24.5 / -, one 8192^2 chain 120 / - / - / 81.  int8 chains of fewer than 2^17
+// row pairs in all (a 2048 x 1024 lattice) take one group per thread instead: 3.5
+// against 4.0 us for 1024 x 512, 5.5 against 4.8 for 1024^2, 11.4 against 10.4 for 2048^2.
+constexpr uint64_t kInt8Pairs = 1u << 17;
 constexpr uint64_t kRowPairThreads = 1u << 18;
 constexpr int kMaxRowPairs = 8;
 
 void ising_plan_grid(mc_ctx *c)
 {
-    c->row_pairs = 1;
-    if (c->layout == MC_LAYOUT_MSC32) {
-        uint64_t pairs = 0;
-        for (const auto &ch : c->ising)
-            pairs += (uint64_t)ch.W * (ch.Ly >> 1);
-        while (c->row_pairs < kMaxRowPairs && pairs / (2 * c->row_pairs) >= kRowPairThreads)
-            c->row_pairs *= 2;
-    }
+    uint64_t pairs = 0;
+    for (const auto &ch : c->ising)
+        pairs += (uint64_t)(c->layout == MC_LAYOUT_INT8 ? ch.Lx / 8 : ch.W) * (ch.Ly >> 1);
+    c->row_pairs = c->layout == MC_LAYOUT_INT8 && pairs < kInt8Pairs ? 0 : 1;
+    while (c->row_pairs && c->row_pairs < kMaxRowPairs && pairs / (2 * c->row_pairs) >= kRowPairThreads)
+        c->row_pairs *= 2;
     c->block_start.assign(c->n_chains + 1, 0);
     uint32_t acc = 0;
     for (int k = 0; k < c->n_chains; ++k) {
@@ -448,6 +458,36 @@ bool ising_resident_fits(const mc_ctx *c, int *smem_bytes)
     return need + 1024 <= (size_t)optin;
 }
 
+// Automatic choice between the resident and the grid launches: estimated us per
+// sweep, from times measured over L = 16 .. 384 and 1 .. 4096 chains.  A resident
+// chain costs its sites at one CTA's rate, and chains beyond one per SM queue up; a
+// grid sweep costs two chained launches and all sites at the chip's rate.
+// Resident / grid, measured us per measured sweep: int8 64^2 x 1 chain 1.9 / 3.4,
+// 96^2 x 1 3.5 / 3.4, 128^2 x 1 4.7 / 3.5, 128^2 x 48 4.8 / 5.3, 256^2 x 1 14.2 / 3.4, 256^2 x 152
+// 14.7 / 18.9, 64^2 x 4096 26 / 63, 130^2 (ragged groups) x 1 7.3 / 5.3; 32-spin words 128^2
+// x 1 4.3 / 5.4, 256^2 x 1 8.0 / 6.5, 256^2 x 152 8.3 / 10.3, 384^2 x 48 17.9 / 10.3.
+bool ising_resident_auto(const mc_ctx *c)
+{
+    if (!ising_resident_fits(c, nullptr))
+        return false;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    double one = 0.0, all = 0.0;
+    bool ragged = false;
+    for (const auto &ch : c->ising) {
+        const double sites = (double)ch.Lx * ch.Ly;
+        one = sites > one ? sites : one;
+        all += sites;
+        ragged = ragged || (ch.Lx & 7u) != 0;
+    }
+    const double rounds = (double)((c->n_chains + sms - 1) / sms);
+    if (c->layout == MC_LAYOUT_MSC32)
+        return std::max(4.2, 0.122e-3 * one * rounds) <= 5.4 + 0.6e-6 * all;
+    return ragged ? 1.0 + 0.38e-3 * one * rounds <= 4.0 + 4.5e-6 * all
+                  : 1.0 + 0.22e-3 * one * rounds <= 3.4 + 2.0e-6 * all;
+}
+
 // Threads of a resident CTA: the work units of the largest chain (int8: groups
 // of four same-colour sites; MSC32: row pairs) rounded up to a warp, at most
 // the block size -- the caller's (mc_set_mode), else 1024 when every chain has
@@ -463,7 +503,7 @@ static int resident_threads(const mc_ctx *c)
 {
     uint32_t units = 0;
     for (const auto &ch : c->ising) {
-        const uint32_t u = c->layout == MC_LAYOUT_INT8 ? ((((ch.Lx * ch.Ly) >> 1) + 3) >> 2) : ch.W * (ch.Ly >> 1);
+        const uint32_t u = c->layout == MC_LAYOUT_INT8 ? int8_units<false>(ch, 1) : ch.W * (ch.Ly >> 1);
         units = u > units ? u : units;
     }
     int dev = 0, sms = 0;
@@ -474,6 +514,11 @@ static int resident_threads(const mc_ctx *c)
     return t < 32 ? 32 : (t < cap ? t : cap);
 }
 
+static void (*resident_kernel(const mc_ctx *c))(SweepArgs, uint32_t, uint32_t)
+{
+    return c->layout == MC_LAYOUT_INT8 ? k_resident<MC_LAYOUT_INT8> : k_resident<MC_LAYOUT_MSC32>;
+}
+
 // Raise the dynamic shared-memory limit of the resident kernels (outside any
 // graph capture).
 cudaError_t ising_prepare_resident(mc_ctx *c)
@@ -481,10 +526,7 @@ cudaError_t ising_prepare_resident(mc_ctx *c)
     int smem = 0;
     if (!ising_resident_fits(c, &smem))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_resident<MC_LAYOUT_INT8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_resident<MC_LAYOUT_MSC32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return e;
+    return cudaFuncSetAttribute(resident_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t ising_init_launch(mc_ctx *c, const mc_chain_desc *desc)
@@ -520,7 +562,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     a.state = c->d_state;
     a.cap = c->cap;
     a.tries = nullptr;
-    a.row_pairs = (uint32_t)c->row_pairs;
+    a.row_pairs = (uint32_t)std::max(c->row_pairs, 1);
     a.release = 1;
     if (mode == MC_MODE_RESIDENT) {
         int smem = 0;
@@ -530,10 +572,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
         cudaError_t e = prof_begin(c);
         if (e != cudaSuccess)
             return e;
-        if (c->layout == MC_LAYOUT_INT8)
-            k_resident<MC_LAYOUT_INT8><<<c->n_chains, threads, smem, c->ls>>>(a, (uint32_t)n, (uint32_t)every);
-        else
-            k_resident<MC_LAYOUT_MSC32><<<c->n_chains, threads, smem, c->ls>>>(a, (uint32_t)n, (uint32_t)every);
+        resident_kernel(c)<<<c->n_chains, threads, smem, c->ls>>>(a, (uint32_t)n, (uint32_t)every);
         e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
@@ -547,17 +586,16 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
             cudaError_t e = prof_begin(c);
             if (e != cudaSuccess)
                 return e;
-            if (c->layout == MC_LAYOUT_INT8) {
-                if (colour == 0)
-                    launch_half_sweep<0, MC_LAYOUT_INT8>(c, a);
-                else
-                    launch_half_sweep<1, MC_LAYOUT_INT8>(c, a);
-            } else {
-                if (colour == 0)
-                    launch_half_sweep<0, MC_LAYOUT_MSC32>(c, a);
-                else
-                    launch_half_sweep<1, MC_LAYOUT_MSC32>(c, a);
-            }
+            const bool pairs = c->row_pairs != 0;
+            if (c->layout == MC_LAYOUT_MSC32)
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_MSC32, true>
+                             : launch_half_sweep<1, MC_LAYOUT_MSC32, true>)(c, a);
+            else if (pairs)
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, true>
+                             : launch_half_sweep<1, MC_LAYOUT_INT8, true>)(c, a);
+            else
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, false>
+                             : launch_half_sweep<1, MC_LAYOUT_INT8, false>)(c, a);
             e = prof_end(c);
             if (e != cudaSuccess)
                 return e;

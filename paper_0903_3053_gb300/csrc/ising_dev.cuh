@@ -40,8 +40,8 @@ __device__ __forceinline__ void block_sum2(uint32_t &a, uint32_t &b)
 }
 
 // ------------------------------------------------------------------ int8 layout
-// Two forms of the same update; both visit the (up to four) sites of colour C
-// that share Philox block g.
+// Two forms of the same update of the (up to four) sites of colour C that share
+// a Philox block.
 //
 // int8_group, any even extents: the sites are consecutive in the colour's
 // raster order and may run over the end of a row, so the row and column are
@@ -103,27 +103,14 @@ __device__ __forceinline__ void ge_chain2(uint32_t &g2, uint32_t &g4, uint32_t r
 // whose xor is 0x00 or 0xFE: the anti-aligned neighbours are counted by
 // bitwise adders on all four sites at once, as in the 32-spin words, and the
 // accept bits of ge_chain2 are spread to bit 1 of the bytes by a multiplication.
-// Three 8-byte loads and one byte (the in-row neighbour of the group's first or
-// last site) replace the 20 byte loads of int8_group.  The other colour's
-// bytes of the 8-byte store hold the values they had.  Bound by the schedulers'
-// dispatch (Philox is 72 of its ~130 cycles per warp and group); against the
-// byte-wise form, measured through the library's calls: 100 measured sweeps of one
-// 64^2 chain 307 -> 194 us, 10 sweeps of 4096 such chains 543 -> 388 us (resident
-// mode), 50 measured sweeps of a 1024 x 512 chain 352 -> 272 us (grid mode, two
-// launches per sweep), the configuration and series read back each time.
-template <int C, bool MEASURE, int LD = kLdPlain>
-__device__ __forceinline__ void int8_oct(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t y,
-                                         uint32_t gx, uint32_t sweep, uint32_t &anti, uint32_t &up)
+// par: parity of the sites' x; w, wu, wd: the eight bytes in the row and in the rows
+// above and below; edge: the in-row neighbour outside the eight bytes.  Returns
+// whether a site flipped; w is then the row's new bytes.
+template <bool MEASURE>
+__device__ __forceinline__ bool int8_oct(uint32_t par, uint2 &w, uint2 wu, uint2 wd, uint32_t edge, const uint4 &r,
+                                         const IsingChain &ch, uint32_t &anti, uint32_t &up)
 {
-    const uint32_t Lx = ch.Lx, Ly = ch.Ly, par = (y + C) & 1u, x0 = 8 * gx; // par: parity of the sites' x
     const uint32_t selA = par ? 0x7531u : 0x6420u, selO = par ? 0x6420u : 0x7531u;
-    int8_t *row = s + y * Lx;
-    const uint2 w = lat_load<LD>(reinterpret_cast<const uint2 *>(row + x0));
-    const uint2 wu = lat_load<LD>(reinterpret_cast<const uint2 *>(s + dec_wrap(y, Ly) * Lx + x0));
-    const uint2 wd = lat_load<LD>(reinterpret_cast<const uint2 *>(s + inc_wrap(y, Ly) * Lx + x0));
-    const uint32_t xs = par ? (x0 + 8 == Lx ? 0u : x0 + 8) : (x0 == 0 ? Lx - 1 : x0 - 1);
-    const uint32_t edge = (uint8_t)lat_load<LD>(row + xs);
-    const uint4 r = philox4x32_10(make_uint4(y * (Lx >> 3) + gx, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
     uint32_t g2 = 0, g4 = 0;
     ge_chain2(g2, g4, r.w, 0u - ch.T2, 0u - ch.T4);
     ge_chain2(g2, g4, r.z, 0u - ch.T2, 0u - ch.T4);
@@ -139,15 +126,10 @@ __device__ __forceinline__ void int8_oct(int8_t *s, const IsingChain &ch, const 
     const uint32_t x = a1 ^ a2 ^ a3, m = (a1 & a2) | (a3 & (a1 | a2)); // 2 m + x = a1 + a2 + a3
     // two or more anti-aligned, or r < T4, or one anti-aligned and r < T2 (T4 <= T2)
     const uint32_t f = ((x & a4) | m | ~G4 | ((x ^ a4) & ~G2)) & 0x02020202u;
-    const uint32_t nv = sv ^ (f * 0x7Fu); // 0x02 -> 0xFE per byte
-    if (f != 0) {
-        uint2 o;
-        o.x = __byte_perm(nv, ns, par ? 0x1504u : 0x5140u);
-        o.y = __byte_perm(nv, ns, par ? 0x3726u : 0x7362u);
-        *reinterpret_cast<uint2 *>(row + x0) = o;
-    }
+    const uint32_t fe = f * 0x7Fu, nv = sv ^ fe; // 0x02 -> 0xFE per byte
+    w.x = __byte_perm(nv, ns, par ? 0x1504u : 0x5140u);
+    w.y = __byte_perm(nv, ns, par ? 0x3726u : 0x7362u);
     if (MEASURE) { // 0xFE = -2 per anti-aligned bond, +-1 per spin
-        const uint32_t fe = f * 0x7Fu;
         int bonds = __dp4a((int)(a1 ^ fe), 0x01010101, 0);
         bonds = __dp4a((int)(a2 ^ fe), 0x01010101, bonds);
         bonds = __dp4a((int)(a3 ^ fe), 0x01010101, bonds);
@@ -155,18 +137,92 @@ __device__ __forceinline__ void int8_oct(int8_t *s, const IsingChain &ch, const 
         anti += (uint32_t)(-bonds) >> 1;
         up += (uint32_t)(8 + __dp4a((int)nv, 0x01010101, __dp4a((int)ns, 0x01010101, 0))) >> 1;
     }
+    return f != 0;
 }
 
-// Philox group g of a chain, in the form its rows allow (uniform over the chain).
+// One group: column gx of row y.  Three 8-byte loads and one byte replace the 20 byte
+// loads of int8_group; the other colour's bytes of the 8-byte store hold the values
+// they had.  Bound by the schedulers' dispatch (Philox is 72 of its ~200 cycles per
+// warp and group); against the byte-wise form 100 measured sweeps of one 64^2 chain
+// 307 -> 194 us, 10 sweeps of 4096 such chains 543 -> 388 us (resident mode,
+// configuration and series read back each time).
 template <int C, bool MEASURE, int LD = kLdPlain>
-__device__ __forceinline__ void int8_unit(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t g,
-                                          uint32_t sweep, uint32_t &anti, uint32_t &up)
+__device__ __forceinline__ void int8_row(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t y,
+                                         uint32_t gx, uint32_t sweep, uint32_t &anti, uint32_t &up)
+{
+    const uint32_t Lx = ch.Lx, Ly = ch.Ly, par = (y + C) & 1u, x0 = 8 * gx;
+    int8_t *row = s + y * Lx;
+    uint2 w = lat_load<LD>(reinterpret_cast<const uint2 *>(row + x0));
+    const uint2 wu = lat_load<LD>(reinterpret_cast<const uint2 *>(s + dec_wrap(y, Ly) * Lx + x0));
+    const uint2 wd = lat_load<LD>(reinterpret_cast<const uint2 *>(s + inc_wrap(y, Ly) * Lx + x0));
+    const uint32_t xs = par ? (x0 + 8 == Lx ? 0u : x0 + 8) : (x0 == 0 ? Lx - 1 : x0 - 1);
+    const uint32_t edge = (uint8_t)lat_load<LD>(row + xs);
+    const uint4 r = philox4x32_10(make_uint4(y * (Lx >> 3) + gx, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+    if (int8_oct<MEASURE>(par, w, wu, wd, edge, r, ch, anti, up))
+        *reinterpret_cast<uint2 *>(row + x0) = w;
+}
+
+// The groups of column gx in the row pairs y = 2 yy, 2 yy + 1, yy0 <= yy < yy1.  A
+// pair's rows have fixed parities, so the byte selectors are constants, and each
+// row is loaded once; a thread's prologue is spread over several groups.  For
+// large grid launches (an 8192^2 chain 141 -> 81 us per measured sweep, 4096^2 37
+// -> 25); with fewer threads than the chip holds int8_row is faster (1024 x 512
+// 3.5 against 4.0 us), as it is in shared memory (4096 chains of 64^2 26 against 28).
+template <int C, bool MEASURE, int LD = kLdPlain>
+__device__ __forceinline__ void int8_row_pairs(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t yy0,
+                                               uint32_t yy1, uint32_t gx, uint32_t sweep, uint32_t &anti, uint32_t &up)
+{
+    const uint32_t Lx = ch.Lx, Ly = ch.Ly, W8 = Lx >> 3, x0 = 8 * gx;
+    const uint32_t xl = x0 == 0 ? Lx - 1 : x0 - 1, xr = x0 + 8 == Lx ? 0u : x0 + 8;
+    const uint32_t e0 = C ? xr : xl, e1 = C ? xl : xr; // row 2 yy holds sites x = 2 j + C, row 2 yy + 1 x = 2 j + 1 - C
+    uint32_t y0 = 2 * yy0, blk = y0 * W8 + gx;
+    int8_t *row = s + y0 * Lx;
+    const auto oct = [&](const int8_t *p) { return lat_load<LD>(reinterpret_cast<const uint2 *>(p + x0)); };
+    uint2 wu = oct(s + dec_wrap(y0, Ly) * Lx), w0 = oct(row);
+#pragma unroll 1
+    for (uint32_t yy = yy0; yy < yy1; ++yy) {
+        int8_t *row1 = row + Lx, *row2 = y0 + 2 == Ly ? s : row1 + Lx;
+        uint2 w1 = oct(row1);
+        const uint2 wd = oct(row2);
+        const uint32_t b0 = (uint8_t)lat_load<LD>(row + e0), b1 = (uint8_t)lat_load<LD>(row1 + e1);
+        const uint4 r0 = philox4x32_10(make_uint4(blk, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+        const uint4 r1 = philox4x32_10(make_uint4(blk + W8, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+        const uint2 v0 = w0; // the other colour's bytes of row 2 yy, neighbours of row 2 yy + 1
+        const uint2 v1 = w1;
+        if (int8_oct<MEASURE>(C, w0, wu, v1, b0, r0, ch, anti, up))
+            *reinterpret_cast<uint2 *>(row + x0) = w0;
+        if (int8_oct<MEASURE>(1 - C, w1, v0, wd, b1, r1, ch, anti, up))
+            *reinterpret_cast<uint2 *>(row1 + x0) = w1;
+        wu = v1;
+        w0 = wd;
+        y0 += 2;
+        blk += 2 * W8;
+        row += 2 * Lx;
+    }
+}
+
+// Work units of a chain's half-sweep: Philox groups, or (PAIRS, rows of whole
+// groups) `row_pairs` row pairs of a group column; and unit u of the chain.
+template <bool PAIRS>
+__host__ __device__ __forceinline__ uint32_t int8_units(const IsingChain &ch, uint32_t row_pairs)
+{
+    if (PAIRS && (ch.Lx & 7u) == 0)
+        return ((ch.Ly >> 1) + row_pairs - 1) / row_pairs * (ch.Lx >> 3);
+    return (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
+}
+template <int C, bool MEASURE, bool PAIRS = false, int LD = kLdPlain>
+__device__ __forceinline__ void int8_unit(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t u,
+                                          uint32_t row_pairs, uint32_t sweep, uint32_t &anti, uint32_t &up)
 {
     if ((ch.Lx & 7u) == 0) {
-        const uint32_t y = fast_div(4 * g, ch.div_half);
-        int8_oct<C, MEASURE, LD>(s, ch, ks, y, g - y * (ch.Lx >> 3), sweep, anti, up);
+        const uint32_t q = fast_div(4 * u, ch.div_half), gx = u - q * (ch.Lx >> 3); // u / (Lx / 8)
+        if (PAIRS)
+            int8_row_pairs<C, MEASURE, LD>(s, ch, ks, q * row_pairs, min(ch.Ly >> 1, (q + 1) * row_pairs), gx, sweep,
+                                           anti, up);
+        else
+            int8_row<C, MEASURE, LD>(s, ch, ks, q, gx, sweep, anti, up);
     } else {
-        int8_group<C, MEASURE, LD>(s, ch, ks, g, sweep, anti, up);
+        int8_group<C, MEASURE, LD>(s, ch, ks, u, sweep, anti, up);
     }
 }
 

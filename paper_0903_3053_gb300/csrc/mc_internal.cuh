@@ -152,7 +152,7 @@ struct SweepArgs {
     int measure;                 // 1: this sweep is measured
     uint32_t rec_k;              // index of this record within the running call
     uint8_t *tries;              // SU(2) try record base, or nullptr
-    uint32_t row_pairs;          // MSC32 grid mode: row pairs per thread
+    uint32_t row_pairs;          // Ising grid mode: row pairs per thread
     int release;                 // let the next kernel's blocks in once this one's are past chain_wait
 };
 
@@ -190,7 +190,7 @@ struct mc_ctx {
     std::vector<mc_chain_desc> desc;
     std::vector<uint32_t> block_start, meas_start;
     uint32_t grid_blocks = 0, meas_blocks = 0;
-    int row_pairs = 1;                   // MSC32 grid mode: row pairs per thread
+    int row_pairs = 1;                   // Ising grid mode: row pairs per thread (0: int8, one group)
     // run bookkeeping
     long long sweeps_done = 0;
     long long rec_written = 0, rec_read = 0;
@@ -217,6 +217,7 @@ cudaError_t ising_measure_launch(mc_ctx *c, int chain, DevRecord *out);
 cudaError_t ising_config_io(mc_ctx *c, int chain, int fmt, void *dev_buf, bool to_lattice);
 size_t ising_config_bytes(const IsingChain &ch, int fmt);
 bool ising_resident_fits(const mc_ctx *c, int *smem_bytes);
+bool ising_resident_auto(const mc_ctx *c);
 cudaError_t ising_prepare_resident(mc_ctx *c);
 void ising_plan_grid(mc_ctx *c);
 

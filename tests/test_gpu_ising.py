@@ -331,22 +331,26 @@ def test_full_size_sampled_sites(L, layout):
     b.close()
 
 
-@pytest.mark.parametrize("shape", [(8192, 8198), (64, 1 << 20), (16384, 8202)])
-def test_msc_several_row_pairs_per_thread(shape):
+@pytest.mark.parametrize("shape,layout", [
+    ((8192, 8198), mc.MC_LAYOUT_MSC32), ((64, 1 << 20), mc.MC_LAYOUT_MSC32), ((16384, 8202), mc.MC_LAYOUT_MSC32),
+    ((1000, 1050), mc.MC_LAYOUT_INT8), ((8, 1 << 18), mc.MC_LAYOUT_INT8), ((4104, 4098), mc.MC_LAYOUT_INT8),
+    ((8192, 4102), mc.MC_LAYOUT_INT8)])
+def test_several_row_pairs_per_thread(shape, layout):
     """Lattices large enough for 2 or 4 row pairs per thread, with a number of row
-    pairs that is no multiple of it (8198, 8202 rows) or one word per row: sites of
+    pairs that is no multiple of it (8198, 8202, ... rows), one word or group per row, or one row pair (int8): sites of
     the first and last rows and columns and random ones against the oracle's local
     rule, and the exact observables."""
     Lx, Ly = shape
-    b = mc.Batch([mc.ising(shape, 0.42, seed=8, chain_id=2)], layout=mc.MC_LAYOUT_MSC32, series_capacity=4)
+    b = mc.Batch([mc.ising(shape, 0.42, seed=8, chain_id=2)], layout=layout, series_capacity=4)
     b.sweep(2, 0)
     pre = b.get_config(0)
     b.sweep(1, 1)
     post = b.get_config(0)
     rec = b.read_series()
     rng = np.random.default_rng(1)
+    cols = np.concatenate([np.arange(8), Lx - 8 + np.arange(8), rng.integers(0, Lx, 48)])
     ys = np.concatenate([np.repeat([0, 1, 2, 3, Ly - 4, Ly - 3, Ly - 2, Ly - 1], 64), rng.integers(0, Ly, 2000)])
-    xs = np.concatenate([np.tile(np.concatenate([np.arange(32), Lx - 32 + np.arange(32)]), 8), rng.integers(0, Lx, 2000)])
+    xs = np.concatenate([np.tile(cols, 8), rng.integers(0, Lx, 2000)])
     sites = ys.astype(np.int64) * Lx + xs
     want = oracle.ising_check_sites(pre, post, 0.42, 8, 2, 2, sites)
     np.testing.assert_array_equal(post.reshape(-1)[sites], want)
