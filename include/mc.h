@@ -234,11 +234,13 @@ MC_API mc_status mc_profile_read(mc_ctx *ctx, int64_t *launches, double *total_m
 MC_API mc_status mc_philox_rate(int32_t blocks, int32_t threads, uint32_t iters, uint64_t seed, uint32_t *dev_out,
                                 void *cuda_stream);
 
-/* ---- Batched chains in one persistent launch ---------------------------------
+/* ---- Batched chains advanced together ----------------------------------------
  * A group advances every chain of up to 16 contexts (any mix of Ising layouts
- * and SU(2)) with ONE persistent kernel launch per call, replayed from a CUDA
- * graph -- the paper runs independent parameter points side by side (Sec. 3);
- * here they share one GPU.  The grid is a set of thread-block clusters; a
+ * and SU(2)) in one call -- the paper runs independent parameter points side by
+ * side (Sec. 3); here they share one GPU.  By default (split_cost < 0) the
+ * members' own launches run side by side, each member in its own mode.  With
+ * split_cost >= 0 all chains run in ONE persistent kernel launch per call,
+ * replayed from a CUDA graph: the grid is a set of thread-block clusters; a
  * host-computed longest-first schedule gives each cluster a list of rounds,
  * each either one large chain split over the cluster's CTAs (phases separated
  * by the hardware cluster barrier) or up to cluster-size small chains, one per
@@ -257,9 +259,11 @@ MC_API mc_status mc_group_create(mc_group **out, int32_t n_ctx, mc_ctx *const *c
  * mc_group_sweep with MC_ECUDA); threads_per_block a
  * multiple of 32 in [64, 256] (0 = keep; default 256); a chain whose estimated
  * cost (MSC spin-flip units per sweep: Ising int8 2 per site, MSC 1 per site,
- * SU(2) 60 per link) is at least split_cost is shared by a whole cluster
- * (split_cost < 0: one CTA's fair share of the total).  Invalidates the
- * schedule; the next mc_group_sweep recomputes it. */
+ * SU(2) 60 per link) is at least split_cost is shared by a whole cluster.
+ * split_cost < 0 (the default): the members' own launches side by side; the
+ * schedule is then the persistent launch's with one CTA's fair share of the
+ * total as the cost that is shared.  Invalidates the schedule; the next
+ * mc_group_sweep recomputes it. */
 MC_API mc_status mc_group_configure(mc_group *g, int32_t cluster_size, int32_t threads_per_block, double split_cost);
 /* Advance every member chain by n_sweeps (async), recording as mc_sweep does. */
 MC_API mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every);

@@ -1,7 +1,14 @@
-// batch.cu -- many uneven chains (Ising in either layout, SU(2)) advanced by
-// ONE persistent kernel launch per call, captured in a CUDA graph.
+// batch.cu -- many uneven chains (Ising in either layout, SU(2)) advanced
+// together.
 //
-// A group borrows the chains of several contexts.  The host computes a
+// A group borrows the chains of several contexts.  By default the members' own
+// launches run side by side on the members' private streams.  us per measured
+// sweep against the persistent launch below (clusters of 8, 256 threads): 256 Ising +
+// 64 SU(2) chains 322 against 364 (the SU(2) phases alone take 280), 64 + 16 58
+// against 237, 8 + 2 21 against 83, 256 + 2 64 against 100, 8 + 64 193 against 292 -- the
+// persistent kernel holds 16 warps per SM, and its phases wait at cluster barriers
+// where chained launches overlap.  A split cost >= 0 (mc_group_configure) asks for
+// ONE persistent kernel launch per call, captured in a CUDA graph: the host computes a
 // schedule once (longest-processing-time first): the grid is a set of
 // thread-block clusters of C CTAs, and each cluster walks a list of rounds.  A
 // round is either
@@ -272,7 +279,7 @@ struct mc_group {
     size_t max_rounds = 0, max_clusters = 0;
     // configuration and schedule
     int C = 4, threads = 256;
-    double split_cost = -1.0; // items at least this costly are shared by a cluster (< 0: automatic)
+    double split_cost = -1.0; // >= 0: persistent launch, items at least this costly shared by a cluster
     int n_clusters = 0;
     std::vector<uint32_t> round_start;
     std::vector<int32_t> rounds;
@@ -596,6 +603,28 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
         mc_status s = plan(g);
         if (s != MC_OK)
             return s;
+    }
+    if (g->split_cost < 0.0) {
+        // Automatic: the members' own launches, side by side.  The SU(2) members, whose
+        // chains of launches are the longest, first.
+        mc_status st = MC_OK;
+        size_t begun = 0;
+        std::vector<mc_ctx *> order(g->members);
+        std::stable_partition(order.begin(), order.end(), [](const mc_ctx *c) { return c->kind == MC_KIND_SU2; });
+        for (; begun < order.size() && st == MC_OK; ++begun)
+            st = sweep_begin(order[begun], n_sweeps, measure_every);
+        for (size_t i = 0; i < begun; ++i) {
+            const mc_status f = sweep_end(order[i]);
+            if (st == MC_OK)
+                st = f;
+        }
+        if (st != MC_OK)
+            return st;
+        for (mc_ctx *c : g->members) {
+            c->sweeps_done += n_sweeps;
+            c->rec_written += recs;
+        }
+        return MC_OK;
     }
     const auto key = std::make_tuple((long long)n_sweeps, (int)measure_every);
     auto it = g->graphs.find(key);

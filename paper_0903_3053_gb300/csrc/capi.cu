@@ -118,7 +118,7 @@ bool validate(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t ca
 }
 
 struct Plan {
-    size_t state, chains, block_start, meas_start, series, scratch_rec, partials, staging, tries, lattice, total;
+    size_t state, chains, block_start, block_chain, block_chain_count, meas_start, series, scratch_rec, partials, staging, tries, lattice, total;
     size_t staging_bytes;
     std::vector<size_t> lat_off, tries_off;
 };
@@ -142,6 +142,17 @@ Plan make_plan(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t c
     p.state = take(sizeof(DevState));
     p.chains = take((size_t)n * (kind == MC_KIND_ISING ? sizeof(IsingChain) : sizeof(Su2Chain)));
     p.block_start = take((size_t)(n + 1) * sizeof(uint32_t));
+    // blocks of a grid-mode launch at the smallest block size (32 threads) and one unit per thread
+    p.block_chain_count = 0;
+    for (int k = 0; k < n; ++k) {
+        const mc_chain_desc &d = chains[k];
+        const size_t sites = (size_t)d.L[0] * d.L[1] * (kind == MC_KIND_ISING ? 1 : (size_t)d.L[2] * d.L[3]);
+        const size_t units = kind == MC_KIND_SU2 ? sites / 2 : layout == MC_LAYOUT_INT8 ? (sites / 2 + 3) / 4 : sites / 128;
+        p.block_chain_count += (units + 31) / 32;
+    }
+    if (n == 1)
+        p.block_chain_count = 0;
+    p.block_chain = take(p.block_chain_count * sizeof(uint32_t));
     p.meas_start = take((size_t)(n + 1) * sizeof(uint32_t));
     p.series = take((size_t)n * (size_t)cap * sizeof(DevRecord));
     p.scratch_rec = take((size_t)n * sizeof(DevRecord));
@@ -292,6 +303,13 @@ mc_status upload_tables(mc_ctx *c)
         su2_plan_grid(c);
     cudaError_t e = cudaMemcpyAsync(c->d_block_start, c->block_start.data(), c->block_start.size() * 4,
                                     cudaMemcpyHostToDevice, c->stream);
+    c->block_chain.clear();
+    if (c->n_chains > 1)
+        for (int k = 0; k < c->n_chains; ++k)
+            c->block_chain.insert(c->block_chain.end(), c->block_start[k + 1] - c->block_start[k], (uint32_t)k);
+    if (e == cudaSuccess && !c->block_chain.empty())
+        e = cudaMemcpyAsync(c->d_block_chain, c->block_chain.data(), c->block_chain.size() * 4, cudaMemcpyHostToDevice,
+                            c->stream);
     if (e == cudaSuccess && !c->meas_start.empty())
         e = cudaMemcpyAsync(c->d_meas_start, c->meas_start.data(), c->meas_start.size() * 4, cudaMemcpyHostToDevice,
                             c->stream);
@@ -327,28 +345,22 @@ bool capturing(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
-// `n` sweeps and the advance of the run state: launched one by one the first
-// time a (n, every, mode, ...) is asked for, captured into a graph the second time
-// and replayed from then on.  A graph pays for itself only when replayed: recording
-// and instantiating one costs ~3 us per launch in it, a launch ~2 us (50 measured
-// sweeps of a 1024 x 512 chain on a new context, configuration and series read
-// back: 551 -> 283 us; 20 of 8^4 at four beta 1159 -> 597).
-mc_status run_chunk(mc_ctx *c, long long n, int every, int mode)
+// `n` sweeps and the advance of the run state on the context's private stream
+// (capture is not permitted on the legacy default stream a caller may pass):
+// launched one by one the first time a (n, every, mode, ...) is asked for, captured
+// into a graph the second time and replayed from then on.  A graph pays for itself
+// only when replayed: recording and instantiating one costs ~3 us per launch in it, a
+// launch ~2 us (50 measured sweeps of a 1024 x 512 chain on a new context,
+// configuration and series read back: 551 -> 283 us; 20 of 8^4 at four beta 1159 ->
+// 597).
+mc_status launch_chunk(mc_ctx *c, long long n, int every, int mode)
 {
-    if (c->profiling) { // direct launches, each sweep kernel bracketed by events
-        cudaError_t ek = enqueue_chunk(c, n, every, mode);
-        if (ek != cudaSuccess)
-            return cuda_fail(ek, "enqueue sweep kernels");
-        return MC_OK;
-    }
-    // Launched, recorded and replayed on a private stream (capture is not
-    // permitted on the legacy default stream a caller may pass), fenced with
-    // events against the caller's stream so stream order is preserved.
     const auto key = std::make_tuple(n, every, mode, c->threads, c->record_tries, c->n_or);
     auto it = c->graphs.find(key);
-    if (it == c->graphs.end() && c->swept.count(key) && !capturing(c->stream)) {
+    cudaError_t e = cudaSuccess;
+    if (it == c->graphs.end() && c->swept.count(key) && !capturing(c->cap_stream)) {
         cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
+        e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess)
             return cuda_fail(e, "begin graph capture");
         c->ls = c->cap_stream;
@@ -369,28 +381,15 @@ mc_status run_chunk(mc_ctx *c, long long n, int every, int mode)
             return cuda_fail(e, "instantiate graph");
         it = c->graphs.emplace(key, ge).first;
     }
-    cudaError_t e = cudaEventRecord(c->fence_in, c->stream);
-    if (e == cudaSuccess)
-        e = cudaStreamWaitEvent(c->cap_stream, c->fence_in, 0);
-    if (e == cudaSuccess) {
-        if (it != c->graphs.end()) {
-            e = cudaGraphLaunch(it->second, c->cap_stream);
-        } else {
-            c->ls = c->cap_stream;
-            e = enqueue_chunk(c, n, every, mode);
-            c->ls = c->stream;
-            c->swept.insert(key);
-        }
+    if (it != c->graphs.end()) {
+        e = cudaGraphLaunch(it->second, c->cap_stream);
+    } else {
+        c->ls = c->cap_stream;
+        e = enqueue_chunk(c, n, every, mode);
+        c->ls = c->stream;
+        c->swept.insert(key);
     }
-    // also after a failed launch: what was enqueued stays ordered before the caller's next work
-    cudaError_t ef = cudaEventRecord(c->fence_out, c->cap_stream);
-    if (ef == cudaSuccess)
-        ef = cudaStreamWaitEvent(c->stream, c->fence_out, 0);
-    if (e == cudaSuccess)
-        e = ef;
-    if (e != cudaSuccess)
-        return cuda_fail(e, "launch sweeps");
-    return MC_OK;
+    return e == cudaSuccess ? MC_OK : cuda_fail(e, "launch sweeps");
 }
 
 const char *kVersion = "mc-gb300 1.0 (sm_103a)";
@@ -412,6 +411,53 @@ static cudaError_t prof_record(mc_ctx *c)
 void set_last_error(const std::string &msg) { g_err = msg; }
 cudaError_t prof_begin(mc_ctx *c) { return c->profiling ? prof_record(c) : cudaSuccess; }
 cudaError_t prof_end(mc_ctx *c) { return c->profiling ? prof_record(c) : cudaSuccess; }
+
+mc_status sweep_begin(mc_ctx *c, long long n, int every)
+{
+    const int mode = resolve_mode(c);
+    cudaError_t e = cudaSuccess;
+    if (mode == MC_MODE_RESIDENT)
+        e = c->kind == MC_KIND_ISING ? ising_prepare_resident(c) : su2_prepare_resident(c);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "configure resident kernel");
+    if (!c->profiling) {
+        e = cudaEventRecord(c->fence_in, c->stream);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(c->cap_stream, c->fence_in, 0);
+        if (e != cudaSuccess)
+            return cuda_fail(e, "order the sweeps after the caller's stream");
+    }
+    // Split long calls into replayable chunks whose length is a multiple of
+    // measure_every, so the record cadence repeats exactly.
+    long long chunk = mode == MC_MODE_RESIDENT ? 4096 : 256;
+    if (every > 0)
+        chunk = std::max<long long>(every, chunk / every * every);
+    mc_status s = MC_OK;
+    for (long long left = n; left > 0 && s == MC_OK;) {
+        const long long m = std::min(left, chunk);
+        if (c->profiling) { // direct launches, each sweep kernel bracketed by events
+            e = enqueue_chunk(c, m, every, mode);
+            s = e == cudaSuccess ? MC_OK : cuda_fail(e, "enqueue sweep kernels");
+        } else {
+            s = launch_chunk(c, m, every, mode);
+        }
+        left -= m;
+    }
+    if (!c->profiling) { // also after a failed launch: what was enqueued stays ordered before the caller's next work
+        e = cudaEventRecord(c->fence_out, c->cap_stream);
+        if (e != cudaSuccess && s == MC_OK)
+            s = cuda_fail(e, "record the end of the sweeps");
+    }
+    return s;
+}
+
+mc_status sweep_end(mc_ctx *c)
+{
+    if (c->profiling)
+        return MC_OK;
+    const cudaError_t e = cudaStreamWaitEvent(c->stream, c->fence_out, 0);
+    return e == cudaSuccess ? MC_OK : cuda_fail(e, "order the caller's stream after the sweeps");
+}
 }  // namespace mc
 
 extern "C" {
@@ -476,6 +522,7 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
     c->d_state = reinterpret_cast<DevState *>(c->ws + p.state);
     c->d_chains = c->ws + p.chains;
     c->d_block_start = reinterpret_cast<uint32_t *>(c->ws + p.block_start);
+    c->d_block_chain = reinterpret_cast<uint32_t *>(c->ws + p.block_chain);
     c->d_meas_start = reinterpret_cast<uint32_t *>(c->ws + p.meas_start);
     c->d_series = reinterpret_cast<DevRecord *>(c->ws + p.series);
     c->d_scratch_rec = reinterpret_cast<DevRecord *>(c->ws + p.scratch_rec);
@@ -621,27 +668,10 @@ mc_status mc_sweep(mc_ctx *c, int64_t n_sweeps, int32_t measure_every)
         return fail(MC_EINVAL, "measurement ring buffer would overflow: read the series first or raise capacity");
     if (c->sweeps_done + n_sweeps > 0xFFFFFFFFll)
         return fail(MC_EINVAL, "sweep counter would exceed 2^32 (the Philox sweep word)");
-    const int mode = resolve_mode(c);
-    if (mode == MC_MODE_RESIDENT) {
-        cudaError_t e = c->kind == MC_KIND_ISING ? ising_prepare_resident(c) : su2_prepare_resident(c);
-        if (e != cudaSuccess)
-            return cuda_fail(e, "configure resident kernel");
-    }
-    // Split long calls into replayable chunks whose length is a multiple of
-    // measure_every, so the record cadence repeats exactly.
-    long long chunk = 256;
-    if (mode == MC_MODE_RESIDENT)
-        chunk = 4096;
-    if (measure_every > 0)
-        chunk = std::max<long long>(measure_every, chunk / measure_every * measure_every);
-    long long left = n_sweeps;
-    while (left > 0) {
-        const long long m = std::min(left, chunk);
-        mc_status s = run_chunk(c, m, measure_every, mode);
-        if (s != MC_OK)
-            return s;
-        left -= m;
-    }
+    const mc_status s = sweep_begin(c, n_sweeps, measure_every);
+    const mc_status f = sweep_end(c);
+    if (s != MC_OK || f != MC_OK)
+        return s != MC_OK ? s : f;
     c->sweeps_done += n_sweeps;
     c->rec_written += recs;
     return MC_OK;

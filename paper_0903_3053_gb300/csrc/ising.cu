@@ -40,7 +40,7 @@ namespace {
 template <int C, int LAYOUT, bool PAIRS>
 __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 {
-    const int k = find_chain(a.block_start, a.n_chains, blockIdx.x);
+    const int k = chain_of_block(a);
     const IsingChain ch = static_cast<const IsingChain *>(a.chains)[k];
     const uint32_t t = (blockIdx.x - a.block_start[k]) * blockDim.x + threadIdx.x;
     const uint32_t sweep = (uint32_t)(a.state->sweep_base + a.k);
@@ -556,6 +556,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     SweepArgs a{};
     a.chains = c->d_chains;
     a.block_start = c->d_block_start;
+    a.block_chain = c->d_block_chain;
     a.n_chains = c->n_chains;
     a.lattice = c->d_lattice;
     a.series = c->d_series;

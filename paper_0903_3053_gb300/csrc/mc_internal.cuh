@@ -125,6 +125,11 @@ __device__ __forceinline__ void chain_wait(bool release)
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Chain of a block of a grid-mode launch: one load (a binary search over the
+// offsets is six dependent ones for 64 chains).
+struct SweepArgs;
+__device__ __forceinline__ int chain_of_block(const SweepArgs &a);
+
 // Largest k in [0, n) with block_start[k] <= b (block_start ascending, [0] = 0).
 __device__ __forceinline__ int find_chain(const uint32_t *__restrict__ block_start, int n, uint32_t b)
 {
@@ -143,6 +148,7 @@ __device__ __forceinline__ int find_chain(const uint32_t *__restrict__ block_sta
 struct SweepArgs {
     const void *chains;          // IsingChain* or Su2Chain*
     const uint32_t *block_start; // grid-mode block offsets per chain (n_chains + 1 entries)
+    const uint32_t *block_chain; // chain of each block (n_chains > 1)
     int n_chains;
     char *lattice;               // lattice region base
     DevRecord *series;           // [chain][cap]
@@ -155,6 +161,11 @@ struct SweepArgs {
     uint32_t row_pairs;          // Ising grid mode: row pairs per thread
     int release;                 // let the next kernel's blocks in once this one's are past chain_wait
 };
+
+__device__ __forceinline__ int chain_of_block(const SweepArgs &a)
+{
+    return a.n_chains == 1 ? 0 : (int)__ldg(&a.block_chain[blockIdx.x]);
+}
 
 }  // namespace mc
 
@@ -174,7 +185,8 @@ struct mc_ctx {
     size_t ws_bytes = 0;
     // carve-out of the workspace
     void *d_chains = nullptr;
-    uint32_t *d_block_start = nullptr;   // grid-mode sweep launches
+    uint32_t *d_block_start = nullptr;   // grid-mode sweep launches: first block of each chain
+    uint32_t *d_block_chain = nullptr;   // and the chain of each block (more than one chain)
     uint32_t *d_meas_start = nullptr;    // measurement launches
     char *d_lattice = nullptr;
     mc::DevRecord *d_series = nullptr;
@@ -188,7 +200,7 @@ struct mc_ctx {
     std::vector<mc::IsingChain> ising;
     std::vector<mc::Su2Chain> su2;
     std::vector<mc_chain_desc> desc;
-    std::vector<uint32_t> block_start, meas_start;
+    std::vector<uint32_t> block_start, block_chain, meas_start;
     uint32_t grid_blocks = 0, meas_blocks = 0;
     int row_pairs = 1;                   // Ising grid mode: row pairs per thread (0: int8, one group)
     // run bookkeeping
@@ -232,6 +244,11 @@ cudaError_t su2_prepare_resident(mc_ctx *c);
 cudaError_t su2_resident_enqueue(mc_ctx *c, long long n, int every);
 
 cudaError_t advance_state_launch(mc_ctx *c, long long n, long long recs);
+
+// A validated sweep call in two parts (capi.cu): everything enqueued on the context's private stream, ordered after
+// the caller's work; then the caller's stream made to wait for it.  Between the two a group starts its other members.
+mc_status sweep_begin(mc_ctx *c, long long n, int every);
+mc_status sweep_end(mc_ctx *c);
 
 // Message returned by mc_last_error() on this thread.
 void set_last_error(const std::string &msg);

@@ -58,9 +58,9 @@ __device__ __forceinline__ const Su2Chain &block_chain(const SweepArgs &, const 
     b0 = tab.start[k];
     return tab.ch[k];
 }
-__device__ __forceinline__ Su2Chain block_chain(const SweepArgs &a, const NoTable &, uint32_t b, int &k, uint32_t &b0)
+__device__ __forceinline__ Su2Chain block_chain(const SweepArgs &a, const NoTable &, uint32_t, int &k, uint32_t &b0)
 {
-    k = find_chain(a.block_start, a.n_chains, b);
+    k = chain_of_block(a);
     b0 = a.block_start[k];
     return static_cast<const Su2Chain *>(a.chains)[k];
 }
@@ -369,6 +369,7 @@ static SweepArgs sweep_args(const mc_ctx *c)
     SweepArgs a{};
     a.chains = c->d_chains;
     a.block_start = c->d_block_start;
+    a.block_chain = c->d_block_chain;
     a.n_chains = c->n_chains;
     a.lattice = c->d_lattice;
     a.series = c->d_series;

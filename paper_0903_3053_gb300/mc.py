@@ -395,7 +395,8 @@ class Batch:
 
 
 class Group:
-    """Chains of several Batches advanced by one persistent launch per call."""
+    """Chains of several Batches advanced together: the batches' own launches side
+    by side, or (configure with split_cost >= 0) one persistent launch per call."""
 
     def __init__(self, batches):
         torch = _torch()
