@@ -253,10 +253,10 @@ mc_status sweep_end(mc_ctx *c);
 // Message returned by mc_last_error() on this thread.
 void set_last_error(const std::string &msg);
 
-// Launch one sweep kernel on the context's launch stream, chained to the kernel before it (chain_wait) unless
-// profiling events separate the launches.
+// Launch a kernel chained to the one before it on the stream (chain_wait), or as a plain launch.
 template <typename... P, typename... A>
-cudaError_t launch_chained(const mc_ctx *c, void (*kernel)(P...), unsigned blocks, unsigned threads, const A &...args)
+cudaError_t launch_chained_on(cudaStream_t stream, bool chained, void (*kernel)(P...), unsigned blocks, unsigned threads,
+                              size_t smem, const A &...args)
 {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
@@ -264,10 +264,18 @@ cudaError_t launch_chained(const mc_ctx *c, void (*kernel)(P...), unsigned block
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(threads);
-    cfg.stream = c->ls;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = c->profiling ? 0 : 1;
+    cfg.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Launch one sweep kernel on the context's launch stream, chained unless profiling events separate the launches.
+template <typename... P, typename... A>
+cudaError_t launch_chained(const mc_ctx *c, void (*kernel)(P...), unsigned blocks, unsigned threads, const A &...args)
+{
+    return launch_chained_on(c->ls, !c->profiling, kernel, blocks, threads, 0, args...);
 }
 
 // Bracket one sweep-kernel launch with events when the context is profiling.

@@ -40,7 +40,17 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr)
            (4ull << 61);
 }
 
-// The same swizzle for an MN-major operand (the M or N index runs along the
+// The same for a K-major operand of 128-byte rows (64 16-bit elements) in the
+// 128-byte swizzle (16-byte chunk c of row r at chunk c ^ (r & 7)): stride offset
+// 1024 bytes (8 rows); a view may start at any row and at any 32-byte K step of a
+// row, as above.
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr)
+{
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
+           (2ull << 61);
+}
+
+// The 64-byte swizzle for an MN-major operand (the M or N index runs along the
 // 64-byte rows, K along the rows): a 512-byte atom holds 32 elements of M or N
 // x 8 values of K; the stride offset (512 bytes) steps K by 8 and the leading
 // offset `atom_stride` steps M or N by 32.  The atoms may overlap: a stride of
@@ -91,6 +101,25 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_taddr, uint64_t a_desc, uint
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_taddr),
                  "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+                 : "memory");
+}
+
+// The same, called by a whole converged warp of which one elected lane issues: the
+// descriptors then come from warp-uniform arithmetic, in the uniform registers that
+// the instruction reads them from.  Issued from a single lane's branch, each MMA
+// waits ~100 cycles for its descriptors to be formed and moved.
+template <bool ACC>
+__device__ __forceinline__ void mma_bf16_warp(uint32_t d_taddr, uint64_t a_desc, uint64_t b_desc, uint32_t idesc)
+{
+    asm volatile("{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_taddr),
+                 "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void commit_warp(uint32_t bar_saddr)
+{
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar_saddr)
                  : "memory");
 }
 
@@ -173,6 +202,40 @@ __device__ __forceinline__ void ld_32x32b_x32(uint32_t taddr, float (&v)[32])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int j = 0; j < 32; ++j)
+        v[j] = __uint_as_float(r[j]);
+}
+
+// 64 consecutive FP32 columns of this thread's tensor-memory lane, complete on
+// return (the wait is part of the statement, so that nothing that uses the values can
+// be scheduled ahead of it).
+__device__ __forceinline__ void ld_32x32b_x64(uint32_t taddr, float (&v)[64])
+{
+    uint32_t r[64];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
+                 "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
+                 "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]),
+                   "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                   "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+                   "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+                   "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+                   "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]),
+                   "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+                   "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]),
+                   "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
+                   "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]),
+                   "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
+                   "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]),
+                   "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int j = 0; j < 64; ++j)
         v[j] = __uint_as_float(r[j]);
 }
 

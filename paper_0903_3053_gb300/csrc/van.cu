@@ -89,57 +89,7 @@ __global__ void k_prep_weights(const float *p, DevParams P, bf16 *wh, float *w1,
 }
 
 // ------------------------------------------------------------------ forward
-// 32 -> 32 masked convolutions on the fifth-generation tensor cores: implicit
-// GEMMs D[q][o] = sum_{t,c} A_t[q][c] W[t][o][c] with tcgen05.mma (M = 128
-// positions, N = 32 channels, K = 16, BF16 in, FP32 accumulator in tensor
-// memory).  Positions are indexed on a padded grid, q = r P + xp with
-// xp = x + 2 and a row pitch P >= L + 4, so that every tap (dy, dx) of output q
-// reads input index q + (dy + 2) P + dx of the staged rows y0-2 .. y0+R-1 -- a
-// shifted view of the same shared-memory chunk planes (see tc_dev.cuh), zero
-// halo columns giving the zero padding.  Outputs on halo columns or past the
-// last row are computed and discarded.  One CTA item = R rows of one sample,
-// cut into 128-position tiles; tiles are issued 3 at a time by one thread into
-// one of two tensor-memory buffers (26 MMAs per tile: 13 taps x 2 k-steps)
-// while 4 warps drain the other (tcgen05.ld, bias, ReLU, BF16, stores).
-//
-// Geometry of the gradient kernel (k_conv32_bwd_tc: P = L + 4, rows staged with
-// cp.async by the CTA's threads, `nplanes` chunk planes, two CTAs per SM).
-struct TcConvGeom {
-    int L, P, R, YB, Qpad, tiles, PL;
-    uint32_t plane_bytes, smem_bytes;
-};
-constexpr uint32_t kTcB = kTapsB * 4 * kCh * 16; // B planes: [tap][chunk][out channel] x 16 bytes
-constexpr int kTcGroup = 3;                       // tiles per commit
-constexpr uint32_t kTcCols = 256;                 // 2 buffers x 3 tiles x 32 columns, rounded to a power of 2
-constexpr int kTcMaxPolls = 1 << 22;              // bounded completion wait
-
-// Rows per CTA item: the R <= 16 whose `nplanes` planes (plus the weights)
-// fit two CTAs per SM and that needs the fewest 128-position tiles per sample.
-TcConvGeom tc_conv_geom(int L, int nplanes)
-{
-    TcConvGeom best{};
-    long best_tiles = -1;
-    for (int R = 1; R <= 16 && R <= L; ++R) {
-        TcConvGeom g{};
-        g.L = L;
-        g.P = L + 4;
-        g.R = R;
-        g.Qpad = (R * g.P + 127) / 128 * 128;
-        g.PL = (g.Qpad + 2 * g.P + 4 + 7) / 8 * 8; // 2-entry guard each side of every tap's view
-        g.plane_bytes = (uint32_t)g.PL * 16;
-        g.smem_bytes = (uint32_t)nplanes * g.plane_bytes + kTcB + 32;
-        g.YB = (L + R - 1) / R;
-        g.tiles = g.Qpad / 128;
-        if (g.smem_bytes > 110u * 1024)
-            continue;
-        const long t = (long)g.YB * g.tiles;
-        if (best_tiles < 0 || t < best_tiles || (t == best_tiles && R > best.R)) {
-            best = g;
-            best_tiles = t;
-        }
-    }
-    return best;
-}
+constexpr int kTcMaxPolls = 1 << 22; // bounded completion wait
 
 // Layer 1 (1 -> 32 channels, mask A, ReLU) on the fifth-generation tensor
 // cores: one MMA per tile of 128 consecutive positions (M = 128, N = 32,
@@ -164,6 +114,7 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5;
+    chain_wait(true);
     if (tid < kCh)
         Bias[tid] = b1[tid];
     if (tid < 2 * kCh) { // w1 is [o][t]
@@ -255,75 +206,151 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
         tc::tmem_free(tbase, kL1Cols);
 }
 
-// ---------------------------------------------------------------- TMA-pipelined forward convolution
-// out = ReLU(conv(in) + bias).  The staging is taken off the threads and the
-// three stages of an item overlap across items: warp 4 streams the
-// input rows of the next item by TMA (one box of all 32 channels: R + 2 rows of
-// P positions from x = -2, everything outside the lattice arriving zero-filled,
-// 64-byte rows in the 64-byte swizzle, which the MMA reads through swizzled
-// descriptors -- a tap is still an offset of whole rows) into the second of two
-// stage buffers, one thread of warp 5 issues the MMAs of the current item, and warps
-// 0-3 drain tensor memory (bias, ReLU, BF16, stores).  They hand over through
-// mbarriers: stage full (TMA bytes), stage free (MMA commit), accumulator full
-// (MMA commit) and accumulator free (epilogue arrivals); every wait is bounded
-// and a timeout latches MC_ETIMEOUT.  Every TMA destination starts on a
-// 1024-byte boundary.  Two CTAs of 6 warps per SM (stages of at most 110 KB,
-// so fewer rows per item) where that costs at most 15% more tiles than one CTA
-// with 200 KB: the other CTA's MMAs fill one CTA's pipeline gaps (L = 64,
-// batch 4096: 4.94 against 5.95 ms per forward pass); else one.
-struct TmaConvGeom {
-    int L, P, R, YB, Qpad, tiles, PL, ctas_per_sm;
+// Gradients travel between the backward kernels as a BF16 hi + lo pair
+// (hi = bf16(v), lo = bf16(v - hi), ~16 mantissa bits): two [n][L][L][32] BF16
+// arrays in the space of one FP32 array, which the tensor cores read directly.
+__device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo)
+{
+    bf16 h[8], l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        h[k] = __float2bfloat16(v[k]);
+        l[k] = __float2bfloat16(v[k] - bf(h[k]));
+    }
+    hi = *reinterpret_cast<uint4 *>(h);
+    lo = *reinterpret_cast<uint4 *>(l);
+}
+
+// ---------------------------------------------------------------- masked 32-channel convolutions
+// The hidden layers' forward and data-gradient convolutions and the last layer's
+// forward, on the fifth-generation tensor cores (tcgen05.mma, BF16 in, FP32
+// accumulator in tensor memory), as implicit GEMMs over runs of G = 4 (L % 4 == 0)
+// or 2 neighbouring positions: row q of the operand A is the run x .. x + G - 1, 64 G
+// bytes, and the accumulator of 128 rows holds the outputs of all its positions, G x
+// 32 columns.  An MMA of one input position and 16 channels (K = 16) feeds all
+// outputs of the run whose window it is in (N = 32 .. 32 G).  What bounds these kernels
+// is the shared-memory read of the operands, 128 bytes per clock and SM: an MMA
+// reads 4 KB of A and N x 32 bytes of B, so that 128 positions cost 1040 cycles with
+// one-position rows (26 MMAs), 740 with G = 2 and 560 with G = 4.  Measured at L = 64,
+// batch 4096, per hidden layer: forward 643 us with one-position rows, 463 with G = 2,
+// 430 with G = 4 (its MMAs alone 370; 2.15 GB of activations, 5.0 TB/s), the data
+// gradient 2600 with one-position rows staged by the CTA's threads, 1070 now (5.4 GB,
+// 5.0 TB/s).
+//
+// Runs are indexed on a padded grid, q = (smp (R + 2) + r) P + pp with P = L / G + 1:
+// pp = 0 is the zero run left of the row, and the run right of it is the next row's
+// pp = 0.  A tap is a shifted view of the staged rows, which lie in G / 2 slabs of
+// 128-byte rows (two positions each; 128-byte swizzle, which follows the absolute
+// shared-memory address): the descriptor's start moves by whole rows, by 64 bytes for
+// the second position of a slab.  Rows of A on the padding are computed and
+// dropped.  B holds each tap's weights once, the taps of a kernel row in the order in
+// which the next position of a run meets them one step later, so that the operand of
+// N = 32 c columns is c consecutive taps.
+//
+//   FWD  : out(p)[o] = ReLU(b[o] + sum_t sum_c W[t][o][c] in(p + d_t)[c]), BF16.
+//   LAST : the 32 -> 1 layer, 16 columns per position (the smallest N) of which
+//          the first holds the logit f; the epilogue forms log sigmoid(s f) and
+//          (training) dF = -(1/n) s sigmoid(-s f).
+//   BWD  : out(p)[c] = [mask(p)[c] > 0] sum_t sum_o W[t][o][c] dz(p - d_t)[o], dz and
+//          out as BF16 hi + lo pairs (two MMAs per K step).
+//
+// Warp-specialised: a producer warp streams an item's rows (R + 2 rows of P runs of
+// S samples, a box per slab, everything outside the lattice zero-filled) by TMA into
+// the second of two stage buffers, one thread of another warp issues the MMAs of the
+// current item, the first EW warps drain tensor memory, 64 columns each (two slots
+// per accumulator buffer: two tiles for G = 2, the halves of a tile for G = 4).  They hand over through mbarriers: stage
+// full (TMA bytes), stage free (MMA commit), accumulator full (MMA commit) and
+// accumulator free (epilogue arrivals); every wait is bounded and a timeout
+// latches MC_ETIMEOUT.  Two CTAs per SM (4 epilogue warps each) where that costs at
+// most 15% more tiles than one, to fill each other's pipeline gaps; else one, with 8
+// epilogue warps for the data gradient.
+constexpr int kFwd = 0, kLast = 1, kBwd = 2;
+constexpr int kRunGuard = 8;                   // rows ahead of staged row 0 (8 x 128 bytes: a box lands 1024-byte aligned)
+constexpr uint32_t kRunMaxSmem1 = 200u * 1024; // two stages + weights + barriers + scratch, one CTA per SM
+constexpr uint32_t kRunMaxSmem2 = 113u * 1024; // the same, two CTAs per SM
+constexpr uint32_t kRunBarBytes = 128;         // 9 mbarriers, tensor-memory slot
+constexpr uint32_t kRunScratch = 1024;         // per epilogue warp: 8 pairs of output on their way to whole lines
+constexpr int kMaxItemRows = 32, kMaxItemSamples = 16, kMaxPackedTiles = 4;
+
+__host__ __device__ constexpr int conv_cols(int mode) { return mode == kLast ? 16 : kCh; } // per position
+__host__ __device__ constexpr uint32_t conv_weight_bytes(int mode) { return kTapsB * 4u * (uint32_t)conv_cols(mode) * 16u; }
+__host__ __device__ constexpr int epilogue_warps(int mode, int ctas) { return mode == kBwd && ctas == 1 ? 8 : 4; }
+
+struct RunGeom {
+    int L, G, P, R, S, YB, tiles, ctas_per_sm; // S samples per item (1 unless an item holds whole lattices)
+    uint32_t inv_p, inv_rows;                  // ceil(2^32 / P), ceil(2^32 / (R + 2)): exact quotients below 2^16
     uint32_t plane_bytes, stage_bytes, smem_bytes;
 };
-constexpr int kTmaGuard = 16;                  // positions ahead of staged row 0 (>= 2; 16 x 64 bytes = one
-                                               // 1024-byte boundary, so that the TMA box lands swizzle-aligned)
-constexpr uint32_t kTmaMaxSmem1 = 200u * 1024; // two stages + weights + barriers, one CTA per SM
-constexpr uint32_t kTmaMaxSmem2 = 110u * 1024; // the same, two CTAs per SM
-constexpr uint32_t kTmaBarBytes = 128;         // 9 mbarriers, tensor-memory slot
 
-// Rows per item: the R whose two stages fit `max_smem` and that needs the
-// fewest 128-position tiles per sample.
-TmaConvGeom tma_conv_geom_cap(int L, uint32_t max_smem)
+RunGeom run_geom_of(int L, int G, int R, int S, int mode, int ctas)
 {
-    TmaConvGeom best{};
-    long best_tiles = -1;
-    for (int R = 1; R <= 32 && R <= L; ++R) {
-        TmaConvGeom g{};
-        g.L = L;
-        g.P = (L + 4 + 7) / 8 * 8;
-        g.R = R;
-        g.Qpad = (R * g.P + 127) / 128 * 128;
-        g.PL = (kTmaGuard + 2 * g.P + g.Qpad + 15) / 16 * 16; // whole 1024-byte swizzle spans
-        g.plane_bytes = (uint32_t)g.PL * 64;                 // 64 bytes (32 channels) per position
-        g.stage_bytes = g.plane_bytes;
-        g.smem_bytes = 2 * g.stage_bytes + kTcB + kTmaBarBytes + 1024; // + alignment slack
-        g.YB = (L + R - 1) / R;
-        g.tiles = g.Qpad / 128;
-        if (g.smem_bytes > max_smem)
-            continue;
-        const long t = (long)g.YB * g.tiles;
-        if (best_tiles < 0 || t < best_tiles || (t == best_tiles && R > best.R)) {
-            best = g;
-            best_tiles = t;
+    RunGeom g{};
+    g.L = L;
+    g.G = G;
+    g.P = L / g.G + 1;
+    g.R = R;
+    g.S = S;
+    g.YB = (L + R - 1) / R;
+    g.ctas_per_sm = ctas;
+    const int q = (S * (R + 2) - 2) * g.P, qpad = (q + 127) / 128 * 128;
+    g.tiles = qpad / 128;
+    // the staged rows and the zero row past them; the views of the last tile's padding rows run on into what
+    // follows (the other planes, the weights), whose products are dropped
+    g.plane_bytes = (uint32_t)((kRunGuard + S * (R + 2) * g.P + 1 + 7) / 8 * 8) * 128u;
+    g.stage_bytes = (mode == kBwd ? 2u : 1u) * (uint32_t)(g.G / 2) * g.plane_bytes;
+    const uint32_t used = 2 * g.stage_bytes + conv_weight_bytes(mode) + kRunBarBytes +
+                          (mode == kLast ? 0u : (uint32_t)epilogue_warps(mode, ctas) * kRunScratch);
+    const uint32_t read = 2 * g.stage_bytes - g.plane_bytes + (uint32_t)(kRunGuard + qpad + 2 * g.P + 2) * 128u;
+    g.smem_bytes = std::max(used, read) + 1024; // + alignment slack
+    g.inv_p = (uint32_t)(((1ull << 32) + g.P - 1) / g.P);
+    g.inv_rows = (uint32_t)(((1ull << 32) + R + 1) / (R + 2));
+    return g;
+}
+
+// Shared-memory cycles of a tile's MMAs: 4 KB of A and 32 bytes per column of B each,
+// at 128 bytes per clock (two channel halves; BWD hi and lo alike for every G).
+int tile_cycles(int mode, int G)
+{
+    int cycles = 0;
+    for (int d = 0; d < 3; ++d)
+        for (int j = -2; j <= G + 1; ++j) {
+            const int ulo = d == 2 && mode != kBwd ? 2 : 0, uhi = d == 2 && mode == kBwd ? 2 : 4;
+            const int n = std::min(uhi - 1 + j, G) - std::max(ulo - 2 + j, 0);
+            cycles += n > 0 ? 2 * (32 + n * conv_cols(mode) / 4) : 0;
         }
+    return cycles;
+}
+
+// Run length, rows and (for lattices that fit an item whole) samples per item: the
+// fewest cycles per sample among those whose two stages fit `max_smem`.
+RunGeom run_geom_cap(int L, int mode, int ctas, uint32_t max_smem, double &cost)
+{
+    RunGeom best{};
+    cost = 1e300;
+    for (int G = 2; G <= 4 && L % G == 0; G += 2) {
+        const int cycles = tile_cycles(mode, G);
+        for (int R = 1; R <= kMaxItemRows && R <= L; ++R)
+            for (int S = 1; S == 1 || (R == L && S <= kMaxItemSamples); ++S) {
+                const RunGeom g = run_geom_of(L, G, R, S, mode, ctas);
+                if (g.smem_bytes > max_smem || (S > 1 && g.tiles > kMaxPackedTiles))
+                    continue;
+                const double c = (double)g.YB * g.tiles / S * cycles;
+                if (c < cost || (c == cost && S == 1 && R > best.R)) {
+                    best = g;
+                    cost = c;
+                }
+            }
     }
     return best;
 }
 
-TmaConvGeom tma_conv_geom(int L)
+RunGeom run_geom(int L, int mode)
 {
-    TmaConvGeom one = tma_conv_geom_cap(L, kTmaMaxSmem1), two = tma_conv_geom_cap(L, kTmaMaxSmem2);
-    one.ctas_per_sm = 1;
-    two.ctas_per_sm = 2;
-    const long t1 = (long)one.YB * one.tiles, t2 = (long)two.YB * two.tiles;
-    return two.R > 0 && 100 * t2 <= 115 * t1 ? two : one;
+    double c1, c2;
+    const RunGeom one = run_geom_cap(L, mode, 1, kRunMaxSmem1, c1), two = run_geom_cap(L, mode, 2, kRunMaxSmem2, c2);
+    return two.R > 0 && c2 <= 1.15 * c1 ? two : one;
 }
 
-// The last layer (32 -> 1) on the same pipeline: B has N = 16 rows (the
-// smallest tile of an M = 128 MMA), the layer's weights -- BF16 values, as
-// k_prep_weights leaves them -- in row 0 and zeros elsewhere, so that the
-// logit is f = D[p][0] + b; the epilogue forms f, log sigmoid(s f) and
-// (training) dF = -(1/n) s sigmoid(-s f) per position.
 struct LastLayerArgs {
     const float *wD; // [t][c], BF16-representable
     const float *bD; // the layer's bias (one value)
@@ -333,48 +360,106 @@ struct LastLayerArgs {
     float inv_n;
 };
 
-template <int MINB, bool LAST>
-__global__ void __launch_bounds__(192, MINB) k_conv32_tma(const __grid_constant__ CUtensorMap in_map,
-                                                       bf16 *__restrict__ out, const bf16 *__restrict__ W,
-                                                       const float *__restrict__ bias, LastLayerArgs la, int n,
-                                                       TmaConvGeom g, int *err)
+struct ConvArgs {
+    const bf16 *W;     // [t][o][c] (FWD, BWD)
+    const float *bias; // FWD
+    const bf16 *mask;  // BWD: the layer's input activations
+    bf16 *out, *out_lo;
+    LastLayerArgs la;
+    int n;
+    int *err;
+};
+
+// Store a warp's 32 rows of 128 bytes (one pair of positions per lane, `row`) to
+// out[pair], pair = ~0 for rows that are dropped.  Eight rows at a time go through
+// shared memory (16-byte chunk c of row r at chunk c ^ r: no bank conflicts), so that
+// eight lanes store one whole 128-byte line; stored by their own lanes, the rows
+// would be 32 lines per instruction (forward, L = 64, batch 512: 81 -> 72 us).  MASK: halves
+// whose activation mk (lane's chunks, in storing order) is not positive become zero.
+template <bool MASK>
+__device__ __forceinline__ void store_pairs(uint4 *scratch, int lane, const uint4 (&row)[8], uint32_t pair,
+                                            const uint4 (&mk)[8], uint4 *out)
 {
-    constexpr int NB = LAST ? 16 : kCh; // output columns of the MMA
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if ((lane >> 3) == k)
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                scratch[(lane & 7) * 8 + (c ^ (lane & 7))] = row[c];
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = 4 * i + (lane >> 3), c = lane & 7;
+            uint4 o = scratch[r * 8 + (c ^ r)];
+            const uint32_t pr = __shfl_sync(0xffffffffu, pair, 8 * k + r);
+            if (MASK) {
+                const uint4 m = mk[2 * k + i];
+                const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+                o.x &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.x), zero);
+                o.y &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.y), zero);
+                o.z &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.z), zero);
+                o.w &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.w), zero);
+            }
+            if (pr != ~0u)
+                out[(size_t)pr * 8 + c] = o;
+        }
+        __syncwarp();
+    }
+}
+
+template <int MODE, int G, int MINB>
+__global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
+    k_conv_runs(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+                const __grid_constant__ ConvArgs a, const __grid_constant__ RunGeom g)
+{
+    constexpr int EW = epilogue_warps(MODE, MINB);
+    constexpr int NB = conv_cols(MODE);             // accumulator columns per position
+    constexpr uint32_t kSlot = 2 * NB;              // columns of a slot: two positions
+    constexpr uint32_t kCols = 4 * kSlot;           // two buffers of two slots
+    constexpr int kGroup = G == 2 ? 2 : 1;          // tiles per commit
+    constexpr int SLABS = G / 2;
+    constexpr uint32_t kTap = NB * 16;              // bytes of one tap in one chunk plane
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // the stages hold 64-byte-swizzled rows: round the base up to 1024 bytes
+    // the stages hold 128-byte-swizzled rows: round the base up to 1024 bytes
     // (the launch reserves 1024 extra bytes)
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t sb = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t boff = 2 * g.stage_bytes, bars = boff + kTcB;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const uint32_t boff = 2 * g.stage_bytes, bars = boff + conv_weight_bytes(MODE);
     const uint32_t full0 = sb + bars, empty0 = full0 + 16, tfull0 = full0 + 32, tempty0 = full0 + 48,
-                   drain = full0 + 64, tslot_off = bars + 80;
-    for (uint32_t i = tid; i < 2 * g.stage_bytes / 16; i += blockDim.x) // padding columns and guards stay zero
-        reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (LAST) {
-        for (int i = tid; i < kTapsB * 4 * NB; i += blockDim.x) { // [t][c8][row]: row 0 the weights
-            const int t = i / (4 * NB), c8 = (i / NB) % 4, o = i % NB;
-            bf16 v[8];
+                   drain = full0 + 64, tslot_off = bars + 80, scratch_off = bars + kRunBarBytes;
+    // the run right of the box's last row is zero (BWD reads it); whatever else lies outside the boxes is met only by
+    // rows of A that are dropped
+    for (uint32_t i = tid; i < 8u * 2u * g.stage_bytes / g.plane_bytes; i += blockDim.x)
+        *reinterpret_cast<uint4 *>(smem + (i >> 3) * g.plane_bytes +
+                                   (uint32_t)(kRunGuard + g.S * (g.R + 2) * g.P) * 128u + (i & 7u) * 16u) =
+            make_uint4(0u, 0u, 0u, 0u);
+    // Weights: [kernel row d][chunk of 8 K values][tap u'][row] x 16 bytes.  Tap order: FWD and LAST dx = 2 .. -2
+    // (row dy = 0: 0, -1, -2), BWD dx = -2 .. 2 (-2, -1, 0).
+    for (int i = tid; i < kTapsB * 4 * NB; i += blockDim.x) {
+        const int d = i < 20 * NB ? 0 : i < 40 * NB ? 1 : 2, nt = d == 2 ? 3 : 5;
+        const int r0 = i - d * 20 * NB, c8 = r0 / (nt * NB), u = (r0 / NB) % nt, o = r0 % NB;
+        const int dx = MODE == kBwd ? u - 2 : (d == 2 ? -u : 2 - u), t = d == 2 ? 12 + dx : 5 * d + dx + 2;
+        bf16 v[8];
+        if (MODE == kFwd) {
+            *reinterpret_cast<uint4 *>(v) =
+                *reinterpret_cast<const uint4 *>(a.W + ((size_t)(t * kCh + o) * kCh + c8 * 8));
+        } else {
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                v[k] = __float2bfloat16(o == 0 ? la.wD[t * kCh + c8 * 8 + k] : 0.f);
-            *reinterpret_cast<uint4 *>(smem + boff + ((t * 4 + c8) * NB + o) * 16) = *reinterpret_cast<uint4 *>(v);
+                v[k] = MODE == kBwd ? a.W[((size_t)t * kCh + c8 * 8 + k) * kCh + o]
+                                    : __float2bfloat16(o == 0 ? a.la.wD[t * kCh + c8 * 8 + k] : 0.f);
         }
-    } else {
-        for (int i = tid; i < kTapsB * kCh * 4; i += blockDim.x) {
-            const int t = i / (kCh * 4), o = (i / 4) % kCh, c8 = i % 4;
-            *reinterpret_cast<uint4 *>(smem + boff + ((t * 4 + c8) * kCh + o) * 16) =
-                *reinterpret_cast<const uint4 *>(W + ((size_t)(t * kCh + o) * kCh + c8 * 8));
-        }
+        *reinterpret_cast<uint4 *>(smem + boff + (uint32_t)i * 16u) = *reinterpret_cast<uint4 *>(v);
     }
     if (warp == 0)
-        tc::tmem_alloc(sb + tslot_off, kTcCols);
+        tc::tmem_alloc(sb + tslot_off, kCols);
     if (tid == 0) {
         for (int k = 0; k < 2; ++k) {
             tc::mbar_init(full0 + 8 * k, 1);
             tc::mbar_init(empty0 + 8 * k, 1);
             tc::mbar_init(tfull0 + 8 * k, 1);
-            tc::mbar_init(tempty0 + 8 * k, 4);
+            tc::mbar_init(tempty0 + 8 * k, EW);
         }
         tc::mbar_init(drain, 1);
     }
@@ -382,12 +467,13 @@ __global__ void __launch_bounds__(192, MINB) k_conv32_tma(const __grid_constant_
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t *>(smem + tslot_off);
-    const int total = n * g.YB, rounds = (g.tiles + kTcGroup - 1) / kTcGroup;
+    chain_wait(true); // only the weights, final before the first kernel of the pass, were read so far
+    const uint32_t tbase = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(smem + tslot_off), 0);
+    const int total = (a.n + g.S - 1) / g.S * g.YB, rounds = (g.tiles + kGroup - 1) / kGroup;
     int ok = 1;
-    if (warp == 4) {
+    if (warp == EW) {
         if (lane == 0) { // producer
-            const uint32_t bytes = (uint32_t)(g.R + 2) * (uint32_t)g.P * 64u;
+            const uint32_t bytes = (uint32_t)(g.S * (g.R + 2) * g.P) * 128u * SLABS * (MODE == kBwd ? 2u : 1u);
             int k = 0, armed[2] = {-1, -1};
             for (int it = blockIdx.x; it < total; it += gridDim.x, ++k) {
                 const int s = k & 1;
@@ -395,127 +481,223 @@ __global__ void __launch_bounds__(192, MINB) k_conv32_tma(const __grid_constant_
                     ok = 0;
                     break;
                 }
-                const int b = it / g.YB, y0 = (it - b * g.YB) * g.R;
+                const int bi = it / g.YB, y0 = (it - bi * g.YB) * g.R, ys = MODE == kBwd ? y0 : y0 - 2;
                 tc::mbar_arrive_expect_tx(full0 + 8 * s, bytes);
-                const uint32_t st = sb + (uint32_t)s * g.stage_bytes;
-                // rows y0-2 .. y0+R-1, columns -2 .. P-3, all 32 channels: one box
-                tc::tma_load_5d(st + (uint32_t)kTmaGuard * 64u, &in_map, 0, 0, -2, y0 - 2, b, full0 + 8 * s);
+                const uint32_t st = sb + (uint32_t)s * g.stage_bytes + kRunGuard * 128u;
+                // rows ys .. ys + R + 1 of P runs from x = -G, S samples: one box per slab of two positions
+#pragma unroll
+                for (int sl = 0; sl < SLABS; ++sl) {
+                    tc::tma_load_5d(st + (uint32_t)sl * g.plane_bytes, &map_hi, 0, sl, -1, ys, bi * g.S, full0 + 8 * s);
+                    if (MODE == kBwd)
+                        tc::tma_load_5d(st + (uint32_t)(SLABS + sl) * g.plane_bytes, &map_lo, 0, sl, -1, ys, bi * g.S,
+                                        full0 + 8 * s);
+                }
                 armed[s] = k;
             }
             for (int s = 0; s < 2; ++s) // the last loads of each stage have landed before the CTA ends
                 if (armed[s] >= 0 && !tc::mbar_wait(full0 + 8 * s, (armed[s] >> 1) & 1, kTcMaxPolls))
                     ok = 0;
         }
-    } else if (warp == 5) {
-        if (lane == 0) { // MMA issuer
-            const uint32_t idesc = tc::idesc_bf16_f32(128, NB);
-            uint64_t adesc[kTapsB * 2], bdesc[kTapsB * 2];
-            for (int t = 0; t < kTapsB; ++t)
-                for (int kc = 0; kc < 2; ++kc) {
-                    adesc[t * 2 + kc] = tc::smem_desc_sw64(
-                        sb + (uint32_t)(kTmaGuard + (tap_dy(t) + 2) * g.P + tap_dx(t)) * 64u + (uint32_t)kc * 32u);
-                    bdesc[t * 2 + kc] = tc::smem_desc(sb + boff + (uint32_t)(t * 4 + 2 * kc) * (NB * 16), NB * 16, 128);
-                }
+    } else if (warp == EW + 1) { // MMA issuer: the whole warp, uniform; an elected lane issues
+        {
+            const uint64_t a0 = tc::smem_desc_sw128(sb + kRunGuard * 128u);
+            uint64_t bd[3]; // kernel row d: its chunk planes are nt kTap bytes apart
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                bd[d] = tc::smem_desc(sb + boff + (uint32_t)d * 20u * kTap, (d == 2 ? 3u : 5u) * kTap, 128);
+            const uint64_t slab = (uint64_t)(g.plane_bytes >> 4), lo_off = SLABS * slab;
             uint32_t tcount = 0;
             int k = 0;
             for (int it = blockIdx.x; ok && it < total; it += gridDim.x, ++k) {
                 const int s = k & 1;
-                if (!tc::mbar_wait(full0 + 8 * s, (k >> 1) & 1, kTcMaxPolls)) {
+                if (!__all_sync(0xffffffffu, tc::mbar_wait(full0 + 8 * s, (k >> 1) & 1, kTcMaxPolls))) {
                     ok = 0;
                     break;
                 }
                 tc::fence_after_sync();
-                const uint64_t soff = (uint64_t)(((uint32_t)s * g.stage_bytes) >> 4);
                 for (int rd = 0; rd < rounds; ++rd, ++tcount) {
                     const uint32_t bb = tcount & 1u;
-                    if (tcount >= 2 && !tc::mbar_wait(tempty0 + 8 * bb, ((tcount >> 1) - 1) & 1u, kTcMaxPolls)) {
+                    if (tcount >= 2 &&
+                        !__all_sync(0xffffffffu,
+                                    tc::mbar_wait(tempty0 + 8 * bb, ((tcount >> 1) - 1) & 1u, kTcMaxPolls))) {
                         ok = 0;
                         break;
                     }
                     tc::fence_after_sync();
-                    const int m0 = rd * kTcGroup, m1 = m0 + kTcGroup < g.tiles ? m0 + kTcGroup : g.tiles;
+                    const int m0 = rd * kGroup, m1 = m0 + kGroup < g.tiles ? m0 + kGroup : g.tiles;
                     for (int m = m0; m < m1; ++m) {
-                        const uint32_t d = tbase + (bb * kTcGroup + (uint32_t)(m - m0)) * NB;
-                        const uint64_t off = soff + (uint64_t)((uint32_t)m * 128u * 4u); // 128 positions x 64 B
+                        const uint32_t dt = tbase + (2 * bb + (uint32_t)(m - m0)) * kSlot;
+                        const uint64_t at = a0 + (uint64_t)(((uint32_t)s * g.stage_bytes) >> 4) +
+                                            (uint64_t)((uint32_t)m * 128u * 8u); // 128 rows x 128 B
+                        // kernel row d, input position x + j of the run x .. x + G - 1, channel half h: tap u = 2 - j + k
+                        // of the run's position k, for the positions k0 <= k < k1 whose window holds it
 #pragma unroll
-                        for (int j = 0; j < kTapsB * 2; ++j)
-                            tc::mma_bf16(d, adesc[j] + off, bdesc[j], idesc, j != 0);
+                        for (int d = 0; d < 3; ++d) {
+                            const int ulo = d == 2 && MODE != kBwd ? 2 : 0, uhi = d == 2 && MODE == kBwd ? 2 : 4;
+                            const uint64_t ar = at + (uint64_t)((uint32_t)(MODE == kBwd ? 2 - d : d) * (uint32_t)g.P * 8u);
+                            const uint64_t bplane = (uint64_t)(((d == 2 ? 3u : 5u) * kTap) >> 4);
+#pragma unroll
+                            for (int j = -2; j <= G + 1; ++j) {
+                                const int k0 = ulo - 2 + j > 0 ? ulo - 2 + j : 0, k1 = uhi - 1 + j < G ? uhi - 1 + j : G;
+                                if (k0 >= k1)
+                                    continue;
+                                const int run = (j + G) / G - 1, pos = (j + G) % G; // the run it lies in, its position there
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) { // 16 channels at 16 h
+                                    const uint64_t A = ar + (uint64_t)(pos >> 1) * slab +
+                                                       (uint64_t)(int64_t)(run * 8 + (pos & 1) * 4 + h * 2);
+                                    const uint64_t B = bd[d] + (uint64_t)(2 * h) * bplane +
+                                                       (uint64_t)((uint32_t)(2 - j + k0 - ulo) * (kTap >> 4));
+                                    // position j + 2 meets its first tap here: its columns do not accumulate yet
+                                    const bool first = d == 0 && h == 0 && j + 2 < G;
+                                    const int ka = first ? k1 - 1 : k1; // accumulating positions k0 .. ka - 1
+                                    if (ka > k0) {
+                                        tc::mma_bf16_warp<true>(dt + k0 * NB, A, B, tc::idesc_bf16_f32(128, (ka - k0) * NB));
+                                        if (MODE == kBwd)
+                                            tc::mma_bf16_warp<true>(dt + k0 * NB, A + lo_off, B,
+                                                                    tc::idesc_bf16_f32(128, (ka - k0) * NB));
+                                    }
+                                    if (first) {
+                                        const uint64_t B1 = B + (uint64_t)((uint32_t)(ka - k0) * (kTap >> 4));
+                                        tc::mma_bf16_warp<false>(dt + ka * NB, A, B1, tc::idesc_bf16_f32(128, NB));
+                                        if (MODE == kBwd)
+                                            tc::mma_bf16_warp<true>(dt + ka * NB, A + lo_off, B1, tc::idesc_bf16_f32(128, NB));
+                                    }
+                                }
+                            }
+                        }
                     }
-                    tc::commit(tfull0 + 8 * bb);
+                    tc::commit_warp(tfull0 + 8 * bb);
                 }
                 if (!ok)
                     break;
-                tc::commit(empty0 + 8 * s); // stage s is free once this item's MMAs have read it
+                tc::commit_warp(empty0 + 8 * s); // stage s is free once this item's MMAs have read it
             }
-            tc::commit(drain); // every MMA issued above has completed before the CTA ends
-            if (!tc::mbar_wait(drain, 0u, kTcMaxPolls))
+            tc::commit_warp(drain); // every MMA issued above has completed before the CTA ends
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(drain, 0u, kTcMaxPolls)))
                 ok = 0;
         }
-    } else { // warps 0-3: epilogue, tensor-memory lanes 32 warp .. 32 warp + 31
+    } else { // epilogue, tensor-memory lanes 32 (warp % 4) .. + 31; 8 warps: slot warp / 4, 4 warps: both slots
         float bv[kCh];
 #pragma unroll
         for (int c = 0; c < kCh; ++c)
-            bv[c] = LAST ? 0.f : __ldg(&bias[c]);
-        const float b0 = LAST ? __ldg(la.bD) : 0.f;
+            bv[c] = MODE == kFwd ? __ldg(&a.bias[c]) : 0.f;
+        const float b0 = MODE == kLast ? __ldg(a.la.bD) : 0.f;
+        uint4 *scratch = reinterpret_cast<uint4 *>(smem + scratch_off + (uint32_t)warp * kRunScratch);
         uint32_t tcount = 0;
         for (int it = blockIdx.x; ok && it < total; it += gridDim.x) {
-            const int b = it / g.YB, y0 = (it - b * g.YB) * g.R;
+            const int bi = it / g.YB, y0 = (it - bi * g.YB) * g.R;
             for (int rd = 0; rd < rounds; ++rd, ++tcount) {
                 const uint32_t bb = tcount & 1u;
-                const bool got =
-                    __any_sync(0xffffffffu, tc::mbar_wait(tfull0 + 8 * bb, (tcount >> 1) & 1u, kTcMaxPolls));
-                tc::fence_after_sync();
-                if (!got) {
-                    ok = 0;
-                    break;
-                }
-                const int m0 = rd * kTcGroup, m1 = m0 + kTcGroup < g.tiles ? m0 + kTcGroup : g.tiles;
-                for (int m = m0; m < m1; ++m) {
-                    const uint32_t col = tbase + ((uint32_t)(32 * warp) << 16) + (bb * kTcGroup + (uint32_t)(m - m0)) * NB;
-                    const int q = m * 128 + 32 * warp + lane, r = q / g.P, xp = q - r * g.P;
-                    if (LAST) {
-                        const float acc = tc::ld_32x32b_x1(col);
-                        if (r < g.R && y0 + r < g.L && xp >= 2 && xp < g.L + 2) {
-                            const size_t p = ((size_t)b * g.L + y0 + r) * g.L + (xp - 2);
-                            const float fv = b0 + acc;
-                            const float sv = la.negate ? -(float)la.spins[p] : (float)la.spins[p];
-                            la.f[p] = fv;
-                            la.ll[p] = log_sigmoid(sv * fv);
-                            if (la.dF)
-                                la.dF[p] = -la.inv_n * sv * sigmoid(-sv * fv);
+                const int m0 = rd * kGroup;
+                const int slot0 = EW == 8 ? warp >> 2 : 0;
+                const int slot1 = EW == 8 ? slot0 + 1 : (G == 4 || m0 + 1 < g.tiles ? 2 : 1);
+                bool waited = false;
+#pragma unroll 1
+                for (int slot = slot0; slot < slot1; ++slot) {
+                    const int m = G == 2 ? m0 + slot : m0;
+                    const uint32_t col = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (2 * bb + (uint32_t)slot) * kSlot;
+                    const uint32_t q = (uint32_t)(m * 128 + 32 * (warp & 3) + lane), row = __umulhi(q, g.inv_p),
+                                   pp = q - row * (uint32_t)g.P;
+                    const uint32_t smp = g.S == 1 ? 0u : __umulhi(row, g.inv_rows), r = row - smp * (uint32_t)(g.R + 2);
+                    const int b = bi * g.S + (int)smp, y = y0 + (int)r;
+                    const bool live = pp >= 1 && (int)r < g.R && y < g.L && (int)smp < g.S && b < a.n && m < g.tiles;
+                    // first position of the slot's pair, and the pair's index for the lanes that store it
+                    const size_t p = ((size_t)b * g.L + y) * g.L + G * (pp - 1) + (G == 4 ? 2 * slot : 0);
+                    const uint32_t pair = live ? (uint32_t)(p >> 1) : ~0u;
+                    uint4 mk[8];
+                    if (MODE == kBwd) { // mask chunks as this lane stores them, in flight during the wait
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const uint32_t pr = __shfl_sync(0xffffffffu, pair, 4 * i + (lane >> 3));
+                            mk[i] = pr == ~0u ? make_uint4(0u, 0u, 0u, 0u)
+                                              : __ldg(reinterpret_cast<const uint4 *>(a.mask) + (size_t)pr * 8 + (lane & 7));
                         }
-                        continue;
                     }
-                    float v[kCh];
-                    tc::ld_32x32b_x32(col, v);
-                    if (r < g.R && y0 + r < g.L && xp >= 2 && xp < g.L + 2) {
-                        uint4 pk[4];
+                    if (!waited) {
+                        waited = true;
+                        ok = __any_sync(0xffffffffu, tc::mbar_wait(tfull0 + 8 * bb, (tcount >> 1) & 1u, kTcMaxPolls));
+                        tc::fence_after_sync();
+                        if (!ok)
+                            break;
+                    }
+                    float v[2 * kCh], acc[2];
+                    if (MODE == kLast) {
+                        acc[0] = tc::ld_32x32b_x1(col);
+                        acc[1] = tc::ld_32x32b_x1(col + NB);
+                    } else {
+                        tc::ld_32x32b_x64(col, v);
+                    }
+                    if (slot + 1 == slot1) { // the accumulator is in registers: the next MMAs may have it
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0)
+                            tc::mbar_arrive(tempty0 + 8 * bb);
+                    }
+                    if (MODE == kLast) {
+                        if (live) {
+                            const char2 s2 = *reinterpret_cast<const char2 *>(a.la.spins + p);
+                            const float sv[2] = {a.la.negate ? -(float)s2.x : (float)s2.x,
+                                                 a.la.negate ? -(float)s2.y : (float)s2.y};
+                            const float f0 = b0 + acc[0], f1 = b0 + acc[1];
+                            *reinterpret_cast<float2 *>(a.la.f + p) = make_float2(f0, f1);
+                            *reinterpret_cast<float2 *>(a.la.ll + p) =
+                                make_float2(log_sigmoid(sv[0] * f0), log_sigmoid(sv[1] * f1));
+                            if (a.la.dF)
+                                *reinterpret_cast<float2 *>(a.la.dF + p) =
+                                    make_float2(-a.la.inv_n * sv[0] * sigmoid(-sv[0] * f0),
+                                                -a.la.inv_n * sv[1] * sigmoid(-sv[1] * f1));
+                        }
+                    } else if (MODE == kFwd) {
+                        uint4 pk[8];
                         uint32_t *pw = reinterpret_cast<uint32_t *>(pk);
 #pragma unroll
-                        for (int c = 0; c < kCh; c += 2) {
-                            const __nv_bfloat162 h =
-                                __floats2bfloat162_rn(fmaxf(v[c] + bv[c], 0.f), fmaxf(v[c + 1] + bv[c + 1], 0.f));
+                        for (int c = 0; c < 2 * kCh; c += 2) {
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(v[c] + bv[c % kCh], 0.f),
+                                                                           fmaxf(v[c + 1] + bv[c % kCh + 1], 0.f));
                             pw[c / 2] = *reinterpret_cast<const uint32_t *>(&h);
                         }
-                        uint4 *dst = reinterpret_cast<uint4 *>(out + (((size_t)b * g.L + y0 + r) * g.L + (xp - 2)) * kCh);
+                        store_pairs<false>(scratch, lane, pk, pair, mk, reinterpret_cast<uint4 *>(a.out));
+                    } else {
+                        uint4 hi[8], lo[8];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            dst[k] = pk[k];
+                        for (int k = 0; k < 8; ++k)
+                            split8(v + 8 * k, hi[k], lo[k]);
+                        store_pairs<true>(scratch, lane, hi, pair, mk, reinterpret_cast<uint4 *>(a.out));
+                        store_pairs<true>(scratch, lane, lo, pair, mk, reinterpret_cast<uint4 *>(a.out_lo));
                     }
                 }
-                tc::fence_before_sync();
-                __syncwarp();
-                if (lane == 0)
-                    tc::mbar_arrive(tempty0 + 8 * bb);
+                if (!ok)
+                    break;
             }
         }
     }
     ok = __syncthreads_and(ok);
     if (!ok && tid == 0)
-        atomicExch(err, 1);
+        atomicExch(a.err, 1);
     tc::fence_after_sync();
     if (warp == 0)
-        tc::tmem_free(tbase, kTcCols);
+        tc::tmem_free(tbase, kCols);
+}
+
+template <int MODE>
+using ConvKernel = void (*)(const CUtensorMap, const CUtensorMap, const ConvArgs, const RunGeom);
+template <int MODE>
+ConvKernel<MODE> conv_kernel(const RunGeom &g)
+{
+    if (g.G == 4)
+        return g.ctas_per_sm == 2 ? k_conv_runs<MODE, 4, 2> : k_conv_runs<MODE, 4, 1>;
+    return g.ctas_per_sm == 2 ? k_conv_runs<MODE, 2, 2> : k_conv_runs<MODE, 2, 1>;
+}
+
+// Launch one convolution; map_lo only for BWD.
+template <int MODE>
+void launch_conv(const RunGeom &g, const CUtensorMap &hi, const CUtensorMap &lo, const ConvArgs &a, int sms,
+                 cudaStream_t st)
+{
+    const unsigned grid = (unsigned)std::min<size_t>((size_t)((a.n + g.S - 1) / g.S) * g.YB, (size_t)sms * g.ctas_per_sm);
+    launch_chained_on(st, true, conv_kernel<MODE>(g), grid, 32u * (epilogue_warps(MODE, g.ctas_per_sm) + 2), g.smem_bytes,
+                      hi, lo, a, g);
 }
 
 // Encoder of tensor maps, from the driver through the runtime (no link
@@ -553,150 +735,23 @@ cudaError_t activation_map(CUtensorMap *m, const bf16 *base, int n, int L, int P
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Gradients travel between the backward kernels as a BF16 hi + lo pair
-// (hi = bf16(v), lo = bf16(v - hi), ~16 mantissa bits): two [n][L][L][32] BF16
-// arrays in the space of one FP32 array, which the tensor cores read directly.
-__device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo)
+// The same tensor as runs of G positions (64 values = two positions, slab, x / G, y,
+// sample); one box is R + 2 rows of P runs of S samples of one slab, landing as
+// 128-byte rows in the 128-byte swizzle.
+cudaError_t run_map(CUtensorMap *m, const bf16 *base, int n, const RunGeom &g)
 {
-    bf16 h[8], l[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        h[k] = __float2bfloat16(v[k]);
-        l[k] = __float2bfloat16(v[k] - bf(h[k]));
-    }
-    hi = *reinterpret_cast<uint4 *>(h);
-    lo = *reinterpret_cast<uint4 *>(l);
-}
-
-// Gradient with respect to a 32 -> 32 layer's input, masked by the previous
-// layer's ReLU, on the fifth-generation tensor cores:
-//   out(p)[c] = [mask(p)[c] > 0] sum_t sum_o W[t][o][c] dz(p - d_t)[o].
-// Same padded-position implicit GEMM as the forward kernel with the taps negated
-// (rows y0 .. y0+R+1 staged) and the weights transposed into the B planes;
-// dz arrives as hi + lo (8 A planes) and each k step issues two MMAs into
-// the same FP32 accumulator; the masked result leaves as hi + lo.
-constexpr int kTcBwdGroup = 2;
-constexpr uint32_t kTcBwdCols = 128;
-
-__global__ void __launch_bounds__(128, 2) k_conv32_bwd_tc(const bf16 *__restrict__ dzh, const bf16 *__restrict__ dzl,
-                                                          bf16 *__restrict__ outh, bf16 *__restrict__ outl,
-                                                          const bf16 *__restrict__ W, const bf16 *__restrict__ mask,
-                                                          int n, TcConvGeom g, int *err)
-{
-    extern __shared__ __align__(128) unsigned char smem[];
-    const uint32_t sb = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t abytes = 8 * g.plane_bytes; // planes 0-3: hi, 4-7: lo
-    const uint32_t boff = abytes, bar0 = sb + boff + kTcB, tslot_off = boff + kTcB + 16;
-    for (uint32_t i = tid; i < abytes / 16; i += blockDim.x)
-        reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = tid; i < kTapsB * 4 * kCh; i += blockDim.x) { // B planes [t][o8][c] = W[t][8 o8 .. +7][c]
-        const int t = i / (4 * kCh), o8 = (i / kCh) % 4, c = i % kCh;
-        bf16 v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            v[k] = W[((size_t)t * kCh + o8 * 8 + k) * kCh + c];
-        *reinterpret_cast<uint4 *>(smem + boff + ((t * 4 + o8) * kCh + c) * 16) = *reinterpret_cast<uint4 *>(v);
-    }
-    if (warp == 0)
-        tc::tmem_alloc(sb + tslot_off, kTcBwdCols);
-    if (tid == 0) {
-        tc::mbar_init(bar0, 1);
-        tc::mbar_init(bar0 + 8, 1);
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t *>(smem + tslot_off);
-    const uint32_t idesc = tc::idesc_bf16_f32(128, kCh);
-    uint64_t adesc[kTapsB * 2], bdesc[kTapsB * 2];
-    if (tid == 0)
-        for (int t = 0; t < kTapsB; ++t)
-            for (int kc = 0; kc < 2; ++kc) {
-                adesc[t * 2 + kc] = tc::smem_desc(sb + (uint32_t)(2 * kc) * g.plane_bytes +
-                                                      (uint32_t)(2 - tap_dy(t) * g.P - tap_dx(t)) * 16u,
-                                                  g.plane_bytes, 128);
-                bdesc[t * 2 + kc] = tc::smem_desc(sb + boff + (uint32_t)(t * 4 + 2 * kc) * (kCh * 16), kCh * 16, 128);
-            }
-    const uint64_t lo_off = (uint64_t)((4u * g.plane_bytes) >> 4);
-    const int rounds = (g.tiles + kTcBwdGroup - 1) / kTcBwdGroup;
-    auto issue = [&](int rd) {
-        const int m0 = rd * kTcBwdGroup, m1 = m0 + kTcBwdGroup < g.tiles ? m0 + kTcBwdGroup : g.tiles;
-        for (int m = m0; m < m1; ++m) {
-            const uint32_t d = tbase + (uint32_t)((rd & 1) * kTcBwdGroup + (m - m0)) * kCh;
-            const uint64_t off = (uint64_t)((uint32_t)m * 128u);
-#pragma unroll
-            for (int j = 0; j < kTapsB * 2; ++j) {
-                tc::mma_bf16(d, adesc[j] + off, bdesc[j], idesc, j != 0);
-                tc::mma_bf16(d, adesc[j] + off + lo_off, bdesc[j], idesc, 1u);
-            }
-        }
-        tc::commit(bar0 + 8u * (uint32_t)(rd & 1));
-    };
-    uint32_t uses[2] = {0u, 0u};
-    int ok = 1;
-    for (int it = blockIdx.x; ok && it < n * g.YB; it += gridDim.x) {
-        const int b = it / g.YB, y0 = (it - b * g.YB) * g.R;
-        for (int i = tid; i < (g.R + 2) * g.L * 8; i += blockDim.x) { // rows y0 .. y0+R+1, hi and lo
-            const int rho = i / (g.L * 8), rem = i - rho * g.L * 8, x = rem >> 3, pl = rem & 7, yy = y0 + rho;
-            const bool inside = yy < g.L;
-            const bf16 *src = (pl < 4 ? dzh : dzl) + (((size_t)b * g.L + (inside ? yy : 0)) * g.L + x) * kCh + (pl & 3) * 8;
-            const uint32_t dst = sb + (uint32_t)pl * g.plane_bytes + (uint32_t)(4 + rho * g.P + x) * 16u;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(inside ? 16 : 0)
-                         : "memory");
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        tc::fence_smem_for_async();
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
-        if (tid == 0)
-            issue(0);
-        for (int rd = 0; rd < rounds; ++rd) {
-            if (tid == 0 && rd + 1 < rounds)
-                issue(rd + 1);
-            const int s = rd & 1;
-            const bool got = tc::mbar_wait(bar0 + 8u * s, uses[s] & 1u, kTcMaxPolls);
-            ++uses[s];
-            tc::fence_after_sync();
-            const int m0 = rd * kTcBwdGroup, m1 = m0 + kTcBwdGroup < g.tiles ? m0 + kTcBwdGroup : g.tiles;
-            for (int m = m0; m < m1; ++m) {
-                float v[kCh];
-                tc::ld_32x32b_x32(tbase + ((uint32_t)(32 * warp) << 16) + (uint32_t)(s * kTcBwdGroup + (m - m0)) * kCh,
-                                  v);
-                const int q = m * 128 + 32 * warp + lane, r = q / g.P, xp = q - r * g.P;
-                if (got && r < g.R && y0 + r < g.L && xp >= 2 && xp < g.L + 2) {
-                    const size_t p = ((size_t)b * g.L + y0 + r) * g.L + (xp - 2);
-                    const uint4 *mk = reinterpret_cast<const uint4 *>(mask + p * kCh);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint4 mv = mk[k];
-                        const bf16 *m8 = reinterpret_cast<const bf16 *>(&mv);
-                        float o[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            o[j] = bf(m8[j]) > 0.f ? v[8 * k + j] : 0.f;
-                        uint4 hi, lo;
-                        split8(o, hi, lo);
-                        reinterpret_cast<uint4 *>(outh + p * kCh)[k] = hi;
-                        reinterpret_cast<uint4 *>(outl + p * kCh)[k] = lo;
-                    }
-                }
-            }
-            tc::fence_before_sync();
-            ok = __syncthreads_and(ok && got);
-            tc::fence_after_sync();
-            if (!ok)
-                break;
-        }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (!ok && tid == 0)
-        atomicExch(err, 1);
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0)
-        tc::tmem_free(tbase, kTcBwdCols);
+    const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc)
+        return cudaErrorNotSupported;
+    const cuuint64_t L = (cuuint64_t)g.L, G = (cuuint64_t)g.G;
+    const cuuint64_t dims[5] = {64, G / 2, L / G, L, (cuuint64_t)n};
+    const cuuint64_t strides[4] = {128, 64 * G, 64 * L, 64 * L * L};
+    const cuuint32_t box[5] = {64, 1, (cuuint32_t)g.P, (cuuint32_t)(g.R + 2), (cuuint32_t)g.S};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // Stage rows y-2..y of a [n][L][L][32] BF16 activation into smem rows of L+4
@@ -718,6 +773,7 @@ __global__ void k_logq(const float *ll, double *logq, int L)
     __shared__ double part[32];
     const int b = blockIdx.x, n = L * L;
     double acc = 0.0;
+    chain_wait(true);
     for (int i = threadIdx.x; i < n; i += blockDim.x)
         acc += (double)ll[(size_t)b * n + i];
 #pragma unroll
@@ -1721,6 +1777,7 @@ struct mc_van {
     const bf16 *zero = nullptr; // 5 kTapBytes of zeros
     float *dwpart = nullptr; // per-CTA partial gradients of k_dw32_tc
     int *err = nullptr;      // device fault latch (a bounded completion wait gave up)
+    RunGeom conv[3];         // geometries of the convolutions (kFwd, kLast, kBwd)
     int sms = 0;
     bool weights_ready = false;
 };
@@ -1831,6 +1888,12 @@ cudaError_t raise_smem_limit(const void *kernel, size_t bytes)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+template <int MODE>
+cudaError_t raise_conv_limit(const RunGeom &g)
+{
+    return raise_smem_limit((const void *)conv_kernel<MODE>(g), g.smem_bytes);
+}
+
 cudaError_t prep(mc_van *w)
 {
     k_prep_weights<<<64, 256, 0, w->stream>>>(w->p, w->dp, w->wh, w->w1, w->wD, w->bias);
@@ -1852,29 +1915,27 @@ cudaError_t forward(mc_van *w, int n, int negate, double *logq, float *dF)
     const unsigned l1g =
         (unsigned)std::min<long long>(((long long)n * L * L + kL1Threads - 1) / kL1Threads, (long long)w->sms * 8);
     k_layer1_tc<<<l1g, kL1Threads, 0, w->stream>>>(w->spins, negate, w->w1, w->bias, w->H, n, L, w->err);
-    const TmaConvGeom tg = tma_conv_geom(L);
-    const unsigned tcg = (unsigned)std::min<size_t>((size_t)n * tg.YB, (size_t)w->sms * tg.ctas_per_sm);
-    const LastLayerArgs none{};
-    const LastLayerArgs last{w->wD, w->bias + (D - 1) * kCh, w->spins, negate, w->f, w->ll, dF, 1.0f / n};
+    const RunGeom &gh = w->conv[kFwd], &gl = w->conv[kLast];
     for (int l = 1; l <= D - 1; ++l) { // hidden layers 1 .. D-2, then the last layer
         CUtensorMap in_map;
-        const cudaError_t e = activation_map(&in_map, w->H + (l - 1) * layer, n, L, tg.P, tg.R + 2);
+        const bool is_last = l == D - 1;
+        const cudaError_t e = run_map(&in_map, w->H + (l - 1) * layer, n, is_last ? gl : gh);
         if (e != cudaSuccess)
             return e;
-        const bool is_last = l == D - 1;
-        bf16 *out = is_last ? nullptr : w->H + l * layer;
-        const bf16 *wl = is_last ? nullptr : w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh;
-        const float *bl = is_last ? nullptr : w->bias + l * kCh;
-        if (tg.ctas_per_sm == 2 && is_last)
-            k_conv32_tma<2, true><<<tcg, 192, tg.smem_bytes, w->stream>>>(in_map, out, wl, bl, last, n, tg, w->err);
-        else if (tg.ctas_per_sm == 2)
-            k_conv32_tma<2, false><<<tcg, 192, tg.smem_bytes, w->stream>>>(in_map, out, wl, bl, none, n, tg, w->err);
-        else if (is_last)
-            k_conv32_tma<1, true><<<tcg, 192, tg.smem_bytes, w->stream>>>(in_map, out, wl, bl, last, n, tg, w->err);
-        else
-            k_conv32_tma<1, false><<<tcg, 192, tg.smem_bytes, w->stream>>>(in_map, out, wl, bl, none, n, tg, w->err);
+        ConvArgs a{};
+        a.n = n;
+        a.err = w->err;
+        if (is_last) {
+            a.la = LastLayerArgs{w->wD, w->bias + (D - 1) * kCh, w->spins, negate, w->f, w->ll, dF, 1.0f / n};
+            launch_conv<kLast>(gl, in_map, in_map, a, w->sms, w->stream);
+        } else {
+            a.W = w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh;
+            a.bias = w->bias + l * kCh;
+            a.out = w->H + l * layer;
+            launch_conv<kFwd>(gh, in_map, in_map, a, w->sms, w->stream);
+        }
     }
-    k_logq<<<n, 256, 0, w->stream>>>(w->ll, logq, L);
+    launch_chained_on(w->stream, true, k_logq, (unsigned)n, 256u, 0, (const float *)w->ll, logq, L);
     return cudaGetLastError();
 }
 
@@ -1897,8 +1958,7 @@ cudaError_t backward(mc_van *w, int n)
     const unsigned eg = (unsigned)std::min<size_t>(rg, (size_t)kMaxDwBlocks * kDwPart / kEdgeOutD);
     k_layerD_bwd_w<<<eg, 256, 0, w->stream>>>(w->dF, hD, w->dwpart, n, L);
     k_edge_grad_reduce<false><<<kEdgeOutD, 256, 0, w->stream>>>(w->dwpart, (int)eg, w->g, w->dp);
-    const TcConvGeom tgb = tc_conv_geom(L, 8);
-    const unsigned tcg = (unsigned)std::min<size_t>((size_t)n * tgb.YB, (size_t)w->sms * 2);
+    const RunGeom &gb = w->conv[kBwd];
     // k_dw32_tc: two CTAs per SM (256 tensor-memory columns and at most 110 KB of stages each)
     const DwTcGeom dg = dw_tc_geom(L);
     const unsigned dwg = (unsigned)std::min<size_t>(std::min<size_t>((size_t)n * L, (size_t)w->sms * 2), kMaxDwBlocks);
@@ -1913,9 +1973,20 @@ cudaError_t backward(mc_van *w, int n)
             return e;
         k_dw32_tc<<<dwg, 192, dg.smem_bytes, w->stream>>>(zh_map, zl_map, x_map, w->dwpart, n, dg, w->err);
         k_dw_reduce<<<(kDwPart + 255) / 256, 256, 0, w->stream>>>(w->dwpart, (int)dwg, w->g, w->dp, l);
-        k_conv32_bwd_tc<<<tcg, 128, tgb.smem_bytes, w->stream>>>(dzh, dzl, nxh, nxl,
-                                                                 w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh,
-                                                                 w->H + (l - 1) * layer, n, tgb, w->err);
+        CUtensorMap hi_map, lo_map;
+        e = run_map(&hi_map, dzh, n, gb);
+        if (e == cudaSuccess)
+            e = run_map(&lo_map, dzl, n, gb);
+        if (e != cudaSuccess)
+            return e;
+        ConvArgs a{};
+        a.W = w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh;
+        a.mask = w->H + (l - 1) * layer;
+        a.out = nxh;
+        a.out_lo = nxl;
+        a.n = n;
+        a.err = w->err;
+        launch_conv<kBwd>(gb, hi_map, lo_map, a, w->sms, w->stream);
         std::swap(dzh, nxh);
         std::swap(dzl, nxl);
     }
@@ -2002,20 +2073,18 @@ mc_status mc_van_create(mc_van **out, int32_t L, int32_t batch, int32_t depth, u
     w->acc = reinterpret_cast<int *>(b + o.acc);
     w->hist = reinterpret_cast<bf16 *>(b + o.hist);
     w->zero = reinterpret_cast<const bf16 *>(b + o.zero);
+    for (int mode = 0; mode < 3; ++mode)
+        w->conv[mode] = run_geom(L, mode);
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaMemsetAsync(w->ws, 0, o.hist, w->stream); // params, Adam state, buffers
     if (e == cudaSuccess)
-        e = raise_smem_limit(tma_conv_geom(L).ctas_per_sm == 2 ? (const void *)k_conv32_tma<2, false>
-                                                               : (const void *)k_conv32_tma<1, false>,
-                             tma_conv_geom(L).smem_bytes);
+        e = raise_conv_limit<kFwd>(w->conv[kFwd]);
     if (e == cudaSuccess)
-        e = raise_smem_limit(tma_conv_geom(L).ctas_per_sm == 2 ? (const void *)k_conv32_tma<2, true>
-                                                               : (const void *)k_conv32_tma<1, true>,
-                             tma_conv_geom(L).smem_bytes);
+        e = raise_conv_limit<kLast>(w->conv[kLast]);
     if (e == cudaSuccess)
-        e = raise_smem_limit((const void *)k_conv32_bwd_tc, tc_conv_geom(L, 8).smem_bytes);
+        e = raise_conv_limit<kBwd>(w->conv[kBwd]);
     if (e == cudaSuccess)
         e = raise_smem_limit((const void *)k_dw32_tc, dw_tc_geom(L).smem_bytes);
     if (e == cudaSuccess)
