@@ -813,14 +813,15 @@ struct Piece {
 // 13 positions p - d_t of every p:
 //   dZ_{D-1}(p)[c] = [h(p)[c] > 0] sum_t wD[t][c] dF(p - d_t),
 //   gW[t][c] = sum_p h(p)[c] dF(p - d_t),  gb = sum_p dF(p), h = h_{D-1}.
-// A warp takes a row, four positions at a time with 8 lanes of 4 channels each; a lane keeps its 52 weights and 52 gradient sums in registers, so that a
-// position costs 13 shared-memory reads (dF) and 104 multiply-adds per lane, and h is
-// read once.  The lanes of a channel, then the warps are added in a fixed order into the CTA's
-// partial sums part[output][CTA] (reduced in a fixed order by k_edge_grad_reduce: the
-// gradient does not depend on the order the CTAs finish in).  L = 64, batch 512:
-// 105 us for the 146 + 190 us of separate kernels that read weights and
-// activations per tap from shared memory; bound by the multiply-adds (47 us) and 400
-// MB of activations and gradients (60 us).
+// A warp takes a row, four positions at a time with 8 lanes of 4 channels each; a lane
+// keeps its 52 weights and 52 gradient sums in registers, so that a position costs 13
+// shared-memory reads (dF) and 104 multiply-adds per lane, and h is read once.  The
+// lanes of a channel, then the warps are added in a fixed order into the CTA's partial
+// sums part[output][CTA] (reduced in a fixed order by k_edge_grad_reduce: the gradient
+// does not depend on the order the CTAs finish in).  L = 64, batch 512: 105 us for the
+// 146 + 190 us of separate kernels that read weights and activations per tap from shared
+// memory (193 with h prefetched one position ahead in registers: latency-bound); bound
+// by the multiply-adds (47 us) and 400 MB of activations and gradients (60 us).
 constexpr int kEdgeOutD = kTapsB * kCh + 1;  // last layer: 13 x 32 weights + bias
 constexpr int kEdgeOut1 = kCh * (kTapsA + 1); // first layer: 32 x (12 weights + bias)
 constexpr int kEdgeThreads = 128, kEdgeCtas = 3;
@@ -1376,6 +1377,19 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(u) : "f"(hi), "f"(lo));
     return u;
 }
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&d);
+}
+// max(., 0) of the pair: the same bits as packing max(lo, 0), max(hi, 0)
+__device__ __forceinline__ uint32_t relu_pack(float lo, float hi)
+{
+    uint32_t u = pack_bf16x2(lo, hi);
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(u) : "r"(0u));
+    return u;
+}
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
@@ -1745,6 +1759,765 @@ __global__ void __launch_bounds__(kSampleThreads, 1) k_sample(const bf16 *__rest
     }
 }
 
+// ------------------------------------------------- sampler, columns streamed
+// The same sampling as k_sample (bit for bit: every hidden value adds its taps in raster
+// order, 16 channels at a time), arranged so that the chain of a step holds nothing that
+// could be computed before it.  The latency of a step is what bounds the sampler: L^2
+// of them follow one another whatever the batch.
+//
+//   * A chain warp owns 16 samples and runs first layer, hidden layers, output layer and
+//     draw in its registers: a layer's accumulator fragment, packed to BF16, is the next
+//     layer's operand fragment (m16n8k16), so that a layer costs 8 matrix instructions
+//     (tap 12) and an epilogue, with no shared-memory round trip between layers.
+//   * For each hidden layer and 16 samples a helper warp prepares the accumulators over
+//     taps 0..11.  Taps 0..9 are of the two rows above, known for a whole row: the helper
+//     computes them for the next block of 4 positions while the chain works on the
+//     current one, a quarter of the block's taps per step, so that a weight fragment
+//     serves 4 positions and a column of activations up to 5 taps.  Taps 10 and 11 (the
+//     two positions just before) are added step by step.
+//   * For each 16 samples a warp prepares the first layer's sum over the spins other than
+//     the last one and the uniforms, and two warps the output layer's sum over taps 0..11
+//     and log q: after a step the terms of its own values first, since the chain waits for
+//     them, then the upper rows' terms of the position after.
+//
+// Activations of earlier rows stay in the ring arrays in global memory, written and read
+// back by the same lane in its own order (an asynchronous 16-byte copy per lane and half
+// a column: nothing crosses lanes).  A helper publishes position k's accumulators, the
+// chain loads them, then publishes the layer's input at k, from which the helper finishes
+// position k + 1: each slot is read before the next value is written.  No register
+// spills and loops short enough to share the instruction cache are what the roles'
+// registers and code are cut for: 12 bytes of spills cost 8%, 56 missed lines a step 15%.
+//
+// us per position at L = 64, depth 6, 4096 samples: 1.68 against 4.45 for k_sample (depth 5:
+// 1.48 / 3.63, depth 4: 1.24 / 2.94, depth 3: 1.18 / 2.18; 1.7 to 2.1 / 4.5 to 4.9 on L = 8
+// to 50).  Tensor throughput would allow 0.87 (832 matrix instructions per step and SM, 208 per
+// sub-core at 8 cycles); the chain's latency is ~3200 cycles, of them ~1300 in its matrix
+// instructions, which share the tensor cores with the helpers'.
+constexpr int kHalf = 16;                     // samples of a chain warp
+constexpr int kColBytes = kHalf * kCh * 2;    // 16 samples of one position: 1 KB
+constexpr int kPipeTiles = 7;                 // columns a helper has staged or in flight
+constexpr int kPipeSide = 6;                  // columns (of two rows) of a side warp
+constexpr int kPipeHidden = 4;                // hidden layers: 8 helper warps
+constexpr int kPipeMinL = 8;                  // a block's columns are known a block ahead
+constexpr int kPipeThreads = 32 * (2 * kPipeHidden + 8); // helpers; chains and first-layer warps; output warps
+constexpr int kPipeRegs = 128; // at launch, a thread; then by warp group: helpers, chains, output warps
+constexpr int kHelperRegs = 184, kChainRegs = 88, kOutRegs = 56;
+static_assert(2 * kHelperRegs + kChainRegs + kOutRegs == 4 * kPipeRegs, "the split is the launch's total");
+// words of a row's spins as bits, from bit 2 on (read two at a time)
+__host__ __device__ inline int spin_words(int L) { return (L - 1) / 32 + 2; }
+
+struct PipeSmem { // byte offsets
+    int w, fifo, p, h, p0, win, hn, po, w1, wd, bias, draw, u, bits, bar, total;
+};
+__host__ __device__ inline PipeSmem pipe_smem(int D, int L)
+{
+    const int nh = D - 2;
+    PipeSmem o{};
+    int at = 0;
+    auto take = [&](int bytes) {
+        const int r = at;
+        at += (bytes + 15) & ~15;
+        return r;
+    };
+    o.w = take(nh * kTapsB * kCh * kCh * 2);       // fragments [l][t][k-step][n-tile pair][lane]
+    o.fifo = take(nh * 2 * kPipeTiles * kColBytes); // per helper
+    o.p = take(nh * 2 * kHalf * kCh * 4);          // accumulators of position k, fragments
+    o.h = take(nh * 2 * kColBytes);                // input of hidden layer l at k, fragments
+    o.p0 = take(2 * 2 * kHalf * kCh * 4);          // first-layer sums, two steps, fragments
+    o.win = take(2 * kPipeSide * 2 * kColBytes);   // the output layer's window of two rows
+    o.hn = take(2 * kColBytes);                    // last hidden layer at k, ring_elem order
+    o.po = take(2 * 32 * 16);                      // output-layer sums, by the chain's lanes
+    o.w1 = take(kTapsA * kCh * 4);
+    o.wd = take(kTapsB * kCh * 4);
+    o.bias = take(((D - 1) * kCh + 1) * 4);
+    o.draw = take(2 * kHalf * 8);                  // s_k, s_k f_k
+    o.u = take(2 * 2 * kHalf * 4);                 // uniforms, two steps
+    o.bits = take(2 * kHalf * 3 * spin_words(L) * 4);
+    o.bar = take((2 * nh + 2) * 8);
+    o.total = at;
+    return o;
+}
+
+// D(16 x 8) += A(16 x 16) B(16 x 8), A as one uint4 fragment.
+__device__ __forceinline__ void mma16(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1)
+{
+    mma_bf16(c, a.x, a.y, a.z, a.w, b0, b1);
+}
+// c += A B over one 16-channel step and all four n-tiles; w: the lane's two weight quads.
+__device__ __forceinline__ void mma_step(float (&c)[4][4], const uint4 &a, const uint4 &w0, const uint4 &w1)
+{
+    mma16(c[0], a, w0.x, w0.y);
+    mma16(c[1], a, w0.z, w0.w);
+    mma16(c[2], a, w1.x, w1.y);
+    mma16(c[3], a, w1.z, w1.w);
+}
+
+// The channel of accumulator column i (n-tile i / 8).  The last hidden layer's columns are
+// ordered so that a lane of the fragment holds four channels of a part of the output layer's
+// sum one after the other (4 t + 0..3 and 16 + 4 t + 0..3 for lane t of a row).
+__host__ __device__ inline int pipe_channel(bool last, int i)
+{
+    return last ? (i >> 4) * 16 + ((i >> 1) & 3) * 4 + ((i >> 3) & 1) * 2 + (i & 1) : i;
+}
+
+// wait_phase for whole warps: the lanes agree before the branch, which is then uniform (a
+// loop that lanes may leave one by one costs ~100 cycles more, and the chain waits
+// six times a step).
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *abort, int *err)
+{
+#pragma unroll 1
+    for (int it = 0; it < kTcMaxPolls; ++it) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        if (__all_sync(0xffffffffu, done))
+            return true;
+        if (__any_sync(0xffffffffu, *abort))
+            return false;
+    }
+    *abort = 1;
+    atomicExch(err, 1);
+    return false;
+}
+
+// What the chain waits for (nh + 2 times a step) is handed over by named barriers, at which
+// the preparing warps arrive and only the chain warp waits: a completed mbarrier wait took
+// it ~200 cycles.  The next arrival always follows from a signal the chain gives after its
+// wait.  The warps that wait for the chain do so by mbarriers, several on the same one.
+constexpr int kReadyHidden = 1, kReadyFirst = kReadyHidden + 2 * kPipeHidden, kReadyOut = kReadyFirst + 2;
+__device__ __forceinline__ void ready(int id, int threads)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// After a wait that gave up: arrive until the chain, which stops at its next step, has left.
+__device__ __forceinline__ void release_chain(int id, int threads, volatile int *done)
+{
+#pragma unroll 1
+    for (int it = 0; it < kTcMaxPolls && !__any_sync(0xffffffffu, *done); ++it)
+        ready(id, threads);
+}
+
+template <int REGS>
+__device__ __forceinline__ void regs_grow()
+{
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+template <int REGS>
+__device__ __forceinline__ void regs_shrink()
+{
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+
+__global__ void __launch_bounds__(kPipeThreads, 1)
+    k_sample_pipe(const bf16 *__restrict__ wh, const float *__restrict__ w1, const float *__restrict__ wD,
+                  const float *__restrict__ bias, int D, int L, int n, bf16 *hist, int8_t *out, double *logq, PhiloxKey key,
+                  uint32_t round, const uint32_t *ids, int *err)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int abort_flag, chain_done[2];
+    volatile int *abort = &abort_flag;
+    const int nh = D - 2, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int s0 = blockIdx.x * kSampleTile, P = L * L;
+    bool ok = true; // no wait has given up
+    const PipeSmem o = pipe_smem(D, L);
+    const int words = spin_words(L);
+    // ---- weights (fragment order), biases, cleared spins, barriers
+    for (int i = tid; i < nh * kTapsB * 512; i += kPipeThreads) { // 32-bit words
+        const int q = i & 3, ln = (i >> 2) & 31, pair = (i >> 7) & 1, ks = (i >> 8) & 1, lt = i >> 9;
+        const int oc = pipe_channel(lt / kTapsB == nh - 1, (2 * pair + (q >> 1)) * 8 + (ln >> 2)),
+                  c = ks * 16 + (q & 1) * 8 + (ln & 3) * 2;
+        reinterpret_cast<uint32_t *>(smem + o.w)[i] =
+            *reinterpret_cast<const uint32_t *>(wh + ((size_t)lt * kCh + oc) * kCh + c);
+    }
+    float *W1 = reinterpret_cast<float *>(smem + o.w1), *WD = reinterpret_cast<float *>(smem + o.wd),
+          *Bs = reinterpret_cast<float *>(smem + o.bias);
+    for (int i = tid; i < kCh * kTapsA; i += kPipeThreads) { // w1 is [o][t]; in the order of a lane's fragment columns
+        const int oc = i / kTapsA;
+        W1[(i % kTapsA) * kCh + ((oc >> 1) & 3) * 8 + (oc >> 3) * 2 + (oc & 1)] = w1[i];
+    }
+    for (int i = tid; i < kTapsB * kCh; i += kPipeThreads)
+        WD[i] = wD[i];
+    for (int i = tid; i < (D - 1) * kCh + 1; i += kPipeThreads)
+        Bs[i] = bias[i / kCh == nh ? nh * kCh + pipe_channel(true, i % kCh) : i];
+    for (int i = tid; i < 2 * kHalf * 3 * words; i += kPipeThreads)
+        reinterpret_cast<uint32_t *>(smem + o.bits)[i] = 0u;
+    const uint32_t bars = smem_u32(smem + o.bar);
+    if (tid == 0) {
+        abort_flag = chain_done[0] = chain_done[1] = 0;
+        for (int j = 0; j < 2 * nh + 2; ++j)
+            tc::mbar_init(bars + 8u * j, 1);
+    }
+    __syncthreads();
+    auto bar_h = [&](int l, int mt) { return bars + 8u * (uint32_t)((l - 1) * 2 + mt); };
+    auto bar_e = [&](int mt) { return bars + 8u * (uint32_t)(2 * nh + mt); };
+    auto signal = [&](uint32_t bar) { // after every lane's shared accesses before it
+        __syncwarp();
+        if (lane == 0)
+            tc::mbar_arrive(bar);
+    };
+    const size_t row_bytes = (size_t)L * kColBytes, ring_bytes = 3 * row_bytes; // of 16 samples and one layer
+    const size_t lstride = (size_t)gridDim.x * 2 * ring_bytes;
+
+    if (warp < 2 * kPipeHidden) { // ------------------------------------------------------------ helpers
+        regs_grow<kHelperRegs>();
+        const int l = 1 + (warp >> 1), mt = warp & 1;
+        if (l > nh)
+            return;
+        unsigned char *ring = reinterpret_cast<unsigned char *>(hist) + (l - 1) * lstride +
+                              ((size_t)blockIdx.x * 2 + mt) * ring_bytes + lane * 16;
+        unsigned char *fifo = smem + o.fifo + warp * kPipeTiles * kColBytes;
+        const uint4 *w = reinterpret_cast<const uint4 *>(smem + o.w) + (l - 1) * kTapsB * 128;
+        float4 *slotP = reinterpret_cast<float4 *>(smem + o.p + warp * (kHalf * kCh * 4)) + lane;
+        const uint4 *slotH = reinterpret_cast<const uint4 *>(smem + o.h + warp * kColBytes) + lane;
+        const uint32_t H = bar_h(l, mt);
+        // The columns of a block: rows y - 2 and y - 1, each x0 - 2 .. x0 + 5, column c of a row in
+        // slot c, the last in slot 0.  Taps dx = -2 .. 0 use columns 0..5 and are the last to use 0..2;
+        // taps dx = 1, 2 use 3..7.  What is free then is filled with the row's column 7 and the next row's.
+        int fy = 0, fx = 0, fr = 0, fm = 1; // the row whose columns are fetched: block, which row, (fy + 1) % 3
+        const unsigned char *rsrc = ring, *psrc = ring;
+        int rx = -2, px = 0; // its first column's x (a row outside the lattice: far outside), and the row's before
+        auto fetch = [&](const unsigned char *src, int x, int c, int s) {
+            const bool in = (unsigned)(x + c) < (unsigned)L;
+            const unsigned char *from = in ? src + c * kColBytes : ring;
+            cp16(fifo + s * kColBytes + lane * 16, from, in ? 16 : 0);
+            cp16(fifo + s * kColBytes + lane * 16 + 512, from + 512, in ? 16 : 0);
+        };
+        auto place = [&] { // where the row's columns are
+            const int m = fm + fr >= 3 ? fm + fr - 3 : fm + fr;
+            rx = fy < L && fy - 2 + fr >= 0 ? fx - 2 : -(1 << 20);
+            rsrc = ring + m * row_bytes + (ptrdiff_t)(fx - 2) * kColBytes;
+        };
+        auto next_row = [&] {
+            psrc = rsrc;
+            px = rx;
+            fr ^= 1;
+            if (fr == 0) {
+                fx += 4;
+                if (fx >= L) {
+                    fx = 0;
+                    ++fy;
+                    fm = fm == 2 ? 0 : fm + 1;
+                }
+            }
+            place();
+        };
+        auto column = [&](uint4(&a)[2], int c) {
+            const uint4 *p = reinterpret_cast<const uint4 *>(fifo + (c == 7 ? 0 : c) * kColBytes) + lane;
+            a[0] = p[0];
+            a[1] = p[32];
+        };
+        float cur[4][4][4], nxt[4][4][4]; // the accumulators of a block's positions; of the next block's
+        auto taps = [&](uint4(&a)[4][2], int r, int d) { // a: columns d .. d + 3, column c in a[c & 3]
+            const uint4 *wt = w + (5 * r + d) * 128 + lane;
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks) {
+                const uint4 w0 = wt[ks * 64], w1 = wt[ks * 64 + 32];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    mma_step(nxt[q], a[(d + q) & 3][ks], w0, w1);
+            }
+        };
+        auto first_taps = [&](int r) {
+            uint4 a[4][2];
+            cp_wait<0>();
+            column(a[0], 0);
+            column(a[1], 1);
+            column(a[2], 2);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                column(a[(d + 3) & 3], d + 3);
+                taps(a, r, d);
+            }
+            next_row();
+            fetch(psrc, px, 7, 0);
+            fetch(rsrc, rx, 1, 1);
+            fetch(rsrc, rx, 2, 2);
+            cp_commit();
+        };
+        auto last_taps = [&](int r) {
+            uint4 a[4][2];
+            cp_wait<0>();
+            column(a[3], 3);
+            column(a[0], 4);
+            column(a[1], 5);
+#pragma unroll
+            for (int d = 3; d < 5; ++d) {
+                column(a[(d + 3) & 3], d + 3);
+                taps(a, r, d);
+            }
+            fetch(rsrc, rx, 0, 0);
+#pragma unroll
+            for (int c = 3; c < 7; ++c)
+                fetch(rsrc, rx, c, c);
+            cp_commit();
+        };
+        uint4 a11[2] = {}; // the layer's input at the position before, in this row
+        int k = 0, stored = 0;
+        unsigned char *dst = ring; // of position k - 1 in the ring (position modulo 3 L)
+        // position k, at x: taps 10, 11, hand over
+        auto finish = [&](float(&c)[4][4], int x) {
+            if ((unsigned)x >= (unsigned)L)
+                return;
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            const uint4 *wt = w + 10 * 128 + lane;
+            if (x == 0)
+                a11[0] = a11[1] = zero;
+            mma_step(c, a11[0], wt[0], wt[32]);
+            mma_step(c, a11[1], wt[64], wt[96]);
+            if (k > 0) {
+                ok = wait_warp(H, (uint32_t)(k - 1) & 1u, abort, err);
+                a11[0] = slotH[0];
+                a11[1] = slotH[32];
+                *reinterpret_cast<uint4 *>(dst) = a11[0];
+                *reinterpret_cast<uint4 *>(dst + 512) = a11[1];
+                dst += kColBytes;
+                if (++stored == 3 * L) {
+                    stored = 0;
+                    dst = ring;
+                }
+                if (x == 0)
+                    a11[0] = a11[1] = zero;
+            }
+            wt += 128;
+            mma_step(c, a11[0], wt[0], wt[32]);
+            mma_step(c, a11[1], wt[64], wt[96]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                slotP[q * 32] = make_float4(c[q][0], c[q][1], c[q][2], c[q][3]);
+            ready(kReadyHidden + warp, 64);
+            ++k;
+        };
+        place();
+#pragma unroll
+        for (int c = 0; c < 7; ++c)
+            fetch(rsrc, rx, c, c);
+        cp_commit();
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    nxt[q][j][e] = 0.f;
+        // Two positions of a block at a time, between them the taps of one row above the next block; the block
+        // before the first has no positions.  (The loop's body stays one row long: the roles' loops have to share
+        // the instruction cache.  With all four positions written out, 56 lines a step missed it.)
+        int x0 = -4, r = 0;
+#pragma unroll 1
+        for (int y = 0; y < L && ok;) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (r == 0) {
+                            cur[q][j][e] = nxt[q][j][e];
+                            nxt[q][j][e] = 0.f;
+                        } else if (q < 2) {
+                            cur[q][j][e] = cur[q + 2][j][e];
+                        }
+                    }
+            finish(cur[0], x0 + 2 * r);
+            first_taps(r);
+            finish(cur[1], x0 + 2 * r + 1);
+            last_taps(r);
+            r ^= 1;
+            if (r == 0) {
+                x0 += 4;
+                if (x0 >= L) {
+                    x0 = 0;
+                    ++y;
+                }
+            }
+        }
+        cp_wait<0>();
+        if (!ok)
+            release_chain(kReadyHidden + warp, 64, chain_done + mt);
+        return;
+    }
+    if (warp >= 2 * kPipeHidden + 4) { // -------------------------------------------------- output layer
+        regs_shrink<kOutRegs>();
+        // two warps per half, 8 samples each: a lane has 8 channels of one (two of the sum's 8 parts)
+        const int mt = warp & 1, sub = (warp >> 1) & 1, ls = 8 * sub + (lane >> 2), qt = lane & 3, s = mt * kHalf + ls;
+        unsigned char *ring = reinterpret_cast<unsigned char *>(hist) + nh * lstride +
+                              ((size_t)blockIdx.x * 2 + mt) * ring_bytes + sub * 512 + lane * 16;
+        unsigned char *win = smem + o.win + mt * kPipeSide * 2 * kColBytes + sub * 512 + lane * 16;
+        const bf16 *Hn = reinterpret_cast<const bf16 *>(smem + o.hn + mt * kColBytes) + ring_elem(ls, qt * 8);
+        const float2 *draw = reinterpret_cast<const float2 *>(smem + o.draw) + s;
+        // part p of the sum goes to the chain's lane 4 (s % 8) + p % 4: float (s / 8) 2 + p / 4 of its four
+        float *Po = reinterpret_cast<float *>(smem + o.po) + mt * 128 + (lane >> 2) * 16 + (2 * qt & 3) * 4 + 2 * sub + (qt >> 1);
+        const float4 *wdl = reinterpret_cast<const float4 *>(WD) + 2 * qt;
+        double lq = 0.0; // of sample s, in the lane of its first channels
+        float po[2];
+        auto tap = [&](const uint4 &h, int t) {
+            const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const float4 w = wdl[t * 8 + p];
+                po[p] = __fmaf_rn(w.x, bf16_lo(hw[2 * p]), po[p]);
+                po[p] = __fmaf_rn(w.y, bf16_hi(hw[2 * p]), po[p]);
+                po[p] = __fmaf_rn(w.z, bf16_lo(hw[2 * p + 1]), po[p]);
+                po[p] = __fmaf_rn(w.w, bf16_hi(hw[2 * p + 1]), po[p]);
+            }
+        };
+        int slot = 0; // of column x - 2 of the position `rows_above` works on
+        auto rows_above = [&](int y, int x) { // taps 0..9 at (y, x)
+            po[0] = po[1] = 0.f;
+            const unsigned char *col[5];
+#pragma unroll
+            for (int d = 0; d < 5; ++d)
+                col[d] = win + (slot + d >= kPipeSide ? slot + d - kPipeSide : slot + d) * 2 * kColBytes;
+            slot = slot + 1 == kPipeSide ? 0 : slot + 1;
+            if (y >= 2 && x >= 2 && x + 2 < L) {
+#pragma unroll 1
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int d = 0; d < 5; ++d)
+                        tap(*reinterpret_cast<const uint4 *>(col[d] + r * kColBytes), 5 * r + d);
+                return;
+            }
+            int s = slot == 0 ? kPipeSide - 1 : slot - 1; // slot of column x - 2
+#pragma unroll 1
+            for (int t = 0, d = 0; t < 10; ++t) {
+                const int r = t >= 5;
+                if (y - 2 + r >= 0 && x - 2 + d >= 0 && x - 2 + d < L)
+                    tap(*reinterpret_cast<const uint4 *>(win + (s * 2 + r) * kColBytes), t);
+                s = s + 1 == kPipeSide ? 0 : s + 1;
+                if (++d == 5) {
+                    d = 0;
+                    s = s + 1 == kPipeSide ? 0 : s + 1; // five on in a ring of six: back to column x - 2
+                }
+            }
+        };
+        int cy = 0, cx = 3, cslot = 5, at = 3; // next column to fetch, its slot, its position modulo 3 L
+        auto fetch = [&] {                     // the next column, rows y - 2 and y - 1 there
+            if (cy < L) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    if (cy - 2 + r >= 0) {
+                        int from = at + (1 + r) * L;
+                        from = from >= 3 * L ? from - 3 * L : from;
+                        cp16(win + (cslot * 2 + r) * kColBytes, ring + (size_t)from * kColBytes);
+                    }
+            }
+            cp_commit();
+            cslot = cslot + 1 == kPipeSide ? 0 : cslot + 1;
+            at = at + 1 == 3 * L ? 0 : at + 1;
+            if (++cx == L) {
+                cx = 0;
+                ++cy;
+            }
+        };
+        // after step k - 1: taps 10, 11 at k, which the chain waits for (R1), then the upper rows' taps at k + 1
+        uint4 h10 = make_uint4(0u, 0u, 0u, 0u), h11 = h10;
+        unsigned char *dst = ring; // of position k - 1
+        int stored = 0;
+        rows_above(0, 0);
+        fetch(); // position 3
+        int y = 0, x = 0;
+#pragma unroll 1
+        for (int k = 0; k < P && ok; ++k) {
+            float lt = 0.f;
+            if (k > 0) {
+                ok = wait_warp(bar_e(mt), (uint32_t)(k - 1) & 1u, abort, err);
+                h10 = h11;
+                h11 = *reinterpret_cast<const uint4 *>(Hn);
+                lt = draw->y;
+            }
+            if (x >= 2)
+                tap(h10, 10);
+            if (x >= 1)
+                tap(h11, 11);
+            Po[0] = po[0];
+            Po[4] = po[1];
+            ready(kReadyOut + mt, 96);
+            if (k > 0) {
+                *reinterpret_cast<uint4 *>(dst) = h11;
+                dst += kColBytes;
+                if (++stored == 3 * L) {
+                    stored = 0;
+                    dst = ring;
+                }
+            }
+            cp_wait<0>(); // columns up to position k + 3
+            fetch();      // and k + 4
+            if (++x == L) {
+                x = 0;
+                ++y;
+            }
+            rows_above(y, x);
+            if (k > 0 && qt == 0)
+                lq += (double)log_sigmoid(lt);
+        }
+        if (ok)
+            wait_warp(bar_e(mt), (uint32_t)(P - 1) & 1u, abort, err);
+        if (qt == 0 && s0 + s < n)
+            logq[s0 + s] = lq + (double)log_sigmoid(draw->y);
+        cp_wait<0>();
+        if (!ok)
+            release_chain(kReadyOut + mt, 96, chain_done + mt);
+        return;
+    }
+    regs_shrink<kChainRegs>();
+
+    if (warp >= 2 * kPipeHidden + 2) { // --------------------------------------------- first layer, uniforms
+        const int mt = warp & 1, g = lane >> 2, qt = lane & 3; // samples g, g + 8; the fragment's columns
+        const int sb = mt * kHalf + g + 8 * (qt & 1), mine = qt < 2; // the sample whose spins and uniforms this lane keeps
+        const int gs = s0 + sb, live = mine && gs < n;
+        const uint32_t *bits = reinterpret_cast<const uint32_t *>(smem + o.bits) + mt * kHalf * 3 * words;
+        uint32_t *my_bits = reinterpret_cast<uint32_t *>(smem + o.bits) + sb * 3 * words;
+        const float2 *draw = reinterpret_cast<const float2 *>(smem + o.draw) + sb;
+        float *u = reinterpret_cast<float *>(smem + o.u) + sb;
+        const float4 *w1l = reinterpret_cast<const float4 *>(W1) + 2 * qt;
+        int8_t *out_g = out + (size_t)gs * P;
+        const uint32_t my_id = live ? (ids ? ids[gs] : (uint32_t)gs) : 0u;
+        uint4 rnd = make_uint4(0u, 0u, 0u, 0u);
+        float a[2][8];
+        auto spins_of = [&](int h, int row, int x) { // bit d: the spin of sample g + 8 h at (row, x - 2 + d)
+            const uint32_t *b = bits + ((g + 8 * h) * 3 + row % 3) * words + (x >> 5);
+            return __funnelshift_r(b[0], b[1], x & 31);
+        };
+        auto tap = [&](int t, uint32_t m0, uint32_t m1) { // bit 0 of m: the tap's spin
+            const float4 wa = w1l[t * 8], wb = w1l[t * 8 + 1];
+            const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            const float v[2] = {m0 & 1u ? 1.f : -1.f, m1 & 1u ? 1.f : -1.f};
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    a[h][e] = __fmaf_rn(w[e], v[h], a[h][e]);
+        };
+        auto rows_above = [&](int y, int x) { // bias and taps 0..9 at (y, x)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 b = *reinterpret_cast<const float2 *>(Bs + 8 * j + 2 * qt);
+                a[0][2 * j] = a[1][2 * j] = b.x;
+                a[0][2 * j + 1] = a[1][2 * j + 1] = b.y;
+            }
+            if (y >= 2 && x >= 2 && x + 2 < L) {
+#pragma unroll 1
+                for (int r = 0; r < 2; ++r) {
+                    const uint32_t m0 = spins_of(0, y + 1 + r, x), m1 = spins_of(1, y + 1 + r, x);
+#pragma unroll
+                    for (int d = 0; d < 5; ++d)
+                        tap(5 * r + d, m0 >> d, m1 >> d);
+                }
+                return;
+            }
+#pragma unroll 1
+            for (int t = 0; t < 10; ++t) {
+                const int r = t / 5, d = t - 5 * r;
+                if (y - 2 + r >= 0 && x - 2 + d >= 0 && x - 2 + d < L)
+                    tap(t, spins_of(0, y + 1 + r, x) >> d, spins_of(1, y + 1 + r, x) >> d);
+            }
+        };
+        auto uniforms = [&](int k) {
+            if ((k & 3) == 0 && mine)
+                rnd = philox4x32_10(make_uint4((uint32_t)k >> 2, round, kTagVanSample, my_id), key);
+        };
+        auto done = [&](int k, int y, int x) { // tap 10 at k = (y, x) (tap 11 is the last spin, left to the chain)
+            if (x >= 2)
+                tap(10, spins_of(0, y, x), spins_of(1, y, x));
+            float4 *dst = reinterpret_cast<float4 *>(smem + o.p0 + ((k & 1) * 2 + mt) * (kHalf * kCh * 4)) + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    dst[(2 * h + q) * 32] = make_float4(a[h][4 * q], a[h][4 * q + 1], a[h][4 * q + 2], a[h][4 * q + 3]);
+            const uint32_t rk = (k & 2) ? ((k & 1) ? rnd.w : rnd.z) : ((k & 1) ? rnd.y : rnd.x);
+            if (mine)
+                u[(k & 1) * 2 * kHalf] = uniform_open0(rk);
+            ready(kReadyFirst + mt, 64);
+        };
+        // after step k - 1: tap 10 at k + 1, which the chain waits for (R0), then the upper rows' taps at k + 2
+        uniforms(0);
+        rows_above(0, 0);
+        done(0, 0, 0);
+        rows_above(0, 1);
+        int y = 0, x = 1, py = 0, px = 0; // positions k + 1, k - 1
+#pragma unroll 1
+        for (int k = 0; k + 1 < P && ok; ++k) {
+            if (k > 0) {
+                ok = wait_warp(bar_e(mt), (uint32_t)(k - 1) & 1u, abort, err);
+                __syncwarp();
+                if (mine) {
+                    const float sp = draw->x;
+                    uint32_t *b = my_bits + (py % 3) * words + ((px + 2) >> 5);
+                    const uint32_t bit = 1u << ((px + 2) & 31);
+                    *b = sp > 0.f ? *b | bit : *b & ~bit;
+                    if (live)
+                        out_g[k - 1] = (int8_t)sp;
+                }
+                if (++px == L) {
+                    px = 0;
+                    ++py;
+                }
+                __syncwarp();
+            } else { // once the chain has taken the sum of step 0
+                ok = wait_warp(bar_h(1, mt), 0u, abort, err);
+            }
+            done(k + 1, y, x);
+            if (++x == L) {
+                x = 0;
+                ++y;
+            }
+            rows_above(y, x);
+            uniforms(k + 2);
+        }
+        for (int k = P - 2; k < P && ok; ++k) { // the last two draws
+            ok = wait_warp(bar_e(mt), (uint32_t)k & 1u, abort, err);
+            if (live)
+                out_g[k] = (int8_t)draw->x;
+            if (k == P - 2)
+                ready(kReadyFirst + mt, 64); // the chain may write its last draw
+        }
+        if (!ok)
+            release_chain(kReadyFirst + mt, 64, chain_done + mt);
+        return;
+    }
+
+    // ------------------------------------------------------------------------------------------- chain
+    // Lane 4 g + t of a fragment holds rows (samples) g and g + 8.  After the output layer's first exchange even
+    // lanes have row g, odd lanes row g + 8; lanes t = 0 and 1 publish the draw.
+    const int mt = warp & 1, g = lane >> 2, t = lane & 3, odd = t & 1;
+    const int sd = mt * kHalf + g + odd * 8;
+    float2 *draw = reinterpret_cast<float2 *>(smem + o.draw) + sd;
+    const float *u = reinterpret_cast<const float *>(smem + o.u) + sd;
+    const float4 *Po = reinterpret_cast<const float4 *>(smem + o.po) + mt * 32 + lane;
+    bf16 *Hn = reinterpret_cast<bf16 *>(smem + o.hn + mt * kColBytes);
+    const uint4 *w12 = reinterpret_cast<const uint4 *>(smem + o.w) + 12 * 128 + lane;
+    const float4 *Pf = reinterpret_cast<const float4 *>(smem + o.p + mt * (kHalf * kCh * 4)) + lane;
+    uint4 *slotH = reinterpret_cast<uint4 *>(smem + o.h + mt * kColBytes) + lane;
+    float v[2] = {0.f, 0.f}; // the last spin of rows g, g + 8
+    uint32_t pk[4][2] = {};  // a layer's values, packed: [n-tile][row]
+    auto load = [&](float(&c)[4][4], int l) { // accumulators of hidden layer l over taps 0..11
+        group_sync(kReadyHidden + (l - 1) * 2 + mt, 64);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 x = Pf[(l - 1) * 256 + q * 32];
+            c[q][0] = x.x, c[q][1] = x.y, c[q][2] = x.z, c[q][3] = x.w;
+        }
+    };
+    // Hidden layer l of the values pk; the next layer's accumulators are fetched meanwhile.
+    auto layer = [&](float(&c)[4][4], float(&cn)[4][4], int l) {
+        const uint4 a0 = make_uint4(pk[0][0], pk[0][1], pk[1][0], pk[1][1]), a1 = make_uint4(pk[2][0], pk[2][1], pk[3][0], pk[3][1]);
+        const uint4 *w = w12 + (l - 1) * kTapsB * 128;
+        mma_step(c, a0, w[0], w[32]);
+        mma_step(c, a1, w[64], w[96]);
+        float2 b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            b[j] = *reinterpret_cast<const float2 *>(Bs + l * kCh + 2 * t + 8 * j);
+        slotH[(l - 1) * 128] = a0;
+        slotH[(l - 1) * 128 + 32] = a1;
+        signal(bar_h(l, mt));
+        if (l < nh)
+            load(cn, l + 1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 s = add2(make_float2(c[j][2 * h], c[j][2 * h + 1]), b[j]);
+                pk[j][h] = relu_pack(s.x, s.y);
+            }
+    };
+    float ca[4][4], cb[4][4], f0[2][8], uk = 0.f;
+    // What the first layer at k needs besides the last spin: its sum, and the uniform of the draw
+    auto first = [&](int k) {
+        const float4 *src = reinterpret_cast<const float4 *>(smem + o.p0 + ((k & 1) * 2 + mt) * (kHalf * kCh * 4)) + lane;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float4 s4 = src[(2 * h + q) * 32];
+                f0[h][4 * q] = s4.x, f0[h][4 * q + 1] = s4.y, f0[h][4 * q + 2] = s4.z, f0[h][4 * q + 3] = s4.w;
+            }
+        uk = u[(k & 1) * 2 * kHalf];
+    };
+    int x = 0;
+    group_sync(kReadyFirst + mt, 64);
+    first(0);
+    load(ca, 1);
+#pragma unroll 1
+    for (int k = 0; k < P; ++k) {
+        // ---- first layer: sum + w s_{k-1}
+        if (x > 0) {
+            const float4 *w11 = reinterpret_cast<const float4 *>(W1 + 11 * kCh + 8 * t);
+            const float4 wa = w11[0], wb = w11[1];
+            const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    f0[h][e] = __fmaf_rn(w[e], v[h], f0[h][e]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                pk[j][h] = relu_pack(f0[h][2 * j], f0[h][2 * j + 1]);
+        // ---- hidden layers
+#pragma unroll 1
+        for (int l = 1; l <= nh; l += 2) {
+            layer(ca, cb, l);
+            if (l < nh)
+                layer(cb, ca, l + 1);
+        }
+        // The next step's sums, on the way while this one's output is computed.  With the first layer's sum at k + 1
+        // there, the warps that keep the draw of step k - 1 have read it.
+        group_sync(kReadyFirst + mt, 64);
+        if (k + 1 < P)
+            load(ca, 1);
+        // ---- output layer: sum + tap 12, parts t and 4 + t of both rows; then the parts in pairs
+        const float4 wd0 = *reinterpret_cast<const float4 *>(WD + 12 * kCh + 4 * t),
+                     wd1 = *reinterpret_cast<const float4 *>(WD + 12 * kCh + 16 + 4 * t);
+        const float bD = Bs[(D - 1) * kCh];
+        group_sync(kReadyOut + mt, 96);
+        const float4 p4 = *Po;
+        float part[2][2] = {{p4.x, p4.y}, {p4.z, p4.w}}; // [row][part t, part 4 + t]
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t lo = pk[2 * q][h], hi = pk[2 * q + 1][h];
+                const float4 wd = q == 0 ? wd0 : wd1;
+                *reinterpret_cast<uint2 *>(Hn + ring_elem(g + 8 * h, 16 * q + 4 * t)) = make_uint2(lo, hi);
+                part[h][q] = __fmaf_rn(wd.x, bf16_lo(lo), part[h][q]);
+                part[h][q] = __fmaf_rn(wd.y, bf16_hi(lo), part[h][q]);
+                part[h][q] = __fmaf_rn(wd.z, bf16_lo(hi), part[h][q]);
+                part[h][q] = __fmaf_rn(wd.w, bf16_hi(hi), part[h][q]);
+            }
+        float f2[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float other = __shfl_xor_sync(0xffffffffu, odd ? part[0][q] : part[1][q], 1);
+            f2[q] = (odd ? part[1][q] : part[0][q]) + other; // parts 2 s + 2 s + 1
+            f2[q] += __shfl_xor_sync(0xffffffffu, f2[q], 2);
+        }
+        float f = f2[0] + f2[1];
+        f += bD;
+        const int stop = *abort;
+        // ---- draw
+        const float sp = uk < sigmoid(f) ? 1.f : -1.f; // lanes t < 2
+        first(k + 1);
+        v[0] = __shfl_sync(0xffffffffu, sp, lane & ~3);
+        v[1] = __shfl_sync(0xffffffffu, sp, (lane & ~3) | 1);
+        if (t < 2)
+            *draw = make_float2(sp, sp * f);
+        signal(bar_e(mt));
+        if (++x == L)
+            x = 0;
+        if (__any_sync(0xffffffffu, stop))
+            break;
+    }
+    if (lane == 0)
+        *(volatile int *)(chain_done + mt) = 1;
+}
+
 // Copy the int8 lattices of every chain of an int8-layout Ising context into
 // one contiguous [n][L][L] buffer (or back, when `back`).
 __global__ void k_gather(const IsingChain *chains, char *lattice, int8_t *buf, int L, int n, int back)
@@ -1859,6 +2632,7 @@ struct mc_van {
     int *err = nullptr;      // device fault latch (a bounded completion wait gave up)
     RunGeom conv[3];         // geometries of the convolutions (kFwd, kLast, kBwd)
     int sms = 0;
+    bool pipe = false;       // the sampler with streamed columns (k_sample_pipe)
     bool weights_ready = false;
 };
 
@@ -1972,6 +2746,22 @@ template <int MODE>
 cudaError_t raise_conv_limit(const RunGeom &g)
 {
     return raise_smem_limit((const void *)conv_kernel<MODE>(g), g.smem_bytes);
+}
+
+// Which sampler: k_sample_pipe wherever its 8 helper warps and its shared memory do
+// (up to 4 hidden layers) and a block's columns are known a block ahead (L >= 8);
+// k_sample otherwise.  The register split of k_sample_pipe needs exactly the registers
+// it was written for.
+cudaError_t sampler_rule(mc_van *w)
+{
+    if (w->D - 2 > kPipeHidden || w->L < kPipeMinL)
+        return cudaSuccess;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, (const void *)k_sample_pipe);
+    if (e != cudaSuccess || a.numRegs != kPipeRegs)
+        return e;
+    w->pipe = true;
+    return raise_smem_limit((const void *)k_sample_pipe, pipe_smem(w->D, w->L).total);
 }
 
 cudaError_t prep(mc_van *w)
@@ -2177,6 +2967,8 @@ mc_status mc_van_create(mc_van **out, int32_t L, int32_t batch, int32_t depth, u
         e = raise_smem_limit((const void *)k_layer1_bwd_w, (size_t)(kEdgeThreads / 32) * edge_bytes_1(L));
     if (e == cudaSuccess)
         e = raise_smem_limit((const void *)k_sample, sample_smem(depth, L, sample_bufs(depth, L)));
+    if (e == cudaSuccess)
+        e = sampler_rule(w);
     if (e != cudaSuccess) {
         delete w;
         return vfail(MC_ECUDA, std::string("mc_van_create: ") + cudaGetErrorString(e));
@@ -2295,6 +3087,10 @@ mc_status mc_van_sample(mc_van *w, int32_t n, uint32_t round, const uint32_t *de
     if (e == cudaSuccess) {
         const unsigned blocks = (unsigned)((n + kSampleTile - 1) / kSampleTile);
         const int nbuf = sample_bufs(w->D, w->L);
+        if (w->pipe)
+            k_sample_pipe<<<blocks, kPipeThreads, pipe_smem(w->D, w->L).total, w->stream>>>(
+                w->wh, w->w1, w->wD, w->bias, w->D, w->L, n, w->hist, out, lq, w->key, round, dev_ids, w->err);
+        else
         k_sample<<<blocks, kSampleThreads, sample_smem(w->D, w->L, nbuf), w->stream>>>(w->wh, w->w1, w->wD, w->bias, w->D, w->L, n,
                                                                       nbuf, w->hist, w->zero, out, lq, w->key, round, dev_ids, w->err);
         e = cudaGetLastError();

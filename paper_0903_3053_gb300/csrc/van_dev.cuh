@@ -61,10 +61,11 @@ __device__ __forceinline__ float bf(const __nv_bfloat16 v) { return __bfloat162f
 __device__ __forceinline__ float log_sigmoid(float t)
 {
     // log(1 / (1 + e^{-t})) = -softplus(-t), written to stay finite for large |t|
-    return t >= 0.f ? -log1pf(expf(-t)) : t - log1pf(expf(t));
+    const float l = log1pf(expf(-fabsf(t)));
+    return t >= 0.f ? -l : t - l;
 }
 
-__device__ __forceinline__ float sigmoid(float t) { return 1.0f / (1.0f + expf(-t)); }
+__device__ __forceinline__ float sigmoid(float t) { return __frcp_rn(1.0f + expf(-t)); }
 
 }  // namespace van
 }  // namespace mc

@@ -419,6 +419,29 @@ def test_sampler_draws_equal_oracle_on_the_kernel_stream(L, n, depth):
     assert 0.1 < (g > 0).mean() < 0.9  # a non-trivial network
 
 
+@pytest.mark.parametrize("L,n,depth", [(8, 33, 3), (10, 17, 4), (14, 48, 5), (22, 5, 6), (34, 31, 6), (64, 16, 5), (128, 3, 4)])
+def test_sampler_edges_of_rows_blocks_and_halves(L, n, depth):
+    """The sampler works in blocks of four positions (a last block of two, rows
+    of one block more than the window), halves of 16 samples (partly filled,
+    empty) and a column window that runs from row to row.  Its log q is the sum
+    over the conditionals it drew from, so one drawn from a wrong tap anywhere
+    (a change of order 0.1 in a sum of at most ~10^4) parts it from the forward
+    network's log q of the same configuration; the same draws come from any
+    place in the batch; no bounded wait gave up."""
+    p = bf16_params(depth=depth, seed=60 + L, scale=1.3, bias=0.4)
+    net = mc.VAN(L, batch=n, depth=depth, seed=55)
+    net.set_params(mc.mc.van_pack(p))
+    s, lq = net.sample(n, round=9)
+    net.sync()
+    lp = net.log_prob(s).cpu().numpy()
+    ids = torch.arange(n - 1, -1, -1, dtype=torch.int32, device="cuda")
+    back, lqb = net.sample(n, round=9, ids=ids)
+    net.sync()
+    net.close()
+    assert np.max(np.abs(lq.cpu().numpy() - lp) / np.abs(lp)) < 1e-5
+    assert torch.equal(back.flip(0), s) and torch.equal(lqb.flip(0), lq)
+
+
 def test_full_size_L64_sampler_draws_per_position():
     """At L = 64 with 4096 proposals, every position of a sample of the GPU's
     draws is the oracle's decision u_k < p(s_k = +1 | s_<k) on the GPU's own
