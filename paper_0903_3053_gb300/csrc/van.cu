@@ -93,14 +93,20 @@ constexpr int kTcMaxPolls = 1 << 22; // bounded completion wait
 
 // Layer 1 (1 -> 32 channels, mask A, ReLU) on the fifth-generation tensor
 // cores: one MMA per tile of 128 consecutive positions (M = 128, N = 32,
-// K = 16: the 12 taps and 4 zeros).  Each thread builds its position's A row
-// from the (negated) spins -- +-1 or 0 outside the lattice, exact in BF16 --
-// into two K-major chunk planes; B holds the layer's weights (BF16 values, as
-// k_prep_weights leaves them) as [chunk][out channel] rows.  After the MMA each
-// thread reads its position's 32 accumulator columns from its tensor-memory
-// lane, adds the bias, applies ReLU and stores the 64-byte BF16 row.  Several
-// CTAs per SM overlap one another's MMA waits; every wait is bounded and a
-// timeout latches *err.
+// K = 16: the 12 taps and 4 zeros).  The A rows hold the (negated) spins --
+// 0 outside the lattice, exact in BF16 -- in two K-major chunk planes; B holds the
+// layer's weights (BF16 values, as k_prep_weights leaves them) as
+// [chunk][out channel] rows.  A warp converts the spins of its 32 positions' three
+// rows once into shared memory (the positions are consecutive, so each row is a
+// run of 36 bytes, fetched a tile ahead), and a lane takes its five neighbours of a
+// row as three words, shifted by half a word at odd positions and masked at the
+// lattice's edges.  After the MMA each thread reads its position's 32 accumulator
+// columns, adds the bias, applies ReLU; the BF16 rows go through shared memory, so
+// that a warp stores whole lines.  Several CTAs per SM overlap one another's MMA
+// waits; every wait is bounded and a timeout latches *err.  L = 64, 4096
+// configurations: 250 us against 436 when every tap was a byte load, a comparison and
+// two conversions and every lane stored its own 64-byte row; the 1.07 GB it writes
+// take 155.
 constexpr int kL1Threads = 128;
 constexpr uint32_t kL1Cols = 32;
 
@@ -110,10 +116,12 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
 {
     __shared__ __align__(128) uint4 A[2][kL1Threads]; // chunk planes: taps 0-7, taps 8-15
     __shared__ __align__(128) uint4 B[2][kCh];        // chunk planes: [out channel] taps 0-7, 8-15
+    __shared__ __align__(16) uint4 Rows[kL1Threads / 32][128]; // a warp's 32 output rows
+    __shared__ __align__(16) bf16 Win[kL1Threads / 32][3 * 40]; // a warp's spins, three rows of 36
     __shared__ float Bias[kCh];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     chain_wait(true);
     if (tid < kCh)
         Bias[tid] = b1[tid];
@@ -139,34 +147,63 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
     const uint64_t adesc = tc::smem_desc(smem_u32(&A[0][0]), kL1Threads * 16, 128);
     const uint64_t bdesc = tc::smem_desc(smem_u32(&B[0][0]), kCh * 16, 128);
     constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kCh);
-    const long long total = (long long)n * L * L, tiles = (total + kL1Threads - 1) / kL1Threads;
+    const uint32_t total = (uint32_t)n * L * L, tiles = (total + kL1Threads - 1) / kL1Threads;
+    const uint32_t step = gridDim.x * kL1Threads, step_y = step / L % L, step_x = step % L;
+    bf16 *const win = Win[warp];
+    uint4 *const rows = Rows[warp];
+    uint32_t p = blockIdx.x * kL1Threads + tid; // this thread's position, its row and column
+    int y = (int)(p / L % L), x = (int)(p % L);
+    // the spins around the warp's positions, rows y - 2, y - 1, y: 36 each, from two left of the first
+    int raw[3][2];
+    auto fetch = [&](uint32_t first) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t i = first + lane + 32 * h - 2 - (2 - r) * L; // wraps below 0: out of range
+                raw[r][h] = (h == 0 || lane < 4) && i < total ? spins[i] : 0;
+            }
+    };
+    fetch(p - lane);
     int ok = 1;
     uint32_t uses = 0;
-    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++uses) {
-        const long long p = tile * kL1Threads + tid;
+    for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++uses) {
         const bool live = p < total;
-        int b = 0, y = 0, x = 0;
-        if (live) {
-            b = (int)(p / ((long long)L * L));
-            const int r = (int)(p - (long long)b * L * L);
-            y = r / L;
-            x = r - y * L;
-        }
-        bf16 a[16];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            float v = 0.f;
-            if (t < kTapsA && live) {
-                const int yy = y + tap_dy(t), xx = x + tap_dx(t);
-                if (yy >= 0 && xx >= 0 && xx < L) {
-                    const int s = spins[((size_t)b * L + yy) * L + xx];
-                    v = (float)(negate ? -s : s);
-                }
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (h == 0 || lane < 4)
+                    win[r * 40 + lane + 32 * h] = __float2bfloat16((float)(negate ? -raw[r][h] : raw[r][h]));
+        __syncwarp();
+        p += step;
+        fetch(p - lane);
+        // neighbours e = 0..4 (dx = e - 2) of a row as pairs, zero outside the lattice
+        const uint32_t m01 = (x >= 2 ? 0xFFFFu : 0u) | (x >= 1 ? 0xFFFF0000u : 0u),
+                       m3 = x + 1 < L ? 0xFFFF0000u : 0u, m4 = x + 2 < L ? 0xFFFFu : 0u;
+        uint32_t e01[3], e23[2], e4[2];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(win + r * 40) + (lane >> 1);
+            const uint32_t w0 = w[0], w1 = w[1], in = y - 2 + r >= 0 ? 0xFFFFFFFFu : 0u;
+            e01[r] = (lane & 1 ? __byte_perm(w0, w1, 0x5432) : w0) & m01 & in;
+            if (r < 2) {
+                const uint32_t w2 = w[2];
+                e23[r] = (lane & 1 ? __byte_perm(w1, w2, 0x5432) : w1) & (0xFFFFu | m3) & in;
+                e4[r] = (lane & 1 ? w2 >> 16 : w2) & m4 & in;
             }
-            a[t] = __float2bfloat16(v);
         }
-        A[0][tid] = *reinterpret_cast<uint4 *>(&a[0]);
-        A[1][tid] = *reinterpret_cast<uint4 *>(&a[8]);
+        // taps 0..4 of row y - 2, 5..9 of row y - 1, 10 and 11 of row y
+        A[0][tid] = make_uint4(e01[0], e23[0], e4[0] | e01[1] << 16, __byte_perm(e01[1], e23[1], 0x5432));
+        A[1][tid] = make_uint4(e23[1] >> 16 | e4[1] << 16, e01[2], 0u, 0u);
+        x += step_x;
+        y += step_y;
+        if (x >= L) {
+            x -= L;
+            ++y;
+        }
+        if (y >= L)
+            y -= L;
         tc::fence_smem_for_async();
         tc::fence_before_sync();
         __syncthreads();
@@ -182,19 +219,25 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
         tc::fence_after_sync();
         float v[kCh];
         tc::ld_32x32b_x32(tbase + ((uint32_t)(32 * warp) << 16), v);
-        if (live) {
-            uint4 pk[4];
-            uint32_t *pw = reinterpret_cast<uint32_t *>(pk);
 #pragma unroll
-            for (int c = 0; c < kCh; c += 2) {
-                const __nv_bfloat162 h =
-                    __floats2bfloat162_rn(fmaxf(v[c] + Bias[c], 0.f), fmaxf(v[c + 1] + Bias[c + 1], 0.f));
-                pw[c / 2] = *reinterpret_cast<const uint32_t *>(&h);
+        for (int k = 0; k < 4; ++k) {
+            uint32_t u[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(v[8 * k + 2 * c] + Bias[8 * k + 2 * c], 0.f),
+                                                               fmaxf(v[8 * k + 2 * c + 1] + Bias[8 * k + 2 * c + 1], 0.f));
+                u[c] = *reinterpret_cast<const uint32_t *>(&h);
             }
-            uint4 *dst = reinterpret_cast<uint4 *>(h1 + (size_t)p * kCh);
+            rows[lane * 4 + (k ^ (lane >> 1 & 3))] = make_uint4(u[0], u[1], u[2], u[3]);
+        }
+        __syncwarp();
+        const uint32_t live_lanes = __popc(__ballot_sync(0xffffffffu, live));
+        uint4 *dst = reinterpret_cast<uint4 *>(h1 + (size_t)(p - step - lane) * kCh);
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                dst[k] = pk[k];
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t row = 8 * k + (lane >> 2);
+            if (row < live_lanes)
+                dst[32 * k + lane] = rows[row * 4 + ((lane & 3) ^ (row >> 1 & 3))];
         }
         tc::fence_before_sync(); // this tile's tensor-memory reads precede the next MMA
     }
