@@ -91,6 +91,70 @@ __global__ void k_prep_weights(const float *p, DevParams P, bf16 *wh, float *w1,
 // ------------------------------------------------------------------ forward
 constexpr int kTcMaxPolls = 1 << 22; // bounded completion wait
 
+// BF16 pair <-> two floats as plain bit operations (BF16 -> FP32 is exact);
+// the pack rounds to nearest even, lo in the low half.
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
+{
+    uint32_t u;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(u) : "f"(hi), "f"(lo));
+    return u;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&d);
+}
+// max(., 0) of the pair: the same bits as packing max(lo, 0), max(hi, 0)
+__device__ __forceinline__ uint32_t relu_pack(float lo, float hi)
+{
+    uint32_t u = pack_bf16x2(lo, hi);
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(u) : "r"(0u));
+    return u;
+}
+__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
+
+// A lane's row of 128 bytes (two positions) to and from global memory, 32 bytes an instruction: whole sectors, so
+// that rows stored by their own lanes need no detour through shared memory, whose bandwidth the
+// convolutions' operands want.  L = 64, batch 512, a forward layer: 58 us; by 16-byte stores 81, by whole lines through
+// shared memory 67.
+__device__ __forceinline__ void store32(void *dst, const uint4 &a, const uint4 &b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void store_row(bf16 *dst, const uint4 (&row)[8])
+{
+#pragma unroll
+    for (int c = 0; c < 8; c += 2)
+        store32(dst + 8 * c, row[c], row[c + 1]);
+}
+__device__ __forceinline__ void load_row(const bf16 *src, bool live, uint4 (&row)[8])
+{
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) {
+        row[c] = row[c + 1] = make_uint4(0u, 0u, 0u, 0u);
+        if (live)
+            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(row[c].x), "=r"(row[c].y), "=r"(row[c].z), "=r"(row[c].w), "=r"(row[c + 1].x),
+                           "=r"(row[c + 1].y), "=r"(row[c + 1].z), "=r"(row[c + 1].w)
+                         : "l"(src + 8 * c));
+    }
+}
+// Zero the halves of hi and lo where the activation m is not positive.
+__device__ __forceinline__ void mask8(const uint4 &m, uint4 &hi, uint4 &lo)
+{
+    const uint32_t w[4] = {m.x, m.y, m.z, m.w};
+    uint32_t on[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        on[k] = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w[k]), __floats2bfloat162_rn(0.f, 0.f));
+    hi.x &= on[0], hi.y &= on[1], hi.z &= on[2], hi.w &= on[3];
+    lo.x &= on[0], lo.y &= on[1], lo.z &= on[2], lo.w &= on[3];
+}
+
 // Layer 1 (1 -> 32 channels, mask A, ReLU) on the fifth-generation tensor
 // cores: one MMA per tile of 128 consecutive positions (M = 128, N = 32,
 // K = 16: the 12 taps and 4 zeros).  The A rows hold the (negated) spins --
@@ -116,9 +180,8 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
 {
     __shared__ __align__(128) uint4 A[2][kL1Threads]; // chunk planes: taps 0-7, taps 8-15
     __shared__ __align__(128) uint4 B[2][kCh];        // chunk planes: [out channel] taps 0-7, 8-15
-    __shared__ __align__(16) uint4 Rows[kL1Threads / 32][128]; // a warp's 32 output rows
     __shared__ __align__(16) bf16 Win[kL1Threads / 32][3 * 40]; // a warp's spins, three rows of 36
-    __shared__ float Bias[kCh];
+    __shared__ __align__(16) float Bias[kCh];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -150,7 +213,6 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
     const uint32_t total = (uint32_t)n * L * L, tiles = (total + kL1Threads - 1) / kL1Threads;
     const uint32_t step = gridDim.x * kL1Threads, step_y = step / L % L, step_x = step % L;
     bf16 *const win = Win[warp];
-    uint4 *const rows = Rows[warp];
     uint32_t p = blockIdx.x * kL1Threads + tid; // this thread's position, its row and column
     int y = (int)(p / L % L), x = (int)(p % L);
     // the spins around the warp's positions, rows y - 2, y - 1, y: 36 each, from two left of the first
@@ -219,25 +281,16 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
         tc::fence_after_sync();
         float v[kCh];
         tc::ld_32x32b_x32(tbase + ((uint32_t)(32 * warp) << 16), v);
+        uint32_t u[kCh / 2];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t u[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(v[8 * k + 2 * c] + Bias[8 * k + 2 * c], 0.f),
-                                                               fmaxf(v[8 * k + 2 * c + 1] + Bias[8 * k + 2 * c + 1], 0.f));
-                u[c] = *reinterpret_cast<const uint32_t *>(&h);
-            }
-            rows[lane * 4 + (k ^ (lane >> 1 & 3))] = make_uint4(u[0], u[1], u[2], u[3]);
+        for (int c = 0; c < kCh; c += 2) {
+            const float2 s = add2(make_float2(v[c], v[c + 1]), *reinterpret_cast<const float2 *>(&Bias[c]));
+            u[c / 2] = relu_pack(s.x, s.y);
         }
-        __syncwarp();
-        const uint32_t live_lanes = __popc(__ballot_sync(0xffffffffu, live));
-        uint4 *dst = reinterpret_cast<uint4 *>(h1 + (size_t)(p - step - lane) * kCh);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t row = 8 * k + (lane >> 2);
-            if (row < live_lanes)
-                dst[32 * k + lane] = rows[row * 4 + ((lane & 3) ^ (row >> 1 & 3))];
+        if (live) {
+            bf16 *dst = h1 + (size_t)(p - step) * kCh;
+            store32(dst, make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7]));
+            store32(dst + 16, make_uint4(u[8], u[9], u[10], u[11]), make_uint4(u[12], u[13], u[14], u[15]));
         }
         tc::fence_before_sync(); // this tile's tensor-memory reads precede the next MMA
     }
@@ -254,14 +307,14 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
 // arrays in the space of one FP32 array, which the tensor cores read directly.
 __device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo)
 {
-    bf16 h[8], l[8];
+    uint32_t h[4], l[4];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        h[k] = __float2bfloat16(v[k]);
-        l[k] = __float2bfloat16(v[k] - bf(h[k]));
+    for (int k = 0; k < 4; ++k) {
+        h[k] = pack_bf16x2(v[2 * k], v[2 * k + 1]);
+        l[k] = pack_bf16x2(v[2 * k] - bf16_lo(h[k]), v[2 * k + 1] - bf16_hi(h[k]));
     }
-    hi = *reinterpret_cast<uint4 *>(h);
-    lo = *reinterpret_cast<uint4 *>(l);
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 // ---------------------------------------------------------------- masked 32-channel convolutions
@@ -312,7 +365,6 @@ constexpr int kRunGuard = 8;                   // rows ahead of staged row 0 (8 
 constexpr uint32_t kRunMaxSmem1 = 200u * 1024; // two stages + weights + barriers + scratch, one CTA per SM
 constexpr uint32_t kRunMaxSmem2 = 113u * 1024; // the same, two CTAs per SM
 constexpr uint32_t kRunBarBytes = 128;         // 9 mbarriers, tensor-memory slot
-constexpr uint32_t kRunScratch = 1024;         // per epilogue warp: 8 pairs of output on their way to whole lines
 constexpr int kMaxItemRows = 32, kMaxItemSamples = 16, kMaxPackedTiles = 4;
 
 __host__ __device__ constexpr int conv_cols(int mode) { return mode == kLast ? 16 : kCh; } // per position
@@ -341,8 +393,7 @@ RunGeom run_geom_of(int L, int G, int R, int S, int mode, int ctas)
     // follows (the other planes, the weights), whose products are dropped
     g.plane_bytes = (uint32_t)((kRunGuard + S * (R + 2) * g.P + 1 + 7) / 8 * 8) * 128u;
     g.stage_bytes = (mode == kBwd ? 2u : 1u) * (uint32_t)(g.G / 2) * g.plane_bytes;
-    const uint32_t used = 2 * g.stage_bytes + conv_weight_bytes(mode) + kRunBarBytes +
-                          (mode == kLast ? 0u : (uint32_t)epilogue_warps(mode, ctas) * kRunScratch);
+    const uint32_t used = 2 * g.stage_bytes + conv_weight_bytes(mode) + kRunBarBytes;
     const uint32_t read = 2 * g.stage_bytes - g.plane_bytes + (uint32_t)(kRunGuard + qpad + 2 * g.P + 2) * 128u;
     g.smem_bytes = std::max(used, read) + 1024; // + alignment slack
     g.inv_p = (uint32_t)(((1ull << 32) + g.P - 1) / g.P);
@@ -413,43 +464,6 @@ struct ConvArgs {
     int *err;
 };
 
-// Store a warp's 32 rows of 128 bytes (one pair of positions per lane, `row`) to
-// out[pair], pair = ~0 for rows that are dropped.  Eight rows at a time go through
-// shared memory (16-byte chunk c of row r at chunk c ^ r: no bank conflicts), so that
-// eight lanes store one whole 128-byte line; stored by their own lanes, the rows
-// would be 32 lines per instruction (forward, L = 64, batch 512: 81 -> 72 us).  MASK: halves
-// whose activation mk (lane's chunks, in storing order) is not positive become zero.
-template <bool MASK>
-__device__ __forceinline__ void store_pairs(uint4 *scratch, int lane, const uint4 (&row)[8], uint32_t pair,
-                                            const uint4 (&mk)[8], uint4 *out)
-{
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if ((lane >> 3) == k)
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                scratch[(lane & 7) * 8 + (c ^ (lane & 7))] = row[c];
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int r = 4 * i + (lane >> 3), c = lane & 7;
-            uint4 o = scratch[r * 8 + (c ^ r)];
-            const uint32_t pr = __shfl_sync(0xffffffffu, pair, 8 * k + r);
-            if (MASK) {
-                const uint4 m = mk[2 * k + i];
-                const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
-                o.x &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.x), zero);
-                o.y &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.y), zero);
-                o.z &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.z), zero);
-                o.w &= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&m.w), zero);
-            }
-            if (pr != ~0u)
-                out[(size_t)pr * 8 + c] = o;
-        }
-        __syncwarp();
-    }
-}
-
 template <int MODE, int G, int MINB>
 __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
     k_conv_runs(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
@@ -470,7 +484,7 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t boff = 2 * g.stage_bytes, bars = boff + conv_weight_bytes(MODE);
     const uint32_t full0 = sb + bars, empty0 = full0 + 16, tfull0 = full0 + 32, tempty0 = full0 + 48,
-                   drain = full0 + 64, tslot_off = bars + 80, scratch_off = bars + kRunBarBytes;
+                   drain = full0 + 64, tslot_off = bars + 80;
     // the run right of the box's last row is zero (BWD reads it); whatever else lies outside the boxes is met only by
     // rows of A that are dropped
     for (uint32_t i = tid; i < 8u * 2u * g.stage_bytes / g.plane_bytes; i += blockDim.x)
@@ -536,6 +550,14 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                                         full0 + 8 * s);
                 }
                 armed[s] = k;
+                if (MODE == kBwd) { // the epilogue's mask, into L2: one run of rows (or of whole lattices)
+                    const int rows = g.S > 1 ? (a.n - bi * g.S < g.S ? a.n - bi * g.S : g.S) * g.L
+                                             : (g.L - y0 < g.R ? g.L - y0 : g.R);
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                                     a.mask + ((size_t)bi * g.S * g.L + y0) * g.L * kCh),
+                                 "r"((uint32_t)(rows * g.L * kCh * 2))
+                                 : "memory");
+                }
             }
             for (int s = 0; s < 2; ++s) // the last loads of each stage have landed before the CTA ends
                 if (armed[s] >= 0 && !tc::mbar_wait(full0 + 8 * s, (armed[s] >> 1) & 1, kTcMaxPolls))
@@ -626,7 +648,6 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
         for (int c = 0; c < kCh; ++c)
             bv[c] = MODE == kFwd ? __ldg(&a.bias[c]) : 0.f;
         const float b0 = MODE == kLast ? __ldg(a.la.bD) : 0.f;
-        uint4 *scratch = reinterpret_cast<uint4 *>(smem + scratch_off + (uint32_t)warp * kRunScratch);
         uint32_t tcount = 0;
         for (int it = blockIdx.x; ok && it < total; it += gridDim.x) {
             const int bi = it / g.YB, y0 = (it - bi * g.YB) * g.R;
@@ -645,18 +666,11 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                     const uint32_t smp = g.S == 1 ? 0u : __umulhi(row, g.inv_rows), r = row - smp * (uint32_t)(g.R + 2);
                     const int b = bi * g.S + (int)smp, y = y0 + (int)r;
                     const bool live = pp >= 1 && (int)r < g.R && y < g.L && (int)smp < g.S && b < a.n && m < g.tiles;
-                    // first position of the slot's pair, and the pair's index for the lanes that store it
+                    // first position of the slot's pair: this lane's row of 2 x 32 channels
                     const size_t p = ((size_t)b * g.L + y) * g.L + G * (pp - 1) + (G == 4 ? 2 * slot : 0);
-                    const uint32_t pair = live ? (uint32_t)(p >> 1) : ~0u;
                     uint4 mk[8];
-                    if (MODE == kBwd) { // mask chunks as this lane stores them, in flight during the wait
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const uint32_t pr = __shfl_sync(0xffffffffu, pair, 4 * i + (lane >> 3));
-                            mk[i] = pr == ~0u ? make_uint4(0u, 0u, 0u, 0u)
-                                              : __ldg(reinterpret_cast<const uint4 *>(a.mask) + (size_t)pr * 8 + (lane & 7));
-                        }
-                    }
+                    if (MODE == kBwd) // the mask, in flight during the wait
+                        load_row(a.mask + p * kCh, live, mk);
                     if (!waited) {
                         waited = true;
                         ok = __any_sync(0xffffffffu, tc::mbar_wait(tfull0 + 8 * bb, (tcount >> 1) & 1u, kTcMaxPolls));
@@ -696,18 +710,22 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                         uint32_t *pw = reinterpret_cast<uint32_t *>(pk);
 #pragma unroll
                         for (int c = 0; c < 2 * kCh; c += 2) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(v[c] + bv[c % kCh], 0.f),
-                                                                           fmaxf(v[c + 1] + bv[c % kCh + 1], 0.f));
-                            pw[c / 2] = *reinterpret_cast<const uint32_t *>(&h);
+                            const float2 s = add2(make_float2(v[c], v[c + 1]), make_float2(bv[c % kCh], bv[c % kCh + 1]));
+                            pw[c / 2] = relu_pack(s.x, s.y);
                         }
-                        store_pairs<false>(scratch, lane, pk, pair, mk, reinterpret_cast<uint4 *>(a.out));
+                        if (live)
+                            store_row(a.out + p * kCh, pk);
                     } else {
                         uint4 hi[8], lo[8];
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
+                        for (int k = 0; k < 8; ++k) {
                             split8(v + 8 * k, hi[k], lo[k]);
-                        store_pairs<true>(scratch, lane, hi, pair, mk, reinterpret_cast<uint4 *>(a.out));
-                        store_pairs<true>(scratch, lane, lo, pair, mk, reinterpret_cast<uint4 *>(a.out_lo));
+                            mask8(mk[k], hi[k], lo[k]);
+                        }
+                        if (live) {
+                            store_row(a.out + p * kCh, hi);
+                            store_row(a.out_lo + p * kCh, lo);
+                        }
                     }
                 }
                 if (!ok)
@@ -1411,30 +1429,6 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-
-// BF16 pair <-> two floats as plain bit operations (BF16 -> FP32 is exact);
-// the pack rounds to nearest even, lo in the low half.
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
-{
-    uint32_t u;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(u) : "f"(hi), "f"(lo));
-    return u;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
-    return *reinterpret_cast<float2 *>(&d);
-}
-// max(., 0) of the pair: the same bits as packing max(lo, 0), max(hi, 0)
-__device__ __forceinline__ uint32_t relu_pack(float lo, float hi)
-{
-    uint32_t u = pack_bf16x2(lo, hi);
-    asm("max.bf16x2 %0, %0, %1;" : "+r"(u) : "r"(0u));
-    return u;
-}
-__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
 // Named barriers of the sampler's warp groups (0 is __syncthreads).
 constexpr int kBarMain = 1, kBarSide = 2;
