@@ -659,8 +659,8 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                 bool waited = false;
 #pragma unroll 1
                 for (int slot = slot0; slot < slot1; ++slot) {
-                    const int m = G == 2 ? m0 + slot : m0;
                     const uint32_t col = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (2 * bb + (uint32_t)slot) * kSlot;
+                    const int m = G == 2 ? m0 + slot : m0;
                     const uint32_t q = (uint32_t)(m * 128 + 32 * (warp & 3) + lane), row = __umulhi(q, g.inv_p),
                                    pp = q - row * (uint32_t)g.P;
                     const uint32_t smp = g.S == 1 ? 0u : __umulhi(row, g.inv_rows), r = row - smp * (uint32_t)(g.R + 2);
@@ -678,20 +678,17 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                         if (!ok)
                             break;
                     }
-                    float v[2 * kCh], acc[2];
+                    auto taken = [&] { // the accumulator is in registers: the next MMAs may have it
+                        if (slot + 1 == slot1) {
+                            tc::fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0)
+                                tc::mbar_arrive(tempty0 + 8 * bb);
+                        }
+                    };
                     if (MODE == kLast) {
-                        acc[0] = tc::ld_32x32b_x1(col);
-                        acc[1] = tc::ld_32x32b_x1(col + NB);
-                    } else {
-                        tc::ld_32x32b_x64(col, v);
-                    }
-                    if (slot + 1 == slot1) { // the accumulator is in registers: the next MMAs may have it
-                        tc::fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0)
-                            tc::mbar_arrive(tempty0 + 8 * bb);
-                    }
-                    if (MODE == kLast) {
+                        const float acc[2] = {tc::ld_32x32b_x1(col), tc::ld_32x32b_x1(col + NB)};
+                        taken();
                         if (live) {
                             const char2 s2 = *reinterpret_cast<const char2 *>(a.la.spins + p);
                             const float sv[2] = {a.la.negate ? -(float)s2.x : (float)s2.x,
@@ -706,6 +703,9 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                                                 -a.la.inv_n * sv[1] * sigmoid(-sv[1] * f1));
                         }
                     } else if (MODE == kFwd) {
+                        float v[2 * kCh];
+                        tc::ld_32x32b_x64(col, v);
+                        taken();
                         uint4 pk[8];
                         uint32_t *pw = reinterpret_cast<uint32_t *>(pk);
 #pragma unroll
@@ -715,16 +715,26 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                         }
                         if (live)
                             store_row(a.out + p * kCh, pk);
-                    } else {
-                        uint4 hi[8], lo[8];
+                    } else { // one position after the other, for the registers
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            split8(v + 8 * k, hi[k], lo[k]);
-                            mask8(mk[k], hi[k], lo[k]);
-                        }
-                        if (live) {
-                            store_row(a.out + p * kCh, hi);
-                            store_row(a.out_lo + p * kCh, lo);
+                        for (int h = 0; h < 2; ++h) {
+                            float v[kCh];
+                            tc::ld_32x32b_x32(col + h * NB, v);
+                            if (h == 1)
+                                taken();
+                            uint4 hi[4], lo[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                split8(v + 8 * k, hi[k], lo[k]);
+                                mask8(mk[4 * h + k], hi[k], lo[k]);
+                            }
+                            if (live) {
+                                bf16 *d = a.out + (p + h) * kCh, *e = a.out_lo + (p + h) * kCh;
+                                store32(d, hi[0], hi[1]);
+                                store32(d + 16, hi[2], hi[3]);
+                                store32(e, lo[0], lo[1]);
+                                store32(e + 16, lo[2], lo[3]);
+                            }
                         }
                     }
                 }
@@ -1167,7 +1177,9 @@ __global__ void __launch_bounds__(192, 2) k_dw32_tc(const __grid_constant__ CUte
             tc::commit(done); // every MMA issued above has completed before the drain
         }
     } else { // warps 0-3: bias gradient per item, then the drain
-        float bsum = 0.f;
+        // a lane sums 8 channels of every 32nd position (16-byte reads: two bytes a lane, one position a warp
+        // at a time, cost as much shared-memory bandwidth as the MMAs' operands)
+        float bsum[8] = {};
         int k = 0;
         for (int it = blockIdx.x; ok && it < total; it += gridDim.x, ++k) {
             const int s = k % NS, use = k / NS;
@@ -1177,16 +1189,28 @@ __global__ void __launch_bounds__(192, 2) k_dw32_tc(const __grid_constant__ CUte
                 break;
             }
             const unsigned char *zh = smem + (size_t)s * g.stage_bytes, *zl = zh + g.zbytes;
-            for (int x = warp; x < g.L; x += 4) { // channel `lane` of position x, 64-byte swizzle
-                const uint32_t off = (uint32_t)x * 64u + ((((uint32_t)lane >> 3) ^ (((uint32_t)x >> 1) & 3u)) << 4) +
-                                     ((uint32_t)lane & 7u) * 2u;
-                bsum += bf(*reinterpret_cast<const bf16 *>(zh + off)) + bf(*reinterpret_cast<const bf16 *>(zl + off));
+            for (int x = 8 * warp + (lane >> 2); x < g.L; x += 32) { // 64-byte swizzle
+                const uint32_t off = (uint32_t)x * 64u + ((((uint32_t)lane & 3u) ^ (((uint32_t)x >> 1) & 3u)) << 4);
+                const uint4 h = *reinterpret_cast<const uint4 *>(zh + off), l = *reinterpret_cast<const uint4 *>(zl + off);
+                const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    bsum[2 * e] += bf16_lo(hw[e]) + bf16_lo(lw[e]);
+                    bsum[2 * e + 1] += bf16_hi(hw[e]) + bf16_hi(lw[e]);
+                }
             }
             __syncwarp();
             if (lane == 0)
                 tc::mbar_arrive(empty0 + 8 * s);
         }
-        bsum_s[warp * 32 + lane] = bsum;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], 4);
+            bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], 8);
+            bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], 16);
+            if (lane < 4)
+                bsum_s[warp * 32 + 8 * lane + e] = bsum[e];
+        }
         const bool got = __any_sync(0xffffffffu, tc::mbar_wait(done, 0u, kTcMaxPolls));
         tc::fence_after_sync();
         if (!got)
@@ -1937,6 +1961,7 @@ __device__ __forceinline__ void release_chain(int id, int threads, volatile int 
         ready(id, threads);
 }
 
+// Registers of a warp group, out of what the block was launched with.
 template <int REGS>
 __device__ __forceinline__ void regs_grow()
 {
