@@ -529,8 +529,9 @@ def run_su2(mc, torch, rank, K, world, issue_peak):
 
 
 def run_batched(mc, torch, rank, K, world, sweeps_per_call=10):
-    """256 Ising + 64 SU(2) chains of uneven sizes in one persistent launch per
-    call (autotuned launch shape); value = site/link updates per second."""
+    """256 Ising + 64 SU(2) chains of uneven sizes advanced together (autotuned:
+    the members' own launches side by side, or one persistent launch of some
+    shape); value = site/link updates per second."""
     from paper_0903_3053_gb300 import autotune, workloads
     spec = workloads.batched_chains(seed=0)
     def chain(d):
@@ -570,7 +571,7 @@ def run_batched(mc, torch, rank, K, world, sweeps_per_call=10):
             "unit": "site+link updates/s",
             "workload": "256 Ising chains L in {32..1024}, beta ~ U[0.35, 0.55] + 64 SU(2) chains L^4, "
                         "L in {4, 6, 8, 12, 16}, beta ~ U[1.8, 2.6] (numpy default_rng(0)); E/M and plaquette "
-                        "every sweep", "launches_per_call": 1 + len(bs), "sweeps_per_call": sweeps_per_call,
+                        "every sweep", "persistent": choice["split"] >= 0, "sweeps_per_call": sweeps_per_call,
             "ms_per_sweep": ms / sweeps, "clusters": nc, "rounds": nr,
             "autotuned": {k: choice[k] for k in ("cluster", "threads", "split", "cached")}}
 
@@ -587,8 +588,8 @@ def run_paper_protocol(mc, torch, ising_sweeps=20000) -> dict:
     (the paper's 10^6 sweeps projected from `ising_sweeps`); SU(2) L_t x L_s^3
     lattices of Table 1, one chain each at beta = 2.3, the paper's protocol of
     1000 thermalisation sweeps then 1000 measurements 5 sweeps apart, run in
-    full, through the per-phase launches (grid) and the persistent launch
-    (group); the faster is reported."""
+    full, through the per-phase launches (grid) and, on the smallest lattices,
+    the resident kernel; the faster is reported."""
     stream = torch.cuda.current_stream()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
@@ -603,8 +604,8 @@ def run_paper_protocol(mc, torch, ising_sweeps=20000) -> dict:
     out = {"ising_1024x512": {}, "su2_table1": []}
     for name, layout in (("msc32", mc.MC_LAYOUT_MSC32), ("int8", mc.MC_LAYOUT_INT8)):
         row = {}
-        # per-colour launches from a CUDA graph; the persistent launch (one cluster for
-        # one chain) measured 3x (MSC) to 37x (int8) slower on this lattice
+        # per-colour launches; the persistent group launch (one cluster for one chain)
+        # measured 3x (MSC) to 37x (int8) slower on this lattice
         for mode in ("grid",):
             b = mc.Batch([mc.ising((1024, 512), 0.4406868, seed=1)], layout=layout, series_capacity=ising_sweeps + 16)
             g = mc.Group([b]) if mode == "group" else None
@@ -628,18 +629,14 @@ def run_paper_protocol(mc, torch, ising_sweeps=20000) -> dict:
     for (lt, ls), paper_s in PAPER_TABLE1_S.items():
         L = (lt, ls, ls, ls)
         row = {"lattice": f"{lt}x{ls}^3", "paper_gpu_s": paper_s}
-        # the persistent launches (group: one cluster for the chain; resident: the SU(2) resident mode)
-        # pay off only for the smallest lattices
-        modes = ("grid",) + (("group",) if ls <= 16 and lt == 4 else ()) + (("resident",) if ls <= 8 else ())
+        # the resident mode (one cluster for the chain, one launch per call) comes near only on the
+        # smallest lattices
+        modes = ("grid",) + (("resident",) if ls <= 8 else ())
         for mode in modes:
             b = mc.Batch([mc.su2(L, 2.3, seed=3, chain_id=0, hot=True)], series_capacity=1100)
-            if mode == "group":
-                g = mc.Group([b])
-                run = lambda n, every: g.sweep(n, every)
-            else:
-                b.set_mode(mc.MC_MODE_GRID if mode == "grid" else mc.MC_MODE_RESIDENT)
-                run = lambda n, every: b.sweep(n, every)
-            run(5, 5)  # graph capture
+            b.set_mode(mc.MC_MODE_GRID if mode == "grid" else mc.MC_MODE_RESIDENT)
+            run = b.sweep
+            run(5, 5)  # first use
             b.read_series()
 
             def protocol():
@@ -648,12 +645,10 @@ def run_paper_protocol(mc, torch, ising_sweeps=20000) -> dict:
 
             t = timed(protocol)
             P = b.read_series()["P"][0]
-            if mode == "group":
-                g.close()
             b.close()
             row[mode + "_s"] = t
             row[mode + "_mean_P"] = float(P.mean())
-        row["gb300_s"] = min(row.get("grid_s", 1e30), row.get("group_s", 1e30), row.get("resident_s", 1e30))
+        row["gb300_s"] = min(row["grid_s"], row.get("resident_s", 1e30))
         row["speedup_vs_paper_gpu"] = paper_s / row["gb300_s"]
         out["su2_table1"].append(row)
     return out

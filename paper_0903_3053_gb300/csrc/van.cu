@@ -1849,11 +1849,12 @@ __global__ void __launch_bounds__(kSampleThreads, 1) k_sample(const bf16 *__rest
 // spills and loops short enough to share the instruction cache are what the roles'
 // registers and code are cut for: 12 bytes of spills cost 8%, 56 missed lines a step 15%.
 //
-// us per position at L = 64, depth 6, 4096 samples: 1.68 against 4.45 for k_sample (depth 5:
-// 1.48 / 3.63, depth 4: 1.24 / 2.94, depth 3: 1.18 / 2.18; 1.7 to 2.1 / 4.5 to 4.9 on L = 8
-// to 50).  Tensor throughput would allow 0.87 (832 matrix instructions per step and SM, 208 per
-// sub-core at 8 cycles); the chain's latency is ~3200 cycles, of them ~1300 in its matrix
-// instructions, which share the tensor cores with the helpers'.
+// us per position at L = 64, depth 6, 4096 samples: 1.64 against 4.45 for k_sample (depth 5:
+// 1.46 / 3.63, depth 4: 1.11 / 2.94, depth 3: 1.10 / 2.18; depth 6 on L = 8 to 50: 1.65 to 2.0
+// / 4.5 to 4.9).  Tensor throughput would allow 0.87 (832 matrix instructions per step and SM,
+// 208 per sub-core at 8 cycles); the chain's latency is ~3100 cycles, of them ~1300 in its
+// matrix instructions, which share the tensor cores with the helpers', and the shared-memory
+// pipe is 85% busy with weights, columns and hand-overs.
 constexpr int kHalf = 16;                     // samples of a chain warp
 constexpr int kColBytes = kHalf * kCh * 2;    // 16 samples of one position: 1 KB
 constexpr int kPipeTiles = 7;                 // columns a helper has staged or in flight
@@ -2203,27 +2204,32 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
     }
     if (warp >= 2 * kPipeHidden + 4) { // -------------------------------------------------- output layer
         regs_shrink<kOutRegs>();
-        // two warps per half, 8 samples each: a lane has 8 channels of one (two of the sum's 8 parts)
-        const int mt = warp & 1, sub = (warp >> 1) & 1, ls = 8 * sub + (lane >> 2), qt = lane & 3, s = mt * kHalf + ls;
+        // Two warps per half, 8 samples each: a lane has 4 channels (one of the sum's 8 parts) of two samples, so that
+        // a tap is one 16-byte read of weights and one of activations (with 8 channels of one sample, three;
+        // the shared-memory pipe is 88% busy).
+        const int mt = warp & 1, sub = (warp >> 1) & 1, part = lane & 7, ls = 8 * sub + (lane >> 3); // samples ls, ls + 4
+        const int s = mt * kHalf + ls + 4 * (part & 1), mine = part < 2; // the sample whose log q this lane keeps
         unsigned char *ring = reinterpret_cast<unsigned char *>(hist) + nh * lstride +
                               ((size_t)blockIdx.x * 2 + mt) * ring_bytes + sub * 512 + lane * 16;
         unsigned char *win = smem + o.win + mt * kPipeSide * 2 * kColBytes + sub * 512 + lane * 16;
-        const bf16 *Hn = reinterpret_cast<const bf16 *>(smem + o.hn + mt * kColBytes) + ring_elem(ls, qt * 8);
+        const bf16 *Hn = reinterpret_cast<const bf16 *>(smem + o.hn + mt * kColBytes);
+        const uint2 *Ha = reinterpret_cast<const uint2 *>(Hn + ring_elem(ls, part * 4)),
+                    *Hb = reinterpret_cast<const uint2 *>(Hn + ring_elem(ls + 4, part * 4));
         const float2 *draw = reinterpret_cast<const float2 *>(smem + o.draw) + s;
         // part p of the sum goes to the chain's lane 4 (s % 8) + p % 4: float (s / 8) 2 + p / 4 of its four
-        float *Po = reinterpret_cast<float *>(smem + o.po) + mt * 128 + (lane >> 2) * 16 + (2 * qt & 3) * 4 + 2 * sub + (qt >> 1);
-        const float4 *wdl = reinterpret_cast<const float4 *>(WD) + 2 * qt;
-        double lq = 0.0; // of sample s, in the lane of its first channels
-        float po[2];
+        float *Po = reinterpret_cast<float *>(smem + o.po) + mt * 128 + (lane >> 3) * 16 + (part & 3) * 4 + 2 * sub + (part >> 2);
+        const float4 *wdl = reinterpret_cast<const float4 *>(WD) + part;
+        double lq = 0.0;
+        float po[2]; // of the two samples
         auto tap = [&](const uint4 &h, int t) {
-            const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
+            const float4 w = wdl[t * 8];
+            const uint32_t lo[2] = {h.x, h.z}, hi[2] = {h.y, h.w};
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                const float4 w = wdl[t * 8 + p];
-                po[p] = __fmaf_rn(w.x, bf16_lo(hw[2 * p]), po[p]);
-                po[p] = __fmaf_rn(w.y, bf16_hi(hw[2 * p]), po[p]);
-                po[p] = __fmaf_rn(w.z, bf16_lo(hw[2 * p + 1]), po[p]);
-                po[p] = __fmaf_rn(w.w, bf16_hi(hw[2 * p + 1]), po[p]);
+                po[p] = __fmaf_rn(w.x, bf16_lo(lo[p]), po[p]);
+                po[p] = __fmaf_rn(w.y, bf16_hi(lo[p]), po[p]);
+                po[p] = __fmaf_rn(w.z, bf16_lo(hi[p]), po[p]);
+                po[p] = __fmaf_rn(w.w, bf16_hi(hi[p]), po[p]);
             }
         };
         int slot = 0; // of column x - 2 of the position `rows_above` works on
@@ -2287,7 +2293,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
             if (k > 0) {
                 ok = wait_warp(bar_e(mt), (uint32_t)(k - 1) & 1u, abort, err);
                 h10 = h11;
-                h11 = *reinterpret_cast<const uint4 *>(Hn);
+                const uint2 ha = *Ha, hb = *Hb;
+                h11 = make_uint4(ha.x, ha.y, hb.x, hb.y);
                 lt = draw->y;
             }
             if (x >= 2)
@@ -2295,7 +2302,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
             if (x >= 1)
                 tap(h11, 11);
             Po[0] = po[0];
-            Po[4] = po[1];
+            Po[64] = po[1];
             ready(kReadyOut + mt, 96);
             if (k > 0) {
                 *reinterpret_cast<uint4 *>(dst) = h11;
@@ -2312,12 +2319,12 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
                 ++y;
             }
             rows_above(y, x);
-            if (k > 0 && qt == 0)
+            if (k > 0 && mine)
                 lq += (double)log_sigmoid(lt);
         }
         if (ok)
             wait_warp(bar_e(mt), (uint32_t)(P - 1) & 1u, abort, err);
-        if (qt == 0 && s0 + s < n)
+        if (mine && s0 + s < n)
             logq[s0 + s] = lq + (double)log_sigmoid(draw->y);
         cp_wait<0>();
         if (!ok)

@@ -12,8 +12,8 @@
 // Activations are BF16, channels innermost ([n][y][x][32]).  Every layer of
 // the forward pass and the 32 -> 32 layers' data and weight gradients run on
 // the fifth-generation tensor cores (tcgen05.mma with a tensor-memory
-// accumulator); the sampler's per-position 32-sample tiles use mma.sync
-// m16n8k16 (M = 32 is below a tcgen05 tile); BF16 in, FP32 accumulate; log q
+// accumulator); the sampler's per-position tiles of 16 or 32 samples use mma.sync
+// m16n8k16 (a tcgen05 tile has 64 or 128 rows); BF16 in, FP32 accumulate; log q
 // is accumulated in FP64.  The edge layers' gradients run on the CUDA cores.
 #pragma once
 #include <cuda_bf16.h>

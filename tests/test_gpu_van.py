@@ -387,6 +387,16 @@ def test_extreme_sides_forward_and_gradients_per_element(L, n, seed):
     _grad_check(L, n, seed)
 
 
+@pytest.mark.parametrize("L,n,seed", [(4, 9, 54), (10, 7, 54), (20, 3, 54), (24, 5, 54), (34, 2, 54), (50, 1, 54)])
+def test_convolution_runs_per_element(L, n, seed):
+    """The convolutions take runs of 2 or 4 positions as tensor-core rows (4 where
+    the side is a multiple), several samples or a few rows per item, the last
+    item of either kind partly filled: every hidden activation and every
+    gradient against the oracle at such sides, with the bounds of the tests
+    above."""
+    _grad_check(L, n, seed)
+
+
 def _sampler_uniforms(seed, rnd, n, L):
     return van.sampler_uniforms(seed, rnd, range(n), L)
 
