@@ -113,7 +113,7 @@ __device__ void run_ising(const GroupMember &m, int chain, int G, int rank, cons
     const unsigned long long base = m.state->sweep_base;
     const uint32_t stride = (uint32_t)G * blockDim.x, start = (uint32_t)rank * blockDim.x + threadIdx.x;
     char *lat = m.lattice + ch.spin_off;
-    const uint32_t units = LAYOUT == MC_LAYOUT_INT8 ? int8_units<false>(ch, 1) : ch.W * (ch.Ly >> 1);
+    const uint32_t units = LAYOUT == MC_LAYOUT_INT8 ? int8_units<false>(ch) : ch.W * (ch.Ly >> 1);
     const uint32_t nw = ch.W * ch.Ly;
     for (uint32_t t = 0; t < g.n_sweeps; ++t) {
         const uint32_t sweep = (uint32_t)(base + t);
@@ -132,14 +132,14 @@ __device__ void run_ising(const GroupMember &m, int chain, int G, int rank, cons
         if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(lat);
             for (uint32_t u = start; u < units; u += stride)
-                int8_unit<0, false, false, kLdBatch>(s, ch, ks, u, 1, sweep, anti, up);
+                int8_unit<0, false, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
             group_barrier(G, cluster);
             if (measure)
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_unit<1, true, false, kLdBatch>(s, ch, ks, u, 1, sweep, anti, up);
+                    int8_unit<1, true, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
             else
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_unit<1, false, false, kLdBatch>(s, ch, ks, u, 1, sweep, anti, up);
+                    int8_unit<1, false, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
         } else {
             uint32_t *p0 = reinterpret_cast<uint32_t *>(lat), *p1 = p0 + nw;
             for (uint32_t u = start; u < units; u += stride) {

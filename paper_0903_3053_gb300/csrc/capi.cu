@@ -303,6 +303,8 @@ mc_status upload_tables(mc_ctx *c)
         su2_plan_grid(c);
     cudaError_t e = cudaMemcpyAsync(c->d_block_start, c->block_start.data(), c->block_start.size() * 4,
                                     cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && c->kind == MC_KIND_ISING) // the plan is part of the chains' descriptors
+        e = cudaMemcpyAsync(c->d_chains, c->ising.data(), sizeof(IsingChain) * c->n_chains, cudaMemcpyHostToDevice, c->stream);
     c->block_chain.clear();
     if (c->n_chains > 1)
         for (int k = 0; k < c->n_chains; ++k)
@@ -547,8 +549,6 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
             ch.spin_off = p.lat_off[k];
             ch.div_half = make_fastdiv(ch.Lx / 2);
         }
-        e = cudaMemcpyAsync(c->d_chains, c->ising.data(), sizeof(IsingChain) * n_chains, cudaMemcpyHostToDevice,
-                            c->stream);
     } else {
         c->su2.resize(n_chains);
         for (int k = 0; k < n_chains; ++k) {

@@ -29,6 +29,7 @@
 // itself with one colour-0 site for the magnetisation; exact integer sums via
 // warp reductions and one 64-bit atomic per CTA.
 #include <algorithm>
+#include <cmath>
 
 #include "ising_dev.cuh"
 
@@ -36,7 +37,7 @@ namespace mc {
 namespace {
 
 // ------------------------------------------------------------------ grid mode
-// PAIRS (int8): threads take a.row_pairs row pairs of a group column, else a group.
+// PAIRS (int8): threads take a run of row pairs of a group column, else a group.
 template <int C, int LAYOUT, bool PAIRS>
 __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 {
@@ -49,23 +50,22 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
     chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between calls)
     if (LAYOUT == MC_LAYOUT_INT8) {
         int8_t *s = reinterpret_cast<int8_t *>(a.lattice + ch.spin_off);
-        if (t < int8_units<PAIRS>(ch, a.row_pairs)) {
+        if (t < int8_units<PAIRS>(ch)) {
             const PhiloxSchedule ks = philox_schedule(ch.key);
             if (measure)
-                int8_unit<C, true, PAIRS>(s, ch, ks, t, a.row_pairs, sweep, anti, up);
+                int8_unit<C, true, PAIRS>(s, ch, ks, t, sweep, anti, up);
             else
-                int8_unit<C, false, PAIRS>(s, ch, ks, t, a.row_pairs, sweep, anti, up);
+                int8_unit<C, false, PAIRS>(s, ch, ks, t, sweep, anti, up);
         }
     } else {
         const uint32_t W = ch.W, nw = W * ch.Ly;
         uint32_t *base = reinterpret_cast<uint32_t *>(a.lattice + ch.spin_off);
         uint32_t *pc = base + (size_t)C * nw;
         const uint32_t *po = base + (size_t)(1 - C) * nw;
-        const uint32_t np = ch.Ly >> 1, nt = (np + a.row_pairs - 1) / a.row_pairs;
-        if (t < W * nt) { // one thread per word column and a.row_pairs row pairs
+        if (t < W * ch.runs) { // one thread per word column and run of row pairs
             const PhiloxSchedule ks = philox_schedule(ch.key);
             const uint32_t q = fast_div(32 * t, ch.div_half), w = t - q * W; // t / W: half a row is 32 W sites
-            const uint32_t yy0 = q * a.row_pairs, yy1 = min(np, yy0 + a.row_pairs);
+            const uint32_t yy0 = run_start(ch, q), yy1 = run_start(ch, q + 1);
             if (measure)
                 msc_row_pairs<C, true>(pc, po, yy0, yy1, w, ch, ks, sweep, anti, up);
             else
@@ -141,16 +141,16 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
         uint32_t anti = 0, up = 0;
         if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(smem);
-            const uint32_t units = int8_units<false>(ch, 1);
+            const uint32_t units = int8_units<false>(ch);
             for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                int8_unit<0, false>(s, ch, ks, u, 1, sweep, anti, up);
+                int8_unit<0, false>(s, ch, ks, u, sweep, anti, up);
             __syncthreads();
             if (measure) {
                 for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                    int8_unit<1, true>(s, ch, ks, u, 1, sweep, anti, up);
+                    int8_unit<1, true>(s, ch, ks, u, sweep, anti, up);
             } else {
                 for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                    int8_unit<1, false>(s, ch, ks, u, 1, sweep, anti, up);
+                    int8_unit<1, false>(s, ch, ks, u, sweep, anti, up);
             }
         } else {
             const uint32_t W = ch.W, nw = W * ch.Ly, pairs = W * (ch.Ly >> 1);
@@ -400,40 +400,60 @@ size_t ising_config_bytes(const IsingChain &ch, int fmt)
 static uint32_t grid_units(const mc_ctx *c, const IsingChain &ch)
 {
     if (c->layout == MC_LAYOUT_INT8)
-        return c->row_pairs ? int8_units<true>(ch, (uint32_t)c->row_pairs) : int8_units<false>(ch, 1);
-    return ((ch.Ly >> 1) + c->row_pairs - 1) / c->row_pairs * ch.W; // runs of row pairs x words
+        return c->row_runs ? int8_units<true>(ch) : int8_units<false>(ch);
+    return ch.runs * ch.W;
 }
 
 // Row pairs per thread: more of them spread a thread's prologue
 // (chain lookup, descriptor, indices, key schedule) over more words and load each
-// neighbour row once, fewer keep the last wave of blocks even.  As many, up to 8,
+// neighbour row once, fewer keep the last wave of blocks even.
+// 32-spin words: as many, a power of two up to 8,
 // as leave 2^18 threads (1.7 full waves of 1024 threads on 152 SMs).  Measured us
 // per measured sweep with 1 / 2 / 4 / 8 row pairs: one 4096^2 chain (131072 row
 // pairs) 18.2 / 20.0 / - / -, one 8192^2 or four 4096^2 chains (524288) 54.6 / 52.3 / 57.7 /
-// 58.8, one 16384^2 chain (2097152) 199.5 / - / - / 189.2; int8, one 4096^2 chain (1048576)
-// 32.3 / - / 24.5 / -, one 8192^2 chain 120 / - / - / 81.  int8 chains of fewer than 2^17
+// 58.8, one 16384^2 chain (2097152) 199.5 / - / - / 189.2.
+// int8: as few waves as 8 allow, filled by runs of two neighbouring lengths, the longer ones first:
+// 2048^2 9.7 against 10.8 us with powers of two, 4096^2 23.1 / 25.4, 8192^2 79 / 82, three of 2000 x 1000
+// 13.0 / 14.4 (32-spin words: 8192^2 50.1 / 51.2, but four 4096^2 54.9 / 51.3).  int8 chains of fewer than 2^17
 // row pairs in all (a 2048 x 1024 lattice) take one group per thread instead: 3.5
-// against 4.0 us for 1024 x 512, 5.5 against 4.8 for 1024^2, 11.4 against 10.4 for 2048^2.
+// against 4.0 us for 1024 x 512, 5.5 against 4.8 for 1024^2, 11.4 against 10.8 for 2048^2.
 constexpr uint64_t kInt8Pairs = 1u << 17;
 constexpr uint64_t kRowPairThreads = 1u << 18;
-constexpr int kMaxRowPairs = 8;
+constexpr uint64_t kWaveThreads = 152 * 1024; // 64 registers a thread
+constexpr uint64_t kMaxRowPairs = 8;
 
 void ising_plan_grid(mc_ctx *c)
 {
+    const bool int8 = c->layout == MC_LAYOUT_INT8;
     uint64_t pairs = 0;
     for (const auto &ch : c->ising)
-        pairs += (uint64_t)(c->layout == MC_LAYOUT_INT8 ? ch.Lx / 8 : ch.W) * (ch.Ly >> 1);
-    c->row_pairs = c->layout == MC_LAYOUT_INT8 && pairs < kInt8Pairs ? 0 : 1;
-    while (c->row_pairs && c->row_pairs < kMaxRowPairs && pairs / (2 * c->row_pairs) >= kRowPairThreads)
-        c->row_pairs *= 2;
+        pairs += (uint64_t)(int8 ? ch.Lx / 8 : ch.W) * (ch.Ly >> 1);
+    c->row_runs = !int8 || pairs >= kInt8Pairs;
+    const uint64_t waves = (pairs + kMaxRowPairs * kWaveThreads - 1) / (kMaxRowPairs * kWaveThreads),
+                   most = waves * (kWaveThreads / (uint64_t)c->threads);
+    double rows = 1.0; // row pairs per thread
+    if (int8)
+        rows = std::max(1.0, (double)pairs / (double)(waves * kWaveThreads));
+    else
+        while (rows < (double)kMaxRowPairs && (double)pairs / (2.0 * rows) >= (double)kRowPairThreads)
+            rows *= 2.0;
     c->block_start.assign(c->n_chains + 1, 0);
-    uint32_t acc = 0;
-    for (int k = 0; k < c->n_chains; ++k) {
-        c->block_start[k] = acc;
-        acc += blocks_for(grid_units(c, c->ising[k]), c->threads);
+    for (;; rows *= 1.004) { // int8: until the last wave is not exceeded
+        uint64_t acc = 0, fit = 0; // blocks; those that take runs
+        for (int k = 0; k < c->n_chains; ++k) {
+            IsingChain &ch = c->ising[k];
+            const uint32_t np = ch.Ly >> 1;
+            ch.runs = int8 ? std::max(1u, (uint32_t)(np / rows)) : (uint32_t)std::ceil(np / rows);
+            ch.run = np / ch.runs;
+            c->block_start[k] = (uint32_t)acc;
+            const uint64_t blocks = blocks_for(grid_units(c, ch), c->threads);
+            acc += blocks;
+            fit += int8 && (ch.Lx & 7u) ? 0 : blocks;
+        }
+        c->block_start[c->n_chains] = c->grid_blocks = (uint32_t)acc;
+        if (!int8 || !c->row_runs || fit <= most || rows <= 1.0 || rows > 2.0 * (double)kMaxRowPairs)
+            break;
     }
-    c->block_start[c->n_chains] = acc;
-    c->grid_blocks = acc;
 }
 
 static size_t resident_bytes(const mc_ctx *c, const IsingChain &ch)
@@ -503,7 +523,7 @@ static int resident_threads(const mc_ctx *c)
 {
     uint32_t units = 0;
     for (const auto &ch : c->ising) {
-        const uint32_t u = c->layout == MC_LAYOUT_INT8 ? int8_units<false>(ch, 1) : ch.W * (ch.Ly >> 1);
+        const uint32_t u = c->layout == MC_LAYOUT_INT8 ? int8_units<false>(ch) : ch.W * (ch.Ly >> 1);
         units = u > units ? u : units;
     }
     int dev = 0, sms = 0;
@@ -563,7 +583,6 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
     a.state = c->d_state;
     a.cap = c->cap;
     a.tries = nullptr;
-    a.row_pairs = (uint32_t)std::max(c->row_pairs, 1);
     a.release = 1;
     if (mode == MC_MODE_RESIDENT) {
         int smem = 0;
@@ -587,7 +606,7 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
             cudaError_t e = prof_begin(c);
             if (e != cudaSuccess)
                 return e;
-            const bool pairs = c->row_pairs != 0;
+            const bool pairs = c->row_runs;
             if (c->layout == MC_LAYOUT_MSC32)
                 (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_MSC32, true>
                              : launch_half_sweep<1, MC_LAYOUT_MSC32, true>)(c, a);

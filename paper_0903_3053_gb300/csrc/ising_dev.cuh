@@ -201,24 +201,29 @@ __device__ __forceinline__ void int8_row_pairs(int8_t *s, const IsingChain &ch, 
     }
 }
 
+// First row pair of run q of a column (run `runs`: their number).
+__device__ __forceinline__ uint32_t run_start(const IsingChain &ch, uint32_t q)
+{
+    return q * ch.run + min(q, (ch.Ly >> 1) - ch.runs * ch.run);
+}
+
 // Work units of a chain's half-sweep: Philox groups, or (PAIRS, rows of whole
-// groups) `row_pairs` row pairs of a group column; and unit u of the chain.
+// groups) runs of row pairs of a group column; and unit u of the chain.
 template <bool PAIRS>
-__host__ __device__ __forceinline__ uint32_t int8_units(const IsingChain &ch, uint32_t row_pairs)
+__host__ __device__ __forceinline__ uint32_t int8_units(const IsingChain &ch)
 {
     if (PAIRS && (ch.Lx & 7u) == 0)
-        return ((ch.Ly >> 1) + row_pairs - 1) / row_pairs * (ch.Lx >> 3);
+        return ch.runs * (ch.Lx >> 3);
     return (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
 }
 template <int C, bool MEASURE, bool PAIRS = false, int LD = kLdPlain>
 __device__ __forceinline__ void int8_unit(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t u,
-                                          uint32_t row_pairs, uint32_t sweep, uint32_t &anti, uint32_t &up)
+                                          uint32_t sweep, uint32_t &anti, uint32_t &up)
 {
     if ((ch.Lx & 7u) == 0) {
         const uint32_t q = fast_div(4 * u, ch.div_half), gx = u - q * (ch.Lx >> 3); // u / (Lx / 8)
         if (PAIRS)
-            int8_row_pairs<C, MEASURE, LD>(s, ch, ks, q * row_pairs, min(ch.Ly >> 1, (q + 1) * row_pairs), gx, sweep,
-                                           anti, up);
+            int8_row_pairs<C, MEASURE, LD>(s, ch, ks, run_start(ch, q), run_start(ch, q + 1), gx, sweep, anti, up);
         else
             int8_row<C, MEASURE, LD>(s, ch, ks, q, gx, sweep, anti, up);
     } else {

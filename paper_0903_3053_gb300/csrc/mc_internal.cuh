@@ -30,7 +30,7 @@ struct IsingChain {
     uint32_t T2, T4;    // Metropolis thresholds for dE = 4 and dE = 8 (floor(e^{-beta dE} 2^32))
     PhiloxKey key;      // seed
     uint32_t chain_id;  // Philox counter word 3
-    uint32_t pad0;
+    uint32_t runs, run; // grid mode: a column's row pairs in `runs` runs of `run` or, the first ones, one more
     uint64_t spin_off;  // byte offset of the chain's spins in the lattice region
     double beta;        // coupling (the Metropolis-Hastings step of the learned proposal needs it)
     FastDiv div_half;   // by Lx / 2: colour-linear site index -> row
@@ -158,7 +158,6 @@ struct SweepArgs {
     int measure;                 // 1: this sweep is measured
     uint32_t rec_k;              // index of this record within the running call
     uint8_t *tries;              // SU(2) try record base, or nullptr
-    uint32_t row_pairs;          // Ising grid mode: row pairs per thread
     int release;                 // let the next kernel's blocks in once this one's are past chain_wait
 };
 
@@ -202,7 +201,7 @@ struct mc_ctx {
     std::vector<mc_chain_desc> desc;
     std::vector<uint32_t> block_start, block_chain, meas_start;
     uint32_t grid_blocks = 0, meas_blocks = 0;
-    int row_pairs = 1;                   // Ising grid mode: row pairs per thread (0: int8, one group)
+    bool row_runs = true;                // Ising grid mode: threads take runs of row pairs (else int8, a group each)
     // run bookkeeping
     long long sweeps_done = 0;
     long long rec_written = 0, rec_read = 0;

@@ -331,6 +331,34 @@ def test_full_size_sampled_sites(L, layout):
     b.close()
 
 
+@pytest.mark.parametrize("extents", [[(2000, 1000)] * 3, [(2000, 1000), (2002, 1000), (1600, 1402)], [(8, 50000)] * 12,
+                                     [(4096, 514), (16, 8), (8, 2)]])
+def test_int8_runs_of_row_pairs(extents):
+    """Large int8 batches give a thread a run of row pairs, of two neighbouring
+    lengths (columns shorter than a run, extents of partial groups beside whole
+    ones): the same spins and records as each chain by itself, where a thread
+    takes one group."""
+    def chains():
+        return [mc.ising(e, 0.42 + 0.01 * k, seed=31, chain_id=k) for k, e in enumerate(extents)]
+
+    b = mc.Batch(chains(), layout=mc.MC_LAYOUT_INT8, series_capacity=8)
+    b.set_mode(mc.MC_MODE_GRID)
+    b.sweep(3, 1)
+    rec = b.read_series()
+    cfg = [b.get_config(k) for k in range(len(extents))]
+    b.close()
+    for k, c in enumerate(chains()):
+        if extents[k] in extents[:k] and k > 1:
+            continue
+        one = mc.Batch([c], layout=mc.MC_LAYOUT_INT8, series_capacity=8)
+        one.set_mode(mc.MC_MODE_GRID)
+        one.sweep(3, 1)
+        r = one.read_series()
+        assert np.array_equal(one.get_config(0), cfg[k])
+        assert all(np.array_equal(r[f][0], rec[f][k]) for f in ("sweep", "E", "M"))
+        one.close()
+
+
 @pytest.mark.parametrize("shape,layout", [
     ((8192, 8198), mc.MC_LAYOUT_MSC32), ((64, 1 << 20), mc.MC_LAYOUT_MSC32), ((16384, 8202), mc.MC_LAYOUT_MSC32),
     ((1000, 1050), mc.MC_LAYOUT_INT8), ((8, 1 << 18), mc.MC_LAYOUT_INT8), ((4104, 4098), mc.MC_LAYOUT_INT8),
