@@ -131,26 +131,26 @@ __device__ __forceinline__ void store_row(bf16 *dst, const uint4 (&row)[8])
     for (int c = 0; c < 8; c += 2)
         store32(dst + 8 * c, row[c], row[c + 1]);
 }
-__device__ __forceinline__ void load_row(const bf16 *src, bool live, uint4 (&row)[8])
+// Which of a position's 32 activations are positive, for the backward pass: bit k for channel 2 k, bit 16 + k for
+// channel 2 k + 1.  The backward convolution reads these 4 bytes per position instead of 64 of activations (a fifth
+// of its traffic): 131 -> 110 us at L = 64, batch 512; the forward layers of a training step write them in
+// 1 to 2 us each.
+__device__ __forceinline__ uint32_t positive_bits(const uint32_t *w) // 16 packed pairs
 {
+    uint32_t bits = 0;
 #pragma unroll
-    for (int c = 0; c < 8; c += 2) {
-        row[c] = row[c + 1] = make_uint4(0u, 0u, 0u, 0u);
-        if (live)
-            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(row[c].x), "=r"(row[c].y), "=r"(row[c].z), "=r"(row[c].w), "=r"(row[c + 1].x),
-                           "=r"(row[c + 1].y), "=r"(row[c + 1].z), "=r"(row[c + 1].w)
-                         : "l"(src + 8 * c));
-    }
+    for (int k = 0; k < 16; ++k)
+        bits |= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(w + k), __floats2bfloat162_rn(0.f, 0.f)) & (0x00010001u << k);
+    return bits;
 }
-// Zero the halves of hi and lo where the activation m is not positive.
-__device__ __forceinline__ void mask8(const uint4 &m, uint4 &hi, uint4 &lo)
+// Zero the halves of channels 8 C .. 8 C + 7 of hi and lo whose bit is not set.
+template <int C>
+__device__ __forceinline__ void mask8(uint32_t bits, uint4 &hi, uint4 &lo)
 {
-    const uint32_t w[4] = {m.x, m.y, m.z, m.w};
-    uint32_t on[4];
+    uint32_t on[4]; // bits k and 16 + k to the signs of the halves, the signs over the halves
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        on[k] = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w[k]), __floats2bfloat162_rn(0.f, 0.f));
+        asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(on[k]) : "r"(bits << (15 - (4 * C + k))));
     hi.x &= on[0], hi.y &= on[1], hi.z &= on[2], hi.w &= on[3];
     lo.x &= on[0], lo.y &= on[1], lo.z &= on[2], lo.w &= on[3];
 }
@@ -176,7 +176,8 @@ constexpr uint32_t kL1Cols = 32;
 
 __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__restrict__ spins, int negate,
                                                              const float *__restrict__ w1, const float *__restrict__ b1,
-                                                             bf16 *__restrict__ h1, int n, int L, int *err)
+                                                             bf16 *__restrict__ h1, uint32_t *__restrict__ bits, int n,
+                                                             int L, int *err)
 {
     __shared__ __align__(128) uint4 A[2][kL1Threads]; // chunk planes: taps 0-7, taps 8-15
     __shared__ __align__(128) uint4 B[2][kCh];        // chunk planes: [out channel] taps 0-7, 8-15
@@ -291,6 +292,8 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
             bf16 *dst = h1 + (size_t)(p - step) * kCh;
             store32(dst, make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7]));
             store32(dst + 16, make_uint4(u[8], u[9], u[10], u[11]), make_uint4(u[12], u[13], u[14], u[15]));
+            if (bits)
+                bits[p - step] = positive_bits(u);
         }
         tc::fence_before_sync(); // this tile's tensor-memory reads precede the next MMA
     }
@@ -457,7 +460,8 @@ struct LastLayerArgs {
 struct ConvArgs {
     const bf16 *W;     // [t][o][c] (FWD, BWD)
     const float *bias; // FWD
-    const bf16 *mask;  // BWD: the layer's input activations
+    const uint32_t *mask; // BWD: positive_bits of the layer's input activations
+    uint32_t *bits;    // FWD: positive_bits of the output, or null
     bf16 *out, *out_lo;
     LastLayerArgs la;
     int n;
@@ -550,14 +554,6 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                                         full0 + 8 * s);
                 }
                 armed[s] = k;
-                if (MODE == kBwd) { // the epilogue's mask, into L2: one run of rows (or of whole lattices)
-                    const int rows = g.S > 1 ? (a.n - bi * g.S < g.S ? a.n - bi * g.S : g.S) * g.L
-                                             : (g.L - y0 < g.R ? g.L - y0 : g.R);
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                                     a.mask + ((size_t)bi * g.S * g.L + y0) * g.L * kCh),
-                                 "r"((uint32_t)(rows * g.L * kCh * 2))
-                                 : "memory");
-                }
             }
             for (int s = 0; s < 2; ++s) // the last loads of each stage have landed before the CTA ends
                 if (armed[s] >= 0 && !tc::mbar_wait(full0 + 8 * s, (armed[s] >> 1) & 1, kTcMaxPolls))
@@ -668,9 +664,9 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                     const bool live = pp >= 1 && (int)r < g.R && y < g.L && (int)smp < g.S && b < a.n && m < g.tiles;
                     // first position of the slot's pair: this lane's row of 2 x 32 channels
                     const size_t p = ((size_t)b * g.L + y) * g.L + G * (pp - 1) + (G == 4 ? 2 * slot : 0);
-                    uint4 mk[8];
-                    if (MODE == kBwd) // the mask, in flight during the wait
-                        load_row(a.mask + p * kCh, live, mk);
+                    uint2 mk = make_uint2(0u, 0u);
+                    if (MODE == kBwd && live) // the masks, in flight during the wait
+                        mk = __ldg(reinterpret_cast<const uint2 *>(a.mask + p));
                     if (!waited) {
                         waited = true;
                         ok = __any_sync(0xffffffffu, tc::mbar_wait(tfull0 + 8 * bb, (tcount >> 1) & 1u, kTcMaxPolls));
@@ -713,8 +709,11 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                             const float2 s = add2(make_float2(v[c], v[c + 1]), make_float2(bv[c % kCh], bv[c % kCh + 1]));
                             pw[c / 2] = relu_pack(s.x, s.y);
                         }
-                        if (live)
+                        if (live) {
                             store_row(a.out + p * kCh, pk);
+                            if (a.bits)
+                                *reinterpret_cast<uint2 *>(a.bits + p) = make_uint2(positive_bits(pw), positive_bits(pw + 16));
+                        }
                     } else { // one position after the other, for the registers
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
@@ -724,10 +723,13 @@ __global__ void __launch_bounds__(32 * (epilogue_warps(MODE, MINB) + 2), MINB)
                                 taken();
                             uint4 hi[4], lo[4];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
+                            for (int k = 0; k < 4; ++k)
                                 split8(v + 8 * k, hi[k], lo[k]);
-                                mask8(mk[4 * h + k], hi[k], lo[k]);
-                            }
+                            const uint32_t on = h ? mk.y : mk.x;
+                            mask8<0>(on, hi[0], lo[0]);
+                            mask8<1>(on, hi[1], lo[1]);
+                            mask8<2>(on, hi[2], lo[2]);
+                            mask8<3>(on, hi[3], lo[3]);
                             if (live) {
                                 bf16 *d = a.out + (p + h) * kCh, *e = a.out_lo + (p + h) * kCh;
                                 store32(d, hi[0], hi[1]);
@@ -2691,6 +2693,7 @@ struct mc_van {
     bf16 *H = nullptr;
     float *dZa = nullptr, *dZb = nullptr;
     float *f = nullptr, *ll = nullptr, *dF = nullptr;
+    uint32_t *bits = nullptr; // positive_bits of hidden layers 0 .. D - 3 of a training step
     int8_t *spins = nullptr, *prop = nullptr;
     double *lq = nullptr, *lq2 = nullptr, *lq3 = nullptr, *lq4 = nullptr, *mh_lr = nullptr;
     long long *E1 = nullptr, *E2 = nullptr;
@@ -2731,7 +2734,7 @@ mc_status check_err(mc_van *w, const char *where)
 }
 
 struct VanLayout {
-    size_t p, m, v, g, wh, w1, wD, bias, H, dZa, dZb, f, ll, dF, spins, prop, lq, lq2, lq3, lq4, lr, E1, E2, acc, zero,
+    size_t p, m, v, g, wh, w1, wD, bias, H, dZa, dZb, f, ll, dF, bits, spins, prop, lq, lq2, lq3, lq4, lr, E1, E2, acc, zero,
         hist, dwpart, err, total;
 };
 
@@ -2762,6 +2765,7 @@ VanLayout van_layout(int L, int nmax, int D)
     o.f = take(pos * 4);
     o.ll = take(pos * 4);
     o.dF = take(pos * 4);
+    o.bits = take((size_t)(D - 2) * pos * 4);
     o.spins = take(pos);
     o.prop = take(pos);
     o.lq = take((size_t)nmax * 8);
@@ -2853,7 +2857,8 @@ cudaError_t forward(mc_van *w, int n, int negate, double *logq, float *dF)
     const size_t layer = (size_t)w->nmax * L * L * kCh;
     const unsigned l1g =
         (unsigned)std::min<long long>(((long long)n * L * L + kL1Threads - 1) / kL1Threads, (long long)w->sms * 8);
-    k_layer1_tc<<<l1g, kL1Threads, 0, w->stream>>>(w->spins, negate, w->w1, w->bias, w->H, n, L, w->err);
+    k_layer1_tc<<<l1g, kL1Threads, 0, w->stream>>>(w->spins, negate, w->w1, w->bias, w->H, dF ? w->bits : nullptr, n, L,
+                                                   w->err);
     const RunGeom &gh = w->conv[kFwd], &gl = w->conv[kLast];
     for (int l = 1; l <= D - 1; ++l) { // hidden layers 1 .. D-2, then the last layer
         CUtensorMap in_map;
@@ -2871,6 +2876,7 @@ cudaError_t forward(mc_van *w, int n, int negate, double *logq, float *dF)
             a.W = w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh;
             a.bias = w->bias + l * kCh;
             a.out = w->H + l * layer;
+            a.bits = dF && l < D - 2 ? w->bits + l * (layer / kCh) : nullptr;
             launch_conv<kFwd>(gh, in_map, in_map, a, w->sms, w->stream);
         }
     }
@@ -2921,7 +2927,7 @@ cudaError_t backward(mc_van *w, int n)
                           (int)dwg, w->g, w->dp, l);
         ConvArgs a{};
         a.W = w->wh + (size_t)(l - 1) * kTapsB * kCh * kCh;
-        a.mask = w->H + (l - 1) * layer;
+        a.mask = w->bits + (l - 1) * (layer / kCh);
         a.out = nxh;
         a.out_lo = nxl;
         a.n = n;
@@ -3004,6 +3010,7 @@ mc_status mc_van_create(mc_van **out, int32_t L, int32_t batch, int32_t depth, u
     w->f = reinterpret_cast<float *>(b + o.f);
     w->ll = reinterpret_cast<float *>(b + o.ll);
     w->dF = reinterpret_cast<float *>(b + o.dF);
+    w->bits = reinterpret_cast<uint32_t *>(b + o.bits);
     w->spins = reinterpret_cast<int8_t *>(b + o.spins);
     w->prop = reinterpret_cast<int8_t *>(b + o.prop);
     w->lq = reinterpret_cast<double *>(b + o.lq);
