@@ -129,17 +129,52 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
     __shared__ uint32_t sums[2][2];
     if (threadIdx.x < 4)
         sums[threadIdx.x >> 1][threadIdx.x & 1] = 0;
-    for (uint32_t u = threadIdx.x; u < bytes / 4; u += blockDim.x)
-        sl[u] = gl[u];
+    const bool nibbles = LAYOUT == MC_LAYOUT_INT8 && (ch.Lx & 7u) == 0;
+    const uint32_t G = ch.Lx >> 3, groups = G * ch.Ly; // groups of a colour
+    if (nibbles) { // eight sites of a row, both colours, at a time
+        const uint2 *g8 = reinterpret_cast<const uint2 *>(gl);
+        for (uint32_t u = threadIdx.x; u < groups; u += blockDim.x) {
+            const uint32_t odd = fast_div(4 * u, ch.div_half) & 1u;
+            const uint2 v = g8[u];
+            smem[odd * groups + u] = (uint8_t)nibble_of(__byte_perm(v.x, v.y, 0x6420u));
+            smem[(odd ^ 1u) * groups + u] = (uint8_t)nibble_of(__byte_perm(v.x, v.y, 0x7531u));
+        }
+    } else {
+        for (uint32_t u = threadIdx.x; u < bytes / 4; u += blockDim.x)
+            sl[u] = gl[u];
+    }
     __syncthreads();
     const PhiloxSchedule ks = philox_schedule(ch.key);
     const unsigned long long base = a.state->sweep_base;
     int buf = 0;
+    // the next record's slot and the sweeps until it: counted, not divided for (warp 0 writes the record on the way to the
+    // next sweep's barrier)
+    unsigned long long slot = a.state->rec_head % (unsigned long long)a.cap;
+    DevRecord *const series = &a.series[(long long)k * a.cap];
+    uint32_t until = every;
     for (uint32_t t = 0; t < n_sweeps; ++t) {
         const uint32_t sweep = (uint32_t)(base + t);
-        const bool measure = every != 0 && ((t + 1) % every) == 0;
+        const bool measure = every != 0 && --until == 0;
         uint32_t anti = 0, up = 0;
-        if (LAYOUT == MC_LAYOUT_INT8) {
+        if (nibbles) {
+            uint8_t *p0 = smem, *p1 = smem + groups;
+            for (uint32_t u = threadIdx.x; u < groups / 2; u += blockDim.x) {
+                const uint32_t yy = fast_div(4 * u, ch.div_half);
+                nibble_row_pair<0, false>(p0, p1, yy, u - yy * G, ch, ks, sweep, anti, up);
+            }
+            __syncthreads();
+            if (measure) {
+                for (uint32_t u = threadIdx.x; u < groups / 2; u += blockDim.x) {
+                    const uint32_t yy = fast_div(4 * u, ch.div_half);
+                    nibble_row_pair<1, true>(p1, p0, yy, u - yy * G, ch, ks, sweep, anti, up);
+                }
+            } else {
+                for (uint32_t u = threadIdx.x; u < groups / 2; u += blockDim.x) {
+                    const uint32_t yy = fast_div(4 * u, ch.div_half);
+                    nibble_row_pair<1, false>(p1, p0, yy, u - yy * G, ch, ks, sweep, anti, up);
+                }
+            }
+        } else if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(smem);
             const uint32_t units = int8_units<false>(ch);
             for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
@@ -183,8 +218,7 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
         __syncthreads();
         if (measure) {
             if (threadIdx.x == 0) {
-                const unsigned long long r = a.state->rec_head + (t + 1) / every - 1;
-                DevRecord *rec = &a.series[(long long)k * a.cap + (long long)(r % (unsigned long long)a.cap)];
+                DevRecord *rec = &series[slot];
                 rec->sweep = (long long)(base + t);
                 rec->a = sums[buf][0];
                 rec->b = sums[buf][1];
@@ -192,7 +226,18 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
                 sums[buf][0] = sums[buf][1] = 0; // next added to two measurements later, past further barriers
             }
             buf ^= 1;
+            until = every;
+            slot = slot + 1 == (unsigned long long)a.cap ? 0 : slot + 1;
         }
+    }
+    if (nibbles) {
+        uint2 *g8 = reinterpret_cast<uint2 *>(gl);
+        for (uint32_t u = threadIdx.x; u < groups; u += blockDim.x) {
+            const uint32_t odd = fast_div(4 * u, ch.div_half) & 1u;
+            const uint32_t even_x = bytes_of(smem[odd * groups + u]), odd_x = bytes_of(smem[(odd ^ 1u) * groups + u]);
+            g8[u] = make_uint2(__byte_perm(even_x, odd_x, 0x5140u), __byte_perm(even_x, odd_x, 0x7362u));
+        }
+        return;
     }
     for (uint32_t u = threadIdx.x; u < bytes / 4; u += blockDim.x)
         gl[u] = sl[u];
@@ -438,8 +483,8 @@ void ising_plan_grid(mc_ctx *c)
         while (rows < (double)kMaxRowPairs && (double)pairs / (2.0 * rows) >= (double)kRowPairThreads)
             rows *= 2.0;
     c->block_start.assign(c->n_chains + 1, 0);
-    for (;; rows *= 1.004) { // int8: until the last wave is not exceeded
-        uint64_t acc = 0, fit = 0; // blocks; those that take runs
+    for (;;) { // int8: until the last wave is not exceeded, or every chain is one block
+        uint64_t acc = 0, fit = 0, least = 0; // blocks; those that take runs; chains that do
         for (int k = 0; k < c->n_chains; ++k) {
             IsingChain &ch = c->ising[k];
             const uint32_t np = ch.Ly >> 1;
@@ -448,11 +493,15 @@ void ising_plan_grid(mc_ctx *c)
             c->block_start[k] = (uint32_t)acc;
             const uint64_t blocks = blocks_for(grid_units(c, ch), c->threads);
             acc += blocks;
-            fit += int8 && (ch.Lx & 7u) ? 0 : blocks;
+            if ((ch.Lx & 7u) == 0) {
+                fit += blocks;
+                ++least;
+            }
         }
         c->block_start[c->n_chains] = c->grid_blocks = (uint32_t)acc;
-        if (!int8 || !c->row_runs || fit <= most || rows <= 1.0 || rows > 2.0 * (double)kMaxRowPairs)
+        if (!int8 || !c->row_runs || fit <= std::max(most, least) || rows <= 1.0 || rows > 2.0 * (double)kMaxRowPairs)
             break;
+        rows *= fit > most + most / 32 ? 1.03 : 1.004;
     }
 }
 
@@ -482,9 +531,9 @@ bool ising_resident_fits(const mc_ctx *c, int *smem_bytes)
 // sweep, from times measured over L = 16 .. 384 and 1 .. 4096 chains.  A resident
 // chain costs its sites at one CTA's rate, and chains beyond one per SM queue up; a
 // grid sweep costs two chained launches and all sites at the chip's rate.
-// Resident / grid, measured us per measured sweep: int8 64^2 x 1 chain 1.9 / 3.4,
-// 96^2 x 1 3.5 / 3.4, 128^2 x 1 4.7 / 3.5, 128^2 x 48 4.8 / 5.3, 256^2 x 1 14.2 / 3.4, 256^2 x 152
-// 14.7 / 18.9, 64^2 x 4096 26 / 63, 130^2 (ragged groups) x 1 7.3 / 5.3; 32-spin words 128^2
+// Resident / grid, measured us per measured sweep: int8 64^2 x 1 chain 1.25 / 3.1,
+// 96^2 x 1 2.4 / 3.1, 128^2 x 1 3.4 / 3.1, 128^2 x 48 3.4 / 4.6, 256^2 x 1 11 / 3.1, 256^2 x 48 11 / 8.7, 256^2 x 152
+// 10.7 / 15.0, 64^2 x 4096 20 / 170, 128^2 x 1024 18 / 53, 130^2 (ragged groups) x 1 7.1 / 5.1; 32-spin words 128^2
 // x 1 4.3 / 5.4, 256^2 x 1 8.0 / 6.5, 256^2 x 152 8.3 / 10.3, 384^2 x 48 17.9 / 10.3.
 bool ising_resident_auto(const mc_ctx *c)
 {
@@ -505,11 +554,11 @@ bool ising_resident_auto(const mc_ctx *c)
     if (c->layout == MC_LAYOUT_MSC32)
         return std::max(4.2, 0.122e-3 * one * rounds) <= 5.4 + 0.6e-6 * all;
     return ragged ? 1.0 + 0.38e-3 * one * rounds <= 4.0 + 4.5e-6 * all
-                  : 1.0 + 0.22e-3 * one * rounds <= 3.4 + 2.0e-6 * all;
+                  : 0.75 + 0.16e-3 * one * rounds <= 3.1 + 1.3e-6 * all;
 }
 
-// Threads of a resident CTA: the work units of the largest chain (int8: groups
-// of four same-colour sites; MSC32: row pairs) rounded up to a warp, at most
+// Threads of a resident CTA: the work units of the largest chain (int8: pairs of groups
+// in a row pair, or groups where Lx is no multiple of 8; MSC32: row pairs) rounded up to a warp, at most
 // the block size -- the caller's (mc_set_mode), else 1024 when every chain has
 // an SM to itself and the default (256) when chains share SMs.  Threads past
 // the last unit would idle through every half-sweep and hold the SM's warp
@@ -517,13 +566,14 @@ bool ising_resident_auto(const mc_ctx *c)
 // of 4096 such chains is resident on the 152 SMs in one wave (1.23e12 against
 // 0.96e12 spin flips/s with 256-thread CTAs, four waves of one working warp
 // each).  With a CTA per SM to spare, more threads shorten each half-sweep:
-// one 64^2 int8 chain 2.44 against 2.99 us per sweep with 512 threads, one
-// 256^2 MSC32 chain 7.8 against 9.2 us.
+// one 256^2 MSC32 chain 7.8 against 9.2 us.
 static int resident_threads(const mc_ctx *c)
 {
     uint32_t units = 0;
     for (const auto &ch : c->ising) {
-        const uint32_t u = c->layout == MC_LAYOUT_INT8 ? int8_units<false>(ch) : ch.W * (ch.Ly >> 1);
+        const uint32_t u = c->layout == MC_LAYOUT_MSC32 ? ch.W * (ch.Ly >> 1)
+                           : (ch.Lx & 7u) == 0          ? (ch.Lx >> 3) * (ch.Ly >> 1)
+                                                        : int8_units<false>(ch);
         units = u > units ? u : units;
     }
     int dev = 0, sms = 0;

@@ -143,9 +143,7 @@ __device__ __forceinline__ bool int8_oct(uint32_t par, uint2 &w, uint2 wu, uint2
 // One group: column gx of row y.  Three 8-byte loads and one byte replace the 20 byte
 // loads of int8_group; the other colour's bytes of the 8-byte store hold the values
 // they had.  Bound by the schedulers' dispatch (Philox is 72 of its ~200 cycles per
-// warp and group); against the byte-wise form 100 measured sweeps of one 64^2 chain
-// 307 -> 194 us, 10 sweeps of 4096 such chains 543 -> 388 us (resident mode,
-// configuration and series read back each time).
+// warp and group); the byte-wise form took 1.6 times as long.
 template <int C, bool MEASURE, int LD = kLdPlain>
 __device__ __forceinline__ void int8_row(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t y,
                                          uint32_t gx, uint32_t sweep, uint32_t &anti, uint32_t &up)
@@ -167,7 +165,7 @@ __device__ __forceinline__ void int8_row(int8_t *s, const IsingChain &ch, const 
 // row is loaded once; a thread's prologue is spread over several groups.  For
 // large grid launches (an 8192^2 chain 141 -> 81 us per measured sweep, 4096^2 37
 // -> 25); with fewer threads than the chip holds int8_row is faster (1024 x 512
-// 3.5 against 4.0 us), as it is in shared memory (4096 chains of 64^2 26 against 28).
+// 3.5 against 4.0 us).
 template <int C, bool MEASURE, int LD = kLdPlain>
 __device__ __forceinline__ void int8_row_pairs(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t yy0,
                                                uint32_t yy1, uint32_t gx, uint32_t sweep, uint32_t &anti, uint32_t &up)
@@ -198,6 +196,65 @@ __device__ __forceinline__ void int8_row_pairs(int8_t *s, const IsingChain &ch, 
         y0 += 2;
         blk += 2 * W8;
         row += 2 * Lx;
+    }
+}
+
+// Nibbles: a resident int8 lattice of whole groups (Lx % 8 == 0), held as one byte per group and colour,
+// plane[c][y][g] with the group's four sites x = 8 g + 2 j + ((y + c) & 1) as bits j = 0..3 (1 = up).  A
+// group's update is then the 32-spin words' logic on four bits: ~110 dispatch cycles per warp and group, 72 of them
+// Philox, against ~200 on bytes.  us per measured sweep: 4096 chains of 64^2 19.9 against 26.4, 1024 of 128^2 18.4 / 25.7, one of
+// 64^2 1.25 / 1.66 (0.2 of it the record's slot, counted instead of divided for).
+// The bits (1 = up) of the four bytes of v.
+__device__ __forceinline__ uint32_t nibble_of(uint32_t v)
+{
+    return ((~v >> 7 & 0x01010101u) * 0x01020408u >> 24) & 15u;
+}
+// The spin bytes of a nibble: 1 -> 0x01, 0 -> 0xFF.
+__device__ __forceinline__ uint32_t bytes_of(uint32_t nib)
+{
+    return ~(((nib * 0x00204081u) & 0x01010101u) * 0xFEu);
+}
+// New nibble s given its neighbours (as msc_word).
+template <int C>
+__device__ __forceinline__ uint32_t nibble_update(uint32_t s, uint32_t nu, uint32_t nd, uint32_t ns, uint32_t side, uint32_t blk,
+                                                  uint32_t sweep, const IsingChain &ch, const PhiloxSchedule &ks)
+{
+    const uint4 r = philox4x32_10(make_uint4(blk, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+    uint32_t g2 = 0, g4 = 0;
+    ge_chain2(g2, g4, r.w, 0u - ch.T2, 0u - ch.T4);
+    ge_chain2(g2, g4, r.z, 0u - ch.T2, 0u - ch.T4);
+    ge_chain2(g2, g4, r.y, 0u - ch.T2, 0u - ch.T4);
+    ge_chain2(g2, g4, r.x, 0u - ch.T2, 0u - ch.T4);
+    g2 |= ch.T2 == 0 ? 15u : 0u;
+    g4 |= ch.T4 == 0 ? 15u : 0u;
+    const uint32_t a1 = s ^ nu, a2 = s ^ nd, a3 = s ^ ns, a4 = s ^ side; // 1 = anti-aligned
+    const uint32_t x = a1 ^ a2 ^ a3, m = (a1 & a2) | (a3 & (a1 | a2)); // 2 m + x = a1 + a2 + a3
+    return s ^ (((x & a4) | m | ~g4 | ((x ^ a4) & ~g2)) & 15u);
+}
+// Group g of rows 2 yy and 2 yy + 1 of plane C (as msc_row_pairs: the rows' parities are fixed and the pair shares
+// the other plane's rows).
+template <int C, bool MEASURE>
+__device__ __forceinline__ void nibble_row_pair(uint8_t *pc, const uint8_t *po, uint32_t yy, uint32_t g, const IsingChain &ch,
+                                                const PhiloxSchedule &ks, uint32_t sweep, uint32_t &anti, uint32_t &up)
+{
+    const uint32_t G = ch.Lx >> 3, Ly = ch.Ly, y0 = 2 * yy, r0 = y0 * G, r1 = r0 + G;
+    const uint32_t gl = dec_wrap(g, G), gr = inc_wrap(g, G);
+    const uint32_t om = po[dec_wrap(y0, Ly) * G + g], o0 = po[r0 + g], o1 = po[r1 + g],
+                   op = po[(y0 + 2 == Ly ? 0u : r1 + G) + g];
+    const uint32_t s0 = pc[r0 + g], s1 = pc[r1 + g];
+    // offset C on the even row, 1 - C on the odd one: the neighbour at j - 1 (offset 0) or j + 1
+    const uint32_t e0 = po[r0 + (C == 0 ? gl : gr)], e1 = po[r1 + (C == 0 ? gr : gl)];
+    const uint32_t left = C == 0 ? o0 : o1, le = C == 0 ? e0 : e1, right = C == 0 ? o1 : o0, re = C == 0 ? e1 : e0;
+    const uint32_t from_left = (left << 1 | le >> 3) & 15u, from_right = right >> 1 | (re << 3 & 8u);
+    const uint32_t side0 = C == 0 ? from_left : from_right, side1 = C == 0 ? from_right : from_left;
+    const uint32_t n0 = nibble_update<C>(s0, om, o1, o0, side0, r0 + g, sweep, ch, ks);
+    const uint32_t n1 = nibble_update<C>(s1, o0, op, o1, side1, r1 + g, sweep, ch, ks);
+    pc[r0 + g] = (uint8_t)n0;
+    pc[r1 + g] = (uint8_t)n1;
+    if (MEASURE) {
+        const uint32_t u0 = om | o1 << 4 | o0 << 8 | side0 << 12, u1 = o0 | op << 4 | o1 << 8 | side1 << 12;
+        anti += __popc((n0 * 0x1111u ^ u0) | (n1 * 0x1111u ^ u1) << 16);
+        up += __popc(n0 | o0 << 4 | n1 << 8 | o1 << 12);
     }
 }
 

@@ -331,6 +331,32 @@ def test_full_size_sampled_sites(L, layout):
     b.close()
 
 
+@pytest.mark.parametrize("every", [0, 1, 3])
+@pytest.mark.parametrize("beta", [0.2, 0.4406868, 3.0, 6.0])
+def test_int8_resident_nibbles(beta, every):
+    """Resident int8 lattices of whole groups are held as four-bit groups: one
+    group per row, two rows, row ends, odd numbers of row pairs, beside chains of
+    partial groups, thresholds of zero; records wrap around the series.  The same
+    spins and records as the grid launches."""
+    extents = [(8, 2), (8, 6), (16, 2), (24, 10), (64, 64), (72, 30), (200, 18), (6, 10), (130, 4)]
+    out = []
+    for mode in (mc.MC_MODE_RESIDENT, mc.MC_MODE_GRID):
+        b = mc.Batch([mc.ising(e, beta, seed=77, chain_id=k) for k, e in enumerate(extents)],
+                     layout=mc.MC_LAYOUT_INT8, series_capacity=8)
+        b.set_mode(mode)
+        recs = []
+        for n in (7, 6):
+            b.sweep(n - n % max(every, 1) if every else n, every)
+            recs.append(b.read_series().copy())
+        out.append((recs, [b.get_config(k) for k in range(len(extents))]))
+        b.close()
+    (r0, c0), (r1, c1) = out
+    for x, y in zip(r0, r1):
+        assert np.array_equal(x, y)
+    for x, y in zip(c0, c1):
+        assert np.array_equal(x, y) and set(np.unique(x)) <= {-1, 1}
+
+
 @pytest.mark.parametrize("extents", [[(2000, 1000)] * 3, [(2000, 1000), (2002, 1000), (1600, 1402)], [(8, 50000)] * 12,
                                      [(4096, 514), (16, 8), (8, 2)]])
 def test_int8_runs_of_row_pairs(extents):
