@@ -132,14 +132,14 @@ __device__ void run_ising(const GroupMember &m, int chain, int G, int rank, cons
         if (LAYOUT == MC_LAYOUT_INT8) {
             int8_t *s = reinterpret_cast<int8_t *>(lat);
             for (uint32_t u = start; u < units; u += stride)
-                int8_unit<0, false, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                int8_unit<0, false, false, kLdBatch, 1>(s, ch, ks, u, sweep, anti, up);
             group_barrier(G, cluster);
             if (measure)
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_unit<1, true, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, true, false, kLdBatch, 1>(s, ch, ks, u, sweep, anti, up);
             else
                 for (uint32_t u = start; u < units; u += stride)
-                    int8_unit<1, false, false, kLdBatch>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, false, false, kLdBatch, 1>(s, ch, ks, u, sweep, anti, up);
         } else {
             uint32_t *p0 = reinterpret_cast<uint32_t *>(lat), *p1 = p0 + nw;
             for (uint32_t u = start; u < units; u += stride) {

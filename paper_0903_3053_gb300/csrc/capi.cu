@@ -147,7 +147,9 @@ Plan make_plan(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t c
     for (int k = 0; k < n; ++k) {
         const mc_chain_desc &d = chains[k];
         const size_t sites = (size_t)d.L[0] * d.L[1] * (kind == MC_KIND_ISING ? 1 : (size_t)d.L[2] * d.L[3]);
-        const size_t units = kind == MC_KIND_SU2 ? sites / 2 : layout == MC_LAYOUT_INT8 ? (sites / 2 + 3) / 4 : sites / 128;
+        const size_t units = kind == MC_KIND_SU2         ? sites / 2
+                             : layout == MC_LAYOUT_INT8 ? (sites / 2 + 3) / 4 + (size_t)d.L[1] // int8: and the rows' ends
+                                                        : sites / 128;
         p.block_chain_count += (units + 31) / 32;
     }
     if (n == 1)
@@ -548,6 +550,7 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
             ch.chain_id = chains[k].chain_id;
             ch.spin_off = p.lat_off[k];
             ch.div_half = make_fastdiv(ch.Lx / 2);
+            ch.div_inner = make_fastdiv(std::max(ch.Lx / 8, 1u));
         }
     } else {
         c->su2.resize(n_chains);

@@ -37,8 +37,12 @@ namespace mc {
 namespace {
 
 // ------------------------------------------------------------------ grid mode
-// PAIRS (int8): threads take a run of row pairs of a group column, else a group.
-template <int C, int LAYOUT, bool PAIRS>
+// What a thread of an int8 launch takes: a group of any chain, a run of row pairs of
+// a group column, or a group of chains that all have rows of whole groups.  A kernel without the
+// code for groups over a row's end has the shorter chain of instructions (1024 x 512 4.1
+// us per measured sweep against 4.5 with both in one, 1024 x 256 twice 4.5 / 4.8).
+enum { kGroups, kRuns, kRows };
+template <int C, int LAYOUT, int FORM>
 __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 {
     const int k = chain_of_block(a);
@@ -50,12 +54,12 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
     chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between calls)
     if (LAYOUT == MC_LAYOUT_INT8) {
         int8_t *s = reinterpret_cast<int8_t *>(a.lattice + ch.spin_off);
-        if (t < int8_units<PAIRS>(ch)) {
+        if (t < int8_units<FORM == kRuns>(ch)) {
             const PhiloxSchedule ks = philox_schedule(ch.key);
             if (measure)
-                int8_unit<C, true, PAIRS>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, true, FORM == kRuns, kLdPlain, FORM == kRows ? 0 : 4>(s, ch, ks, t, sweep, anti, up);
             else
-                int8_unit<C, false, PAIRS>(s, ch, ks, t, sweep, anti, up);
+                int8_unit<C, false, FORM == kRuns, kLdPlain, FORM == kRows ? 0 : 4>(s, ch, ks, t, sweep, anti, up);
         }
     } else {
         const uint32_t W = ch.W, nw = W * ch.Ly;
@@ -96,23 +100,24 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
 // threads with 4 resident per SM (64 registers, so that the Philox key schedule
 // stays in registers; the kernel is bound by the schedulers' dispatch, which 32
 // warps per SM keep busy: a 32768^2 chain in 32-spin words 730 us per sweep against
-// 757 with 8 blocks and 32 registers) or 6 for int8 groups (40 registers, no
-// spills), and blocks of up to 1024 threads for callers that ask for them.
-template <int C, int LAYOUT, bool PAIRS>
-__global__ void __launch_bounds__(256, LAYOUT == MC_LAYOUT_MSC32 || PAIRS ? 4 : 6) k_half_sweep(SweepArgs a)
+// 757 with 8 blocks and 32 registers, int8 groups need them for the bytes loaded ahead) or 5 for
+// int8 rows of whole groups (48 registers; with 4 or 8 1024 x 512 takes 4.3 or 4.5 us against
+// 4.1), and blocks of up to 1024 threads for callers that ask for them.
+template <int C, int LAYOUT, int FORM>
+__global__ void __launch_bounds__(256, FORM == kRows ? 5 : 4) k_half_sweep(SweepArgs a)
 {
-    half_sweep<C, LAYOUT, PAIRS>(a);
+    half_sweep<C, LAYOUT, FORM>(a);
 }
-template <int C, int LAYOUT, bool PAIRS>
+template <int C, int LAYOUT, int FORM>
 __global__ void __launch_bounds__(1024) k_half_sweep_big(SweepArgs a)
 {
-    half_sweep<C, LAYOUT, PAIRS>(a);
+    half_sweep<C, LAYOUT, FORM>(a);
 }
 
-template <int C, int LAYOUT, bool PAIRS>
+template <int C, int LAYOUT, int FORM>
 void launch_half_sweep(mc_ctx *c, const SweepArgs &a)
 {
-    launch_chained(c, c->threads <= 256 ? k_half_sweep<C, LAYOUT, PAIRS> : k_half_sweep_big<C, LAYOUT, PAIRS>,
+    launch_chained(c, c->threads <= 256 ? k_half_sweep<C, LAYOUT, FORM> : k_half_sweep_big<C, LAYOUT, FORM>,
                    c->grid_blocks, (unsigned)c->threads, a);
 }
 
@@ -178,14 +183,14 @@ __global__ void __launch_bounds__(1024) k_resident(SweepArgs a, uint32_t n_sweep
             int8_t *s = reinterpret_cast<int8_t *>(smem);
             const uint32_t units = int8_units<false>(ch);
             for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                int8_unit<0, false>(s, ch, ks, u, sweep, anti, up);
+                int8_unit<0, false, false, kLdPlain, 1>(s, ch, ks, u, sweep, anti, up);
             __syncthreads();
             if (measure) {
                 for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                    int8_unit<1, true>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, true, false, kLdPlain, 1>(s, ch, ks, u, sweep, anti, up);
             } else {
                 for (uint32_t u = threadIdx.x; u < units; u += blockDim.x)
-                    int8_unit<1, false>(s, ch, ks, u, sweep, anti, up);
+                    int8_unit<1, false, false, kLdPlain, 1>(s, ch, ks, u, sweep, anti, up);
             }
         } else {
             const uint32_t W = ch.W, nw = W * ch.Ly, pairs = W * (ch.Ly >> 1);
@@ -474,6 +479,7 @@ void ising_plan_grid(mc_ctx *c)
     for (const auto &ch : c->ising)
         pairs += (uint64_t)(int8 ? ch.Lx / 8 : ch.W) * (ch.Ly >> 1);
     c->row_runs = !int8 || pairs >= kInt8Pairs;
+    c->whole_rows = std::all_of(c->ising.begin(), c->ising.end(), [](const IsingChain &ch) { return (ch.Lx & 7u) == 0; });
     const uint64_t waves = (pairs + kMaxRowPairs * kWaveThreads - 1) / (kMaxRowPairs * kWaveThreads),
                    most = waves * (kWaveThreads / (uint64_t)c->threads);
     double rows = 1.0; // row pairs per thread
@@ -656,16 +662,15 @@ cudaError_t ising_sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
             cudaError_t e = prof_begin(c);
             if (e != cudaSuccess)
                 return e;
-            const bool pairs = c->row_runs;
             if (c->layout == MC_LAYOUT_MSC32)
-                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_MSC32, true>
-                             : launch_half_sweep<1, MC_LAYOUT_MSC32, true>)(c, a);
-            else if (pairs)
-                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, true>
-                             : launch_half_sweep<1, MC_LAYOUT_INT8, true>)(c, a);
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_MSC32, kRuns> : launch_half_sweep<1, MC_LAYOUT_MSC32, kRuns>)(c, a);
+            else if (c->row_runs)
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, kRuns> : launch_half_sweep<1, MC_LAYOUT_INT8, kRuns>)(c, a);
+            else if (c->whole_rows)
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, kRows> : launch_half_sweep<1, MC_LAYOUT_INT8, kRows>)(c, a);
             else
-                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, false>
-                             : launch_half_sweep<1, MC_LAYOUT_INT8, false>)(c, a);
+                (colour == 0 ? launch_half_sweep<0, MC_LAYOUT_INT8, kGroups>
+                             : launch_half_sweep<1, MC_LAYOUT_INT8, kGroups>)(c, a);
             e = prof_end(c);
             if (e != cudaSuccess)
                 return e;

@@ -45,39 +45,62 @@ __device__ __forceinline__ void block_sum2(uint32_t &a, uint32_t &b)
 //
 // int8_group, any even extents: the sites are consecutive in the colour's
 // raster order and may run over the end of a row, so the row and column are
-// carried from site to site (one division per group, by a multiplication).
-template <int C, bool MEASURE, int LD = kLdPlain>
+// carried from site to site (one division per group, by a multiplication).  The bytes of
+// AHEAD sites are loaded before the first of them is updated: loads that follow a store
+// wait for it, and a launch of few blocks is one such chain (us per measured sweep with 1 / 4
+// ahead: 620 x 170 5.6 / 4.0, four of them 6.1 / 4.7, 1022 x 512 5.6 / 4.7; in shared memory the
+// registers cost more than the wait: 512 lattices of 50^2 6.5 / 7.0).
+template <int C, bool MEASURE, int LD = kLdPlain, int AHEAD = 4>
 __device__ __forceinline__ void int8_group(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t g,
                                            uint32_t sweep, uint32_t &anti, uint32_t &up)
 {
     const uint32_t Lx = ch.Lx, Ly = ch.Ly, half = Lx >> 1, nc = (Lx * Ly) >> 1;
-    const uint4 r4 = philox4x32_10(make_uint4(g, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
-    const uint32_t rr[4] = {r4.x, r4.y, r4.z, r4.w};
-    uint32_t y, j;
-    fast_divmod(4 * g, ch.div_half, y, j);
     const uint32_t live = nc - 4 * g < 4u ? nc - 4 * g : 4u;
+    uint32_t y, j, rr[4];
+    static_assert(AHEAD == 1 || AHEAD == 4, "the draws are made once");
+    const auto draw = [&]() {
+        const uint4 r = philox4x32_10(make_uint4(g, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+        rr[0] = r.x, rr[1] = r.y, rr[2] = r.z, rr[3] = r.w;
+    };
+    if (AHEAD == 1)
+        draw();
+    fast_divmod(4 * g, ch.div_half, y, j);
 #pragma unroll
-    for (uint32_t q = 0; q < 4; ++q) {
-        if (q >= live)
+    for (uint32_t q0 = 0; q0 < 4; q0 += AHEAD) {
+        if (q0 >= live)
             break;
-        const uint32_t x = 2 * j + ((y + C) & 1u);
-        const uint32_t row = y * Lx, rowp = inc_wrap(y, Ly) * Lx, rowm = dec_wrap(y, Ly) * Lx;
-        const int sv = lat_load<LD>(&s[row + x]);
-        const int ne = lat_load<LD>(&s[row + inc_wrap(x, Lx)]), nw = lat_load<LD>(&s[row + dec_wrap(x, Lx)]);
-        const int nn = lat_load<LD>(&s[rowm + x]), ns = lat_load<LD>(&s[rowp + x]);
-        const int local = sv * (ne + nw + nn + ns); // dE / 2
-        const bool flip = local <= 0 || rr[q] < (local == 2 ? ch.T2 : ch.T4);
-        const int nv = flip ? -sv : sv;
-        if (flip)
-            s[row + x] = (int8_t)nv;
-        if (MEASURE) {
-            anti += (uint32_t)(ne != nv) + (uint32_t)(nw != nv) + (uint32_t)(nn != nv) + (uint32_t)(ns != nv);
-            const int partner = (x & 1u) ? nw : ne; // colour-0 site (x ^ 1, y)
-            up += (uint32_t)(nv > 0) + (uint32_t)(partner > 0);
+        uint32_t at[AHEAD];
+        int sv[AHEAD], ne[AHEAD], nw[AHEAD], nn[AHEAD], ns[AHEAD];
+#pragma unroll
+        for (uint32_t q = 0; q < AHEAD; ++q) {
+            const uint32_t x = 2 * j + ((y + C) & 1u), row = y * Lx;
+            at[q] = row + x;
+            sv[q] = lat_load<LD>(&s[row + x]);
+            ne[q] = lat_load<LD>(&s[row + inc_wrap(x, Lx)]);
+            nw[q] = lat_load<LD>(&s[row + dec_wrap(x, Lx)]);
+            nn[q] = lat_load<LD>(&s[dec_wrap(y, Ly) * Lx + x]);
+            ns[q] = lat_load<LD>(&s[inc_wrap(y, Ly) * Lx + x]);
+            if (q0 + q + 1 < live && ++j == half) { // the last site of the colour is loaded again
+                j = 0;
+                ++y;
+            }
         }
-        if (++j == half) {
-            j = 0;
-            ++y;
+        if (AHEAD > 1)
+            draw();
+#pragma unroll
+        for (uint32_t q = 0; q < AHEAD; ++q) {
+            if (q0 + q >= live)
+                break;
+            const int local = sv[q] * (ne[q] + nw[q] + nn[q] + ns[q]); // dE / 2
+            const bool flip = local <= 0 || rr[q0 + q] < (local == 2 ? ch.T2 : ch.T4);
+            const int nv = flip ? -sv[q] : sv[q];
+            if (flip)
+                s[at[q]] = (int8_t)nv;
+            if (MEASURE) {
+                anti += (uint32_t)(ne[q] != nv) + (uint32_t)(nw[q] != nv) + (uint32_t)(nn[q] != nv) + (uint32_t)(ns[q] != nv);
+                const int partner = (at[q] & 1u) ? nw[q] : ne[q]; // colour-0 site (x ^ 1, y)
+                up += (uint32_t)(nv > 0) + (uint32_t)(partner > 0);
+            }
         }
     }
 }
@@ -264,27 +287,71 @@ __device__ __forceinline__ uint32_t run_start(const IsingChain &ch, uint32_t q)
     return q * ch.run + min(q, (ch.Ly >> 1) - ch.runs * ch.run);
 }
 
-// Work units of a chain's half-sweep: Philox groups, or (PAIRS, rows of whole
-// groups) runs of row pairs of a group column; and unit u of the chain.
+// Rows of partial groups (Lx no multiple of 8, at least 8): a group that lies inside a row is updated as in
+// int8_row, its eight bytes loaded and stored as four pairs (rows start on even bytes).  The groups over a row's end
+// take int8_group, in warps of their own: units 0 .. Ly n - 1 are the slots y n + i of at most n = Lx / 8 inner groups of a
+// row, then follows the group at each row's end.  For large grid launches: 4094 x 4098 63.7 -> 52.1 us per measured
+// sweep, three of 998 x 1050 16.4 -> 14.6, 2046^2 18.3 -> 17.1; smaller launches and resident lattices are
+// faster with one form for all (1022 x 512 4.7 against 6.5, resident 50^2 2.3 against 2.9).
+template <int C, bool MEASURE, int LD>
+__device__ __forceinline__ void int8_inner(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t y, uint32_t g,
+                                           uint32_t sweep, uint32_t &anti, uint32_t &up)
+{
+    const uint32_t Lx = ch.Lx, Ly = ch.Ly, par = (y + C) & 1u, x0 = 2 * (4 * g - y * (Lx >> 1));
+    int8_t *row = s + y * Lx;
+    auto eight = [&](const int8_t *p) {
+        const uint16_t *h = reinterpret_cast<const uint16_t *>(p + x0);
+        const uint32_t a = lat_load<LD>(h), b = lat_load<LD>(h + 1), c = lat_load<LD>(h + 2), d = lat_load<LD>(h + 3);
+        return make_uint2(__byte_perm(a, b, 0x5410u), __byte_perm(c, d, 0x5410u));
+    };
+    uint2 w = eight(row);
+    const uint2 wu = eight(s + dec_wrap(y, Ly) * Lx), wd = eight(s + inc_wrap(y, Ly) * Lx);
+    const uint32_t xs = par ? (x0 + 8 == Lx ? 0u : x0 + 8) : (x0 == 0 ? Lx - 1 : x0 - 1);
+    const uint32_t edge = (uint8_t)lat_load<LD>(row + xs);
+    const uint4 r = philox4x32_10(make_uint4(g, sweep, kTagIsingMetro | (uint32_t)C, ch.chain_id), ks);
+    if (int8_oct<MEASURE>(par, w, wu, wd, edge, r, ch, anti, up)) {
+        uint16_t *h = reinterpret_cast<uint16_t *>(row + x0);
+        h[0] = (uint16_t)w.x;
+        h[1] = (uint16_t)(w.x >> 16);
+        h[2] = (uint16_t)w.y;
+        h[3] = (uint16_t)(w.y >> 16);
+    }
+}
+
+// Work units of a chain's half-sweep: Philox groups, or (PAIRS, large grid launches) runs of
+// row pairs of a group column or, rows of partial groups, inner groups and row ends; and unit u of the chain.
 template <bool PAIRS>
 __host__ __device__ __forceinline__ uint32_t int8_units(const IsingChain &ch)
 {
     if (PAIRS && (ch.Lx & 7u) == 0)
         return ch.runs * (ch.Lx >> 3);
+    if (PAIRS && ch.Lx > 8)
+        return ch.Ly * ((ch.Lx >> 3) + 1);
     return (((ch.Lx * ch.Ly) >> 1) + 3) >> 2;
 }
-template <int C, bool MEASURE, bool PAIRS = false, int LD = kLdPlain>
+template <int C, bool MEASURE, bool PAIRS = false, int LD = kLdPlain, int AHEAD = 4>
 __device__ __forceinline__ void int8_unit(int8_t *s, const IsingChain &ch, const PhiloxSchedule &ks, uint32_t u,
                                           uint32_t sweep, uint32_t &anti, uint32_t &up)
 {
-    if ((ch.Lx & 7u) == 0) {
+    if (AHEAD == 0 || (ch.Lx & 7u) == 0) { // AHEAD 0: known by the launch
         const uint32_t q = fast_div(4 * u, ch.div_half), gx = u - q * (ch.Lx >> 3); // u / (Lx / 8)
         if (PAIRS)
             int8_row_pairs<C, MEASURE, LD>(s, ch, ks, run_start(ch, q), run_start(ch, q + 1), gx, sweep, anti, up);
         else
             int8_row<C, MEASURE, LD>(s, ch, ks, q, gx, sweep, anti, up);
+    } else if (PAIRS && ch.Lx > 8) {
+        const uint32_t n = ch.Lx >> 3, half = ch.Lx >> 1;
+        if (u < ch.Ly * n) {
+            const uint32_t y = fast_div(u, ch.div_inner), g = ((y * half + 3) >> 2) + u - y * n;
+            if (4 * g + 4 <= (y + 1) * half)
+                int8_inner<C, MEASURE, LD>(s, ch, ks, y, g, sweep, anti, up);
+        } else {
+            const uint32_t end = (u - ch.Ly * n + 1) * half; // the first site of the next row
+            if (end & 3u)
+                int8_group<C, MEASURE, LD>(s, ch, ks, end >> 2, sweep, anti, up);
+        }
     } else {
-        int8_group<C, MEASURE, LD>(s, ch, ks, u, sweep, anti, up);
+        int8_group<C, MEASURE, LD, AHEAD ? AHEAD : 4>(s, ch, ks, u, sweep, anti, up);
     }
 }
 

@@ -34,6 +34,7 @@ struct IsingChain {
     uint64_t spin_off;  // byte offset of the chain's spins in the lattice region
     double beta;        // coupling (the Metropolis-Hastings step of the learned proposal needs it)
     FastDiv div_half;   // by Lx / 2: colour-linear site index -> row
+    FastDiv div_inner;  // int8, Lx no multiple of 8: by Lx / 8, the groups inside a row (Lx >= 8)
 };
 
 // Per-chain descriptor of a 4D SU(2) chain.
@@ -202,6 +203,7 @@ struct mc_ctx {
     std::vector<uint32_t> block_start, block_chain, meas_start;
     uint32_t grid_blocks = 0, meas_blocks = 0;
     bool row_runs = true;                // Ising grid mode: threads take runs of row pairs (else int8, a group each)
+    bool whole_rows = false;             // int8: every chain has rows of whole Philox groups
     // run bookkeeping
     long long sweeps_done = 0;
     long long rec_written = 0, rec_read = 0;

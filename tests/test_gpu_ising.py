@@ -358,12 +358,13 @@ def test_int8_resident_nibbles(beta, every):
 
 
 @pytest.mark.parametrize("extents", [[(2000, 1000)] * 3, [(2000, 1000), (2002, 1000), (1600, 1402)], [(8, 50000)] * 12,
-                                     [(4096, 514), (16, 8), (8, 2)]])
+                                     [(4096, 514), (16, 8), (8, 2)], [(4094, 514), (10, 4), (14, 6), (4, 4)],
+                                     [(1998, 1050)] * 2, [(12, 20002)] * 10])
 def test_int8_runs_of_row_pairs(extents):
     """Large int8 batches give a thread a run of row pairs, of two neighbouring
     lengths (columns shorter than a run, extents of partial groups beside whole
-    ones): the same spins and records as each chain by itself, where a thread
-    takes one group."""
+    ones), and take the groups at the row ends of partial ones apart: the same spins
+    and records as each chain by itself, where a thread takes one group."""
     def chains():
         return [mc.ising(e, 0.42 + 0.01 * k, seed=31, chain_id=k) for k, e in enumerate(extents)]
 
@@ -383,6 +384,30 @@ def test_int8_runs_of_row_pairs(extents):
         assert np.array_equal(one.get_config(0), cfg[k])
         assert all(np.array_equal(r[f][0], rec[f][k]) for f in ("sweep", "E", "M"))
         one.close()
+
+
+@pytest.mark.parametrize("extents", [[(4, 4), (6, 6), (10, 4), (14, 2), (62, 18), (170, 62)], [(8, 2), (16, 6), (256, 30)],
+                                     [(64, 64), (62, 62), (8, 8)], [(6, 2)], [(620, 170)]])
+def test_int8_small_grid_launches(extents):
+    """Small int8 launches have a kernel of their own where every row is whole groups, and load a
+    partial group's sites ahead of its first update (a last group of one or two sites
+    too): the same spins and records as each chain by itself held in shared memory."""
+    def chains():
+        return [mc.ising(e, 0.42 + 0.01 * k, seed=37, chain_id=k) for k, e in enumerate(extents)]
+
+    b = mc.Batch(chains(), layout=mc.MC_LAYOUT_INT8, series_capacity=8)
+    b.set_mode(mc.MC_MODE_GRID)
+    b.sweep(4, 1)
+    rec = b.read_series()
+    for k, c in enumerate(chains()):
+        one = mc.Batch([c], layout=mc.MC_LAYOUT_INT8, series_capacity=8)
+        one.set_mode(mc.MC_MODE_RESIDENT)
+        one.sweep(4, 1)
+        r = one.read_series()
+        assert np.array_equal(one.get_config(0), b.get_config(k))
+        assert all(np.array_equal(r[f][0], rec[f][k]) for f in ("sweep", "E", "M"))
+        one.close()
+    b.close()
 
 
 @pytest.mark.parametrize("shape,layout", [
