@@ -194,34 +194,6 @@ Plan make_plan(int32_t n, const mc_chain_desc *chains, int32_t layout, int64_t c
     return p;
 }
 
-// Wait for the context's stream and report a latched device fault.  The run state
-// comes back in stream order into the context's page-locked block, so that one wait
-// serves both (12 us for a kernel and its check; 19 with a second, pageable copy
-// after the wait).
-mc_status check_device(mc_ctx *c)
-{
-    cudaError_t e = cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "stream synchronize");
-    const DevState &st = *c->h_state;
-    if (st.err_code != 0) {
-        char buf[160];
-        snprintf(buf, sizeof buf, "device fault latched: code %d info %d", st.err_code, st.err_info);
-        return fail(st.err_code == kErrTimeout ? MC_ETIMEOUT : MC_EDEVICE, buf);
-    }
-    return MC_OK;
-}
-
-void destroy_graphs(mc_ctx *c)
-{
-    for (auto &kv : c->graphs)
-        cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
-    c->swept.clear();
-}
-
 // Page-locked run-state copies of the contexts, 64 to an allocation (registering a
 // page takes ~40 us); an allocation goes back when its last context is destroyed.
 struct StateSlab {
@@ -266,6 +238,39 @@ void give_host_state(DevState *p)
     }
 }
 
+// Wait for the context's stream and report a latched device fault.  The run state
+// comes back in stream order, so that one wait serves both (a kernel and its check: 15
+// us, 12 through a page-locked block; 19 with a second copy after the wait).
+mc_status check_device(mc_ctx *c)
+{
+    // a context that is asked often gets a page-locked block for the answer (it costs a lone context ~150 us)
+    if (!c->h_state && ++c->checks == 64 && take_host_state(&c->h_state) != cudaSuccess) {
+        c->h_state = nullptr;
+        cudaGetLastError();
+    }
+    DevState *const to = c->h_state ? c->h_state : &c->state_copy;
+    cudaError_t e = cudaMemcpyAsync(to, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "stream synchronize");
+    const DevState &st = c->state_copy = *to;
+    if (st.err_code != 0) {
+        char buf[160];
+        snprintf(buf, sizeof buf, "device fault latched: code %d info %d", st.err_code, st.err_info);
+        return fail(st.err_code == kErrTimeout ? MC_ETIMEOUT : MC_EDEVICE, buf);
+    }
+    return MC_OK;
+}
+
+void destroy_graphs(mc_ctx *c)
+{
+    for (auto &kv : c->graphs)
+        cudaGraphExecDestroy(kv.second);
+    c->graphs.clear();
+    c->swept.clear();
+}
+
 void free_ctx(mc_ctx *c)
 {
     destroy_graphs(c);
@@ -303,17 +308,24 @@ mc_status upload_tables(mc_ctx *c)
         ising_plan_grid(c);
     else
         su2_plan_grid(c);
-    cudaError_t e = cudaMemcpyAsync(c->d_block_start, c->block_start.data(), c->block_start.size() * 4,
-                                    cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess && c->kind == MC_KIND_ISING) // the plan is part of the chains' descriptors
-        e = cudaMemcpyAsync(c->d_chains, c->ising.data(), sizeof(IsingChain) * c->n_chains, cudaMemcpyHostToDevice, c->stream);
     c->block_chain.clear();
     if (c->n_chains > 1)
         for (int k = 0; k < c->n_chains; ++k)
             c->block_chain.insert(c->block_chain.end(), c->block_start[k + 1] - c->block_start[k], (uint32_t)k);
-    if (e == cudaSuccess && !c->block_chain.empty())
-        e = cudaMemcpyAsync(c->d_block_chain, c->block_chain.data(), c->block_chain.size() * 4, cudaMemcpyHostToDevice,
-                            c->stream);
+    // descriptors (the Ising plan is part of them), block starts and block chains follow one another in the workspace: one
+    // copy, which a new context would otherwise wait for three times
+    const char *const desc = c->kind == MC_KIND_ISING ? reinterpret_cast<const char *>(c->ising.data())
+                                                      : reinterpret_cast<const char *>(c->su2.data());
+    const size_t desc_bytes = (size_t)c->n_chains * (c->kind == MC_KIND_ISING ? sizeof(IsingChain) : sizeof(Su2Chain)),
+                 at_start = (size_t)(reinterpret_cast<char *>(c->d_block_start) - static_cast<char *>(c->d_chains)),
+                 at_chain = (size_t)(reinterpret_cast<char *>(c->d_block_chain) - static_cast<char *>(c->d_chains));
+    std::vector<char> tables(c->block_chain.empty() ? at_start + c->block_start.size() * 4
+                                                    : at_chain + c->block_chain.size() * 4);
+    memcpy(tables.data(), desc, desc_bytes);
+    memcpy(tables.data() + at_start, c->block_start.data(), c->block_start.size() * 4);
+    if (!c->block_chain.empty())
+        memcpy(tables.data() + at_chain, c->block_chain.data(), c->block_chain.size() * 4);
+    cudaError_t e = cudaMemcpyAsync(c->d_chains, tables.data(), tables.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess && !c->meas_start.empty())
         e = cudaMemcpyAsync(c->d_meas_start, c->meas_start.data(), c->meas_start.size() * 4, cudaMemcpyHostToDevice,
                             c->stream);
@@ -515,8 +527,6 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
         e = cudaEventCreateWithFlags(&c->fence_in, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&c->fence_out, cudaEventDisableTiming);
-    if (e == cudaSuccess)
-        e = take_host_state(&c->h_state);
     if (e != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(e, "create capture stream");
@@ -574,8 +584,6 @@ mc_status mc_batch_init(mc_ctx **out, int32_t n_chains, const mc_chain_desc *cha
             ch.step0 = ch.step3 * (uint32_t)ch.L[3];
             ch.bytes = ch.step0 * (uint32_t)ch.L[0];
         }
-        e = cudaMemcpyAsync(c->d_chains, c->su2.data(), sizeof(Su2Chain) * n_chains, cudaMemcpyHostToDevice,
-                            c->stream);
     }
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->d_state, 0, sizeof(DevState), c->stream);
@@ -956,7 +964,7 @@ mc_status mc_su2_failed_updates(mc_ctx *c, int64_t *count)
     mc_status s = check_device(c);
     if (s != MC_OK)
         return s;
-    *count = (int64_t)c->h_state->hb_failures;
+    *count = (int64_t)c->state_copy.hb_failures;
     return MC_OK;
 }
 

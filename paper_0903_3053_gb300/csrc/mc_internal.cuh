@@ -215,7 +215,9 @@ struct mc_ctx {
     int su2_res_cluster = 0;             // SU(2) resident mode: CTAs per chain (0 = not prepared)
     std::map<std::tuple<long long, int, int, int, bool, int>, cudaGraphExec_t> graphs;
     std::set<std::tuple<long long, int, int, int, bool, int>> swept; // launched once, not recorded yet
-    mc::DevState *h_state = nullptr;     // page-locked copy of the run state (check_device)
+    mc::DevState state_copy{};           // the run state as of the last check_device
+    mc::DevState *h_state = nullptr;     // page-locked block it comes back through, once there have been many
+    int checks = 0;
     // kernel timing (mc_profile_enable)
     bool profiling = false;
     std::vector<cudaEvent_t> events; // pairs: [2i] before, [2i+1] after launch i
