@@ -119,11 +119,18 @@ __device__ __forceinline__ T lat_load(const T *p)
 // start likewise, so that at most one kernel is ever waiting: let off from the
 // first instruction, kernels piled up several deep and displaced the running one's
 // blocks (3.1 -> 7.3 us per half-sweep of a 2048^2 chain).
+//
+// A kernel that uses tensor memory releases its successor only after its own allocation,
+// and a barrier of the block behind it.  The successor's blocks allocate before they wait, and hold
+// what they have until they end: let in earlier, two of them can take all 512 columns of an SM
+// on which a block of the running kernel has yet to allocate, and each side waits for the other
+// for ever (tcgen05.alloc has no limit).
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait(bool release)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (release)
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        chain_release();
 }
 
 // Chain of a block of a grid-mode launch: one load (a binary search over the

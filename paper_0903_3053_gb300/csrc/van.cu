@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    chain_wait(true);
+    chain_wait(false); // the next kernel's blocks come in only after this block's tensor memory is allocated (below)
     if (tid < kCh)
         Bias[tid] = b1[tid];
     if (tid < 2 * kCh) { // w1 is [o][t]
@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(kL1Threads, 8) k_layer1_tc(const int8_t *__res
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    chain_release();
     const uint32_t tbase = *reinterpret_cast<volatile uint32_t *>(&tslot);
     const uint64_t adesc = tc::smem_desc(smem_u32(&A[0][0]), kL1Threads * 16, 128);
     const uint64_t bdesc = tc::smem_desc(smem_u32(&B[0][0]), kCh * 16, 128);
