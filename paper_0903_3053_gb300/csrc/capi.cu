@@ -346,6 +346,7 @@ cudaError_t sweep_enqueue(mc_ctx *c, long long n, int every, int mode)
 
 cudaError_t enqueue_chunk(mc_ctx *c, long long n, int every, int mode)
 {
+    c->in_chunk = false;
     const cudaError_t e = sweep_enqueue(c, n, every, mode);
     return e != cudaSuccess ? e : advance_state_launch(c, n, every > 0 ? n / every : 0);
 }

@@ -51,7 +51,7 @@ __device__ __forceinline__ void half_sweep(const SweepArgs &a)
     const uint32_t sweep = (uint32_t)(a.state->sweep_base + a.k);
     const bool measure = (C == 1) && a.measure;
     uint32_t anti = 0, up = 0;
-    chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between calls)
+    chain_wait(a.release != 0); // the other colour's half-sweep is done (the run state changes only between chunks)
     if (LAYOUT == MC_LAYOUT_INT8) {
         int8_t *s = reinterpret_cast<int8_t *>(a.lattice + ch.spin_off);
         if (t < int8_units<FORM == kRuns>(ch)) {

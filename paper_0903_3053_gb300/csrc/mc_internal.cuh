@@ -120,6 +120,9 @@ __device__ __forceinline__ T lat_load(const T *p)
 // first instruction, kernels piled up several deep and displaced the running one's
 // blocks (3.1 -> 7.3 us per half-sweep of a 2048^2 chain).
 //
+// The sweep counter is read before the wait.  k_advance writes it at the end of each chunk of a
+// call, so the first kernel of a chunk is launched plainly (launch_chained).
+//
 // A kernel that uses tensor memory releases its successor only after its own allocation,
 // and a barrier of the block behind it.  The successor's blocks allocate before they wait, and hold
 // what they have until they end: let in earlier, two of them can take all 512 columns of an SM
@@ -222,6 +225,7 @@ struct mc_ctx {
     int su2_res_cluster = 0;             // SU(2) resident mode: CTAs per chain (0 = not prepared)
     std::map<std::tuple<long long, int, int, int, bool, int>, cudaGraphExec_t> graphs;
     std::set<std::tuple<long long, int, int, int, bool, int>> swept; // launched once, not recorded yet
+    bool in_chunk = false;               // a sweep kernel of the chunk being enqueued has been launched
     mc::DevState state_copy{};           // the run state as of the last check_device
     mc::DevState *h_state = nullptr;     // page-locked block it comes back through, once there have been many
     int checks = 0;
@@ -281,11 +285,14 @@ cudaError_t launch_chained_on(cudaStream_t stream, bool chained, void (*kernel)(
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Launch one sweep kernel on the context's launch stream, chained unless profiling events separate the launches.
+// Launch one sweep kernel on the context's launch stream, chained to the sweep kernel before it: not the
+// first of a chunk, which reads what k_advance wrote before it waits, nor between profiling events.
 template <typename... P, typename... A>
-cudaError_t launch_chained(const mc_ctx *c, void (*kernel)(P...), unsigned blocks, unsigned threads, const A &...args)
+cudaError_t launch_chained(mc_ctx *c, void (*kernel)(P...), unsigned blocks, unsigned threads, const A &...args)
 {
-    return launch_chained_on(c->ls, !c->profiling, kernel, blocks, threads, 0, args...);
+    const bool chained = c->in_chunk && !c->profiling;
+    c->in_chunk = true;
+    return launch_chained_on(c->ls, chained, kernel, blocks, threads, 0, args...);
 }
 
 // Bracket one sweep-kernel launch with events when the context is profiling.
