@@ -121,8 +121,9 @@ MC_API mc_status mc_su2_init(mc_ctx **out, const int32_t L[4], double beta, uint
  * record is appended after the k-th sweep of this call (k = 1..n_sweeps) for
  * every k divisible by measure_every (the measuring kernels of Sec. 2.3/2.4);
  * MC_EINVAL if that would overrun the unread part of the ring buffer.
- * Repeated calls with the same (n_sweeps, measure_every) replay one captured
- * CUDA graph. */
+ * From the second call with the same (n_sweeps, measure_every) on, a recorded
+ * CUDA graph is replayed.  The library records its own: on a stream that is being
+ * captured, sweeps (mc_group_sweep alike) are refused with MC_ECUDA. */
 MC_API mc_status mc_sweep(mc_ctx *ctx, int64_t n_sweeps, int32_t measure_every);
 
 /* Execution mode for later sweeps: MC_MODE_GRID (one launch per half-sweep /

@@ -583,6 +583,8 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
         if (c->sweeps_done + n_sweeps > 0xFFFFFFFFll)
             return gfail(MC_EINVAL, "sweep counter would exceed 2^32");
     }
+    if (refuse_capture(g->stream))
+        return MC_ECUDA;
     bool or_changed = false; // a member context changed its overrelaxation count since the last call
     for (size_t i = 0; i < g->members.size(); ++i)
         if (g->hm[i].n_or != g->members[i]->n_or) {

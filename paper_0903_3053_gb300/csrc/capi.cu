@@ -351,17 +351,6 @@ cudaError_t enqueue_chunk(mc_ctx *c, long long n, int every, int mode)
     return e != cudaSuccess ? e : advance_state_launch(c, n, every > 0 ? n / every : 0);
 }
 
-// Whether work issued on `s` is being captured into a graph of the caller's.
-bool capturing(cudaStream_t s)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return st != cudaStreamCaptureStatusNone;
-}
-
 // `n` sweeps and the advance of the run state on the context's private stream
 // (capture is not permitted on the legacy default stream a caller may pass):
 // launched one by one the first time a (n, every, mode, ...) is asked for, captured
@@ -375,7 +364,7 @@ mc_status launch_chunk(mc_ctx *c, long long n, int every, int mode)
     const auto key = std::make_tuple(n, every, mode, c->threads, c->record_tries, c->n_or);
     auto it = c->graphs.find(key);
     cudaError_t e = cudaSuccess;
-    if (it == c->graphs.end() && c->swept.count(key) && !capturing(c->cap_stream)) {
+    if (it == c->graphs.end() && c->swept.count(key)) {
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess)
@@ -428,6 +417,19 @@ static cudaError_t prof_record(mc_ctx *c)
 void set_last_error(const std::string &msg) { g_err = msg; }
 cudaError_t prof_begin(mc_ctx *c) { return c->profiling ? prof_record(c) : cudaSuccess; }
 cudaError_t prof_end(mc_ctx *c) { return c->profiling ? prof_record(c) : cudaSuccess; }
+
+bool refuse_capture(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (st == cudaStreamCaptureStatusNone)
+        return false;
+    g_err = "sweeps cannot be captured into a graph: the host counts them when they are asked for";
+    return true;
+}
 
 mc_status sweep_begin(mc_ctx *c, long long n, int every)
 {
@@ -680,6 +682,8 @@ mc_status mc_sweep(mc_ctx *c, int64_t n_sweeps, int32_t measure_every)
         return fail(MC_EINVAL, "measurement ring buffer would overflow: read the series first or raise capacity");
     if (c->sweeps_done + n_sweeps > 0xFFFFFFFFll)
         return fail(MC_EINVAL, "sweep counter would exceed 2^32 (the Philox sweep word)");
+    if (!c->profiling && refuse_capture(c->stream))
+        return MC_ECUDA;
     const mc_status s = sweep_begin(c, n_sweeps, measure_every);
     const mc_status f = sweep_end(c);
     if (s != MC_OK || f != MC_OK)

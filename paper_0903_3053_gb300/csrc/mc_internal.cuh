@@ -264,6 +264,11 @@ cudaError_t advance_state_launch(mc_ctx *c, long long n, long long recs);
 mc_status sweep_begin(mc_ctx *c, long long n, int every);
 mc_status sweep_end(mc_ctx *c);
 
+// Whether `s` is being captured into a graph of the caller's (with the error message set).  A captured sweep would be
+// counted on the host once and run once per launch of the graph, so the sweep counter and the records kept
+// would no longer be the device's.
+bool refuse_capture(cudaStream_t s);
+
 // Message returned by mc_last_error() on this thread.
 void set_last_error(const std::string &msg);
 

@@ -38,3 +38,28 @@ result = launches()
     for r in runs:
         assert r[0] == "plain"
         assert set(r[1:]) == {"programmatic"}
+
+
+@pytest.mark.parametrize("call", ["lib.mc_sweep(b, 4, 1)", "lib.mc_group_sweep(g, 4, 1)", "lib.mc_group_sweep(p, 4, 1)"])
+def test_sweeps_are_refused_on_a_capturing_stream(call):
+    """Before a graph of theirs is recorded as well as after: nothing is launched or counted."""
+    result = run(f"""
+st = stream()
+b = batch([mc.ising((64, 64), 0.44, 1)], st=st)
+g, p = group([b], st), group([b], st)
+assert lib.mc_group_configure(p, 4, 256, 0.0) == 0
+out = []
+for warm in range(3):
+    launches()
+    before = swept(b)
+    assert fake.cudaStreamBeginCapture(st, 1) == 0
+    status = {call}
+    h = ctypes.c_void_p()
+    fake.cudaStreamEndCapture(st, ctypes.byref(h))
+    out.append([status, lib.mc_last_error().decode(), swept(b) - before, launches()])
+    assert {call} == 0
+result = [mc.MC_ECUDA, out]
+""")
+    for status, message, counted, log in result[1]:
+        assert status == result[0] and "captured" in message
+        assert counted == 0 and log == []
