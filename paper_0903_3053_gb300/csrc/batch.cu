@@ -613,6 +613,8 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
         size_t begun = 0;
         std::vector<mc_ctx *> order(g->members);
         std::stable_partition(order.begin(), order.end(), [](const mc_ctx *c) { return c->kind == MC_KIND_SU2; });
+        for (size_t i = 0; i < order.size() && st == MC_OK; ++i)
+            st = sweep_prepare(order[i]);
         for (; begun < order.size() && st == MC_OK; ++begun)
             st = sweep_begin(order[begun], n_sweeps, measure_every);
         for (size_t i = 0; i < begun; ++i) {
@@ -620,13 +622,7 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
             if (st == MC_OK)
                 st = f;
         }
-        if (st != MC_OK)
-            return st;
-        for (mc_ctx *c : g->members) {
-            c->sweeps_done += n_sweeps;
-            c->rec_written += recs;
-        }
-        return MC_OK;
+        return st;
     }
     const auto key = std::make_tuple((long long)n_sweeps, (int)measure_every);
     auto it = g->graphs.find(key);

@@ -431,14 +431,18 @@ bool refuse_capture(cudaStream_t s)
     return true;
 }
 
+mc_status sweep_prepare(mc_ctx *c)
+{
+    if (resolve_mode(c) != MC_MODE_RESIDENT)
+        return MC_OK;
+    const cudaError_t e = c->kind == MC_KIND_ISING ? ising_prepare_resident(c) : su2_prepare_resident(c);
+    return e == cudaSuccess ? MC_OK : cuda_fail(e, "configure resident kernel");
+}
+
 mc_status sweep_begin(mc_ctx *c, long long n, int every)
 {
     const int mode = resolve_mode(c);
     cudaError_t e = cudaSuccess;
-    if (mode == MC_MODE_RESIDENT)
-        e = c->kind == MC_KIND_ISING ? ising_prepare_resident(c) : su2_prepare_resident(c);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "configure resident kernel");
     if (!c->profiling) {
         e = cudaEventRecord(c->fence_in, c->stream);
         if (e == cudaSuccess)
@@ -459,6 +463,10 @@ mc_status sweep_begin(mc_ctx *c, long long n, int every)
             s = e == cudaSuccess ? MC_OK : cuda_fail(e, "enqueue sweep kernels");
         } else {
             s = launch_chunk(c, m, every, mode);
+        }
+        if (s == MC_OK) { // what has been launched counts, whatever becomes of the rest
+            c->sweeps_done += m;
+            c->rec_written += every > 0 ? m / every : 0;
         }
         left -= m;
     }
@@ -684,13 +692,12 @@ mc_status mc_sweep(mc_ctx *c, int64_t n_sweeps, int32_t measure_every)
         return fail(MC_EINVAL, "sweep counter would exceed 2^32 (the Philox sweep word)");
     if (!c->profiling && refuse_capture(c->stream))
         return MC_ECUDA;
-    const mc_status s = sweep_begin(c, n_sweeps, measure_every);
+    mc_status s = sweep_prepare(c);
+    if (s != MC_OK)
+        return s;
+    s = sweep_begin(c, n_sweeps, measure_every);
     const mc_status f = sweep_end(c);
-    if (s != MC_OK || f != MC_OK)
-        return s != MC_OK ? s : f;
-    c->sweeps_done += n_sweeps;
-    c->rec_written += recs;
-    return MC_OK;
+    return s != MC_OK ? s : f;
 }
 
 mc_status mc_sync(mc_ctx *c)

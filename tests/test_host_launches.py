@@ -63,3 +63,27 @@ result = [mc.MC_ECUDA, out]
     for status, message, counted, log in result[1]:
         assert status == result[0] and "captured" in message
         assert counted == 0 and log == []
+
+
+def test_host_counters_follow_what_was_launched():
+    """A launch that fails in a later chunk, or in a later member of a group: the sweeps launched before are counted (the
+    device's counter has advanced by them), those of the failed chunk are not, and nothing follows them."""
+    result = run("""
+b = batch([mc.ising((64, 64), 0.44, 1)])
+lib.mc_set_mode(b, 1, 0)
+fake.fake_fail_launch(2 * 256 + 1 + 5)        # within the second chunk
+one = [lib.mc_sweep(b, 300, 1), swept(b)]
+two = batch([mc.ising((64, 64), 0.44, 1)]), batch([mc.ising((128, 64), 0.44, 1)])
+for c in two:
+    lib.mc_set_mode(c, 1, 0)
+g = group(two)
+launches()
+fake.fake_fail_launch(2 * 4 + 1 + 2)          # within the second member
+st = lib.mc_group_sweep(g, 4, 1)
+advanced = sum("k_advance" in e[0] for e in launches())
+rec = (mc.mc_record * 4)()
+n = ctypes.c_int64()
+assert lib.mc_read_series(two[0], rec, 4, ctypes.byref(n)) == 0
+result = [one, [st, swept(two[0]), swept(two[1]), advanced, n.value]]
+""")
+    assert result == [[-3, 256], [-3, 4, 0, 1, 4]]
