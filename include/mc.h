@@ -238,9 +238,9 @@ MC_API mc_status mc_philox_rate(int32_t blocks, int32_t threads, uint32_t iters,
 /* ---- Batched chains advanced together ----------------------------------------
  * A group advances every chain of up to 16 contexts (any mix of Ising layouts
  * and SU(2)) in one call -- the paper runs independent parameter points side by
- * side (Sec. 3); here they share one GPU.  By default (split_cost < 0) the
- * members' own launches run side by side, each member in its own mode.  With
- * split_cost >= 0 all chains run in ONE persistent kernel launch per call,
+ * side (Sec. 3); here they share one GPU.  By default (MC_GROUP_SIDE_BY_SIDE)
+ * the members' own launches run side by side, each member in its own mode.  With
+ * split_cost >= 0 or MC_GROUP_FAIR_SHARE all chains run in ONE persistent kernel launch per call,
  * replayed from a CUDA graph: the grid is a set of thread-block clusters; a
  * host-computed longest-first schedule gives each cluster a list of rounds,
  * each either one large chain split over the cluster's CTAs (phases separated
@@ -250,25 +250,28 @@ MC_API mc_status mc_philox_rate(int32_t blocks, int32_t threads, uint32_t iters,
  * Member contexts must have been created on the group's stream and stay alive
  * until mc_group_destroy; records go to each member's own ring buffer. */
 typedef struct mc_group mc_group; /* opaque, owned by the library */
+#define MC_GROUP_SIDE_BY_SIDE (-1.0) /* split_cost: the members' own launches */
+#define MC_GROUP_FAIR_SHARE (-2.0)   /* split_cost: persistent launch, one CTA's fair share of the total cost */
 
 /* Device workspace the group needs for its schedule and scratch (0 = error). */
 MC_API size_t mc_group_workspace_bytes(int32_t n_ctx, mc_ctx *const *ctxs);
 MC_API mc_status mc_group_create(mc_group **out, int32_t n_ctx, mc_ctx *const *ctxs, void *workspace,
                                  size_t workspace_bytes, void *cuda_stream);
 /* cluster_size in {1, 2, 4, 8, 16} (0 = keep; default 4; 16 is a non-portable
- * cluster size: a device that cannot co-schedule it fails the next
+ * cluster size: a device that cannot co-schedule it fails the next persistent
  * mc_group_sweep with MC_ECUDA); threads_per_block a
  * multiple of 32 in [64, 256] (0 = keep; default 256); a chain whose estimated
  * cost (MSC spin-flip units per sweep: Ising int8 2 per site, MSC 1 per site,
  * SU(2) 60 per link) is at least split_cost is shared by a whole cluster.
- * split_cost < 0 (the default): the members' own launches side by side; the
- * schedule is then the persistent launch's with one CTA's fair share of the
- * total as the cost that is shared.  Invalidates the schedule; the next
- * mc_group_sweep recomputes it. */
+ * MC_GROUP_FAIR_SHARE (and anything below it) takes one CTA's fair share of the
+ * total as that cost.  MC_GROUP_SIDE_BY_SIDE (the default, and any other negative
+ * value): the members' own launches, to which the sizes do not apply.
+ * Invalidates the schedule. */
 MC_API mc_status mc_group_configure(mc_group *g, int32_t cluster_size, int32_t threads_per_block, double split_cost);
 /* Advance every member chain by n_sweeps (async), recording as mc_sweep does. */
 MC_API mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every);
-/* Clusters in the launch and rounds in the schedule (0 before the first sweep). */
+/* Clusters in the persistent launch and rounds in its schedule (0 before the first
+ * sweep since the configuration; side by side, what MC_GROUP_FAIR_SHARE would take). */
 MC_API mc_status mc_group_schedule(const mc_group *g, int32_t *n_clusters, int32_t *n_rounds);
 MC_API mc_status mc_group_destroy(mc_group *g);
 

@@ -1,13 +1,14 @@
 // batch.cu -- many uneven chains (Ising in either layout, SU(2)) advanced
 // together.
 //
-// A group borrows the chains of several contexts.  By default the members' own
-// launches run side by side on the members' private streams.  us per measured
+// A group borrows the chains of several contexts.  By default (MC_GROUP_SIDE_BY_SIDE)
+// the members' own launches run side by side on the members' private streams.  us per measured
 // sweep against the persistent launch below (clusters of 8, 256 threads): 256 Ising +
 // 64 SU(2) chains 322 against 364 (the SU(2) phases alone take 280), 64 + 16 58
 // against 237, 8 + 2 21 against 83, 256 + 2 64 against 100, 8 + 64 193 against 292 -- the
 // persistent kernel holds 16 warps per SM, and its phases wait at cluster barriers
-// where chained launches overlap.  A split cost >= 0 (mc_group_configure) asks for
+// where chained launches overlap.  A split cost >= 0, or MC_GROUP_FAIR_SHARE for one CTA's share
+// of the total, (mc_group_configure) asks for
 // ONE persistent kernel launch per call, captured in a CUDA graph: the host computes a
 // schedule once (longest-processing-time first): the grid is a set of
 // thread-block clusters of C CTAs, and each cluster walks a list of rounds.  A
@@ -279,12 +280,15 @@ struct mc_group {
     size_t max_rounds = 0, max_clusters = 0;
     // configuration and schedule
     int C = 4, threads = 256;
-    double split_cost = -1.0; // >= 0: persistent launch, items at least this costly shared by a cluster
+    // MC_GROUP_SIDE_BY_SIDE, or the persistent launch: items at least this costly shared by a cluster
+    // (MC_GROUP_FAIR_SHARE and below: one CTA's share of the total)
+    double split_cost = MC_GROUP_SIDE_BY_SIDE;
+    bool persistent() const { return !(split_cost < 0.0 && split_cost > MC_GROUP_FAIR_SHARE); }
     int n_clusters = 0;
     std::vector<uint32_t> round_start;
     std::vector<int32_t> rounds;
     std::vector<uint8_t> round_shared;
-    bool planned = false;
+    bool swept = false, planned = false, uploaded = false; // since the last configuration
     std::vector<GroupMember> hm; // host copy of d_members
     std::map<std::tuple<long long, int>, cudaGraphExec_t> graphs;
 };
@@ -340,7 +344,7 @@ void destroy_group_graphs(mc_group *g)
     g->graphs.clear();
 }
 
-// Longest-processing-time schedule of the items over n_clusters clusters of C CTAs.
+// Longest-processing-time schedule of the items over n_clusters clusters of C CTAs (host only).
 mc_status plan(mc_group *g)
 {
     int dev = 0, sms = 0;
@@ -415,8 +419,18 @@ mc_status plan(mc_group *g)
     g->round_start[NC] = (uint32_t)g->round_shared.size();
     if (g->round_shared.size() > g->max_rounds)
         return gfail(MC_ENOMEM, "group schedule exceeds its workspace");
-    e = cudaMemcpyAsync(g->d_round_start, g->round_start.data(), g->round_start.size() * 4, cudaMemcpyHostToDevice,
-                        g->stream);
+    g->planned = true;
+    return MC_OK;
+}
+
+// The schedule and the members to the device, for the persistent launch.
+mc_status upload(mc_group *g)
+{
+    cudaError_t e = cudaMemcpyAsync(g->d_members, g->hm.data(), g->hm.size() * sizeof(GroupMember), cudaMemcpyHostToDevice,
+                                    g->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(g->d_round_start, g->round_start.data(), g->round_start.size() * 4, cudaMemcpyHostToDevice,
+                            g->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(g->d_rounds, g->rounds.data(), g->rounds.size() * 4, cudaMemcpyHostToDevice, g->stream);
     if (e == cudaSuccess)
@@ -426,7 +440,7 @@ mc_status plan(mc_group *g)
         e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess)
         return gfail(MC_ECUDA, std::string("upload group schedule: ") + cudaGetErrorString(e));
-    g->planned = true;
+    g->uploaded = true;
     destroy_group_graphs(g);
     return MC_OK;
 }
@@ -536,8 +550,6 @@ mc_status mc_group_create(mc_group **out, int32_t n_ctx, mc_ctx *const *ctxs, vo
         e = cudaFuncSetAttribute(k_group, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     g->hm = hm;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(g->d_members, g->hm.data(), hm.size() * sizeof(GroupMember), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
         e = cudaMemcpyAsync(g->d_items, g->items.data(), g->items.size() * sizeof(int2), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(st);
@@ -563,7 +575,7 @@ mc_status mc_group_configure(mc_group *g, int32_t cluster_size, int32_t threads_
     if (threads_per_block)
         g->threads = threads_per_block;
     g->split_cost = split_cost;
-    g->planned = false;
+    g->swept = g->planned = g->uploaded = false;
     destroy_group_graphs(g);
     return MC_OK;
 }
@@ -585,29 +597,8 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
     }
     if (refuse_capture(g->stream))
         return MC_ECUDA;
-    bool or_changed = false; // a member context changed its overrelaxation count since the last call
-    for (size_t i = 0; i < g->members.size(); ++i)
-        if (g->hm[i].n_or != g->members[i]->n_or) {
-            g->hm[i].n_or = g->members[i]->n_or;
-            or_changed = true;
-        }
-    if (or_changed) {
-        cudaError_t e = cudaMemcpyAsync(g->d_members, g->hm.data(), g->hm.size() * sizeof(GroupMember),
-                                        cudaMemcpyHostToDevice, g->stream);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(g->stream);
-        if (e != cudaSuccess)
-            return gfail(MC_ECUDA, std::string("update group members: ") + cudaGetErrorString(e));
-        g->planned = false;
-        destroy_group_graphs(g);
-    }
-    if (!g->planned) {
-        mc_status s = plan(g);
-        if (s != MC_OK)
-            return s;
-    }
-    if (g->split_cost < 0.0) {
-        // Automatic: the members' own launches, side by side.  The SU(2) members, whose
+    if (!g->persistent()) {
+        // The members' own launches, side by side.  The SU(2) members, whose
         // chains of launches are the longest, first.
         mc_status st = MC_OK;
         size_t begun = 0;
@@ -622,7 +613,23 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
             if (st == MC_OK)
                 st = f;
         }
+        g->swept = g->swept || st == MC_OK;
         return st;
+    }
+    for (size_t i = 0; i < g->members.size(); ++i)
+        if (g->hm[i].n_or != g->members[i]->n_or) { // changed since the last call
+            g->hm[i].n_or = g->members[i]->n_or;
+            g->uploaded = false;
+        }
+    if (!g->planned) {
+        const mc_status s = plan(g);
+        if (s != MC_OK)
+            return s;
+    }
+    if (!g->uploaded) {
+        const mc_status s = upload(g);
+        if (s != MC_OK)
+            return s;
     }
     const auto key = std::make_tuple((long long)n_sweeps, (int)measure_every);
     auto it = g->graphs.find(key);
@@ -656,6 +663,7 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
         e = cudaStreamWaitEvent(g->stream, g->fence_out, 0);
     if (e != cudaSuccess)
         return gfail(MC_ECUDA, std::string("group graph launch: ") + cudaGetErrorString(e));
+    g->swept = true;
     for (mc_ctx *c : g->members) {
         c->sweeps_done += n_sweeps;
         c->rec_written += recs;
@@ -667,8 +675,16 @@ mc_status mc_group_schedule(const mc_group *g, int32_t *n_clusters, int32_t *n_r
 {
     if (!g || !n_clusters || !n_rounds)
         return gfail(MC_EINVAL, "NULL argument");
-    *n_clusters = g->planned ? g->n_clusters : 0;
-    *n_rounds = g->planned ? (int32_t)g->round_shared.size() : 0;
+    *n_clusters = *n_rounds = 0;
+    if (!g->swept)
+        return MC_OK;
+    if (!g->planned) { // side by side: the persistent launch's schedule, made when it is asked for
+        const mc_status s = plan(const_cast<mc_group *>(g));
+        if (s != MC_OK)
+            return s;
+    }
+    *n_clusters = g->n_clusters;
+    *n_rounds = (int32_t)g->round_shared.size();
     return MC_OK;
 }
 

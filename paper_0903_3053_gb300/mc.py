@@ -21,6 +21,7 @@ MC_KIND_ISING, MC_KIND_SU2 = 1, 2
 MC_LAYOUT_INT8, MC_LAYOUT_MSC32 = 0, 1
 MC_FMT_INT8, MC_FMT_BITS, MC_FMT_F32, MC_FMT_NATIVE = 0, 1, 2, 3
 MC_MODE_AUTO, MC_MODE_GRID, MC_MODE_RESIDENT = 0, 1, 2
+MC_GROUP_SIDE_BY_SIDE, MC_GROUP_FAIR_SHARE = -1.0, -2.0  # split_cost of Group.configure
 
 #: every symbol include/mc.h declares (checked by the ABI test)
 EXPORTS = [
@@ -396,7 +397,8 @@ class Batch:
 
 class Group:
     """Chains of several Batches advanced together: the batches' own launches side
-    by side, or (configure with split_cost >= 0) one persistent launch per call."""
+    by side, or one persistent launch per call (configure with the cost from which a
+    chain is shared by a cluster as split_cost, or MC_GROUP_FAIR_SHARE)."""
 
     def __init__(self, batches):
         torch = _torch()
@@ -417,7 +419,7 @@ class Group:
                                  ctypes.c_void_p(self.workspace.data_ptr()), nbytes,
                                  ctypes.c_void_p(self.stream.cuda_stream)))
 
-    def configure(self, cluster_size: int = 0, threads_per_block: int = 0, split_cost: float = -1.0):
+    def configure(self, cluster_size: int = 0, threads_per_block: int = 0, split_cost: float = MC_GROUP_SIDE_BY_SIDE):
         _check(load().mc_group_configure(self._g, int(cluster_size), int(threads_per_block), float(split_cost)))
 
     def sweep(self, n: int, measure_every: int = 0):

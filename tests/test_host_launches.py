@@ -87,3 +87,50 @@ assert lib.mc_read_series(two[0], rec, 4, ctypes.byref(n)) == 0
 result = [one, [st, swept(two[0]), swept(two[1]), advanced, n.value]]
 """)
     assert result == [[-3, 256], [-3, 4, 0, 1, 4]]
+
+
+def test_group_launches_what_its_split_cost_asks_for():
+    """MC_GROUP_SIDE_BY_SIDE: the members' own kernels, and nothing of the persistent launch (no schedule, so that a cluster
+    size the device cannot place does not matter).  MC_GROUP_FAIR_SHARE, anything below it and costs >= 0: one
+    persistent kernel a call, also after a member's overrelaxation count has changed."""
+    result = run("""
+a = batch([mc.ising((64, 64), 0.44, 1)])
+b = batch([mc.su2((4, 4, 4, 4), 2.3, 1)])
+g = group([a, b])
+nc, nr = ctypes.c_int32(), ctypes.c_int32()
+
+def schedule():
+    st = lib.mc_group_schedule(g, ctypes.byref(nc), ctypes.byref(nr))
+    return [st, nc.value > 0, nr.value > 0]
+
+def call(split, n=1):
+    out = []
+    for _ in range(n):
+        launches()
+        st = lib.mc_group_sweep(g, 2, 1)
+        names = {e[0] for e in launches()} - {"wait", "graph", "end"}
+        out.append([st, any("7k_groupE" in s for s in names), any("k_phase" in s for s in names)])
+    return out
+
+result = {}
+for split in (-1.0, -0.5, mc.MC_GROUP_FAIR_SHARE, -9.0, 0.0, 1e300):
+    assert lib.mc_group_configure(g, 4, 256, split) == 0
+    before = schedule()
+    result[str(split)] = [before, call(split, 2), schedule()]
+assert lib.mc_group_configure(g, 4, 256, mc.MC_GROUP_FAIR_SHARE) == 0
+assert lib.mc_su2_set_overrelax(b, 2) == 0
+result["overrelax"] = call(-2.0, 2)
+fake.fake_set_clusters(0)
+result["no cluster"] = []
+for split in (-1.0, -2.0):
+    assert lib.mc_group_configure(g, 16, 256, split) == 0
+    result["no cluster"].append(call(split))
+""")
+    ok = [0, True, True]
+    for split in ("-1.0", "-0.5"):
+        assert result[split] == [[0, False, False], [[0, False, True]] * 2, ok]
+    for split in ("-2.0", "-9.0", "0.0", "1e+300"):
+        assert result[split] == [[0, False, False], [[0, True, False]] * 2, ok]
+    assert result["overrelax"] == [[0, True, False]] * 2
+    assert result["no cluster"][0] == [[0, False, True]]
+    assert result["no cluster"][1][0][0] == -3
