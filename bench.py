@@ -561,7 +561,8 @@ def run_batched(mc, torch, rank, K, world, sweeps_per_call=10):
     torch.cuda.synchronize()
     barrier(world)
     ms = max_over_ranks(t0.elapsed_time(t1), world)
-    nc, nr = g.schedule()
+    persistent = choice["split"] != mc.MC_GROUP_SIDE_BY_SIDE
+    nc, nr = g.schedule() if persistent else (None, None)
     for b in bs:
         b.read_series()
     g.close()
@@ -571,7 +572,7 @@ def run_batched(mc, torch, rank, K, world, sweeps_per_call=10):
             "unit": "site+link updates/s",
             "workload": "256 Ising chains L in {32..1024}, beta ~ U[0.35, 0.55] + 64 SU(2) chains L^4, "
                         "L in {4, 6, 8, 12, 16}, beta ~ U[1.8, 2.6] (numpy default_rng(0)); E/M and plaquette "
-                        "every sweep", "persistent": choice["split"] >= 0, "sweeps_per_call": sweeps_per_call,
+                        "every sweep", "persistent": persistent, "sweeps_per_call": sweeps_per_call,
             "ms_per_sweep": ms / sweeps, "clusters": nc, "rounds": nr,
             "autotuned": {k: choice[k] for k in ("cluster", "threads", "split", "cached")}}
 

@@ -65,18 +65,22 @@ def _time(fn, reps: int) -> float:
 
 
 def group_candidates():
+    """(cluster size, threads, split cost): the members' own launches once (the sizes do not apply to them), then the
+    persistent launch with chains above a CTA's fair share, or every chain, shared by a cluster."""
+    yield 8, 256, mc.MC_GROUP_SIDE_BY_SIDE
     for C in (1, 2, 4, 8, 16):
         for threads in (128, 256):
-            for split in (-1.0, 0.0):
+            for split in (mc.MC_GROUP_FAIR_SHARE, 0.0):
                 if C == 1 and split == 0.0:
-                    continue
+                    continue  # nothing to share
                 yield C, threads, split
 
 
 def tune_group(group: "mc.Group", n_sweeps: int = 4, reps: int = 3, use_cache: bool = True, verbose=False) -> dict:
     """Pick (cluster size, threads, split cost) for a group; returns the choice
-    with its time per sweep.  The group is left configured with it."""
-    key = f"group|{_gpu_name()}|{_signature(group.batches)}|{n_sweeps}"
+    with its time per sweep.  The group is left configured with it.  (Entries of
+    "group|" keys are of a time when a split cost of -1 meant a persistent launch.)"""
+    key = f"group2|{_gpu_name()}|{_signature(group.batches)}|{n_sweeps}"
     cache = _load_cache() if use_cache else {}
     if key in cache:
         c = cache[key]
@@ -94,7 +98,7 @@ def tune_group(group: "mc.Group", n_sweeps: int = 4, reps: int = 3, use_cache: b
         results.append((ms, C, threads, split))
         if verbose:
             print(f"  cluster {C} threads {threads} split {split}: {ms:.3f} ms/sweep", flush=True)
-    ms, C, threads, split = min(results)
+    ms, C, threads, split = min(results, key=lambda r: r[0])
     group.configure(C, threads, split)
     choice = {"cluster": C, "threads": threads, "split": split, "ms_per_sweep": ms,
               "tried": [list(r) for r in results], "when": time.strftime("%Y-%m-%dT%H:%M:%S")}
