@@ -134,3 +134,21 @@ for split in (-1.0, -2.0):
     assert result["overrelax"] == [[0, True, False]] * 2
     assert result["no cluster"][0] == [[0, False, True]]
     assert result["no cluster"][1][0][0] == -3
+
+
+@pytest.mark.parametrize("L,depth,pipe", [(8, 3, True), (8, 6, True), (10, 5, True), (6, 6, False), (2, 3, False), (8, 7, False)])
+def test_sampler_rule(L, depth, pipe):
+    """k_sample_pipe from L = 8 and for up to four hidden layers where it has exactly the registers its split is written
+    for (a split of more than the launch's registers would wait for ever); else k_sample."""
+    result = run(f"""
+result = []
+for regs in (128, 126):
+    fake.fake_set_regs(regs)
+    st, w = van({L}, 32, {depth})
+    assert st == 0
+    launches()
+    assert lib.mc_van_sample(w, 32, 0, None, None, None) == 0
+    result.append([e[0] for e in launches() if "k_sample" in e[0]])
+""")
+    assert [len(r) for r in result] == [1, 1]
+    assert ["k_sample_pipe" in r[0] for r in result] == [pipe, False]
