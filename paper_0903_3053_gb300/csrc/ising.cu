@@ -19,8 +19,8 @@
 // (integer thresholds, no floating point on the path).
 //
 // Execution modes:
-//   grid     : one launch per colour over every chain of the batch; chain of a
-//              block found by binary search over per-chain block offsets.
+//   grid     : one launch per colour over every chain of the batch; the chain of
+//              a block is looked up in a table with an entry per block.
 //   resident : one CTA per chain holding its whole lattice in shared memory and
 //              running all sweeps of a call in one launch (small lattices).
 // The energy/magnetisation measurement (the paper's sweep+measure kernels) is

@@ -37,10 +37,10 @@ namespace {
 
 // Chain descriptors of small batches as kernel parameters: the block's chain is
 // found by comparisons with parameters, and the extents, steps, divisors and keys
-// come from the constant bank instead of a binary search and some twenty dependent
-// loads per thread: 16 against 20 us per measured sweep of 16 chains of 4^4, 55 against
+// come from the constant bank instead of a lookup (by binary search, at that
+// time) and some twenty dependent loads per thread: 16 against 20 us per measured sweep of 16 chains of 4^4, 55 against
 // 61 for one 4 x 24^3 chain with overrelaxation; no difference where the launch is long
-// (4 x 32^4).  Larger batches look the chain up in memory.
+// (4 x 32^4).  Larger batches look the block's chain up in a table in memory.
 constexpr int kTableChains = 16;
 struct ChainTable {
     uint32_t start[kTableChains]; // first block of each chain (2^32 - 1 past the last)

@@ -165,12 +165,12 @@ __device__ __forceinline__ void mask8(uint32_t bits, uint4 &hi, uint4 &lo)
 // run of 36 bytes, fetched a tile ahead), and a lane takes its five neighbours of a
 // row as three words, shifted by half a word at odd positions and masked at the
 // lattice's edges.  After the MMA each thread reads its position's 32 accumulator
-// columns, adds the bias, applies ReLU; the BF16 rows go through shared memory, so
-// that a warp stores whole lines.  Several CTAs per SM overlap one another's MMA
-// waits; every wait is bounded and a timeout latches *err.  L = 64, 4096
-// configurations: 250 us against 436 when every tap was a byte load, a comparison and
-// two conversions and every lane stored its own 64-byte row; the 1.07 GB it writes
-// take 155.
+// columns, adds the bias, applies ReLU and stores its BF16 row (store32).  Several CTAs per SM overlap
+// one another's MMA waits; every wait on an mbarrier is bounded and a timeout latches *err (the tensor-memory
+// allocation has no limit: see chain_wait for why it ends).  L = 64, 4096
+// configurations: ~230 us against 436 when every tap was a byte load, a comparison and
+// two conversions and every lane stored its own row 16 bytes an instruction (250 with the rows
+// through shared memory into whole lines); the 1.07 GB it writes take 155.
 constexpr int kL1Threads = 128;
 constexpr uint32_t kL1Cols = 32;
 
@@ -3168,8 +3168,8 @@ mc_status mc_van_sample(mc_van *w, int32_t n, uint32_t round, const uint32_t *de
             k_sample_pipe<<<blocks, kPipeThreads, pipe_smem(w->D, w->L).total, w->stream>>>(
                 w->wh, w->w1, w->wD, w->bias, w->D, w->L, n, w->hist, out, lq, w->key, round, dev_ids, w->err);
         else
-        k_sample<<<blocks, kSampleThreads, sample_smem(w->D, w->L, nbuf), w->stream>>>(w->wh, w->w1, w->wD, w->bias, w->D, w->L, n,
-                                                                      nbuf, w->hist, w->zero, out, lq, w->key, round, dev_ids, w->err);
+            k_sample<<<blocks, kSampleThreads, sample_smem(w->D, w->L, nbuf), w->stream>>>(
+                w->wh, w->w1, w->wD, w->bias, w->D, w->L, n, nbuf, w->hist, w->zero, out, lq, w->key, round, dev_ids, w->err);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)
