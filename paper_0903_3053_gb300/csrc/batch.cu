@@ -604,10 +604,11 @@ mc_status mc_group_sweep(mc_group *g, int64_t n_sweeps, int32_t measure_every)
         size_t begun = 0;
         std::vector<mc_ctx *> order(g->members);
         std::stable_partition(order.begin(), order.end(), [](const mc_ctx *c) { return c->kind == MC_KIND_SU2; });
+        std::vector<int> mode(order.size(), MC_MODE_GRID);
         for (size_t i = 0; i < order.size() && st == MC_OK; ++i)
-            st = sweep_prepare(order[i]);
+            st = sweep_prepare(order[i], mode[i]);
         for (; begun < order.size() && st == MC_OK; ++begun)
-            st = sweep_begin(order[begun], n_sweeps, measure_every);
+            st = sweep_begin(order[begun], n_sweeps, measure_every, mode[begun]);
         for (size_t i = 0; i < begun; ++i) {
             const mc_status f = sweep_end(order[i]);
             if (st == MC_OK)

@@ -431,17 +431,17 @@ bool refuse_capture(cudaStream_t s)
     return true;
 }
 
-mc_status sweep_prepare(mc_ctx *c)
+mc_status sweep_prepare(mc_ctx *c, int &mode)
 {
-    if (resolve_mode(c) != MC_MODE_RESIDENT)
+    mode = resolve_mode(c);
+    if (mode != MC_MODE_RESIDENT)
         return MC_OK;
     const cudaError_t e = c->kind == MC_KIND_ISING ? ising_prepare_resident(c) : su2_prepare_resident(c);
     return e == cudaSuccess ? MC_OK : cuda_fail(e, "configure resident kernel");
 }
 
-mc_status sweep_begin(mc_ctx *c, long long n, int every)
+mc_status sweep_begin(mc_ctx *c, long long n, int every, int mode)
 {
-    const int mode = resolve_mode(c);
     cudaError_t e = cudaSuccess;
     if (!c->profiling) {
         e = cudaEventRecord(c->fence_in, c->stream);
@@ -692,10 +692,11 @@ mc_status mc_sweep(mc_ctx *c, int64_t n_sweeps, int32_t measure_every)
         return fail(MC_EINVAL, "sweep counter would exceed 2^32 (the Philox sweep word)");
     if (!c->profiling && refuse_capture(c->stream))
         return MC_ECUDA;
-    mc_status s = sweep_prepare(c);
+    int mode = MC_MODE_GRID;
+    mc_status s = sweep_prepare(c, mode);
     if (s != MC_OK)
         return s;
-    s = sweep_begin(c, n_sweeps, measure_every);
+    s = sweep_begin(c, n_sweeps, measure_every, mode);
     const mc_status f = sweep_end(c);
     return s != MC_OK ? s : f;
 }

@@ -259,12 +259,13 @@ cudaError_t su2_resident_enqueue(mc_ctx *c, long long n, int every);
 
 cudaError_t advance_state_launch(mc_ctx *c, long long n, long long recs);
 
-// A validated sweep call in three parts (capi.cu): what can be refused before anything is launched; everything enqueued
+// A validated sweep call in three parts (capi.cu): the mode, and what can be refused before anything is launched (once a
+// call: it looks at every chain, ~4 us for 4096); everything enqueued
 // on the context's private stream, ordered after the caller's work, the host's counters advanced with each chunk that
 // is launched; then the caller's stream made to wait for it.  A group prepares all its members first, and
 // starts all of them before the last part.
-mc_status sweep_prepare(mc_ctx *c);
-mc_status sweep_begin(mc_ctx *c, long long n, int every);
+mc_status sweep_prepare(mc_ctx *c, int &mode);
+mc_status sweep_begin(mc_ctx *c, long long n, int every, int mode);
 mc_status sweep_end(mc_ctx *c);
 
 // Whether `s` is being captured into a graph of the caller's (with the error message set).  A captured sweep would be
